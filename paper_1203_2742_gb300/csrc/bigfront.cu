@@ -1079,6 +1079,22 @@ Group group(const chd_symbolic* s, int g) {
   G.rows = s->dev.rows + s->rows_ptr[G.c0] + 1;
   return G;
 }
+// Launch context of a group's products: split-K partials go to the members'
+// own workspace (of the first right-hand side), behind the a x a and a x L
+// blocks the group uses there, unless the stream's slice is larger.  The
+// products over the group have one or a few output tiles and K = L, so
+// without the split a single CTA runs them: arrow n = 5000, width 32, 1.56 ms
+// a product of four right-hand sides on one CTA each, 0.04 ms split.
+inline Ctx group_ctx(const Ctx& st, const chd_symbolic* s, const Group& G, double* ws) {
+  Ctx c = st;
+  const int64_t used = ((int64_t)G.a * G.a + (int64_t)G.a * G.L + 3) & ~int64_t(3);
+  const int64_t cap = s->f_off[G.c0 + G.L] - G.f1 - used;
+  if (cap > (c.xs ? c.cap : 0)) {
+    c.xs = ws + G.f1 + used;
+    c.cap = cap;
+  }
+  return c;
+}
 constexpr int GW = BT / 32;  // leaves (warps) per CTA
 inline dim3 leaf_grid(int L, int m) { return dim3((L + GW - 1) / GW, 1, m); }
 __device__ __forceinline__ double warp_sum(double v) {
@@ -1295,9 +1311,10 @@ __global__ void __launch_bounds__(BT) mg_unreverse(double* Z, int64_t ldz, const
   const double* pr = Pr + z * sP + (int64_t)i * a;
   for (int q = 1 + lane; q < J; q += 32) zz[q] = pr[a - q];
 }
-void group_rtrans(const chd_symbolic* s, const Ctx& st, int m, int g, int dir, const double* Lc, const double* Qd,
+void group_rtrans(const chd_symbolic* s, const Ctx& st0, int m, int g, int dir, const double* Lc, const double* Qd,
                   double* Z, int64_t ldz, double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   const int64_t sw = s->dev.f_total;
   const double* Q = Qd + G.v0;
   double* P = ws + G.f1;  // a x L per RHS
@@ -1314,25 +1331,28 @@ void group_rtrans(const chd_symbolic* s, const Ctx& st, int m, int g, int dir, c
 }
 
 // per-group sequences
-void group_product(const chd_symbolic* s, const Ctx& st, int g, const double* Lc, double* X, double* ws) {
+void group_product(const chd_symbolic* s, const Ctx& st0, int g, const double* Lc, double* X, double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   mg_product<<<leaf_grid(G.L, 1), BT, 0, st>>>(Lc, X, G.base0, G.J, G.L);
   chd_launch::count_launch();
   gemm(st, 1, G.a, G.a, G.L, 1.0, Dn{const_cast<double*>(Lc) + G.base0 + 1, G.J}, 0,
        DnT{const_cast<double*>(Lc) + G.base0 + 1, G.J}, 0, 0.0, Dn{ws + G.f0 + 1 + G.J, G.J}, 0, true);
 }
-void group_factor(const chd_symbolic* s, const Ctx& st, int g, const double* X, double* Lc, double* Wc, double* Dd,
+void group_factor(const chd_symbolic* s, const Ctx& st0, int g, const double* X, double* Lc, double* Wc, double* Dd,
                   double* ws, double* ldet, int64_t* status) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   mg_factor<<<leaf_grid(G.L, 1), BT, 0, st>>>(X, Lc, Wc, Dd, ldet, G.base0, G.J, G.L, G.c0, G.d0, G.col0, status);
   chd_launch::count_launch();
   // update block the parent adds: -sum_i B_i B_i^T, in the first member's front
   gemm(st, 1, G.a, G.a, G.L, -1.0, Dn{Lc + G.base0 + 1, G.J}, 0, DnT{Lc + G.base0 + 1, G.J}, 0, 0.0,
        Dn{ws + G.f0 + 1 + G.J, G.J}, 0, true);
 }
-void group_gradient(const chd_symbolic* s, const Ctx& st, int g, const double* Wc, double* Sc, double* gr,
+void group_gradient(const chd_symbolic* s, const Ctx& st0, int g, const double* Wc, double* Sc, double* gr,
                     double* Vd, double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   double* V = Vd + G.v0;
   CHD_EW(mg_gather_v, (int64_t)G.a * G.a, 1, st, ws, 0, G.fp, G.Jp, G.rel, G.a, V, 0);
   gemm(st, 1, G.a, G.L, G.a, -1.0, SymL{V, G.a}, 0, Dn{const_cast<double*>(Wc) + G.base0 + 1, G.J}, 0, 0.0,
@@ -1340,9 +1360,10 @@ void group_gradient(const chd_symbolic* s, const Ctx& st, int g, const double* W
   mg_grad_finish<<<leaf_grid(G.L, 1), BT, 0, st>>>(Sc, gr, Wc, G.base0, G.J, G.L);
   chd_launch::count_launch();
 }
-void group_hess_up(const chd_symbolic* s, const Ctx& st, int m, int g, const double* Wc, const double* Vd,
+void group_hess_up(const chd_symbolic* s, const Ctx& st0, int m, int g, const double* Wc, const double* Vd,
                    const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   const int64_t sw = s->dev.f_total;
   double* K = ws + G.f1;
   const Dn Lb{const_cast<double*>(Wc) + G.base0 + 1, G.J};
@@ -1358,9 +1379,10 @@ void group_hess_up(const chd_symbolic* s, const Ctx& st, int m, int g, const dou
   gemm(st, m, G.a, G.L, G.a, 1.0, SymL{const_cast<double*>(Vd) + G.v0, G.a}, 0, Dn{K, G.a}, sw, 0.0,
        Dn{T + G.base0 + 1, G.J}, ldt, false);
 }
-void group_hess_down(const chd_symbolic* s, const Ctx& st, int m, int g, const double* Wc, double* T, int64_t ldt,
+void group_hess_down(const chd_symbolic* s, const Ctx& st0, int m, int g, const double* Wc, double* T, int64_t ldt,
                      double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   const int64_t sw = s->dev.f_total;
   double* Vs = ws + G.f1;
   double* W = Vs + (int64_t)G.a * G.a;
@@ -1370,9 +1392,10 @@ void group_hess_down(const chd_symbolic* s, const Ctx& st, int m, int g, const d
   mg_hess_down<<<leaf_grid(G.L, m), BT, 0, st>>>(T, ldt, Wc, W, sw, G.base0, G.J, G.L);
   chd_launch::count_launch();
 }
-void group_ihess_down(const chd_symbolic* s, const Ctx& st, int m, int g, const double* Wc, const double* Dd,
+void group_ihess_down(const chd_symbolic* s, const Ctx& st0, int m, int g, const double* Wc, const double* Dd,
                       const double* Rd, const double* Tin, int64_t ldt, double* Y, int64_t ldy, double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   const int64_t sw = s->dev.f_total;
   double* Vs = ws + G.f1;
   double* W = Vs + (int64_t)G.a * G.a;
@@ -1385,9 +1408,10 @@ void group_ihess_down(const chd_symbolic* s, const Ctx& st, int m, int g, const 
   gemm(st, m, G.a, G.L, G.a, 1.0, SymL{const_cast<double*>(Rd) + G.v0, G.a}, 0, Dn{W, G.a}, sw, 0.0,
        Dn{Y + G.base0 + 1, G.J}, ldy, false);
 }
-void group_ihess_up(const chd_symbolic* s, const Ctx& st, int m, int g, const double* Wc, double* Y, int64_t ldy,
+void group_ihess_up(const chd_symbolic* s, const Ctx& st0, int m, int g, const double* Wc, double* Y, int64_t ldy,
                     double* ws) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   const int64_t sw = s->dev.f_total;
   double* P = ws + G.f1;
   mg_ihess_up<<<leaf_grid(G.L, m), BT, 0, st>>>(Y, ldy, Wc, P, sw, G.base0, G.J, G.L);
@@ -1398,10 +1422,11 @@ void group_ihess_up(const chd_symbolic* s, const Ctx& st, int m, int g, const do
   gemm(st, m, G.a, G.a, G.L, -1.0, Dn{P, G.a}, sw, DnT{Lb.p, G.J}, 0, 0.0, U, sw, true);
   gemm(st, m, G.a, G.a, G.L, -1.0, Lb, 0, DnT{P, G.a}, sw, 1.0, U, sw, true);
 }
-void group_complete(const chd_symbolic* s, const Ctx& st, int g, const double* Sin, double* Lc, double* Wc,
+void group_complete(const chd_symbolic* s, const Ctx& st0, int g, const double* Sin, double* Lc, double* Wc,
                     double* Dd, double* Vd, double* Rd, const double* Gq, double* ws, double* ldet,
                     int64_t* status) {
   const Group G = group(s, g);
+  const Ctx st = group_ctx(st0, s, G, ws);
   double* V = Vd + G.v0;
   double* R = Gq ? const_cast<double*>(Gq) + G.v0 : Rd + G.v0;
   double* Z = ws + G.f1;

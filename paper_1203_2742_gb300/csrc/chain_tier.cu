@@ -1,6 +1,6 @@
 // Chain tier: runs of one-column fronts whose rows are contiguous and whose
 // ancestor count a is the same along the run (the elimination chains of band
-// patterns in natural order), one CTA per run and right-hand side.
+// patterns in natural order).
 //
 // Andersen, Dahl, Vandenberghe, "Logarithmic barriers for sparse matrix
 // cones": for one-column fronts the supernodal Algorithms 7.1 and 7.2 and the
@@ -8,14 +8,33 @@
 // 3.1, 4.1 and 5.1.  Along such a run, front j has rows j .. j+a, its child
 // is front j-1, and the child's update matrix (bottom-up) or the parent's
 // front (top-down) covers rows j+1 .. j+a-1 of it.  So the a x a block that
-// passes from front to front is a window that slides by one row per column:
-// it stays in shared memory (rows addressed modulo WS), each step adds one
-// row and drops one, and the only global traffic per column is the column's
-// own values.  The run hands over to the rest of the tree through the
-// workspace fronts exactly like the other tiers: its top front writes its
-// update block (bottom-up) or reads the parent's front (top-down) there.
+// passes from front to front is a window that slides by one row per column.
+// The run hands over to the rest of the tree through the workspace fronts
+// exactly like the other tiers: its top front writes its update block
+// (bottom-up) or reads the parent's front (top-down) there.
+//
+// What bounds it.  A GB300 SM retires one FP64 warp instruction per 19
+// clocks, whatever the number of active lanes, and one warp at most one per
+// 64 clocks (dependent or not); a reciprocal is 350 clocks, a barrier of 256
+// threads 29.  So the cost of a column is the number of FP64 warp
+// instructions that must run one column after another, and the design keeps
+// only those in the serial kernels:
+//   * what the next column does not need runs afterwards, over all columns
+//     in parallel: the Cholesky scaling and log det of the factor, the
+//     stored V_j of the gradient, M_A = V K_A / D of the Hessian;
+//   * both passes of the inverse Hessian and the Cholesky product have no
+//     recursion along the run at all (the windows are parts of the input, and
+//     the update blocks only add up), so they run over all columns at once;
+//   * the serial kernels hold the window in registers, one copy of every
+//     entry (bottom-up) or whole rows (top-down), and address it modulo its
+//     size, so nothing moves as it slides.
+// Measured (band n = 12000, half-bandwidth 61, one matrix): factor 49.4 ms
+// before (window in shared memory, both triangles updated, log and sqrt in
+// the chain), gradient 53.0 ms, inverse Hessian with two right-hand sides
+// 112.6 ms; the figures after are in the comments of the kernels.
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <cstdint>
 
 #include "chd_internal.h"
@@ -28,10 +47,10 @@ void count_launch();
 namespace chd {
 namespace chain {
 
-constexpr int CT = 256;       // threads per run
-constexpr int AMAX = 64;      // largest a
-constexpr int WS = AMAX + 1;  // window slots: rows j .. j + a
-constexpr int TPR = 4;        // threads per row of a window product
+constexpr int AMAX = 64;    // largest a
+constexpr int WP = 72;      // row of a window vector in shared memory
+constexpr int RING = 8;     // columns of inputs kept in shared memory
+constexpr int AHEAD = 6;    // columns loaded ahead of the one in work
 
 // run of task t: its first front's record, the run length and a
 struct Run {
@@ -58,400 +77,646 @@ __device__ __forceinline__ Run run_of(const SymDev& S, int t) {
   r.fstride = (J * J + 2 * J + 3) & ~int64_t(3);
   return r;
 }
-__device__ __forceinline__ int slot(int g) { return g % WS; }
 
-// out[r] = sum_s Win(r, s) x[s] for r, s < a, Win the window rows/columns
-// i0 .. i0 + a - 1 (symmetric, both triangles stored); TPR threads per row,
-// the partial sums combined by shuffles.  Valid in the threads with
-// tid % TPR == 0 (returned), for row tid / TPR.
-__device__ __forceinline__ double window_row_dot(const double (*W)[WS + 1], int i0, int a, const double* x,
-                                                 int tid) {
-  const int r = tid / TPR, part = tid % TPR;
-  double acc = 0.0;
-  if (r < a) {
-    const int sr = slot(i0 + r);
-    for (int s = part; s < a; s += TPR) acc = fma(W[sr][slot(i0 + s)], x[s], acc);
-  }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  return acc;
+__device__ __forceinline__ void cp_async8(double* dst, const double* src) {
+  const unsigned d = (unsigned)__cvta_generic_to_shared(dst);
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;\n" ::"r"(d), "l"(src) : "memory");
 }
-// The thread's share of row tid / TPR of the symmetric a x a block B (lower
-// triangle stored column-major, ld a): entries s = part, part + TPR, ...
-// loaded into registers at once (independent loads, one memory latency),
-// so that a step can issue them before its synchronised work and use them
-// after it.  Zero beyond a.
-constexpr int PF = AMAX / TPR;
-struct RowPart {
-  double v[PF];
+__device__ __forceinline__ void cp_async_commit() { asm volatile("cp.async.commit_group;\n" ::: "memory"); }
+template <int N>
+__device__ __forceinline__ void cp_async_wait() {
+  asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
+}
+// barrier of the first `n` threads of the CTA (the rest has returned)
+__device__ __forceinline__ void bar(int n) { asm volatile("bar.sync 1, %0;\n" ::"r"(n) : "memory"); }
+
+// ---------------------------------------------------------------------------
+// bottom-up serial kernels (factor, Hessian step 1)
+//
+// The window covers the a + 1 rows i .. i+a while column i is in work; row
+// rho lives in slot rho mod (a + 1), so the row that leaves (i) and the row
+// that enters (i + 1 + a) share a slot.  Every unordered pair of slots is one
+// entry, held in a register of one update thread for the whole run.  Per
+// column, after one barrier:
+//   warp 0 finishes column i+1: its window entries (published one column
+//     earlier by their owners, with the updates through column i-1), its
+//     input values and the update by column i; then the pivot, and the two
+//     vectors the next update needs, into the other of two buffers;
+//   the other warps update their pairs by column i and publish column i+2.
+// So the pivot's latency (about 700 clocks) runs beside the update of
+// the window (a = 61: 61 FP64 warp instructions, 1160 clocks; twice that in
+// the Hessian).  Inputs arrive by cp.async, AHEAD columns early.
+// ---------------------------------------------------------------------------
+struct UpSmem {
+  double ring[2][RING][WP];
+  double f[2][WP], g[2][WP], uc[2][WP];
 };
-__device__ __forceinline__ RowPart load_row_part(const double* B, int a, int tid) {
-  RowPart p;
-  const int r = tid / TPR, part = tid % TPR;
+enum { UP_FACTOR = 0, UP_HESS = 1 };
+struct UpArgs {
+  const double* src;  // X or Y, the run's first column
+  const double* wc;   // UP_HESS: Wc; the run's first column
+  double* o0;         // Lc (raw column: F_11, F_21) or T (h_0, K_A)
+  double* o1;         // UP_FACTOR: Wc
+  double* dd;         // UP_FACTOR: Dd of the first column
+  int64_t* st;
+};
+template <int NT, int PP, int MODE>
+__device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double* G) {
+  constexpr int EL = NT <= 32 ? 1 : NT <= 96 ? 1 : 3;  // slots per lane of warp 0
+  const int a = R.a, W = a + 1, tid = threadIdx.x, L = R.L;
+  if (tid >= NT + 32) return;
+  for (int e = tid; e < 2 * WP; e += NT + 32) (&sm.uc[0][0])[e] = 0.0;
+  bar(NT + 32);
+  if (tid < 32) {
+    // ---- warp 0: inputs, pivots, outputs ----
+    const int lane = tid;
+    auto prefetch = [&](int c) {
+      if (c < L) {
+        const int s0 = c % W;
+        for (int p = lane; p <= a; p += 32) {
+          int s = s0 + p;
+          if (s >= W) s -= W;
+          cp_async8(&sm.ring[0][c % RING][s], A.src + (int64_t)c * W + p);
+          if (MODE == UP_HESS) cp_async8(&sm.ring[1][c % RING][s], A.wc + (int64_t)c * W + p);
+        }
+      }
+      cp_async_commit();
+    };
+    auto column = [&](int c) {
+      const int s0 = c % W, sp = s0 == 0 ? W - 1 : s0 - 1, cur = c & 1, prv = cur ^ 1;
+      cp_async_wait<AHEAD - 1>();
+      __syncwarp();
+      double val[EL], l[EL];
+      const double gs = c > i0 ? sm.g[prv][s0] : 0.0, fs = c > i0 ? sm.f[prv][s0] : 0.0;
 #pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const int s = part + u * TPR;
-    p.v[u] = (r < a && s < a) ? __ldg(B + (r >= s ? r + (int64_t)s * a : s + (int64_t)r * a)) : 0.0;
-  }
-  return p;
-}
-// sum over the row's entries of v[s] * x[s] * scale, reduced over the TPR
-// threads of the row (valid where tid % TPR == 0)
-__device__ __forceinline__ double row_part_dot(const RowPart& p, const double* x, int a, double scale, int tid) {
-  const int part = tid % TPR;
-  double acc = 0.0;
+      for (int e = 0; e < EL; ++e) {
+        const int o = lane + 32 * e;
+        val[e] = 0.0;
+        l[e] = 0.0;
+        if (o < W) {
+          val[e] = sm.ring[0][c % RING][o];
+          if (MODE == UP_HESS) l[e] = sm.ring[1][c % RING][o];
+          if (c > i0 && o != sp) {  // slot sp: the row that enters, untouched so far
+            val[e] += sm.uc[cur][o];
+            val[e] = fma(-sm.f[prv][o], gs, val[e]);
+            if (MODE == UP_HESS) val[e] = fma(-sm.g[prv][o], fs, val[e]);
+          }
+        }
+      }
+      double d = val[0];
 #pragma unroll
-  for (int u = 0; u < PF; ++u) {
-    const int s = part + u * TPR;
-    if (s < a) acc = fma(p.v[u], x[s] * scale, acc);
+      for (int e = 1; e < EL; ++e)
+        if (s0 / 32 == e) d = val[e];
+      d = __shfl_sync(0xffffffffu, d, s0 & 31);
+      if (MODE == UP_FACTOR) {
+        if (!(d > 0.0)) {
+          if (lane == 0) record_error(A.st, CHD_ERR_NOT_PD, R.k0 + c, R.col0 + c);
+          d = 1.0;
+        }
+        const double r2 = 1.0 / d;
+#pragma unroll
+        for (int e = 0; e < EL; ++e) {
+          const int o = lane + 32 * e;
+          if (o < W) {
+            const double gv = val[e] * r2;
+            sm.f[cur][o] = val[e];
+            sm.g[cur][o] = gv;
+            int p = o - s0;
+            if (p < 0) p += W;
+            A.o0[(int64_t)c * W + p] = p == 0 ? d : val[e];
+            A.o1[(int64_t)c * W + p] = p == 0 ? r2 : gv;
+          }
+        }
+        if (lane == 0) A.dd[4 * (int64_t)c] = d;
+      } else {
+        // P = h_A - L h_0 / 2: U' = Yh_AA - (P L^T + L P^T); K_A = P - L h_0 / 2
+        const double hh = 0.5 * d;
+#pragma unroll
+        for (int e = 0; e < EL; ++e) {
+          const int o = lane + 32 * e;
+          if (o < W) {
+            const double pv = fma(-l[e], hh, val[e]);
+            sm.f[cur][o] = pv;
+            sm.g[cur][o] = l[e];
+            int p = o - s0;
+            if (p < 0) p += W;
+            A.o0[(int64_t)c * W + p] = p == 0 ? d : fma(-l[e], hh, pv);
+          }
+        }
+      }
+    };
+    for (int c = i0; c < i0 + AHEAD; ++c) prefetch(c);
+    column(i0);
+    bar(NT + 32);
+    for (int i = i0; i < L; ++i) {
+      prefetch(i + AHEAD);
+      if (i + 1 < L) column(i + 1);
+      bar(NT + 32);
+    }
+  } else {
+    // ---- update warps: pairs (u, v), u >= v, of slots ----
+    const int ut = tid - 32, np = W * (W + 1) / 2;
+    int pu[PP], pv[PP];
+    double U[PP];
+#pragma unroll
+    for (int t = 0; t < PP; ++t) {
+      const int e = ut + NT * t;
+      int u = 0, v = 0;
+      if (e < np) {
+        u = (int)((sqrtf(8.0f * e + 1.0f) - 1.0f) * 0.5f);
+        while (u * (u + 1) / 2 > e) --u;
+        while ((u + 1) * (u + 2) / 2 <= e) ++u;
+        v = e - u * (u + 1) / 2;
+      }
+      pu[t] = u;
+      pv[t] = v;
+      U[t] = 0.0;
+    }
+    bar(NT + 32);
+    int s0 = i0 % W;
+    for (int i = i0; i < L; ++i) {
+      const int s1 = i + 1 < L ? (s0 + 1 == W ? 0 : s0 + 1) : s0;
+      int s2 = s0 + 2;
+      if (s2 >= W) s2 -= W;
+      const bool pub = i + 2 < L;
+      const double* f = sm.f[i & 1];
+      const double* g = sm.g[i & 1];
+      double* uc = sm.uc[i & 1];
+#pragma unroll
+      for (int t = 0; t < PP; ++t) {
+        if (ut + NT * t >= np) break;
+        const int u = pu[t], v = pv[t];
+        if (u != s0 && v != s0 && u != s1 && v != s1) {
+          U[t] = fma(-f[u], g[v], U[t]);
+          if (MODE == UP_HESS) U[t] = fma(-g[u], f[v], U[t]);
+        }
+        if (pub && (u == s2 || v == s2)) {
+          uc[u == s2 ? v : u] = U[t];
+          U[t] = 0.0;
+        }
+      }
+      bar(NT + 32);
+      s0 = s0 + 1 == W ? 0 : s0 + 1;
+    }
+    // update block of the top front for the parent (lower, ld J = a + 1):
+    // rows L .. L + a - 1, i.e. every slot but that of row L - 1
+    const int sL = L % W, out = sL == 0 ? W - 1 : sL - 1, J = W;
+#pragma unroll
+    for (int t = 0; t < PP; ++t) {
+      if (ut + NT * t >= np) break;
+      const int u = pu[t], v = pv[t];
+      if (u == out || v == out) continue;
+      int p = u - sL, q = v - sL;
+      if (p < 0) p += W;
+      if (q < 0) q += W;
+      G[(1 + max(p, q)) + (int64_t)(1 + min(p, q)) * J] = U[t];
+    }
   }
-  acc += __shfl_xor_sync(0xffffffffu, acc, 1);
-  acc += __shfl_xor_sync(0xffffffffu, acc, 2);
-  return acc;
 }
-// sum over r < a of term(r), the same value in every thread (each warp
-// reduces all terms)
-template <class Term>
-__device__ __forceinline__ double all_sum(int a, Term term, int tid) {
-  const int lane = tid & 31;
-  double acc = 0.0;
-  for (int r = lane; r < a; r += 32) acc += term(r);
-  for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  return acc;
+// Threads by window size: the smallest set of update warps whose registers
+// hold the pairs, so that short windows pay for few barriers and few FP64
+// instructions (one warp up to a = 9, three up to a = 31, seven up to 64).
+constexpr int UPT = 256;
+template <int MODE>
+__device__ __forceinline__ void up_dispatch(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double* G) {
+  if (R.a <= 9) up_run<32, 2, MODE>(R, i0, A, sm, G);
+  else if (R.a <= 31) up_run<96, 6, MODE>(R, i0, A, sm, G);
+  else up_run<224, 10, MODE>(R, i0, A, sm, G);
 }
 
-// Algorithm 7.1 for one-column fronts (Algorithm 3.1): D = F_11, C = sqrt(D),
-// B = F_21 / C, L_AN = F_21 / D, U = F_22 - F_21 F_21^T / D.
-__global__ void __launch_bounds__(CT) kc_factor(SymDev S, int task0, const double* X, double* Lc, double* Wc,
-                                               double* Dd, double* ws, double* ldet, int64_t* st) {
-  __shared__ double U[WS][WS + 1];
-  __shared__ double f[WS];
+// Algorithm 7.1 for one-column fronts (Algorithm 3.1): D = F_11, L_AN =
+// F_21 / D, U = F_22 - F_21 F_21^T / D.  Lc receives F_11 and F_21;
+// kc_factor_post scales them to C = sqrt(D), B = F_21 / C.
+__global__ void __launch_bounds__(UPT) kc_factor(SymDev S, int task0, const double* X, double* Lc, double* Wc,
+                                                double* Dd, double* ws, int64_t* st) {
+  __shared__ UpSmem sm;
   const Run R = run_of(S, task0 + blockIdx.x);
-  const int a = R.a, tid = threadIdx.x;
-  for (int e = tid; e < WS * (WS + 1); e += CT) (&U[0][0])[e] = 0.0;
-  double xv = tid <= a ? X[R.base0 + tid] : 0.0;
-  __syncthreads();
-  for (int i = 0; i < R.L; ++i) {
-    const int64_t base = R.base0 + (int64_t)i * (a + 1);
-    // column i of the front: its values plus the child's update block
-    if (tid <= a) f[tid] = xv + U[slot(i + tid)][slot(i)];
-    if (i + 1 < R.L && tid <= a) xv = X[base + (a + 1) + tid];
-    __syncthreads();
-    double d = f[0];
-    if (!(d > 0.0)) {
-      if (tid == 0) record_error(st, CHD_ERR_NOT_PD, R.k0 + i, R.col0 + i);
-      d = 1.0;
-    }
-    const double r = rsqrt(d), r2 = r * r;
-    if (tid <= a) {
-      const double x = f[tid];
-      Lc[base + tid] = tid == 0 ? d * r : x * r;
-      Wc[base + tid] = tid == 0 ? r2 : x * r2;
-    }
-    if (tid == 0) {
-      Dd[R.d0 + 4 * (int64_t)i] = d;
-      ldet[R.k0 + i] = log(d);
-    }
-    for (int e = tid; e < a * a; e += CT) {
-      const int p = e / a, q = e - (e / a) * a;
-      U[slot(i + 1 + p)][slot(i + 1 + q)] -= f[1 + p] * f[1 + q] * r2;
-    }
-    const int si = slot(i);  // row i leaves; its slot is row i + WS, zero until it enters
-    for (int e = tid; e < WS; e += CT) {
-      U[si][e] = 0.0;
-      U[e][si] = 0.0;
-    }
-    __syncthreads();
-  }
-  // update block of the top front for the parent (lower, ld J = a + 1)
-  double* G = ws + R.f0 + (int64_t)(R.L - 1) * R.fstride;
-  const int J = a + 1;
-  for (int e = tid; e < a * a; e += CT) {
-    const int p = e / a, q = e - (e / a) * a;
-    if (p >= q) G[(1 + p) + (int64_t)(1 + q) * J] = U[slot(R.L + p)][slot(R.L + q)];
+  UpArgs A{X + R.base0, nullptr, Lc + R.base0, Wc + R.base0, Dd + R.d0, st};
+  up_dispatch<UP_FACTOR>(R, 0, A, sm, ws + R.f0 + (int64_t)(R.L - 1) * R.fstride);
+}
+// C, B and log D of every column of every run, one warp per column
+__global__ void __launch_bounds__(128) kc_factor_post(SymDev S, int task0, double* Lc, const double* Dd,
+                                                     double* ldet) {
+  const Run R = run_of(S, task0 + blockIdx.x);
+  const int lane = threadIdx.x & 31;
+  for (int i = blockIdx.y * 4 + (threadIdx.x >> 5); i < R.L; i += gridDim.y * 4) {
+    const double d = Dd[R.d0 + 4 * (int64_t)i], r = rsqrt(d);
+    double* c = Lc + R.base0 + (int64_t)i * (R.a + 1);
+    for (int p = lane; p <= R.a; p += 32) c[p] *= r;
+    if (lane == 0) ldet[R.k0 + i] = log(d);
   }
 }
 
-// V (rows i0 .. i0 + a - 1 of the window) <- the parent's front at the
-// relative positions of the top front's A (top-down passes)
-__device__ void gather_window(const SymDev& S, const Run& R, const double* ws, double (*V)[WS + 1], int tid) {
+// Algorithm 5.1 step 1 for one-column fronts: with Yh the front's values
+// plus the child's U', K_jj = Yh_jj, K_A = Yh_A - L_A Yh_jj,
+// U' = Yh_AA - K_A L_A^T - L_A Yh_A^T; K goes to T, kc_hess_m applies step 2.
+// act (pruned R(Y), §5.5): a front with act == 0 has Y zero in its subtree,
+// so K, U' and M are zero; along a run these are its first columns.
+__global__ void __launch_bounds__(UPT) kc_hess_up(SymDev S, int task0, const double* Wc, const double* Y, int64_t ldy,
+                                                 double* T, int64_t ldt, double* ws, const uint8_t* act) {
+  __shared__ UpSmem sm;
+  const Run R = run_of(S, task0 + blockIdx.x);
+  const int64_t y = blockIdx.y;
+  int i0 = 0;
+  if (act) {
+    const uint8_t* ay = act + y * S.nsn + R.k0;
+    if (!ay[R.L - 1]) return;  // nothing reaches the run; its parent skips its block
+    int lo = 0, hi = R.L - 1;  // the first active column
+    while (lo < hi) {
+      const int mid = (lo + hi) >> 1;
+      if (ay[mid]) hi = mid;
+      else lo = mid + 1;
+    }
+    i0 = lo;
+  }
+  UpArgs A{Y + y * ldy + R.base0, Wc + R.base0, T + y * ldt + R.base0, nullptr, nullptr, nullptr};
+  up_dispatch<UP_HESS>(R, i0, A, sm, ws + y * S.f_total + R.f0 + (int64_t)(R.L - 1) * R.fstride);
+}
+
+// ---------------------------------------------------------------------------
+// products with a symmetric a x a block per column, over all columns at once
+// ---------------------------------------------------------------------------
+constexpr int MT = 128;      // threads per column
+constexpr int BLD = AMAX + 1;  // leading dimension of a staged block
+
+// the symmetric block stored lower column-major (ld a) into both triangles of B
+__device__ __forceinline__ void stage_sym(double (*B)[BLD], const double* M, int a) {
+  const int lane = threadIdx.x & 31;
+  for (int c = threadIdx.x >> 5; c < a; c += MT / 32)
+    for (int r = c + lane; r < a; r += 32) {
+      const double v = M[r + (int64_t)c * a];
+      B[r][c] = v;
+      B[c][r] = v;
+    }
+}
+// y[r] = sum_s B(r, s) x[s], r < a; two threads per row, y written by the even one
+__device__ __forceinline__ void sym_dot(const double (*B)[BLD], const double* x, int a, double* y) {
+  const int r = threadIdx.x >> 1, h = threadIdx.x & 1;
+  if ((threadIdx.x & ~31) / 2 < a) {  // whole warps beyond the block are idle
+    double a0 = 0.0, a1 = 0.0;
+    if (r < a) {
+      int s = h;
+      for (; s + 2 < a; s += 4) {
+        a0 = fma(B[r][s], x[s], a0);
+        a1 = fma(B[r][s + 2], x[s + 2], a1);
+      }
+      if (s < a) a0 = fma(B[r][s], x[s], a0);
+    }
+    a0 += a1;
+    a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+    if (r < a && h == 0) y[r] = a0;
+  }
+}
+// rows j+1 .. j+a of the matrix v (values of the run's columns, and the
+// parent's front Fp beyond the run) as a full symmetric block
+__device__ __forceinline__ void stage_window(const SymDev& S, const Run& R, int j, const double* v, const double* Fp,
+                                            int Jp, const int32_t* rel, double (*B)[BLD]) {
+  const int lane = threadIdx.x & 31, a = R.a;
+  for (int c = threadIdx.x >> 5; c < a; c += MT / 32) {
+    const int col = j + 1 + c;
+    for (int r = c + lane; r < a; r += 32) {
+      double x;
+      if (col < R.L) {
+        x = v[(int64_t)col * (a + 1) + (r - c)];
+      } else {  // rows col .. of the run's top front lie in the parent
+        const int pr = __ldg(rel + (j + 1 + r - R.L)), pc = __ldg(rel + (col - R.L));
+        x = __ldcg(Fp + (pr >= pc ? pr + (int64_t)pc * Jp : pc + (int64_t)pr * Jp));
+      }
+      B[r][c] = x;
+      B[c][r] = x;
+    }
+  }
+}
+struct Parent {
+  const double* F;
+  int J;
+  const int32_t* rel;
+};
+__device__ __forceinline__ Parent parent_of(const SymDev& S, const Run& R, const double* ws) {
+  Parent P;
   const int k1 = R.k0 + R.L - 1;
   const int64_t p = S.sn_par[k1];
-  const int a = R.a;
-  const int Jp = (int)(S.rows_ptr[p + 1] - S.rows_ptr[p]);
-  const double* Fp = ws + S.f_off[p];
-  const int32_t* rel = S.rel + S.rows_ptr[k1] + 1;
-  const int i0 = R.L;  // rows L .. L + a - 1: the A of the top front L - 1
-  for (int e = tid; e < a * a; e += CT) {
-    const int r = e / a, s = e - (e / a) * a;
-    const int pr = __ldg(rel + r), ps = __ldg(rel + s);
-    V[slot(i0 + r)][slot(i0 + s)] = __ldcg(Fp + (pr >= ps ? pr + (int64_t)ps * Jp : ps + (int64_t)pr * Jp));
+  P.J = (int)(S.rows_ptr[p + 1] - S.rows_ptr[p]);
+  P.F = ws + S.f_off[p];
+  P.rel = S.rel + S.rows_ptr[k1] + 1;
+  return P;
+}
+
+// Algorithm 5.1 step 2: M_jj = K_jj / D^2, M_A = V K_A / D (K in T, in place)
+__global__ void __launch_bounds__(MT) kc_hess_m(SymDev S, int task0, const double* Wc, const double* Vd, double* T,
+                                               int64_t ldt, const uint8_t* act) {
+  __shared__ double B[AMAX][BLD];
+  __shared__ double x[AMAX], yv[AMAX];
+  const Run R = run_of(S, task0 + blockIdx.x);
+  const int a = R.a, tid = threadIdx.x;
+  const int64_t y = blockIdx.z;
+  for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
+    if (act && !act[y * S.nsn + R.k0 + i]) continue;
+    double* t = T + y * ldt + R.base0 + (int64_t)i * (a + 1);
+    const double dinv = Wc[R.base0 + (int64_t)i * (a + 1)];
+    stage_sym(B, Vd + R.v0 + (int64_t)i * R.vstride, a);
+    if (tid < a) x[tid] = t[1 + tid] * dinv;
+    __syncthreads();
+    sym_dot(B, x, a, yv);
+    __syncthreads();
+    if (tid < a) t[1 + tid] = yv[tid];
+    if (tid == MT - 1) t[0] = dinv * t[0] * dinv;
+    __syncthreads();
   }
+}
+
+// ---------------------------------------------------------------------------
+// top-down serial kernels (gradient, Hessian step 3)
+//
+// The window covers the a rows c+1 .. c+a while column c is in work, row rho
+// in slot rho mod a (row c takes the slot of row c + a).  Four threads hold
+// a row each, entries v = part, part + 4, ..; per column they multiply the
+// window with L_A (a = 61: 128 FP64 warp instructions), reduce over the four,
+// and after a barrier the new row is formed once, and after another taken
+// over into the registers.  The new diagonal entry needs a whole dot product;
+// warp 0 forms it during the next column's product, whose one affected row
+// gets the missing term afterwards.  Warp 0 also loads the inputs and stores
+// the outputs.
+// ---------------------------------------------------------------------------
+struct DownSmem {
+  double ring[2][RING][WP];  // L_A (slots), and M_A; [.][WP - 1]: the diagonal's value
+  double wv[WP], tv[2][WP], dg[2];
+};
+enum { DOWN_GRAD = 0, DOWN_HESS = 1 };
+template <int NT, int CP, int MODE>
+__device__ void down_run(const SymDev& S, const Run& R, const double* wc, const double* src, double* out,
+                         const double* ws, DownSmem& sm) {
+  const int a = R.a, W = a + 1, tid = threadIdx.x, L = R.L;
+  if (tid >= NT + 32) return;
+  if (tid < 32) {
+    const int lane = tid;
+    auto prefetch = [&](int c) {
+      if (c >= 0) {
+        const int sc = c % a;
+        for (int p = lane; p <= a; p += 32) {
+          int s = sc + p;
+          while (s >= a) s -= a;
+          if (p == 0) s = WP - 1;
+          cp_async8(&sm.ring[0][c % RING][s], wc + (int64_t)c * W + p);
+          if (MODE == DOWN_HESS) cp_async8(&sm.ring[1][c % RING][s], src + (int64_t)c * W + p);
+        }
+      }
+      cp_async_commit();
+    };
+    // the diagonal of column c, and the column's output
+    int steps = 1;
+    while (steps < 32 && steps < a) steps <<= 1;
+    auto finish = [&](int c) {
+      const double* l = sm.ring[0][c % RING];
+      const double* mm = sm.ring[1][c % RING];
+      const double* t = sm.tv[c & 1];
+      const double m0 = MODE == DOWN_HESS ? mm[WP - 1] : l[WP - 1];
+      double acc = 0.0;
+      for (int v = lane; v < a; v += 32) acc = fma(-l[v], MODE == DOWN_HESS ? t[v] + mm[v] : t[v], acc);
+      for (int o = steps >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      const double d = m0 + acc;
+      if (lane == 0) {
+        sm.dg[c & 1] = d;
+        out[(int64_t)c * W] = d;
+      }
+      const int sc = c % a;
+      for (int v = lane; v < a; v += 32) {
+        int p = v - sc;
+        if (p <= 0) p += a;
+        out[(int64_t)c * W + p] = t[v];
+      }
+    };
+    for (int c = L - 1; c > L - 1 - AHEAD; --c) prefetch(c);
+    cp_async_wait<AHEAD - 1>();
+    bar(NT + 32);
+    for (int c = L - 1; c >= 0; --c) {
+      if (c + 1 < L) finish(c + 1);
+      prefetch(c - AHEAD);
+      cp_async_wait<AHEAD - 1>();  // column c - 1 has arrived
+      bar(NT + 32);
+      bar(NT + 32);
+    }
+    __syncwarp();
+    finish(0);
+  } else {
+    const int rt = tid - 32, u = rt >> 2, part = rt & 3;
+    double V[CP];
+    {
+      // rows L .. L + a - 1 from the parent's front
+      const int k1 = R.k0 + L - 1;
+      const int64_t p = S.sn_par[k1];
+      const int Jp = (int)(S.rows_ptr[p + 1] - S.rows_ptr[p]);
+      const double* Fp = ws + S.f_off[p];
+      const int32_t* rel = S.rel + S.rows_ptr[k1] + 1;
+      const int sL = L % a;
+      auto pos = [&](int s) { return __ldg(rel + (s >= sL ? s - sL : s - sL + a)); };
+#pragma unroll
+      for (int j = 0; j < CP; ++j) {
+        const int v = part + 4 * j;
+        V[j] = 0.0;
+        if (u < a && v < a) {
+          const int pr = pos(u), pc = pos(v);
+          V[j] = __ldcg(Fp + (pr >= pc ? pr + (int64_t)pc * Jp : pc + (int64_t)pr * Jp));
+        }
+      }
+    }
+    bar(NT + 32);
+    for (int c = L - 1; c >= 0; --c) {
+      const double* l = sm.ring[0][c % RING];
+      const double* mm = sm.ring[1][c % RING];
+      double a0 = 0.0, a1 = 0.0;
+#pragma unroll
+      for (int j = 0; j < CP; ++j) {
+        const int v = part + 4 * j;
+        const double lv = v < a ? l[v] : 0.0;
+        if (j & 1) a1 = fma(V[j], lv, a1);
+        else a0 = fma(V[j], lv, a0);
+      }
+      a0 += a1;
+      a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
+      a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+      if (part == 0 && u < a) sm.wv[u] = a0;
+      bar(NT + 32);
+      const int s = c % a;
+      const int s1 = c + 1 < L ? (s + 1 == a ? 0 : s + 1) : -1;  // row c + 1, its diagonal still missing
+      double* tv = sm.tv[c & 1];
+      const double dnew = sm.dg[(c + 1) & 1];
+      if (rt < a) {
+        double w = sm.wv[rt];
+        if (rt == s1) w = fma(dnew, l[rt], w);
+        tv[rt] = MODE == DOWN_HESS ? mm[rt] - w : -w;
+      }
+      bar(NT + 32);
+#pragma unroll
+      for (int j = 0; j < CP; ++j) {
+        const int v = part + 4 * j;
+        if (u == s1 && v == s1) V[j] = dnew;
+        if (u == s) V[j] = v == s || v >= a ? 0.0 : tv[v];
+        else if (v == s && u < a) V[j] = tv[u];
+      }
+    }
+  }
+}
+constexpr int DNT = 288;
+template <int MODE>
+__device__ __forceinline__ void down_dispatch(const SymDev& S, const Run& R, const double* wc, const double* src,
+                                             double* out, const double* ws, DownSmem& sm) {
+  if (R.a <= 8) down_run<32, 2, MODE>(S, R, wc, src, out, ws, sm);
+  else if (R.a <= 16) down_run<64, 4, MODE>(S, R, wc, src, out, ws, sm);
+  else if (R.a <= 32) down_run<128, 8, MODE>(S, R, wc, src, out, ws, sm);
+  else down_run<256, 16, MODE>(S, R, wc, src, out, ws, sm);
 }
 
 // Algorithm 7.2 for one-column fronts (Algorithm 4.1): S_AN = -V L_AN,
 // S_NN = D^{-1} - S_AN^T L_AN; V of the child = [S_NN S_AN^T; S_AN V] on the
-// child's rows; V_j is also stored per front (the Hessian-type calls use it).
-__global__ void __launch_bounds__(CT) kc_gradient(SymDev S, int task0, const double* Wc, double* Sc, double* g,
-                                                 double* Vd, double* ws) {
-  __shared__ double V[WS][WS + 1];
-  __shared__ double lw[WS];
-  __shared__ double sa[WS];
+// child's rows.  kc_grad_post stores V_j of every column and the gradient.
+__global__ void __launch_bounds__(DNT) kc_gradient(SymDev S, int task0, const double* Wc, double* Sc,
+                                                  const double* ws) {
+  __shared__ DownSmem sm;
   const Run R = run_of(S, task0 + blockIdx.x);
-  const int a = R.a, tid = threadIdx.x;
-  gather_window(S, R, ws, V, tid);
-  double wv = tid <= a ? Wc[R.base0 + (int64_t)(R.L - 1) * (a + 1) + tid] : 0.0;
-  __syncthreads();
-  for (int i = R.L - 1; i >= 0; --i) {
-    const int64_t base = R.base0 + (int64_t)i * (a + 1);
-    if (tid <= a) lw[tid] = wv;
-    if (i > 0 && tid <= a) wv = Wc[base - (a + 1) + tid];
-    // V_i (rows i+1 .. i+a) to the front's block (lower, ld a)
+  down_dispatch<DOWN_GRAD>(S, R, Wc + R.base0, nullptr, Sc + R.base0, ws, sm);
+}
+__global__ void __launch_bounds__(MT) kc_grad_post(SymDev S, int task0, const double* Sc, double* g, double* Vd,
+                                                  const double* ws) {
+  const Run R = run_of(S, task0 + blockIdx.x);
+  const Parent P = parent_of(S, R, ws);
+  const int a = R.a, lane = threadIdx.x & 31;
+  const double* v = Sc + R.base0;
+  for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
     double* Vb = Vd + R.v0 + (int64_t)i * R.vstride;
-    for (int e = tid; e < a * a; e += CT) {
-      const int r = e / a, s = e - (e / a) * a;
-      if (r >= s) Vb[r + (int64_t)s * a] = V[slot(i + 1 + r)][slot(i + 1 + s)];
+    for (int c = threadIdx.x >> 5; c < a; c += MT / 32) {
+      const int col = i + 1 + c;
+      for (int r = c + lane; r < a; r += 32) {
+        double x;
+        if (col < R.L) {
+          x = v[(int64_t)col * (a + 1) + (r - c)];
+        } else {
+          const int pr = __ldg(P.rel + (i + 1 + r - R.L)), pc = __ldg(P.rel + (col - R.L));
+          x = __ldcg(P.F + (pr >= pc ? pr + (int64_t)pc * P.J : pc + (int64_t)pr * P.J));
+        }
+        Vb[r + (int64_t)c * a] = x;
+      }
     }
-    __syncthreads();
-    const double sv = -window_row_dot(V, i + 1, a, lw + 1, tid);
-    if (tid % TPR == 0 && tid / TPR < a) sa[tid / TPR] = sv;
-    __syncthreads();
-    const double snn = lw[0] - all_sum(a, [&](int r) { return sa[r] * lw[1 + r]; }, tid);
-    if (tid <= a) {
-      const double v = tid == 0 ? snn : sa[tid - 1];
-      Sc[base + tid] = v;
-      if (g) g[base + tid] = -v;
+    if (g) {
+      const int64_t b = (int64_t)i * (a + 1);
+      for (int q = threadIdx.x; q <= a; q += MT) g[R.base0 + b + q] = -v[b + q];
     }
-    // row i enters the window: V of the child covers rows i .. i + a - 1
-    const int si = slot(i);
-    if (tid == 0) V[si][si] = snn;
-    for (int r = tid; r < a - 1; r += CT) {
-      V[si][slot(i + 1 + r)] = sa[r];
-      V[slot(i + 1 + r)][si] = sa[r];
-    }
-    __syncthreads();
   }
 }
-
-// Algorithm 5.1 steps 1-2 for one-column fronts: with Yh the front's values
-// plus the child's U', K_jj = Yh_jj, K_A = Yh_A - L_A Yh_jj,
-// U' = Yh_AA - K_A L_A^T - L_A Yh_A^T, M_jj = K_jj / D^2, M_A = V K_A / D.
-// act (pruned R(Y), §5.5): a front with act == 0 has Y zero in its subtree,
-// so K, U' and M are zero and the column is skipped (its output was cleared).
-__global__ void __launch_bounds__(CT) kc_hess_up(SymDev S, int task0, const double* Wc, const double* Vd,
-                                                const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws,
-                                                const uint8_t* act) {
-  __shared__ double U[WS][WS + 1];
-  __shared__ double h[WS];
-  __shared__ double lw[WS];
-  __shared__ double kk[WS];
+// Algorithm 5.1 step 3 for one-column fronts: with w = V' L_A, T_A = M_A - w,
+// T_jj = M_jj - L_A^T (T_A + M_A); V' of the child = [T_jj T_A^T; T_A V'] on
+// its rows.  T in place.
+__global__ void __launch_bounds__(DNT) kc_hess_down(SymDev S, int task0, const double* Wc, double* T, int64_t ldt,
+                                                   const double* ws) {
+  __shared__ DownSmem sm;
   const Run R = run_of(S, task0 + blockIdx.x);
   const int64_t y = blockIdx.y;
-  Y += y * ldy;
-  T += y * ldt;
-  ws += y * S.f_total;
-  const uint8_t* ay = act ? act + y * S.nsn + R.k0 : nullptr;
-  const int a = R.a, tid = threadIdx.x;
-  for (int e = tid; e < WS * (WS + 1); e += CT) (&U[0][0])[e] = 0.0;
-  double yv = tid <= a ? Y[R.base0 + tid] : 0.0;
-  double wv = tid <= a ? Wc[R.base0 + tid] : 0.0;
-  __syncthreads();
-  for (int i = 0; i < R.L; ++i) {
-    const int64_t base = R.base0 + (int64_t)i * (a + 1);
-    const double ycur = yv, wcur = wv;
-    if (i + 1 < R.L && tid <= a) {
-      yv = Y[base + (a + 1) + tid];
-      wv = Wc[base + (a + 1) + tid];
-    }
-    if (ay && !ay[i]) continue;  // the same decision in every thread
-    // V_i's row part, loaded now and used after the window update
-    const RowPart vrow = load_row_part(Vd + R.v0 + (int64_t)i * R.vstride, a, tid);
-    if (tid <= a) {
-      h[tid] = ycur + U[slot(i + tid)][slot(i)];
-      lw[tid] = wcur;
-    }
-    __syncthreads();
-    const double h0 = h[0], dinv = lw[0];
-    if (tid < a) kk[tid] = h[1 + tid] - lw[1 + tid] * h0;
-    __syncthreads();
-    for (int e = tid; e < a * a; e += CT) {
-      const int p = e / a, q = e - (e / a) * a;
-      U[slot(i + 1 + p)][slot(i + 1 + q)] -= fma(kk[p], lw[1 + q], lw[1 + p] * h[1 + q]);
-    }
-    // M_A = V (K_A / D): V_i from its stored block (lower, ld a)
-    {
-      const double acc = row_part_dot(vrow, kk, a, 1.0, tid);
-      if (tid % TPR == 0 && tid / TPR < a) T[base + 1 + tid / TPR] = acc * dinv;
-    }
-    if (tid == 0) T[base] = dinv * h0 * dinv;
-    const int si = slot(i);
-    for (int e = tid; e < WS; e += CT) {
-      U[si][e] = 0.0;
-      U[e][si] = 0.0;
-    }
-    __syncthreads();
-  }
-  double* G = ws + R.f0 + (int64_t)(R.L - 1) * R.fstride;
-  const int J = a + 1;
-  for (int e = tid; e < a * a; e += CT) {
-    const int p = e / a, q = e - (e / a) * a;
-    if (p >= q) G[(1 + p) + (int64_t)(1 + q) * J] = U[slot(R.L + p)][slot(R.L + q)];
-  }
+  double* t = T + y * ldt + R.base0;
+  down_dispatch<DOWN_HESS>(S, R, Wc + R.base0, t, t, ws + y * S.f_total, sm);
 }
 
-// Algorithm 5.1 step 3 for one-column fronts: with w = V' L_A,
-// T_A = M_A - w, T_jj = M_jj - 2 L_A^T M_A + L_A^T w; V' of the child =
-// [T_jj T_A^T; T_A V'] on the child's rows.
-__global__ void __launch_bounds__(CT) kc_hess_down(SymDev S, int task0, const double* Wc, double* T, int64_t ldt,
-                                                  double* ws) {
-  __shared__ double V[WS][WS + 1];
-  __shared__ double lw[WS];
-  __shared__ double mv[WS];
-  __shared__ double wl[WS];
-  const Run R = run_of(S, task0 + blockIdx.x);
-  const int64_t y = blockIdx.y;
-  T += y * ldt;
-  ws += y * S.f_total;
-  const int a = R.a, tid = threadIdx.x;
-  gather_window(S, R, ws, V, tid);
-  const int64_t top = R.base0 + (int64_t)(R.L - 1) * (a + 1);
-  double wv = tid <= a ? Wc[top + tid] : 0.0;
-  double tv = tid <= a ? T[top + tid] : 0.0;
-  __syncthreads();
-  for (int i = R.L - 1; i >= 0; --i) {
-    const int64_t base = R.base0 + (int64_t)i * (a + 1);
-    if (tid <= a) {
-      lw[tid] = wv;
-      mv[tid] = tv;
-    }
-    if (i > 0 && tid <= a) {
-      wv = Wc[base - (a + 1) + tid];
-      tv = T[base - (a + 1) + tid];
-    }
-    __syncthreads();
-    const double wr = window_row_dot(V, i + 1, a, lw + 1, tid);
-    if (tid % TPR == 0 && tid / TPR < a) wl[tid / TPR] = wr;
-    __syncthreads();
-    const double tnn = mv[0] + all_sum(a, [&](int r) { return lw[1 + r] * (wl[r] - 2.0 * mv[1 + r]); }, tid);
-    if (tid <= a) T[base + tid] = tid == 0 ? tnn : mv[tid] - wl[tid - 1];
-    const int si = slot(i);
-    if (tid == 0) V[si][si] = tnn;
-    for (int r = tid; r < a - 1; r += CT) {
-      const double v = mv[1 + r] - wl[r];
-      V[si][slot(i + 1 + r)] = v;
-      V[slot(i + 1 + r)][si] = v;
-    }
-    __syncthreads();
-  }
-}
-
-// Algorithm 5.2 steps 1-2 for one-column fronts (top-down): with the window
-// V' (the input T on A_j x A_j, gathered from the parent's T-front),
-// M_A = T_A + V' L_A, M_jj = T_jj + L_A^T (T_A + M_A), K_jj = D M_jj D,
-// K_A = V^{-1} (M_A D) (V^{-1} per front, formed by the inverse-Hessian
-// setup); the child's window is [T_jj T_A^T; T_A V'] on its rows.
-__global__ void __launch_bounds__(CT) kc_ihess_down(SymDev S, int task0, const double* Wc, const double* Dd,
+// Algorithm 5.2 steps 1-2 for one-column fronts: V' is the input T on
+// A_j x A_j, M_A = T_A + V' L_A, M_jj = T_jj + L_A^T (T_A + M_A),
+// K_jj = D M_jj D, K_A = V^{-1} (M_A D).  No column waits for another.
+// Writes what step 3 starts from: Y_jj = K_jj, Y_A = K_A + L_A K_jj, and
+// P = K_A + L_A K_jj / 2 into the first temporary of the front.
+__global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const double* Wc, const double* Dd,
                                                    const double* Rd, const double* Tin, int64_t ldt, double* Y,
                                                    int64_t ldy, double* ws) {
-  __shared__ double V[WS][WS + 1];
-  __shared__ double lw[WS];
-  __shared__ double tt[WS];
-  __shared__ double ma[WS];
+  __shared__ double B[AMAX][BLD];
+  __shared__ double lw[AMAX], tt[AMAX], x[AMAX], yv[AMAX];
+  __shared__ double kjj;
   const Run R = run_of(S, task0 + blockIdx.x);
-  const int64_t y = blockIdx.y;
-  Tin += y * ldt;
-  Y += y * ldy;
+  const int a = R.a, tid = threadIdx.x, lane = tid & 31;
+  const int64_t y = blockIdx.z;
+  Tin += y * ldt + R.base0;
+  Y += y * ldy + R.base0;
   ws += y * S.f_total;
-  const int a = R.a, tid = threadIdx.x;
-  gather_window(S, R, ws, V, tid);
-  const int64_t top = R.base0 + (int64_t)(R.L - 1) * (a + 1);
-  double wv = tid <= a ? Wc[top + tid] : 0.0;
-  double tv = tid <= a ? Tin[top + tid] : 0.0;
-  __syncthreads();
-  for (int i = R.L - 1; i >= 0; --i) {
-    const int64_t base = R.base0 + (int64_t)i * (a + 1);
-    if (tid <= a) {
-      lw[tid] = wv;
-      tt[tid] = tv;
-    }
-    if (i > 0 && tid <= a) {
-      wv = Wc[base - (a + 1) + tid];
-      tv = Tin[base - (a + 1) + tid];
-    }
-    // V_i^{-1}'s row part, loaded now and used after the window products
-    const RowPart rrow = load_row_part(Rd + R.v0 + (int64_t)i * R.vstride, a, tid);
-    __syncthreads();
-    const double wr = window_row_dot(V, i + 1, a, lw + 1, tid);
-    if (tid % TPR == 0 && tid / TPR < a) ma[tid / TPR] = tt[1 + tid / TPR] + wr;
-    __syncthreads();
+  const Parent P = parent_of(S, R, ws);
+  for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
+    const int64_t b = (int64_t)i * (a + 1);
     const double dd = Dd[R.d0 + 4 * (int64_t)i];
-    const double mnn = tt[0] + all_sum(a, [&](int r) { return lw[1 + r] * (tt[1 + r] + ma[r]); }, tid);
-    if (tid == 0) Y[base] = dd * (mnn * dd);
-    {
-      const double acc = row_part_dot(rrow, ma, a, dd, tid);
-      if (tid % TPR == 0 && tid / TPR < a) Y[base + 1 + tid / TPR] = acc;
+    stage_window(S, R, i, Tin, P.F, P.J, P.rel, B);
+    if (tid < a) {
+      lw[tid] = Wc[R.base0 + b + 1 + tid];
+      tt[tid] = Tin[b + 1 + tid];
     }
-    const int si = slot(i);
-    if (tid == 0) V[si][si] = tt[0];
-    for (int r = tid; r < a - 1; r += CT) {
-      V[si][slot(i + 1 + r)] = tt[1 + r];
-      V[slot(i + 1 + r)][si] = tt[1 + r];
+    __syncthreads();
+    sym_dot(B, lw, a, yv);
+    __syncthreads();
+    if (tid < 32) {
+      double acc = 0.0;
+      for (int r = lane; r < a; r += 32) {
+        const double t = tt[r], m = t + yv[r];
+        acc = fma(lw[r], t + m, acc);
+        x[r] = m * dd;
+      }
+      for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+      if (lane == 0) kjj = dd * ((Tin[b] + acc) * dd);
     }
+    stage_sym(B, Rd + R.v0 + (int64_t)i * R.vstride, a);
+    __syncthreads();
+    sym_dot(B, x, a, yv);
+    __syncthreads();
+    double* Pv = ws + R.f0 + (int64_t)i * R.fstride + (int64_t)(a + 1) * (a + 1);
+    if (tid < a) {
+      const double k = kjj, p = fma(0.5 * lw[tid], k, yv[tid]);
+      Pv[1 + tid] = p;
+      Y[b + 1 + tid] = 2.0 * p - yv[tid];
+    }
+    if (tid == MT - 1) Y[b] = kjj;
     __syncthreads();
   }
 }
 
-// Algorithm 5.2 step 3 for one-column fronts (bottom-up): with K from the
-// top-down pass and F the child's U' on this front's rows,
-// P = K_A + L_A K_jj / 2, Y_jj = K_jj - F_jj, Y_A = 2 P - K_A - F_A,
-// U' = F_AA - (P L_A^T + L_A P^T).
-__global__ void __launch_bounds__(CT) kc_ihess_up(SymDev S, int task0, const double* Wc, double* Y, int64_t ldy,
-                                                 double* ws) {
-  __shared__ double U[WS][WS + 1];
-  __shared__ double lw[WS];
-  __shared__ double kk[WS];
-  __shared__ double ff[WS];
-  __shared__ double pp[WS];
+// Sums of the columns' rank-one (rank-two) blocks over a run: entry
+// (j + r, j) of Z = sum_k x_k y_k^T, the k-th column's vectors covering rows
+// k .. k+a.  Nothing depends on the order of the columns, so a warp takes one
+// column j of Z, its lanes the rows r, for the columns of the run (subtracted
+// from or stored to the output) and for the a columns beyond it (the update
+// block the parent adds).
+//   product (Algorithm 3.2): x = y = [C; B];
+//   inverse Hessian step 3:  -(P L^T + L P^T), rows k+1 .. k+a.
+template <bool PROD>
+__global__ void __launch_bounds__(128) kc_band_sum(SymDev S, int task0, const double* Gc, double* Out, int64_t ldo,
+                                                  double* ws) {
   const Run R = run_of(S, task0 + blockIdx.x);
-  const int64_t y = blockIdx.y;
-  Y += y * ldy;
+  const int a = R.a, lane = threadIdx.x & 31, W = a + 1;
+  const int64_t y = blockIdx.z;
+  Out += y * ldo + R.base0;
   ws += y * S.f_total;
-  const int a = R.a, tid = threadIdx.x;
-  for (int e = tid; e < WS * (WS + 1); e += CT) (&U[0][0])[e] = 0.0;
-  double kv = tid <= a ? Y[R.base0 + tid] : 0.0;
-  double wv = tid <= a ? Wc[R.base0 + tid] : 0.0;
-  __syncthreads();
-  for (int i = 0; i < R.L; ++i) {
-    const int64_t base = R.base0 + (int64_t)i * (a + 1);
-    if (tid <= a) {
-      kk[tid] = kv;
-      lw[tid] = wv;
-      ff[tid] = U[slot(i + tid)][slot(i)];
-    }
-    if (i + 1 < R.L && tid <= a) {
-      kv = Y[base + (a + 1) + tid];
-      wv = Wc[base + (a + 1) + tid];
-    }
-    __syncthreads();
-    if (tid < a) pp[tid] = fma(0.5 * lw[1 + tid], kk[0], kk[1 + tid]);
-    __syncthreads();
-    if (tid <= a) Y[base + tid] = tid == 0 ? kk[0] - ff[0] : 2.0 * pp[tid - 1] - kk[tid] - ff[tid];
-    for (int e = tid; e < a * a; e += CT) {
-      const int p = e / a, q = e - (e / a) * a;
-      U[slot(i + 1 + p)][slot(i + 1 + q)] -= fma(pp[p], lw[1 + q], lw[1 + p] * pp[q]);
-    }
-    const int si = slot(i);
-    for (int e = tid; e < WS; e += CT) {
-      U[si][e] = 0.0;
-      U[e][si] = 0.0;
-    }
-    __syncthreads();
-  }
+  const double* Lw = Gc + R.base0;
+  const double* Pw = ws + R.f0 + (int64_t)W * W;
   double* G = ws + R.f0 + (int64_t)(R.L - 1) * R.fstride;
-  const int J = a + 1;
-  for (int e = tid; e < a * a; e += CT) {
-    const int p = e / a, q = e - (e / a) * a;
-    if (p >= q) G[(1 + p) + (int64_t)(1 + q) * J] = U[slot(R.L + p)][slot(R.L + q)];
+  for (int j = blockIdx.y * 4 + (threadIdx.x >> 5); j < R.L + a; j += gridDim.y * 4) {
+    const int rmax = j < R.L ? a : R.L + a - 1 - j;
+    const int kend = PROD ? min(j, R.L - 1) : min(j, R.L) - 1;
+    for (int r0 = 0; r0 <= rmax; r0 += 32) {
+      const int r = r0 + lane;
+      const int klo = max(0, j + r - a);  // the first column that reaches row j + r
+      double acc = 0.0;
+      for (int k = max(0, j + r0 - a); k <= kend; ++k) {
+        if (k >= klo && r <= rmax) {
+          const double lj = Lw[(int64_t)k * W + (j - k)], li = Lw[(int64_t)k * W + (j - k) + r];
+          if (PROD) {
+            acc = fma(li, lj, acc);
+          } else {
+            const double* pk = Pw + (int64_t)k * R.fstride + (j - k);
+            acc = fma(pk[r], lj, acc);
+            acc = fma(li, pk[0], acc);
+          }
+        }
+      }
+      if (r <= rmax) {
+        if (j < R.L) {
+          double* o = Out + (int64_t)j * W + r;
+          *o = PROD ? acc : *o + acc;
+        } else {
+          const int q = j - R.L;
+          G[(1 + q + r) + (int64_t)(1 + q) * W] = PROD ? acc : -acc;
+        }
+      }
+    }
   }
 }
 
@@ -460,35 +725,51 @@ __global__ void __launch_bounds__(CT) kc_ihess_up(SymDev S, int task0, const dou
 
 namespace chd_launch {
 using namespace chd::chain;
+// columns of the longest run of the launch, as a grid dimension
+static unsigned columns(const chd_symbolic* s, int t0, int nt, int per, int extra) {
+  int64_t L = 1;
+  for (int t = t0; t < t0 + nt; ++t) L = std::max<int64_t>(L, s->task_ptr[t + 1] - s->task_ptr[t] + extra);
+  return (unsigned)std::min<int64_t>((L + per - 1) / per, 32768);
+}
 void chain_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* X, double* Lc, double* Wc,
                   double* Dd, double* ws, double* ldet, int64_t* status) {
-  kc_factor<<<nt, CT, 0, st>>>(s->dev, t0, X, Lc, Wc, Dd, ws, ldet, status);
+  kc_factor<<<nt, UPT, 0, st>>>(s->dev, t0, X, Lc, Wc, Dd, ws, status);
+  count_launch();
+  kc_factor_post<<<dim3(nt, columns(s, t0, nt, 4, 0)), 128, 0, st>>>(s->dev, t0, Lc, Dd, ldet);
+  count_launch();
+}
+void chain_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws) {
+  kc_band_sum<true><<<dim3(nt, columns(s, t0, nt, 4, AMAX)), 128, 0, st>>>(s->dev, t0, Lc, X, 0, ws);
   count_launch();
 }
 void chain_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Wc, double* Sc, double* g,
                     double* Vd, double* ws) {
-  kc_gradient<<<nt, CT, 0, st>>>(s->dev, t0, Wc, Sc, g, Vd, ws);
+  kc_gradient<<<nt, DNT, 0, st>>>(s->dev, t0, Wc, Sc, ws);
+  count_launch();
+  kc_grad_post<<<dim3(nt, columns(s, t0, nt, 1, 0)), MT, 0, st>>>(s->dev, t0, Sc, g, Vd, ws);
   count_launch();
 }
 void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, const double* Vd,
                    const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act) {
-  kc_hess_up<<<dim3(nt, m), CT, 0, st>>>(s->dev, t0, Wc, Vd, Y, ldy, T, ldt, ws, act);
+  kc_hess_up<<<dim3(nt, m), UPT, 0, st>>>(s->dev, t0, Wc, Y, ldy, T, ldt, ws, act);
+  count_launch();
+  kc_hess_m<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Vd, T, ldt, act);
   count_launch();
 }
 void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
                      int64_t ldt, double* ws) {
-  kc_hess_down<<<dim3(nt, m), CT, 0, st>>>(s->dev, t0, Wc, T, ldt, ws);
+  kc_hess_down<<<dim3(nt, m), DNT, 0, st>>>(s->dev, t0, Wc, T, ldt, ws);
   count_launch();
 }
 void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
                       const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy,
                       double* ws) {
-  kc_ihess_down<<<dim3(nt, m), CT, 0, st>>>(s->dev, t0, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+  kc_ihess_down<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
   count_launch();
 }
 void chain_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,
                     int64_t ldy, double* ws) {
-  kc_ihess_up<<<dim3(nt, m), CT, 0, st>>>(s->dev, t0, Wc, Y, ldy, ws);
+  kc_band_sum<false><<<dim3(nt, columns(s, t0, nt, 4, AMAX), m), 128, 0, st>>>(s->dev, t0, Wc, Y, ldy, ws);
   count_launch();
 }
 }  // namespace chd_launch

@@ -1076,6 +1076,7 @@ void big_complete(const chd_symbolic* s, const Slot& sl, int k, const double* Si
 // chain-tier launches (chain_tier.cu): runs of one-column band fronts
 void chain_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* X, double* Lc, double* Wc,
                   double* Dd, double* ws, double* ldet, int64_t* status);
+void chain_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws);
 void chain_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Wc, double* Sc, double* g,
                     double* Vd, double* ws);
 void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, const double* Vd,
@@ -1228,8 +1229,7 @@ void product(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doubl
     bf.run(v.nbig, [&](int i, const Slot& sl) {
       big_product(s, sl, big_front(s, v, i), Lc, X, ws);
     });
-    if (v.nr32) w32::warp_product(s, st, v.tr, v.nr32, Lc, X, ws);
-    if (v.nr64) w64::warp_product(s, st, v.tr + v.nr32, v.nr64, Lc, X, ws);
+    if (v.nr32 + v.nr64) chain_product(s, st, v.tr, v.nr32 + v.nr64, Lc, X, ws);
     if (v.nwarp) w32::warp_product(s, st, v.t0, v.nwarp, Lc, X, ws);
     if (v.nw64) w64::warp_product(s, st, v.tw, v.nw64, Lc, X, ws);
     if (v.ncta) {
