@@ -14,6 +14,7 @@
 
 #include "chd_internal.h"
 #include "front_views.cuh"
+#include "panel.cuh"
 #include "tc_gemm.cuh"
 #include "fc_body.cuh"
 
@@ -275,64 +276,31 @@ void gemm(const Ctx& st, int batch, int M, int N, int K, double alpha, MA A, int
 }
 
 // ---------------------------------------------------------------------------
-// Blocked right-looking Cholesky (panels of PP columns) and triangular
-// solves (panels of TW columns).  On GB300 an SM retires about 1.6 FP64
-// lane-operations per clock, spread over its four sub-partitions: a single
-// warp issuing FP64 instructions keeps one sub-partition busy and leaves
-// three idle.  The panel kernels therefore run four warps per CTA and only
-// PR = 8 rows per CTA (two rows per warp, sixteen lanes per row, lane q
-// owning the panel columns c = q mod 16), so that a panel of R rows keeps
-// R / 2 warps issuing; the substitution along the panel columns passes each
-// solved entry within its 16-lane group by a shuffle.
+// Blocked right-looking Cholesky (panels of PP columns, panel.cuh) and
+// triangular solves (panels of TW columns).  A GB300 SM retires one FP64 warp
+// instruction per 19 clocks, one warp one per 64, so the solve panels run
+// four warps per CTA and only PR = 8 rows per CTA (two rows per warp, sixteen
+// lanes per row, lane q owning the panel columns c = q mod 16); the
+// substitution along the panel columns passes each solved entry within its
+// 16-lane group by a shuffle.
 // ---------------------------------------------------------------------------
 constexpr int PP = 32;   // Cholesky panel width
 constexpr int TW = 64;   // triangular-solve panel width
 constexpr int PR = 8;    // panel rows per CTA
 constexpr int PT = 128;  // threads per panel CTA
 
-// Cooperative Cholesky of the pb x pb block held in shared memory (ld
-// PP + 1, identity beyond pb) by the CTA's PT threads: column by column,
-// pivot, scale of the column below it, rank-one update of the trailing
-// lower triangle.  On return Ls holds the lower factor C and rinv the
-// reciprocal pivots; a non-positive pivot is recorded and replaced by 1.
-// Every CTA of a launch computes the same values in the same order.
-__device__ __forceinline__ void cta_potrf32(double (*Ls)[PP + 1], double* rinv, int pb, int64_t* st, int64_t code,
-                                            int64_t snode, int64_t col) {
-  const int tid = threadIdx.x;
-  for (int j = 0; j < pb; ++j) {
-    if (tid == 0) {
-      double d = Ls[j][j];
-      if (!(d > 0.0)) {
-        record_error(st, code, snode, col < 0 ? -1 : col + j);
-        d = 1.0;
-      }
-      Ls[j][j] = sqrt(d);
-      rinv[j] = rsqrt(d);
-    }
-    __syncthreads();
-    const double r = rinv[j];
-    for (int i = j + 1 + tid; i < pb; i += PT) Ls[i][j] *= r;
-    __syncthreads();
-    const int w = pb - j - 1;
-    for (int e = tid; e < w * w; e += PT) {
-      const int i = j + 1 + e % w, k = j + 1 + e / w;
-      if (k <= i) Ls[i][k] = fma(-Ls[i][j], Ls[k][j], Ls[i][k]);
-    }
-    __syncthreads();
-  }
-}
-
 // One panel of the Cholesky of F (ld): the pb x pb block at (j0, j0) and the
 // R rows below it (rows j0+pb ..).  Every CTA factors the diagonal block
 // (the same arithmetic in every CTA, so the copies agree bitwise) and
-// solves its PR rows, B := B C^{-T}.  The CTA that arrives last at the
+// solves its CR rows, B := B C^{-T}.  The CTA that arrives last at the
 // counter -- when every CTA has read the unfactored block -- writes the
 // factored block back and resets the counter.  ctr == nullptr is allowed
 // for a single-CTA launch with R == 0.
+constexpr int CR = 32;  // rows per CTA, four lanes each
 __global__ void __launch_bounds__(PT) mk_potrf_panel(double* F, int64_t ld, int j0, int pb, int R, int* ctr,
                                                      int64_t* st, int64_t code, int64_t snode, int64_t col0) {
   __shared__ double Ls[PP][PP + 1];
-  __shared__ double rinv[PP];
+  __shared__ double rinv[PP], col[3][PP];
   __shared__ int last;
   const int tid = threadIdx.x;
   double* D = F + j0 + (int64_t)j0 * ld;
@@ -340,39 +308,25 @@ __global__ void __launch_bounds__(PT) mk_potrf_panel(double* F, int64_t ld, int 
     const int i = e % PP, c = e / PP;
     Ls[i][c] = (i < pb && c < pb && i >= c) ? D[i + (int64_t)c * ld] : (i == c ? 1.0 : 0.0);
   }
+  // the rows of this CTA, in flight while the diagonal block is factored
+  const int lane = tid & 31, q = lane & 3, i = blockIdx.x * CR + (tid >> 2);
+  const bool ok = i < R;
+  double* Bi = F + (j0 + pb + (ok ? i : 0)) + (int64_t)j0 * ld;
+  double b[PP / 4];
+#pragma unroll
+  for (int u = 0; u < PP / 4; ++u) b[u] = (ok && q + 4 * u < pb) ? Bi[(int64_t)(q + 4 * u) * ld] : 0.0;
   __syncthreads();
   if (tid == 0) {
     __threadfence();
     last = (ctr == nullptr) ? 1 : (atomicAdd(ctr, 1) == (int)gridDim.x - 1);
   }
-  cta_potrf32(Ls, rinv, pb, st, code, snode, col0 < 0 ? -1 : col0 + j0);
-  const int lane = tid & 31, q = lane & 15;
-  const int i = blockIdx.x * PR + 2 * (tid >> 5) + (lane >> 4);
-  const bool ok = i < R;
-  double* Bi = F + (j0 + pb + (ok ? i : 0)) + (int64_t)j0 * ld;
-  double b[PP / 16];
+  panel::chol32(Ls, rinv, col, pb, tid, 1, st, code, snode, col0 < 0 ? -1 : col0 + j0);
+  __syncthreads();
+  if (R > 0) {
+    panel::solve_row(b, Ls, rinv, pb, lane);
 #pragma unroll
-  for (int u = 0; u < PP / 16; ++u) {
-    const int c = 16 * u + q;
-    b[u] = (ok && c < pb) ? Bi[(int64_t)c * ld] : 0.0;
-  }
-#pragma unroll
-  for (int c = 0; c < PP; ++c) {
-    if (c < pb) {
-      double x = b[c / 16] * rinv[c];
-      x = __shfl_sync(0xffffffffu, x, (lane & 16) | (c & 15));
-      if (q == (c & 15)) b[c / 16] = x;
-#pragma unroll
-      for (int u = c / 16; u < PP / 16; ++u) {
-        const int t = 16 * u + q;
-        if (t > c && t < pb) b[u] = fma(-Ls[t][c], x, b[u]);
-      }
-    }
-  }
-#pragma unroll
-  for (int u = 0; u < PP / 16; ++u) {
-    const int c = 16 * u + q;
-    if (ok && c < pb) Bi[(int64_t)c * ld] = b[u];
+    for (int u = 0; u < PP / 4; ++u)
+      if (ok && q + 4 * u < pb) Bi[(int64_t)(q + 4 * u) * ld] = b[u];
   }
   if (last) {
     for (int e = tid; e < pb * pb; e += PT) {
@@ -511,8 +465,8 @@ void potrf_partial(const Ctx& st, double* F, int64_t ld, int J, int n, int64_t* 
       const int pb = std::min(PP, b0 + bw - j0);
       const int R = J - j0 - pb;
       if (st.ctr) {
-        mk_potrf_panel<<<std::max(1, (R + PR - 1) / PR), PT, 0, st>>>(F, ld, j0, pb, R, st.ctr, status, code,
-                                                                        snode, col0);
+        mk_potrf_panel<<<std::max(1, (R + CR - 1) / CR), PT, 0, st>>>(F, ld, j0, pb, R, st.ctr, status, code, snode,
+                                                                      col0);
         chd_launch::count_launch();
       } else {
         mk_potrf_panel<<<1, PT, 0, st>>>(F, ld, j0, pb, 0, nullptr, status, code, snode, col0);
