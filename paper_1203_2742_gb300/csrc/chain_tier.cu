@@ -130,9 +130,12 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
   if (tid < 32) {
     // ---- warp 0: inputs, pivots, outputs ----
     const int lane = tid;
+    // slots of the column being loaded and of the column being finished
+    int sload = i0 % W, scol = i0 % W;
     auto prefetch = [&](int c) {
       if (c < L) {
-        const int s0 = c % W;
+        const int s0 = sload;
+        sload = sload + 1 == W ? 0 : sload + 1;
         for (int p = lane; p <= a; p += 32) {
           int s = s0 + p;
           if (s >= W) s -= W;
@@ -143,7 +146,8 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
       cp_async_commit();
     };
     auto column = [&](int c) {
-      const int s0 = c % W, sp = s0 == 0 ? W - 1 : s0 - 1, cur = c & 1, prv = cur ^ 1;
+      const int s0 = scol, sp = s0 == 0 ? W - 1 : s0 - 1, cur = c & 1, prv = cur ^ 1;
+      scol = scol + 1 == W ? 0 : scol + 1;
       cp_async_wait<AHEAD - 1>();
       __syncwarp();
       double val[EL], l[EL];
@@ -443,16 +447,21 @@ struct DownSmem {
   double wv[WP], tv[2][WP], dg[2];
 };
 enum { DOWN_GRAD = 0, DOWN_HESS = 1 };
-template <int NT, int CP, int MODE>
+template <int NT, int CP, int TP, int MODE>
 __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const double* src, double* out,
                          const double* ws, DownSmem& sm) {
   const int a = R.a, W = a + 1, tid = threadIdx.x, L = R.L;
   if (tid >= NT + 32) return;
+  // slots past the window are multiplied by zeros: they must hold numbers
+  for (int e = tid; e < RING * WP; e += NT + 32) (&sm.ring[0][0][0])[e] = 0.0;
+  bar(NT + 32);
   if (tid < 32) {
     const int lane = tid;
+    int sload = (L - 1) % a, sfin = (L - 1) % a;
     auto prefetch = [&](int c) {
       if (c >= 0) {
-        const int sc = c % a;
+        const int sc = sload;
+        sload = sload == 0 ? a - 1 : sload - 1;
         for (int p = lane; p <= a; p += 32) {
           int s = sc + p;
           while (s >= a) s -= a;
@@ -479,7 +488,8 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
         sm.dg[c & 1] = d;
         out[(int64_t)c * W] = d;
       }
-      const int sc = c % a;
+      const int sc = sfin;
+      sfin = sfin == 0 ? a - 1 : sfin - 1;
       for (int v = lane; v < a; v += 32) {
         int p = v - sc;
         if (p <= 0) p += a;
@@ -499,7 +509,7 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
     __syncwarp();
     finish(0);
   } else {
-    const int rt = tid - 32, u = rt >> 2, part = rt & 3;
+    const int rt = tid - 32, u = rt / TP, part = rt % TP;
     double V[CP];
     {
       // rows L .. L + a - 1 from the parent's front
@@ -512,7 +522,7 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
       auto pos = [&](int s) { return __ldg(rel + (s >= sL ? s - sL : s - sL + a)); };
 #pragma unroll
       for (int j = 0; j < CP; ++j) {
-        const int v = part + 4 * j;
+        const int v = part + TP * j;
         V[j] = 0.0;
         if (u < a && v < a) {
           const int pr = pos(u), pc = pos(v);
@@ -521,23 +531,20 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
       }
     }
     bar(NT + 32);
+    int s = (L - 1) % a;
     for (int c = L - 1; c >= 0; --c) {
       const double* l = sm.ring[0][c % RING];
       const double* mm = sm.ring[1][c % RING];
-      double a0 = 0.0, a1 = 0.0;
+      // one accumulator: a warp issues an FP64 instruction every 64 clocks at
+      // best, dependent or not
+      double a0 = 0.0;
 #pragma unroll
-      for (int j = 0; j < CP; ++j) {
-        const int v = part + 4 * j;
-        const double lv = v < a ? l[v] : 0.0;
-        if (j & 1) a1 = fma(V[j], lv, a1);
-        else a0 = fma(V[j], lv, a0);
-      }
-      a0 += a1;
-      a0 += __shfl_xor_sync(0xffffffffu, a0, 1);
-      a0 += __shfl_xor_sync(0xffffffffu, a0, 2);
+      for (int j = 0; j < CP; ++j)
+        if (TP * j < a) a0 = fma(V[j], l[part + TP * j], a0);  // slots beyond the window: V = 0
+#pragma unroll
+      for (int o = 1; o < TP; o <<= 1) a0 += __shfl_xor_sync(0xffffffffu, a0, o);
       if (part == 0 && u < a) sm.wv[u] = a0;
       bar(NT + 32);
-      const int s = c % a;
       const int s1 = c + 1 < L ? (s + 1 == a ? 0 : s + 1) : -1;  // row c + 1, its diagonal still missing
       double* tv = sm.tv[c & 1];
       const double dnew = sm.dg[(c + 1) & 1];
@@ -547,13 +554,27 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
         tv[rt] = MODE == DOWN_HESS ? mm[rt] - w : -w;
       }
       bar(NT + 32);
+      // the new row into the registers: column slot s of every row, the four
+      // threads of row slot s, and the diagonal entry of the row before
+      const double mine = u < a ? tv[u] : 0.0;
+      const int js = s / TP, ps = s % TP;
+      if (part == ps) {
 #pragma unroll
-      for (int j = 0; j < CP; ++j) {
-        const int v = part + 4 * j;
-        if (u == s1 && v == s1) V[j] = dnew;
-        if (u == s) V[j] = v == s || v >= a ? 0.0 : tv[v];
-        else if (v == s && u < a) V[j] = tv[u];
+        for (int j = 0; j < CP; ++j)
+          if (j == js) V[j] = mine;
       }
+      if (u == s) {
+#pragma unroll
+        for (int j = 0; j < CP; ++j) {
+          const int v = part + TP * j;
+          V[j] = v == s || v >= a ? 0.0 : tv[v];
+        }
+      } else if (u == s1 && part == s1 % TP) {
+#pragma unroll
+        for (int j = 0; j < CP; ++j)
+          if (j == s1 / TP) V[j] = dnew;
+      }
+      s = s == 0 ? a - 1 : s - 1;
     }
   }
 }
@@ -561,10 +582,10 @@ constexpr int DNT = 288;
 template <int MODE>
 __device__ __forceinline__ void down_dispatch(const SymDev& S, const Run& R, const double* wc, const double* src,
                                              double* out, const double* ws, DownSmem& sm) {
-  if (R.a <= 8) down_run<32, 2, MODE>(S, R, wc, src, out, ws, sm);
-  else if (R.a <= 16) down_run<64, 4, MODE>(S, R, wc, src, out, ws, sm);
-  else if (R.a <= 32) down_run<128, 8, MODE>(S, R, wc, src, out, ws, sm);
-  else down_run<256, 16, MODE>(S, R, wc, src, out, ws, sm);
+  if (R.a <= 8) down_run<32, 2, 4, MODE>(S, R, wc, src, out, ws, sm);
+  else if (R.a <= 16) down_run<64, 4, 4, MODE>(S, R, wc, src, out, ws, sm);
+  else if (R.a <= 32) down_run<128, 8, 4, MODE>(S, R, wc, src, out, ws, sm);
+  else down_run<256, 16, 4, MODE>(S, R, wc, src, out, ws, sm);
 }
 
 // Algorithm 7.2 for one-column fronts (Algorithm 4.1): S_AN = -V L_AN,
