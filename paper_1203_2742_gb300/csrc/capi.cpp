@@ -995,6 +995,18 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   size_t iIs = add(s->inst_sn.data(), s->inst_sn.size() * 8);
   size_t iFo = add(s->fc_off.data(), s->fc_off.size() * 8);
   size_t iFf = add(s->fc_fronts.data(), s->fc_fronts.size() * 4);
+  size_t iGf = add(s->gf.data(), s->gf.size() * sizeof(GFront));
+  size_t iGc = add(s->gch.data(), s->gch.size() * sizeof(GChild));
+  size_t iGp = add(s->gptr.data(), s->gptr.size() * 4);
+  size_t iGt[9];
+  const std::vector<int32_t>* gt[9] = {&s->gt_up,  &s->gt_row,  &s->gt_asm, &s->gt_p, &s->gt_gat,
+                                       &s->gt_nn, &s->gt_asmf, &s->gt_wb,  &s->gt_fr};
+  for (int i = 0; i < 9; ++i) iGt[i] = add(gt[i]->data(), gt[i]->size() * 4);
+  size_t iGl = add(s->gleg.data(), s->gleg.size() * 4);
+  size_t iGj = add(s->gj.data(), s->gj.size() * sizeof(GJob));
+  size_t iGva = add(s->gv_all.data(), s->gv_all.size() * 4);
+  size_t iGvs = add(s->gv_sol.data(), s->gv_sol.size() * 4);
+  size_t iGvu = add(s->gv_upd.data(), s->gv_upd.size() * 4);
   std::vector<char> host(off, 0);
   for (auto& p : pcs)
     if (p.bytes) std::memcpy(host.data() + p.off, p.src, p.bytes);
@@ -1059,6 +1071,16 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   d.inst_sn = reinterpret_cast<const int64_t*>(b + pcs[iIs].off);
   d.fc_off = reinterpret_cast<const int64_t*>(b + pcs[iFo].off);
   d.fc_fronts = reinterpret_cast<const int32_t*>(b + pcs[iFf].off);
+  d.gf = reinterpret_cast<const GFront*>(b + pcs[iGf].off);
+  d.gch = reinterpret_cast<const GChild*>(b + pcs[iGc].off);
+  d.gptr = reinterpret_cast<const int32_t*>(b + pcs[iGp].off);
+  const int2** dgt[9] = {&d.gt_up, &d.gt_row, &d.gt_asm, &d.gt_p, &d.gt_gat, &d.gt_nn, &d.gt_asmf, &d.gt_wb, &d.gt_fr};
+  for (int i = 0; i < 9; ++i) *dgt[i] = reinterpret_cast<const int2*>(b + pcs[iGt[i]].off);
+  d.gleg = reinterpret_cast<const int32_t*>(b + pcs[iGl].off);
+  d.gj = reinterpret_cast<const GJob*>(b + pcs[iGj].off);
+  d.gv_all = reinterpret_cast<const int2*>(b + pcs[iGva].off);
+  d.gv_sol = reinterpret_cast<const int2*>(b + pcs[iGvs].off);
+  d.gv_upd = reinterpret_cast<const int2*>(b + pcs[iGvu].off);
   d.ninst = (int64_t)s->inst_sn.size() - 1;
   d.f_total = s->f_off[s->nsn];
   d.d_total = s->d_off[s->nsn];

@@ -27,6 +27,35 @@ struct alignas(16) WMeta {
   int32_t pad[2];
 };
 
+// Grouped tier (group_tier.cu): the fronts whose gradient, Hessian and
+// inverse-Hessian steps run as one launch per step over many fronts.
+constexpr int kGroupBlock = 32;       // rows per block of the assembly and of the update tiles
+constexpr int kGroupThin = 16;        // thin fronts: up to this many columns
+constexpr int kGroupFactor = 32;      // fronts up to this many columns factor in one launch per sub-level
+constexpr int kGroupCols = 128;       // widest front of the tier
+constexpr int kGroupSmem = 200 << 10; // dynamic shared memory a kernel of the tier may use
+struct alignas(16) GFront {
+  int64_t base, f_off, fp_off, d_off, v_off, rel_off;  // values, workspace, parent's workspace, D_NN, V_k, rel of A_k
+  int32_t k, n, a, J, Jp;
+  int32_t lrb, nb;         // row blocks of 8 << lrb rows of A_k, nb of them (at least one)
+  int32_t nbn;             // blocks of N_k
+  int32_t ch_beg, ch_end;  // children (extend-add order) in gch
+  int32_t pad[2];
+};
+struct alignas(16) GChild {
+  int64_t u_off;    // workspace offset of the child's update block
+  int64_t rel_off;  // positions of its A in the parent, in `rel`
+  int32_t Jc, k;
+  int32_t ptr_off;  // gptr[ptr_off + b]: its first row in block b of the parent
+  int32_t pad;
+};
+
+// grouped inverse of V_k: one front
+struct alignas(16) GJob {
+  int64_t v_off, w_off;  // V_k slot, workspace (a x a)
+  int32_t a, k;
+};
+
 // Device copy of the symbolic data, passed by value to every kernel.
 struct SymDev {
   int64_t n = 0;
@@ -65,6 +94,16 @@ struct SymDev {
   const uint8_t* act = nullptr;
   const int64_t* fc_off = nullptr;        // factored completion: scratch offsets (per front)
   const int32_t* fc_fronts = nullptr;     // factored completion: CTA-handled fronts by level
+  // grouped tier: fronts by sub-level, their children, and the work lists
+  // (front, low/high 16 bits or block index)
+  const GFront* gf = nullptr;
+  const GChild* gch = nullptr;
+  const int32_t* gptr = nullptr;
+  const int2 *gt_up = nullptr, *gt_row = nullptr, *gt_asm = nullptr, *gt_p = nullptr, *gt_gat = nullptr,
+             *gt_nn = nullptr, *gt_asmf = nullptr, *gt_wb = nullptr, *gt_fr = nullptr;
+  const int32_t* gleg = nullptr;
+  const GJob* gj = nullptr;
+  const int2 *gv_all = nullptr, *gv_sol = nullptr, *gv_upd = nullptr;
   const int64_t* inst_sn = nullptr;       // instances x supernode ranges
   int64_t ninst = 1;
   int64_t f_total = 0;               // workspace doubles per right-hand side
@@ -135,6 +174,23 @@ struct chd_symbolic {
   std::vector<int32_t> fc_fronts, fc_lvl, fc_big, fc_big_lvl;
   int64_t fc_total = 0;
   double fc_flops[2] = {0, 0};
+  // grouped tier: sub-levels glvl[l] .. glvl[l+1]) of level l (the i-th fronts
+  // of the level's CTA tasks, and with the first the thin dense fronts);
+  // gidx: index in gf or -1.  Work lists as (front, code) pairs with the
+  // sub-levels' ranges gs_*; gs_rn: largest row block (doubles) of a
+  // sub-level, gs_np: most factor panels, gs_thin: whether it has fronts of
+  // at most kGroupFactor columns; gleg: CTA-tier fronts outside the tier.
+  std::vector<GFront> gf;
+  std::vector<GChild> gch;
+  std::vector<int32_t> gptr, gidx, glvl;
+  std::vector<int32_t> gt_up, gt_row, gt_asm, gt_p, gt_gat, gt_nn, gt_asmf, gt_wb, gt_fr, gleg;
+  std::vector<int32_t> gs_up, gs_row, gs_asm, gs_p, gs_gat, gs_asmf, gs_wb, gs_rn, gs_np, gs_thin, gs_leg;
+  int g_rnmax = 0, g_nmax = 0;
+  // grouped inverse: fronts by decreasing a, their lower tiles, and per panel
+  // of 32 columns the row blocks to solve and the tiles to update
+  std::vector<GJob> gj;
+  std::vector<char> in_gj;  // per supernode
+  std::vector<int32_t> gv_all, gv_sol, gv_upd, gv_sol_ptr, gv_upd_ptr;
   // device mirror
   SymDev dev;
   void* dev_buf = nullptr;
@@ -163,15 +219,20 @@ struct Exec {
   int tc_mode = 0;
 };
 
+// Formation of V_k^{-1} by the size a of V_k: up to kInvVGroupMin - 1 rows one
+// CTA per front (k_inv_v; on one SM the a^3 FP64 operations of a larger V_k
+// take milliseconds), up to kInvVGroup rows the grouped kernels over all
+// fronts at once (kv_* in group_tier.cu), beyond that a launch sequence per
+// front whose trailing products run on the tensor cores.  The upper factor
+// of V_k alone (Hessian factor) has no grouped form: one CTA below
+// kInvVMulti rows, else a sequence per front.
+constexpr int kInvVMulti = 96;
+constexpr int kInvVGroupMin = 65;
+constexpr int kInvVGroup = 512;
+
 // What one dense-tier front sequence runs with: its stream, the split-K
 // scratch slice (may be null), the tensor-core scratch (may be null), the
 // factor's status and the tensor-core mode of the analysis.
-// Fronts outside the dense tier whose ancestor set has at least this many
-// rows get V_k^{-1} from the multi-CTA kernels (blocked Cholesky, blocked
-// triangular inverse, tensor-core product) instead of one CTA: on one SM
-// the a^3 FP64 operations of a large V_k take milliseconds.
-constexpr int kInvVMulti = 96;
-
 struct Slot {
   cudaStream_t st = nullptr;
   double* xs = nullptr;

@@ -753,57 +753,47 @@ __device__ void complete_front(const SymDev& S, int k, const double* Sin, double
 // ---------------------------------------------------------------------------
 // kernels: blockIdx.x = task within the launch, blockIdx.y = right-hand side
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) k_factor(SymDev S, int task0, const double* X, double* Lc,
-                                               double* Wc, double* Dd, double* ws, double* ldet,
-                                               int64_t* st) {
-  const int t = task0 + blockIdx.x;
-  for (int q = S.task_ptr[t]; q < S.task_ptr[t + 1]; ++q)
-    factor_front(S, S.task_fronts[q], X, Lc, Wc, Dd, ws, ldet, st);
-}
 __global__ void __launch_bounds__(NT) k_product(SymDev S, int task0, const double* Lc, double* X, double* ws) {
   const int t = task0 + blockIdx.x;
   for (int q = S.task_ptr[t]; q < S.task_ptr[t + 1]; ++q) product_front(S, S.task_fronts[q], Lc, X, ws);
 }
-__global__ void __launch_bounds__(NT) k_gradient(SymDev S, int task0, const double* Wc, double* Sc,
-                                                 double* g, double* Vd, double* ws) {
-  const int t = task0 + blockIdx.x;
-  for (int q = S.task_ptr[t + 1] - 1; q >= S.task_ptr[t]; --q)
-    gradient_front(S, S.task_fronts[q], Wc, Sc, g, Vd, ws);
+// The factor, the gradient and the Hessian-type passes of the CTA-tier fronts
+// that the grouped tier leaves out (wider than kGroupCols columns):
+// blockIdx.x = front of a sub-level's list
+__global__ void __launch_bounds__(NT) k_factor(SymDev S, const int32_t* list, const double* X, double* Lc,
+                                               double* Wc, double* Dd, double* ws, double* ldet,
+                                               int64_t* st) {
+  factor_front(S, list[blockIdx.x], X, Lc, Wc, Dd, ws, ldet, st);
 }
-__global__ void __launch_bounds__(NT) k_hess_up(SymDev S, int task0, const double* Wc,
+__global__ void __launch_bounds__(NT) k_gradient(SymDev S, const int32_t* list, const double* Wc, double* Sc,
+                                                 double* g, double* Vd, double* ws) {
+  gradient_front(S, list[blockIdx.x], Wc, Sc, g, Vd, ws);
+}
+__global__ void __launch_bounds__(NT) k_hess_up(SymDev S, const int32_t* list, const double* Wc,
                                                 const double* Vd, const double* Y, int64_t ldy,
                                                 double* T, int64_t ldt, double* ws) {
-  const int t = task0 + blockIdx.x;
   const int64_t y = blockIdx.y;
   const uint8_t* act = S.act ? S.act + y * S.nsn : nullptr;
-  for (int q = S.task_ptr[t]; q < S.task_ptr[t + 1]; ++q) {
-    const int k = S.task_fronts[q];
-    if (act && !act[k]) continue;  // pruned (§5.5): K, U' and M are zero here
-    hess_up_front(S, k, Wc, Vd, Y + y * ldy, T + y * ldt, ws + y * S.f_total, act);
-  }
+  const int k = list[blockIdx.x];
+  if (act && !act[k]) return;  // pruned (§5.5): K, U' and M are zero here
+  hess_up_front(S, k, Wc, Vd, Y + y * ldy, T + y * ldt, ws + y * S.f_total, act);
 }
-__global__ void __launch_bounds__(NT) k_hess_down(SymDev S, int task0, const double* Wc, double* T,
+__global__ void __launch_bounds__(NT) k_hess_down(SymDev S, const int32_t* list, const double* Wc, double* T,
                                                   int64_t ldt, double* ws) {
-  const int t = task0 + blockIdx.x;
   const int64_t y = blockIdx.y;
-  for (int q = S.task_ptr[t + 1] - 1; q >= S.task_ptr[t]; --q)
-    hess_down_front(S, S.task_fronts[q], Wc, T + y * ldt, ws + y * S.f_total);
+  hess_down_front(S, list[blockIdx.x], Wc, T + y * ldt, ws + y * S.f_total);
 }
-__global__ void __launch_bounds__(NT) k_ihess_down(SymDev S, int task0, const double* Wc,
+__global__ void __launch_bounds__(NT) k_ihess_down(SymDev S, const int32_t* list, const double* Wc,
                                                    const double* Dd, const double* Rd,
                                                    const double* Tin, int64_t ldt, double* Y,
                                                    int64_t ldy, double* ws) {
-  const int t = task0 + blockIdx.x;
   const int64_t y = blockIdx.y;
-  for (int q = S.task_ptr[t + 1] - 1; q >= S.task_ptr[t]; --q)
-    ihess_down_front(S, S.task_fronts[q], Wc, Dd, Rd, Tin + y * ldt, Y + y * ldy, ws + y * S.f_total);
+  ihess_down_front(S, list[blockIdx.x], Wc, Dd, Rd, Tin + y * ldt, Y + y * ldy, ws + y * S.f_total);
 }
-__global__ void __launch_bounds__(NT) k_ihess_up(SymDev S, int task0, const double* Wc, double* Y,
+__global__ void __launch_bounds__(NT) k_ihess_up(SymDev S, const int32_t* list, const double* Wc, double* Y,
                                                  int64_t ldy, double* ws) {
-  const int t = task0 + blockIdx.x;
   const int64_t y = blockIdx.y;
-  for (int q = S.task_ptr[t]; q < S.task_ptr[t + 1]; ++q)
-    ihess_up_front(S, S.task_fronts[q], Wc, Y + y * ldy, ws + y * S.f_total);
+  ihess_up_front(S, list[blockIdx.x], Wc, Y + y * ldy, ws + y * S.f_total);
 }
 // M <-> W of every front of the warp and CTA tiers, one CTA per (front, RHS)
 __global__ void __launch_bounds__(NT) k_rtrans(SymDev S, int dir, const double* Lc, const double* Qd, double* Z,
@@ -912,7 +902,7 @@ __global__ void __launch_bounds__(NT) k_inv_v(SymDev S, const double* Vd, double
   const int k = front_list[blockIdx.x];
   const int n = (int)(S.sn_ptr[k + 1] - S.sn_ptr[k]);
   const int a = (int)(S.rows_ptr[k + 1] - S.rows_ptr[k]) - n;
-  if (a == 0 || a >= kInvVMulti) return;  // large V_k: multi-CTA kernels (big_inv_v)
+  if (a == 0 || a >= (what == 1 ? kInvVGroupMin : kInvVMulti)) return;  // large V_k: multi-CTA kernels
   double* R = Rd + S.v_off[k];
   double* Ri = ws + S.f_off[k];  // a x a scratch inside the front's J x J region
   const double* V = Vd + S.v_off[k];
@@ -1089,6 +1079,28 @@ void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, in
 void chain_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,
                     int64_t ldy, double* ws);
 
+// grouped-tier launches (group_tier.cu); q: sub-level
+void group_factor(const chd_symbolic* s, cudaStream_t st, int q, const double* X, double* Lc, double* Dd, double* ws,
+                  int64_t* status);
+void group_factor_post(const chd_symbolic* s, cudaStream_t st, const double* Lc, double* Wc, double* ws,
+                       double* ldet);
+void group_zero(const chd_symbolic* s, cudaStream_t st, int m, double* ws);
+void group_gradient(const chd_symbolic* s, cudaStream_t st, int q, const double* Wc, double* Sc, double* g, double* Vd,
+                    double* ws);
+void group_hess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const double* Wc, const double* Y,
+                   int64_t ldy, double* ws, const uint8_t* act);
+void group_hess_m(const chd_symbolic* s, cudaStream_t st, int m, const double* Wc, const double* Vd, double* T,
+                  int64_t ldt, double* ws, const uint8_t* act);
+void group_hess_down(const chd_symbolic* s, cudaStream_t st, int q, int m, const double* Wc, double* T, int64_t ldt,
+                     double* ws);
+void group_ihess_gather(const chd_symbolic* s, cudaStream_t st, int q, int m, const double* T, int64_t ldt,
+                        double* ws);
+void group_ihess_k(const chd_symbolic* s, cudaStream_t st, int m, const double* Wc, const double* Dd, const double* Rd,
+                   double* Y, int64_t ldy, double* ws);
+void group_ihess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const double* Wc, double* Y, int64_t ldy,
+                    double* ws);
+void group_inv_v(const chd_symbolic* s, cudaStream_t st, const double* Vd, double* Rd, double* ws, int64_t* status);
+
 // warp-tier launches (warp_tier.cu): w32 for |J| <= 32, w64 for |J| <= 64
 namespace w32 {
 void warp_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws);
@@ -1200,6 +1212,20 @@ static inline Level level(const chd_symbolic* s, int l) {
 static inline int big_front(const chd_symbolic* s, const Level& v, int i) {
   return s->task_fronts[s->task_ptr[v.tc + v.ncta + i]];
 }
+// the level's dense fronts and leaf groups that the grouped tier leaves out
+static std::vector<int> dense_fronts(const chd_symbolic* s, const Level& v) {
+  std::vector<int> d;
+  for (int i = 0; i < v.nbig; ++i) {
+    const int k = big_front(s, v, i);
+    if (s->gidx[k] < 0) d.push_back(k);
+  }
+  return d;
+}
+// the CTA-tier fronts of sub-level q outside the grouped tier
+static inline const int32_t* left_out(const chd_symbolic* s, int q, int& count) {
+  count = s->gs_leg[q + 1] - s->gs_leg[q];
+  return s->dev.gleg + s->gs_leg[q];
+}
 
 void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* X, double* Lc, double* Wc,
             double* Dd, double* ws, double* ldet, int64_t* status) {
@@ -1207,18 +1233,25 @@ void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_factor(s, sl, big_front(s, v, i), X, Lc, Wc, Dd, ws, ldet, status);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_factor(s, sl, dense[i], X, Lc, Wc, Dd, ws, ldet, status);
     });
     if (v.nr32 + v.nr64) chain_factor(s, st, v.tr, v.nr32 + v.nr64, X, Lc, Wc, Dd, ws, ldet, status);
     if (v.nwarp) w32::warp_factor(s, st, v.t0, v.nwarp, X, Lc, Wc, Dd, ws, ldet, status);
     if (v.nw64) w64::warp_factor(s, st, v.tw, v.nw64, X, Lc, Wc, Dd, ws, ldet, status);
-    if (v.ncta) {
-      k_factor<<<v.ncta, NT, 0, st>>>(s->dev, v.tc, X, Lc, Wc, Dd, ws, ldet, status);
-      count();
+    for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
+      group_factor(s, st, q, X, Lc, Dd, ws, status);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_factor<<<nleft, NT, 0, st>>>(s->dev, left, X, Lc, Wc, Dd, ws, ldet, status);
+        count();
+      }
     }
     bf.join_now();
   }
+  group_factor_post(s, st, Lc, Wc, ws, ldet);
 }
 // Cholesky product X = L D L^T on V (Algorithm 3.2), bottom-up like the factor.
 void product(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Lc, double* X, double* ws) {
@@ -1242,15 +1275,22 @@ void product(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doubl
 void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Wc, double* Sc, double* g,
               double* Vd, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  group_zero(s, st, 1, ws);
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_gradient(s, sl, big_front(s, v, i), Wc, Sc, g, Vd, ws);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_gradient(s, sl, dense[i], Wc, Sc, g, Vd, ws);
     });
-    if (v.ncta) {
-      k_gradient<<<v.ncta, NT, 0, st>>>(s->dev, v.tc, Wc, Sc, g, Vd, ws);
-      count();
+    for (int q = s->glvl[l + 1] - 1; q >= s->glvl[l]; --q) {
+      group_gradient(s, st, q, Wc, Sc, g, Vd, ws);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_gradient<<<nleft, NT, 0, st>>>(s->dev, left, Wc, Sc, g, Vd, ws);
+        count();
+      }
     }
     if (v.nr32 + v.nr64) chain_gradient(s, st, v.tr, v.nr32 + v.nr64, Wc, Sc, g, Vd, ws);
     if (v.nwarp) w32::warp_gradient(s, st, v.t0, v.nwarp, Wc, Sc, g, Vd, ws);
@@ -1266,31 +1306,45 @@ void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m,
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_hess_up(s, sl, m, big_front(s, v, i), Wc, Vd, Y, ldy, T, ldt, ws, act);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_hess_up(s, sl, m, dense[i], Wc, Vd, Y, ldy, T, ldt, ws, act);
     });
     if (v.nr32 + v.nr64) chain_hess_up(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
     if (v.nwarp) w32::warp_hess_up(s, st, v.t0, v.nwarp, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
     if (v.nw64) w64::warp_hess_up(s, st, v.tw, v.nw64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
-    if (v.ncta) {
-      k_hess_up<<<dim3(v.ncta, m), NT, 0, st>>>(D, v.tc, Wc, Vd, Y, ldy, T, ldt, ws);
-      count();
+    for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
+      group_hess_up(s, st, q, m, Wc, Y, ldy, ws, act);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_hess_up<<<dim3(nleft, m), NT, 0, st>>>(D, left, Wc, Vd, Y, ldy, T, ldt, ws);
+        count();
+      }
     }
     bf.join_now();
   }
+  group_hess_m(s, st, m, Wc, Vd, T, ldt, ws, act);
 }
 void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, double* T,
                     int64_t ldt, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  group_zero(s, st, m, ws);
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_hess_down(s, sl, m, big_front(s, v, i), Wc, T, ldt, ws);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_hess_down(s, sl, m, dense[i], Wc, T, ldt, ws);
     });
-    if (v.ncta) {
-      k_hess_down<<<dim3(v.ncta, m), NT, 0, st>>>(s->dev, v.tc, Wc, T, ldt, ws);
-      count();
+    for (int q = s->glvl[l + 1] - 1; q >= s->glvl[l]; --q) {
+      group_hess_down(s, st, q, m, Wc, T, ldt, ws);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_hess_down<<<dim3(nleft, m), NT, 0, st>>>(s->dev, left, Wc, T, ldt, ws);
+        count();
+      }
     }
     if (v.nr32 + v.nr64) chain_hess_down(s, st, v.tr, v.nr32 + v.nr64, m, Wc, T, ldt, ws);
     if (v.nwarp) w32::warp_hess_down(s, st, v.t0, v.nwarp, m, Wc, T, ldt, ws);
@@ -1338,30 +1392,43 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_ihess_down(s, sl, m, big_front(s, v, i), Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_ihess_down(s, sl, m, dense[i], Wc, Dd, Rd, T, ldt, Y, ldy, ws);
     });
-    if (v.ncta) {
-      k_ihess_down<<<dim3(v.ncta, m), NT, 0, st>>>(s->dev, v.tc, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
-      count();
+    for (int q = s->glvl[l + 1] - 1; q >= s->glvl[l]; --q) {
+      group_ihess_gather(s, st, q, m, T, ldt, ws);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_ihess_down<<<dim3(nleft, m), NT, 0, st>>>(s->dev, left, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+        count();
+      }
     }
     if (v.nr32 + v.nr64) chain_ihess_down(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
     if (v.nwarp) w32::warp_ihess_down(s, st, v.t0, v.nwarp, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
     if (v.nw64) w64::warp_ihess_down(s, st, v.tw, v.nw64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
     bf.join_now();
   }
+  group_ihess_k(s, st, m, Wc, Dd, Rd, Y, ldy, ws);
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_ihess_up(s, sl, m, big_front(s, v, i), Wc, Y, ldy, ws);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_ihess_up(s, sl, m, dense[i], Wc, Y, ldy, ws);
     });
     if (v.nr32 + v.nr64) chain_ihess_up(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Y, ldy, ws);
     if (v.nwarp) w32::warp_ihess_up(s, st, v.t0, v.nwarp, m, Wc, Y, ldy, ws);
     if (v.nw64) w64::warp_ihess_up(s, st, v.tw, v.nw64, m, Wc, Y, ldy, ws);
-    if (v.ncta) {
-      k_ihess_up<<<dim3(v.ncta, m), NT, 0, st>>>(s->dev, v.tc, Wc, Y, ldy, ws);
-      count();
+    for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
+      group_ihess_up(s, st, q, m, Wc, Y, ldy, ws);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_ihess_up<<<dim3(nleft, m), NT, 0, st>>>(s->dev, left, Wc, Y, ldy, ws);
+        count();
+      }
     }
     bf.join_now();
   }
@@ -1412,17 +1479,20 @@ void big_inv_v(const chd_symbolic* s, const Slot& sl, int k, const double* Vd,
                double* Rd, double* Qd, double* ws, int64_t* status, int what);
 void inv_v(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Vd, double* Rd, double* Qd,
            double* ws, int64_t* status, int what) {
-  // dense-tier fronts and the other fronts with a large V_k: multi-CTA
-  // kernels on the side streams; the rest: one CTA per front (k_inv_v)
+  // V^{-1} of the fronts of the grouped inverse: launches over all of them;
+  // other dense-tier fronts and large V_k: launch sequences on the side
+  // streams; the rest: one CTA per front (k_inv_v)
+  const bool grouped = what == 1;
   std::vector<int> bigs;
   for (int64_t k = 0; k < s->nsn; ++k)
-    if (s->is_big[k]) bigs.push_back((int)k);
+    if (s->is_big[k] && !(grouped && s->in_gj[k])) bigs.push_back((int)k);
   for (int32_t k : s->small_fronts)
-    if (front_J(s, k) - front_n(s, k) >= kInvVMulti) bigs.push_back((int)k);
+    if (front_J(s, k) - front_n(s, k) >= kInvVMulti && !(grouped && s->in_gj[k])) bigs.push_back((int)k);
   BigFork bf{ex, st};
   bf.run((int)bigs.size(), [&](int i, const Slot& sl) {
     big_inv_v(s, sl, bigs[i], Vd, Rd, Qd, ws, status, what);
   });
+  if (grouped) group_inv_v(s, st, Vd, Rd, ws, status);
   if (s->dev.small_count > 0) {
     k_inv_v<<<(int)s->dev.small_count, NT, 0, st>>>(s->dev, Vd, Rd, Qd, ws, status, s->dev.small_fronts, what);
     count();

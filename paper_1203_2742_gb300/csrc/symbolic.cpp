@@ -386,6 +386,193 @@ void factored_completion_plan(chd_symbolic* s) {
   }
 }
 
+// Work lists of the grouped tier (group_tier.cu): CTA-tier fronts, and dense
+// fronts of at most kGroupThin columns unless every dense product is forced
+// onto the tensor cores -- their products are skinny, 50 to 250 us each as
+// launches of their own on a 5000-vertex random pattern.
+static void group_plan(chd_symbolic* s) {
+  const int64_t nsn = s->nsn;
+  s->gidx.assign(nsn, -1);
+  for (auto* v : {&s->gptr, &s->gt_up, &s->gt_row, &s->gt_asm, &s->gt_p, &s->gt_gat, &s->gt_nn, &s->gt_asmf, &s->gt_wb,
+                  &s->gt_fr, &s->gleg, &s->gs_rn, &s->gs_np, &s->gs_thin})
+    v->clear();
+  for (auto* v : {&s->gs_up, &s->gs_row, &s->gs_asm, &s->gs_p, &s->gs_gat, &s->gs_asmf, &s->gs_wb, &s->gs_leg, &s->glvl})
+    v->assign(1, 0);
+  s->gf.clear();
+  s->gch.clear();
+  s->g_rnmax = s->g_nmax = 0;
+  auto blocks = [](int64_t v) { return (v + kGroupBlock - 1) / kGroupBlock; };
+  // rows per block of the row-block kernels: as few as the front's second
+  // temporary holds partial n x n sums for (and a counter); 16 or more for
+  // wide fronts, whose rows carry enough work
+  auto row_block = [](int64_t n, int64_t a) {
+    const int64_t J = n + a, np = n * (n + 1) / 2;
+    for (int l = n > kGroupThin ? 1 : 0; l <= 4; ++l) {
+      const int64_t R = int64_t(8) << l, nb = std::max<int64_t>(1, (a + R - 1) / R);
+      const int64_t part = a > 0 ? nb * np : 0;
+      if (part + 1 <= J * n && (4608 + 2 * R * n) * 8 <= kGroupSmem) return l;
+    }
+    return -1;
+  };
+  auto add = [&](int64_t k) {
+    const int64_t n = front_n(s, k), J = front_J(s, k), a = J - n;
+    const int l = row_block(n, a);
+    GFront f{};
+    f.base = s->colptr[s->sn_ptr[k]];
+    f.f_off = s->f_off[k];
+    const int64_t p = s->sn_par[k];
+    f.fp_off = p >= 0 ? s->f_off[p] : 0;
+    f.Jp = p >= 0 ? (int32_t)front_J(s, p) : 0;
+    f.d_off = s->d_off[k];
+    f.v_off = s->v_off[k];
+    f.rel_off = s->rows_ptr[k] + n;
+    f.k = (int32_t)k;
+    f.n = (int32_t)n;
+    f.a = (int32_t)a;
+    f.J = (int32_t)J;
+    f.lrb = l;
+    const int64_t R = int64_t(8) << l;
+    f.nb = (int32_t)std::max<int64_t>(1, (a + R - 1) / R);
+    f.nbn = (int32_t)blocks(n);
+    f.ch_beg = (int32_t)s->gch.size();
+    const int64_t nblk = f.nbn + blocks(a);
+    auto first_row = [&](int64_t b) { return b < f.nbn ? b * kGroupBlock : std::min(J, n + (b - f.nbn) * kGroupBlock); };
+    for (int64_t q = s->ea_ptr[k]; q < s->ea_ptr[k + 1]; ++q) {
+      const int64_t c = s->ea[q], nc = front_n(s, c), Jc = front_J(s, c);
+      GChild g{};
+      g.u_off = s->f_off[c] + nc + nc * Jc;
+      g.rel_off = s->rows_ptr[c] + nc;
+      g.Jc = (int32_t)Jc;
+      g.k = (int32_t)c;
+      g.ptr_off = (int32_t)s->gptr.size();
+      const int32_t* rel = s->rel.data() + g.rel_off;
+      for (int64_t b = 0; b <= nblk; ++b)
+        s->gptr.push_back(b == nblk ? (int32_t)(Jc - nc)
+                                    : (int32_t)(std::lower_bound(rel, rel + (Jc - nc), (int32_t)first_row(b)) - rel));
+      s->gch.push_back(g);
+    }
+    f.ch_end = (int32_t)s->gch.size();
+    const int32_t id = (int32_t)s->gf.size();
+    s->gidx[k] = id;
+    s->gf.push_back(f);
+    auto push = [&](std::vector<int32_t>& v, int64_t lo, int64_t hi) {
+      v.push_back(id);
+      v.push_back((int32_t)(lo | (hi << 16)));
+    };
+    const int64_t ba = std::max<int64_t>(1, blocks(a));
+    for (int64_t j = 0; j < ba; ++j)
+      for (int64_t i = j; i < ba; ++i) push(s->gt_up, i, j);
+    for (int64_t b = 0; b < f.nb; ++b) push(s->gt_row, b, 0);
+    for (int64_t j = 0; j < nblk; ++j)
+      for (int64_t i = j; i < nblk; ++i) {
+        push(s->gt_gat, i, j);
+        if (n > kGroupThin) push(s->gt_asm, i, j);
+        if (n > kGroupFactor) push(s->gt_asmf, i, j);
+      }
+    if (n > kGroupThin)
+      for (int64_t i = 0; i < blocks(a); ++i)
+        for (int64_t j = 0; j < f.nbn; ++j) push(s->gt_p, i, j);
+    for (int64_t b = 0; b < (n + 15) / 16; ++b) push(s->gt_nn, b, 0);
+    for (int64_t b = 0; b < nblk; ++b) {
+      push(s->gt_fr, b, 0);  // the blocks of A_k, then those of the identity
+      if (n > kGroupFactor) push(s->gt_wb, b, 0);
+    }
+    if (n > kGroupFactor) s->gs_np.back() = std::max(s->gs_np.back(), f.nbn);
+    else s->gs_thin.back() = 1;
+    s->gs_rn.back() = std::max(s->gs_rn.back(), (int32_t)(R * n));
+    s->g_rnmax = std::max(s->g_rnmax, (int)(R * n));
+    s->g_nmax = std::max(s->g_nmax, (int)n);
+  };
+  auto eligible = [&](int64_t k) {
+    const int64_t n = front_n(s, k), a = front_J(s, k) - n;
+    if (n > kGroupCols || a > 65535 * (int64_t)kGroupBlock / 2 || row_block(n, a) < 0) return false;
+    if (s->tier[k] == 1) return true;
+    return s->tier[k] == 2 && n <= kGroupThin && s->tc_mode != 1;
+  };
+  const int64_t nlev = (int64_t)s->lvl_ptr.size() - 1;
+  for (int64_t l = 0; l < nlev; ++l) {
+    const int32_t* c = s->lvl_counts.data() + 5 * l;
+    const int32_t t1 = s->lvl_ptr[l + 1] - c[4], t0 = s->lvl_ptr[l] + c[0] + c[1] + c[2] + c[3];
+    for (int32_t i = 0;; ++i) {
+      std::vector<int64_t> in, out;
+      for (int32_t t = t0; t < t1; ++t)
+        if (s->task_ptr[t] + i < s->task_ptr[t + 1]) {
+          const int64_t k = s->task_fronts[s->task_ptr[t] + i];
+          (eligible(k) ? in : out).push_back(k);
+        }
+      if (i == 0)
+        for (int32_t t = t1; t < s->lvl_ptr[l + 1]; ++t) {
+          const int64_t k = s->task_fronts[s->task_ptr[t]];
+          if (eligible(k)) in.push_back(k);
+        }
+      if (in.empty() && out.empty()) break;
+      s->gs_rn.push_back(0);
+      s->gs_np.push_back(0);
+      s->gs_thin.push_back(0);
+      for (int64_t k : in) add(k);
+      for (int64_t k : out) s->gleg.push_back((int32_t)k);
+      s->gs_up.push_back((int32_t)s->gt_up.size() / 2);
+      s->gs_row.push_back((int32_t)s->gt_row.size() / 2);
+      s->gs_asm.push_back((int32_t)s->gt_asm.size() / 2);
+      s->gs_p.push_back((int32_t)s->gt_p.size() / 2);
+      s->gs_gat.push_back((int32_t)s->gt_gat.size() / 2);
+      s->gs_asmf.push_back((int32_t)s->gt_asmf.size() / 2);
+      s->gs_wb.push_back((int32_t)s->gt_wb.size() / 2);
+      s->gs_leg.push_back((int32_t)s->gleg.size());
+    }
+    s->glvl.push_back((int32_t)s->gs_rn.size());
+  }
+}
+
+// Work lists of the grouped inverse of V_k (kv_* in group_tier.cu).
+static void group_inverse_plan(chd_symbolic* s) {
+  s->gj.clear();
+  s->in_gj.assign(s->nsn, 0);
+  for (auto* v : {&s->gv_all, &s->gv_sol, &s->gv_upd}) v->clear();
+  s->gv_sol_ptr.assign(1, 0);
+  s->gv_upd_ptr.assign(1, 0);
+  for (int64_t k = 0; k < s->nsn; ++k) {
+    const int64_t a = front_J(s, k) - front_n(s, k);
+    if (a < kInvVGroupMin || a > kInvVGroup || (s->is_big[k] && s->tc_mode == 1)) continue;
+    if (s->grp_of[k] >= 0 && s->grp_first[s->grp_of[k]] != k) continue;  // a leaf group shares one V
+    s->in_gj[k] = 1;
+    GJob j{};
+    j.v_off = s->v_off[k];
+    j.w_off = s->f_off[k];
+    j.a = (int32_t)a;
+    j.k = (int32_t)k;
+    s->gj.push_back(j);
+  }
+  std::stable_sort(s->gj.begin(), s->gj.end(), [](const GJob& x, const GJob& y) { return x.a > y.a; });
+  if (s->gj.empty()) return;
+  const int32_t nj = (int32_t)s->gj.size();
+  auto nblk = [&](int32_t f) { return (s->gj[f].a + kGroupBlock - 1) / kGroupBlock; };
+  auto push = [](std::vector<int32_t>& v, int32_t f, int32_t i, int32_t j, int32_t x) {
+    v.push_back(f);
+    v.push_back(i | (j << 10) | (x << 20));
+  };
+  for (int32_t f = 0; f < nj; ++f)
+    for (int32_t j = 0; j < nblk(f); ++j)
+      for (int32_t i = j; i < nblk(f); ++i) push(s->gv_all, f, i, j, 0);
+  const int32_t np = nblk(0);
+  for (int32_t p = 0; p < np; ++p) {
+    for (int32_t f = 0; f < nj && nblk(f) > p; ++f) {
+      for (int32_t i = p + 1; i < nblk(f); ++i) push(s->gv_sol, f, i, 0, 0);
+      for (int32_t i = 0; i <= p; ++i) push(s->gv_sol, f, i, 0, 1);
+    }
+    s->gv_sol_ptr.push_back((int32_t)(s->gv_sol.size() / 2));
+    // the diagonal blocks first: their CTAs go on to factor them
+    for (int32_t f = 0; f < nj && nblk(f) > p + 1; ++f) push(s->gv_upd, f, p + 1, p + 1, 0);
+    for (int32_t f = 0; f < nj && nblk(f) > p + 1; ++f)
+      for (int32_t j = p + 1; j < nblk(f); ++j) {
+        for (int32_t i = j; i < nblk(f); ++i)
+          if (i > p + 1 || j > p + 1) push(s->gv_upd, f, i, j, 0);
+        for (int32_t i = 0; i <= p; ++i) push(s->gv_upd, f, i, j, 1);
+      }
+    s->gv_upd_ptr.push_back((int32_t)(s->gv_upd.size() / 2));
+  }
+}
+
 chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* rowind,
                               const chd_opts& opts, chd_symbolic* s) {
   if (n < 1 || !colptr || !rowind) return CHD_ERR_INVALID;
@@ -932,5 +1119,7 @@ chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* r
     }
   }
   factored_completion_plan(s);
+  group_plan(s);
+  group_inverse_plan(s);
   return CHD_OK;
 }
