@@ -148,8 +148,6 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
     auto column = [&](int c) {
       const int s0 = scol, sp = s0 == 0 ? W - 1 : s0 - 1, cur = c & 1, prv = cur ^ 1;
       scol = scol + 1 == W ? 0 : scol + 1;
-      cp_async_wait<AHEAD - 1>();
-      __syncwarp();
       double val[EL], l[EL];
       const double gs = c > i0 ? sm.g[prv][s0] : 0.0, fs = c > i0 ? sm.f[prv][s0] : 0.0;
 #pragma unroll
@@ -210,12 +208,18 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
       }
     };
     for (int c = i0; c < i0 + AHEAD; ++c) prefetch(c);
+    cp_async_wait<AHEAD - 1>();
+    __syncwarp();
     column(i0);
     bar(NT + 32);
     for (int i = i0; i < L; ++i) {
-      prefetch(i + AHEAD);
-      if (i + 1 < L) column(i + 1);
+      if (i + 1 < L) {
+        cp_async_wait<AHEAD - 2>();  // column i + 1
+        __syncwarp();
+        column(i + 1);
+      }
       bar(NT + 32);
+      prefetch(i + AHEAD);
     }
   } else {
     // ---- update warps: pairs (u, v), u >= v, of slots ----
@@ -434,30 +438,37 @@ __global__ void __launch_bounds__(MT) kc_hess_m(SymDev S, int task0, const doubl
 //
 // The window covers the a rows c+1 .. c+a while column c is in work, row rho
 // in slot rho mod a (row c takes the slot of row c + a).  Four threads hold
-// a row each, entries v = part, part + 4, ..; per column they multiply the
-// window with L_A (a = 61: 128 FP64 warp instructions), reduce over the four,
-// and after a barrier the new row is formed once, and after another taken
-// over into the registers.  The new diagonal entry needs a whole dot product;
-// warp 0 forms it during the next column's product, whose one affected row
-// gets the missing term afterwards.  Warp 0 also loads the inputs and stores
-// the outputs.
+// a row each, entries v = part, part + 4, ..  Per column:
+//   phase 1: they multiply the window with L_A (a = 61: 128 FP64 warp
+//     instructions) and reduce over the four;
+//   barrier; phase 2: T_A = M_A - w, once per entry; barrier; the new row
+//     goes into the registers.
+// The new diagonal entry, T_cc = (M_cc - 2 L_A^T M_A) + L_A^T w, needs a dot
+// product over all rows: warp 0 takes w after the first barrier, passes the
+// second without waiting and has until the next column's phase 2, where the
+// one product that the missing entry enters is corrected.  (The bracket does
+// not depend on the recursion: kc_down_pre forms it for all columns.)  Warp 0
+// also loads the inputs.
 // ---------------------------------------------------------------------------
 struct DownSmem {
-  double ring[2][RING][WP];  // L_A (slots), and M_A; [.][WP - 1]: the diagonal's value
+  double ring[2][RING][WP];  // L_A (slots), and M_A; [.][WP - 1]: the diagonal's part known beforehand
   double wv[WP], tv[2][WP], dg[2];
 };
 enum { DOWN_GRAD = 0, DOWN_HESS = 1 };
+// second barrier of a column: the window threads wait, warp 0 only arrives
+__device__ __forceinline__ void bar2_sync(int n) { asm volatile("bar.sync 2, %0;\n" ::"r"(n) : "memory"); }
+__device__ __forceinline__ void bar2_arrive(int n) { asm volatile("bar.arrive 2, %0;\n" ::"r"(n) : "memory"); }
 template <int NT, int CP, int TP, int MODE>
 __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const double* src, double* out,
                          const double* ws, DownSmem& sm) {
   const int a = R.a, W = a + 1, tid = threadIdx.x, L = R.L;
   if (tid >= NT + 32) return;
   // slots past the window are multiplied by zeros: they must hold numbers
-  for (int e = tid; e < RING * WP; e += NT + 32) (&sm.ring[0][0][0])[e] = 0.0;
+  for (int e = tid; e < 2 * RING * WP; e += NT + 32) (&sm.ring[0][0][0])[e] = 0.0;
   bar(NT + 32);
   if (tid < 32) {
     const int lane = tid;
-    int sload = (L - 1) % a, sfin = (L - 1) % a;
+    int sload = (L - 1) % a;
     auto prefetch = [&](int c) {
       if (c >= 0) {
         const int sc = sload;
@@ -472,42 +483,37 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
       }
       cp_async_commit();
     };
-    // the diagonal of column c, and the column's output
     int steps = 1;
     while (steps < 32 && steps < a) steps <<= 1;
-    auto finish = [&](int c) {
+    for (int c = L - 1; c > L - 1 - AHEAD; --c) prefetch(c);
+    cp_async_wait<AHEAD - 1>();
+    bar(NT + 32);
+    int s1 = -1;  // slot of row c + 1, whose diagonal entry d the window lacks
+    double d = 0.0;
+    for (int c = L - 1; c >= 0; --c) {
+      cp_async_wait<AHEAD - 2>();  // column c - 1 has arrived
+      bar(NT + 32);
       const double* l = sm.ring[0][c % RING];
-      const double* mm = sm.ring[1][c % RING];
-      const double* t = sm.tv[c & 1];
-      const double m0 = MODE == DOWN_HESS ? mm[WP - 1] : l[WP - 1];
-      double acc = 0.0;
-      for (int v = lane; v < a; v += 32) acc = fma(-l[v], MODE == DOWN_HESS ? t[v] + mm[v] : t[v], acc);
+      const double q = MODE == DOWN_HESS ? sm.ring[1][c % RING][WP - 1] : l[WP - 1];
+      const bool two = lane + 32 < a;
+      double w0 = lane < a ? sm.wv[lane] : 0.0, w1 = two ? sm.wv[lane + 32] : 0.0;
+      const double l0 = lane < a ? l[lane] : 0.0, l1 = two ? l[lane + 32] : 0.0;
+      bar2_arrive(NT + 32);
+      if (s1 >= 0) {
+        if (s1 < 32) w0 = lane == s1 ? fma(d, l0, w0) : w0;
+        else w1 = lane == s1 - 32 ? fma(d, l1, w1) : w1;
+      }
+      double acc = fma(l0, w0, lane == 0 ? q : 0.0);
+      if (a > 32) acc = fma(l1, w1, acc);
       for (int o = steps >> 1; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-      const double d = m0 + acc;
+      d = __shfl_sync(0xffffffffu, acc, 0);
       if (lane == 0) {
         sm.dg[c & 1] = d;
         out[(int64_t)c * W] = d;
       }
-      const int sc = sfin;
-      sfin = sfin == 0 ? a - 1 : sfin - 1;
-      for (int v = lane; v < a; v += 32) {
-        int p = v - sc;
-        if (p <= 0) p += a;
-        out[(int64_t)c * W + p] = t[v];
-      }
-    };
-    for (int c = L - 1; c > L - 1 - AHEAD; --c) prefetch(c);
-    cp_async_wait<AHEAD - 1>();
-    bar(NT + 32);
-    for (int c = L - 1; c >= 0; --c) {
-      if (c + 1 < L) finish(c + 1);
+      s1 = s1 < 0 ? (L - 1) % a : (s1 == 0 ? a - 1 : s1 - 1);
       prefetch(c - AHEAD);
-      cp_async_wait<AHEAD - 1>();  // column c - 1 has arrived
-      bar(NT + 32);
-      bar(NT + 32);
     }
-    __syncwarp();
-    finish(0);
   } else {
     const int rt = tid - 32, u = rt / TP, part = rt % TP;
     double V[CP];
@@ -551,10 +557,14 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
       if (rt < a) {
         double w = sm.wv[rt];
         if (rt == s1) w = fma(dnew, l[rt], w);
-        tv[rt] = MODE == DOWN_HESS ? mm[rt] - w : -w;
+        const double t = MODE == DOWN_HESS ? mm[rt] - w : -w;
+        tv[rt] = t;
+        int p = rt - s;
+        if (p <= 0) p += a;
+        out[(int64_t)c * W + p] = t;
       }
-      bar(NT + 32);
-      // the new row into the registers: column slot s of every row, the four
+      bar2_sync(NT + 32);
+      // the new row into the registers: column slot s of every row, the
       // threads of row slot s, and the diagonal entry of the row before
       const double mine = u < a ? tv[u] : 0.0;
       const int js = s / TP, ps = s % TP;
@@ -625,8 +635,22 @@ __global__ void __launch_bounds__(MT) kc_grad_post(SymDev S, int task0, const do
   }
 }
 // Algorithm 5.1 step 3 for one-column fronts: with w = V' L_A, T_A = M_A - w,
-// T_jj = M_jj - L_A^T (T_A + M_A); V' of the child = [T_jj T_A^T; T_A V'] on
-// its rows.  T in place.
+// T_jj = M_jj - 2 L_A^T M_A + L_A^T w; V' of the child = [T_jj T_A^T; T_A V']
+// on its rows.  T in place; first
+// what of T_jj does not depend on the recursion, in place: M_jj - 2 L_A^T M_A
+__global__ void __launch_bounds__(128) kc_down_pre(SymDev S, int task0, const double* Wc, double* T, int64_t ldt) {
+  const Run R = run_of(S, task0 + blockIdx.x);
+  const int lane = threadIdx.x & 31, W = R.a + 1;
+  T += (int64_t)blockIdx.z * ldt + R.base0;
+  for (int i = blockIdx.y * 4 + (threadIdx.x >> 5); i < R.L; i += gridDim.y * 4) {
+    double* t = T + (int64_t)i * W;
+    const double* l = Wc + R.base0 + (int64_t)i * W;
+    double acc = 0.0;
+    for (int p = 1 + lane; p < W; p += 32) acc = fma(l[p], t[p], acc);
+    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+    if (lane == 0) t[0] = fma(-2.0, acc, t[0]);
+  }
+}
 __global__ void __launch_bounds__(DNT) kc_hess_down(SymDev S, int task0, const double* Wc, double* T, int64_t ldt,
                                                    const double* ws) {
   __shared__ DownSmem sm;
@@ -779,6 +803,8 @@ void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m
 }
 void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
                      int64_t ldt, double* ws) {
+  kc_down_pre<<<dim3(nt, columns(s, t0, nt, 4, 0), m), 128, 0, st>>>(s->dev, t0, Wc, T, ldt);
+  count_launch();
   kc_hess_down<<<dim3(nt, m), DNT, 0, st>>>(s->dev, t0, Wc, T, ldt, ws);
   count_launch();
 }
