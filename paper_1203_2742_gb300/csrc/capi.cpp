@@ -1003,6 +1003,11 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
                                        &s->gt_nn, &s->gt_asmf, &s->gt_wb,  &s->gt_fr};
   for (int i = 0; i < 9; ++i) iGt[i] = add(gt[i]->data(), gt[i]->size() * 4);
   size_t iGl = add(s->gleg.data(), s->gleg.size() * 4);
+  size_t iGc2 = add(s->gc.data(), s->gc.size() * sizeof(GComp));
+  size_t iGq[8];
+  const std::vector<int32_t>* gq[8] = {&s->gc_all, &s->gc_sol,  &s->gc_upd,  &s->gc_back,
+                                       &s->gc_b,   &s->gc_thin, &s->gc_wide, &s->gc_rest};
+  for (int i = 0; i < 8; ++i) iGq[i] = add(gq[i]->data(), gq[i]->size() * 4);
   size_t iGj = add(s->gj.data(), s->gj.size() * sizeof(GJob));
   size_t iGva = add(s->gv_all.data(), s->gv_all.size() * 4);
   size_t iGvs = add(s->gv_sol.data(), s->gv_sol.size() * 4);
@@ -1077,6 +1082,11 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   const int2** dgt[9] = {&d.gt_up, &d.gt_row, &d.gt_asm, &d.gt_p, &d.gt_gat, &d.gt_nn, &d.gt_asmf, &d.gt_wb, &d.gt_fr};
   for (int i = 0; i < 9; ++i) *dgt[i] = reinterpret_cast<const int2*>(b + pcs[iGt[i]].off);
   d.gleg = reinterpret_cast<const int32_t*>(b + pcs[iGl].off);
+  d.gc = reinterpret_cast<const GComp*>(b + pcs[iGc2].off);
+  const int2** dq[5] = {&d.gc_all, &d.gc_sol, &d.gc_upd, &d.gc_back, &d.gc_b};
+  for (int i = 0; i < 5; ++i) *dq[i] = reinterpret_cast<const int2*>(b + pcs[iGq[i]].off);
+  const int32_t** dl[3] = {&d.gc_thin, &d.gc_wide, &d.gc_rest};
+  for (int i = 0; i < 3; ++i) *dl[i] = reinterpret_cast<const int32_t*>(b + pcs[iGq[5 + i]].off);
   d.gj = reinterpret_cast<const GJob*>(b + pcs[iGj].off);
   d.gv_all = reinterpret_cast<const int2*>(b + pcs[iGva].off);
   d.gv_sol = reinterpret_cast<const int2*>(b + pcs[iGvs].off);

@@ -56,6 +56,12 @@ struct alignas(16) GJob {
   int32_t a, k;
 };
 
+// grouped completion: one front, blocks of its S-front in the order (A, N)
+struct alignas(16) GComp {
+  int64_t base, f_off, v_off, d_off, rows_off;
+  int32_t k, n, a, J, nA, pad;
+};
+
 // Device copy of the symbolic data, passed by value to every kernel.
 struct SymDev {
   int64_t n = 0;
@@ -104,6 +110,9 @@ struct SymDev {
   const int32_t* gleg = nullptr;
   const GJob* gj = nullptr;
   const int2 *gv_all = nullptr, *gv_sol = nullptr, *gv_upd = nullptr;
+  const GComp* gc = nullptr;
+  const int2 *gc_all = nullptr, *gc_sol = nullptr, *gc_upd = nullptr, *gc_back = nullptr, *gc_b = nullptr;
+  const int32_t *gc_thin = nullptr, *gc_wide = nullptr, *gc_rest = nullptr;
   const int64_t* inst_sn = nullptr;       // instances x supernode ranges
   int64_t ninst = 1;
   int64_t f_total = 0;               // workspace doubles per right-hand side
@@ -191,6 +200,13 @@ struct chd_symbolic {
   std::vector<GJob> gj;
   std::vector<char> in_gj;  // per supernode
   std::vector<int32_t> gv_all, gv_sol, gv_upd, gv_sol_ptr, gv_upd_ptr;
+  // grouped completion: fronts by decreasing a and the lists of its steps;
+  // gc_thin: indices of fronts of at most 32 columns, gc_wide: supernodes of
+  // the others, gc_rest: CTA-tier supernodes outside the grouped form
+  std::vector<GComp> gc;
+  std::vector<char> in_gc;
+  std::vector<int32_t> gc_all, gc_sol, gc_upd, gc_sol_ptr, gc_upd_ptr, gc_back, gc_b, gc_thin, gc_wide, gc_rest;
+  int gc_amax = 0;
   // device mirror
   SymDev dev;
   void* dev_buf = nullptr;

@@ -1152,6 +1152,307 @@ __global__ void __launch_bounds__(RT) kg_factor_nn(SymDev S, const int2* blocks,
   }
 }
 
+// ---------------------------------------------------------------------------
+// Cholesky product (Algorithm 3.2): block pair (bi, bj) of the front =
+// children's blocks + G G^T, G = [C; B] (Lc); N columns to the output, the
+// A x A block to F for the parent.  Only the additions wait for the children,
+// so the product G G^T comes first in each CTA.  17 x 20 x 13 grid: 23.1 ms
+// (one CTA per front) before.
+// ---------------------------------------------------------------------------
+__global__ void __launch_bounds__(256) kg_product(SymDev S, const int2* tiles, const double* Lc, double* Xo,
+                                                 double* ws) {
+  __shared__ double t[GB][GB + 1], A[GB][GB + 1], B[GB][GB + 1];
+  const int2 d = tiles[blockIdx.x];
+  const GFront f = S.gf[d.x];
+  const int bi = d.y & 0xffff, bj = d.y >> 16, tid = threadIdx.x, n = f.n, J = f.J;
+  int fi, ni, fj, nj;
+  block_range(f, bi, fi, ni);
+  block_range(f, bj, fj, nj);
+  const double* L = Lc + f.base;
+  Acc2 s{};
+  const int kmax = min(n, fj + nj);  // G(c, k) = 0 for k > c
+  const int r = tid & 31;
+  for (int k0 = 0; k0 < kmax; k0 += GB) {
+    const int kc = min(GB, kmax - k0);
+    for (int k = tid >> 5; k < GB; k += 8) {
+      const int kk = k0 + k;
+      A[k][r] = k < kc && r < ni && fi + r >= kk ? L[csc_off(J, fi + r, kk)] : 0.0;
+      if (bi != bj) B[k][r] = k < kc && r < nj && fj + r >= kk ? L[csc_off(J, fj + r, kk)] : 0.0;
+    }
+    __syncthreads();
+    block_product(s, A, bi == bj ? A : B, 0, kc);
+    __syncthreads();
+  }
+  const int tr = tid & 15, tc = tid >> 4;
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int w = 0; w < 2; ++w) t[tr + 16 * u][tc + 16 * w] = s.v[u][w];
+  __syncthreads();
+  for (int q = f.ch_beg; q < f.ch_end; ++q) {
+    add_child(S, S.gch[q], ws, bi, fi, bj, fj, &t[0][0], GB + 1);
+    __syncthreads();
+  }
+  double* F = ws + f.f_off;
+  if (r < ni)
+    for (int c = tid >> 5; c < nj; c += 8) {
+      const int row = fi + r, col = fj + c;
+      if (row < col) continue;
+      if (col < n) Xo[f.base + csc_off(J, row, col)] = t[r][c];
+      else F[row + (int64_t)col * J] = t[r][c];
+    }
+}
+
+// ---------------------------------------------------------------------------
+// Completion (Algorithm 7.3) of all the tier's fronts at once: the S-front in
+// the order (A_k, N_k) goes through a partial Cholesky factorisation of its A
+// columns in panels of 32, which leaves R = chol(V_k), Z^T = (R^{-1} S_AN)^T
+// in the N rows and P = S_NN - Z^T Z = D_NN^{-1} in the N block; then
+// L_AN^T = -Z^T R^{-1} by back substitution, D_NN = P^{-1}, C = chol(D_NN) and
+// B = L_AN C.  No front waits for another, so a panel step is one launch over
+// every front that still has one (fronts come by decreasing a), as in the
+// grouped inverse; one CTA per front took 4.0 ms on er5000 and left 40 dense
+// fronts to 5000 launches, 6.7 ms on a 17 x 20 x 13 grid.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void comp_block(const GComp& f, int b, int& first, int& count) {
+  if (b < f.nA) {
+    first = b * GB;
+    count = min(GB, f.a - first);
+  } else {
+    first = f.a + (b - f.nA) * GB;
+    count = min(GB, f.J - first);
+  }
+}
+__device__ __forceinline__ void comp_diag(double (*T)[GB + 1], double* rinv, double (*col)[GB], const GComp& f, int p,
+                                          double* F, int64_t* st) {
+  const int pb = min(GB, f.a - p * GB), tid = threadIdx.x;
+  __syncthreads();
+  if (tid < panel::PTH) panel::chol32(T, rinv, col, pb, tid, 1, st, CHD_ERR_NOT_COMPLETABLE, f.k, -1);
+  __syncthreads();
+  double* D = F + (int64_t)p * GB * (f.J + 1);
+  const int r = tid & 31;
+  for (int c = tid >> 5; c < pb; c += 8)
+    if (r < pb && r >= c) D[r + (int64_t)c * f.J] = T[r][c];
+}
+__global__ void __launch_bounds__(256) kp_init(SymDev S, const int2* tiles, const double* Sin, double* Vd, double* ws,
+                                              int64_t* st) {
+  __shared__ double T[GB][GB + 1], rinv[GB], col[3][GB];
+  const int2 d = tiles[blockIdx.x];
+  const GComp f = S.gc[d.x];
+  const int i = d.y & 1023, j = (d.y >> 10) & 1023, r = threadIdx.x & 31;
+  int fi, ni, fj, nj;
+  comp_block(f, i, fi, ni);
+  comp_block(f, j, fj, nj);
+  double* F = ws + f.f_off;
+  const int32_t* A = S.rows + f.rows_off + f.n;
+  for (int c = threadIdx.x >> 5; c < GB; c += 8) {
+    const int row = fi + r, cc = fj + c;
+    const bool in = r < ni && c < nj && row >= cc;
+    double v = i == j && r == c ? 1.0 : 0.0;
+    if (in) {
+      if (cc >= f.a) v = Sin[f.base + csc_off(f.J, row - f.a, cc - f.a)];         // N x N
+      else if (row >= f.a) v = Sin[f.base + csc_off(f.J, f.n + cc, row - f.a)];   // N x A
+      else {
+        v = Sin[csc_find(S, __ldg(A + row), __ldg(A + cc))];
+        Vd[f.v_off + row + (int64_t)cc * f.a] = v;
+      }
+      if (i > 0 || j > 0 || f.a == 0) F[row + (int64_t)cc * f.J] = v;
+    }
+    T[r][c] = v;
+  }
+  if (i == 0 && j == 0 && f.a > 0) comp_diag(T, rinv, col, f, 0, F, st);
+}
+__global__ void __launch_bounds__(128) kp_solve(SymDev S, const int2* blocks, int p, double* ws) {
+  __shared__ double Ls[GB][GB + 1], rinv[GB];
+  const int2 d = blocks[blockIdx.x];
+  const GComp f = S.gc[d.x];
+  const int tid = threadIdx.x, J = f.J, pb = min(GB, f.a - p * GB);
+  int fi, ni;
+  comp_block(f, d.y & 1023, fi, ni);
+  double* F = ws + f.f_off;
+  const double* D = F + (int64_t)p * GB * (J + 1);
+  for (int e = tid; e < GB * GB; e += 128) {
+    const int i = e & 31, c = e >> 5;
+    Ls[i][c] = i < pb && c < pb && i >= c ? D[i + (int64_t)c * J] : 0.0;
+  }
+  const int row = tid >> 2, q = tid & 3;
+  const bool ok = row < ni;
+  double* B = F + fi + (ok ? row : 0) + (int64_t)p * GB * J;
+  double b[8];
+#pragma unroll
+  for (int u = 0; u < 8; ++u) b[u] = ok && q + 4 * u < pb ? B[(int64_t)(q + 4 * u) * J] : 0.0;
+  __syncthreads();
+  if (tid < GB) rinv[tid] = tid < pb ? 1.0 / Ls[tid][tid] : 0.0;
+  __syncthreads();
+  if ((tid & ~31) / 4 >= ni) return;  // whole warps beyond the block's rows
+  panel::solve_row(b, Ls, rinv, pb, tid & 31);
+#pragma unroll
+  for (int u = 0; u < 8; ++u)
+    if (ok && q + 4 * u < pb) B[(int64_t)(q + 4 * u) * J] = b[u];
+}
+__global__ void __launch_bounds__(256) kp_update(SymDev S, const int2* tiles, int p, double* ws, int64_t* st) {
+  __shared__ double A[GB][GB + 1], B[GB][GB + 1], rinv[GB], col[3][GB];
+  const int2 d = tiles[blockIdx.x];
+  const GComp f = S.gc[d.x];
+  const int i = d.y & 1023, j = (d.y >> 10) & 1023, tid = threadIdx.x, J = f.J;
+  const bool diag = i == p + 1 && j == p + 1 && p + 1 < f.nA;
+  int fi, ni, fj, nj;
+  comp_block(f, i, fi, ni);
+  comp_block(f, j, fj, nj);
+  double* F = ws + f.f_off;
+  const int p0 = p * GB, pe = min(f.a, p0 + GB);
+  stage_block(A, F, J, fi, p0, fi + ni, pe);
+  if (i != j) stage_block(B, F, J, fj, p0, fj + nj, pe);
+  __syncthreads();
+  Acc2 s{};
+  block_product(s, A, i == j ? A : B, 0, pe - p0);
+  if (diag) __syncthreads();  // A is reused for the block to factor
+  const int tr = tid & 15, tc = tid >> 4;
+#pragma unroll
+  for (int u = 0; u < 2; ++u)
+#pragma unroll
+    for (int w = 0; w < 2; ++w) {
+      const int r = tr + 16 * u, c = tc + 16 * w;
+      double v = r == c ? 1.0 : 0.0;
+      if (r < ni && c < nj) {
+        v = 0.0;
+        if (fi + r >= fj + c) {
+          double* o = F + (fi + r) + (int64_t)(fj + c) * J;
+          v = *o - s.v[u][w];
+          if (!diag) *o = v;
+        }
+      }
+      if (diag) A[r][c] = v;
+    }
+  if (diag) comp_diag(A, rinv, col, f, p + 1, F, st);
+}
+// L_AN^T = -Z^T R^{-1}, eight rows (columns of N_k) per CTA, through all panels
+constexpr int BR = 8;
+__global__ void __launch_bounds__(128) kp_back(SymDev S, const int2* blocks, double* Wc, const double* ws) {
+  extern __shared__ double rows[];  // BR x (a + 1)
+  __shared__ double Ls[GB][GB + 1], rinv[GB];
+  const int2 d = blocks[blockIdx.x];
+  const GComp f = S.gc[d.x];
+  const int tid = threadIdx.x, lane = tid & 31, J = f.J, a = f.a, ld = a + 1;
+  const int r0 = d.y * BR, nr = min(BR, f.n - r0);
+  const double* F = ws + f.f_off;
+  for (int c = tid / BR; c < a; c += 128 / BR) {
+    const int r = tid & (BR - 1);
+    if (r < nr) rows[r * ld + c] = -F[a + r0 + r + (int64_t)c * J];
+  }
+  for (int p = f.nA - 1; p >= 0; --p) {
+    const int p0 = p * GB, pb = min(GB, a - p0);
+    __syncthreads();
+    for (int e = tid; e < GB * GB; e += 128) {
+      const int i = e & 31, c = e >> 5;
+      Ls[i][c] = i < pb && c <= i ? F[(p0 + i) + (int64_t)(p0 + c) * J] : 0.0;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      rinv[lane] = lane < pb ? 1.0 / Ls[lane][lane] : 0.0;
+      __syncwarp();
+      const int row = lane >> 2, q = lane & 3;
+      double b[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) b[u] = row < nr && q + 4 * u < pb ? rows[row * ld + p0 + q + 4 * u] : 0.0;
+#pragma unroll
+      for (int c = GB - 1; c >= 0; --c) {
+        if (c < pb) {
+          double x = b[c >> 2] * rinv[c];
+          x = __shfl_sync(0xffffffffu, x, (lane & 28) | (c & 3));
+          if (q == (c & 3)) b[c >> 2] = x;
+#pragma unroll
+          for (int u = 0; u <= c >> 2; ++u)
+            if (4 * u < c) b[u] = fma(4 * u + q < c ? -Ls[c][4 * u + q] : 0.0, x, b[u]);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (row < nr && q + 4 * u < pb) rows[row * ld + p0 + q + 4 * u] = b[u];
+    }
+    __syncthreads();
+    // the columns left of the panel: b_c -= x_p R_pc
+    for (int e = tid; e < nr * p0; e += 128) {
+      const int r = e % nr, c = e / nr;
+      const double* R = F + p0 + (int64_t)c * J;
+      double acc = 0.0;
+      for (int k = 0; k < pb; ++k) acc = fma(rows[r * ld + p0 + k], __ldg(R + k), acc);
+      rows[r * ld + c] -= acc;
+    }
+  }
+  __syncthreads();
+  for (int r = 0; r < nr; ++r)
+    for (int c = tid; c < a; c += 128) Wc[f.base + csc_off(J, f.n + c, r0 + r)] = rows[r * ld + c];
+}
+// fronts of up to 32 columns: P to Wc, D_NN = P^{-1}, C = chol(D_NN), log det
+__global__ void __launch_bounds__(128) kp_nn(SymDev S, const int32_t* list, double* Lc, double* Wc, double* Dd,
+                                            const double* ws, double* ldet, int64_t* st) {
+  __shared__ double P[GB][GB + 1], X[GB][GB + 1], rinv[GB], col[3][GB];
+  const GComp f = S.gc[list[blockIdx.x]];
+  const int tid = threadIdx.x, n = f.n, a = f.a, J = f.J;
+  const double* F = ws + f.f_off;
+  for (int e = tid; e < GB * GB; e += 128) {
+    const int i = e & 31, j = e >> 5;
+    double v = i == j ? 1.0 : 0.0;
+    if (i < n && j <= i) {
+      v = F[(a + i) + (int64_t)(a + j) * J];
+      Wc[f.base + csc_off(J, i, j)] = v;
+    }
+    P[i][j] = v;
+  }
+  __syncthreads();
+  panel::chol32(P, rinv, col, n, tid, 1, st, CHD_ERR_NOT_COMPLETABLE, f.k, S.sn_ptr[f.k]);
+  __syncthreads();
+  {  // X = Q^{-T} (rows of the identity)
+    const int row = tid >> 2, q = tid & 3;
+    double b[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) b[u] = row == q + 4 * u ? 1.0 : 0.0;
+    panel::solve_row(b, P, rinv, n, tid & 31);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) X[row][q + 4 * u] = b[u];
+  }
+  __syncthreads();
+  for (int e = tid; e < GB * GB; e += 128) {
+    const int i = e & 31, j = e >> 5;
+    double v = i == j ? 1.0 : 0.0;
+    if (i < n && j <= i) {
+      v = 0.0;
+      for (int k = i; k < n; ++k) v = fma(X[i][k], X[j][k], v);
+      Dd[f.d_off + i + (int64_t)j * n] = v;
+    } else if (j > i) {
+      v = 0.0;
+    }
+    P[i][j] = v;
+  }
+  __syncthreads();
+  panel::chol32(P, rinv, col, n, tid, 1, st, CHD_ERR_NOT_COMPLETABLE, f.k, S.sn_ptr[f.k]);
+  __syncthreads();
+  for (int e = tid; e < GB * GB; e += 128) {
+    const int i = e & 31, j = e >> 5;
+    if (i < n && j <= i) Lc[f.base + csc_off(J, i, j)] = P[i][j];
+  }
+  if (tid < 32) {
+    double s = tid < n ? 2.0 * log(P[tid][tid]) : 0.0;
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (tid == 0) ldet[f.k] = s;
+  }
+}
+// B = L_AN C, 32 rows per CTA
+__global__ void __launch_bounds__(128) kp_b(SymDev S, const int2* blocks, double* Lc, const double* Wc) {
+  const int2 d = blocks[blockIdx.x];
+  const GComp f = S.gc[d.x];
+  const int n = f.n, J = f.J, r0 = d.y * GB, nr = min(GB, f.a - r0);
+  const int r = threadIdx.x & 31;
+  if (r >= nr) return;
+  const int row = n + r0 + r;
+  for (int c = threadIdx.x >> 5; c < n; c += 4) {
+    double s = 0.0;
+    for (int k = c; k < n; ++k) s = fma(Wc[f.base + csc_off(J, row, k)], Lc[f.base + csc_off(J, k, c)], s);
+    Lc[f.base + csc_off(J, row, c)] = s;
+  }
+}
+
 }  // namespace grp
 }  // namespace chd
 
@@ -1323,5 +1624,45 @@ void group_factor_post(const chd_symbolic* s, cudaStream_t st, const double* Lc,
   count_launch();
   kg_factor_nn<<<nn, RT, 0, st>>>(s->dev, s->dev.gt_nn, Lc, Wc, ws, ldet);
   count_launch();
+}
+// Cholesky product of sub-level q
+void group_product(const chd_symbolic* s, cudaStream_t st, int q, const double* Lc, double* X, double* ws) {
+  const int t0 = s->gs_gat[q], nt = s->gs_gat[q + 1] - t0;
+  if (nt == 0) return;
+  kg_product<<<nt, 256, 0, st>>>(s->dev, s->dev.gt_gat + t0, Lc, X, ws);
+  count_launch();
+}
+// completion of the tier's fronts up to L_AN, and of those of at most 32
+// columns to the end
+void group_complete(const chd_symbolic* s, cudaStream_t st, const double* Sin, double* Lc, double* Wc, double* Dd,
+                    double* Vd, double* ws, double* ldet, int64_t* status) {
+  if (s->gc.empty()) return;
+  kp_init<<<(unsigned)(s->gc_all.size() / 2), 256, 0, st>>>(s->dev, s->dev.gc_all, Sin, Vd, ws, status);
+  count_launch();
+  for (size_t p = 0; p + 1 < s->gc_sol_ptr.size(); ++p) {
+    const int s0 = s->gc_sol_ptr[p], s1 = s->gc_sol_ptr[p + 1];
+    if (s1 > s0) {
+      kp_solve<<<s1 - s0, 128, 0, st>>>(s->dev, s->dev.gc_sol + s0, (int)p, ws);
+      count_launch();
+    }
+    const int u0 = s->gc_upd_ptr[p], u1 = s->gc_upd_ptr[p + 1];
+    if (u1 > u0) {
+      kp_update<<<u1 - u0, 256, 0, st>>>(s->dev, s->dev.gc_upd + u0, (int)p, ws, status);
+      count_launch();
+    }
+  }
+  if (!s->gc_back.empty()) {
+    kp_back<<<(unsigned)(s->gc_back.size() / 2), 128, (size_t)BR * (s->gc_amax + 1) * 8, st>>>(
+        s->dev, s->dev.gc_back, Wc, ws);
+    count_launch();
+  }
+  if (!s->gc_thin.empty()) {
+    kp_nn<<<(unsigned)s->gc_thin.size(), 128, 0, st>>>(s->dev, s->dev.gc_thin, Lc, Wc, Dd, ws, ldet, status);
+    count_launch();
+  }
+  if (!s->gc_b.empty()) {
+    kp_b<<<(unsigned)(s->gc_b.size() / 2), 128, 0, st>>>(s->dev, s->dev.gc_b, Lc, Wc);
+    count_launch();
+  }
 }
 }  // namespace chd_launch

@@ -686,6 +686,37 @@ __device__ void complete_load_front(const SymDev& S, int k, const double* Sin, d
   __syncthreads();
 }
 
+// ... from P = D_NN^{-1} (lower, in T1) and L_AN (in T2) on: D_NN, C, B and
+// the front's log det
+__device__ void complete_nn(const SymDev& S, const FrontInfo& f, double* Lc, double* Dd, double* ldet, int64_t* st) {
+  const int J = f.J, n = f.n, a = f.a, k = f.k;
+  // T2[0:n] = chol(P) = Q ; D = P^{-1} = Q^{-T} Q^{-1}
+  copy_lower(f.T2, J, f.T1, J, n);
+  __syncthreads();
+  cta_potrf_partial(f.T2, J, n, n, st, CHD_ERR_NOT_COMPLETABLE, k, f.col0);
+  double* Dk = Dd + S.d_off[k];
+  set_identity(Dk, n, n);
+  __syncthreads();
+  cta_trsm_rLT(n, n, DnTW{Dk, n}, f.T2, J);  // Dk = Q^{-1}
+  cta_gemm(n, n, n, 1.0, TriLT{Dk, n}, TriL{Dk, n}, 0.0, Dn{f.T1, J}, true);  // T1 = D (lower)
+  copy_lower(Dk, n, f.T1, J, n);
+  __syncthreads();
+  // C = chol(D) in T1[0:n]; B = L_AN C
+  cta_potrf_partial(f.T1, J, n, n, st, CHD_ERR_NOT_COMPLETABLE, k, f.col0);
+  for (int e = threadIdx.x; e < n * n; e += NT) {
+    int r = e % n, c = e / n;
+    if (r >= c) Lc[f.base + csc_off(J, r, c)] = f.T1[r + (int64_t)c * J];
+  }
+  cta_gemm(a, n, n, 1.0, Dn{f.T2 + n, J}, TriL{f.T1, J}, 0.0, Csc{Lc + f.base, J, n}, false);
+  if (threadIdx.x < 32) {
+    double s = 0.0;
+    for (int i = threadIdx.x; i < n; i += 32) s += 2.0 * log(f.T1[i + (int64_t)i * J]);
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x == 0) ldet[k] = s;
+  }
+  __syncthreads();
+}
+
 // Algorithm 7.3 arithmetic for one front whose S-front is loaded.  With Gq
 // (completion with factored update matrices), G = P R_k P of V_k = R_k R_k^T
 // is read from Gq instead of factoring V_k: the solves then run on S_AN and
@@ -723,47 +754,23 @@ __device__ void complete_front(const SymDev& S, int k, const double* Sin, double
     int r = e % J, c = e / J;
     if (r >= c) Wc[f.base + csc_off(J, r, c)] = (r < n) ? f.T1[r + (int64_t)c * J] : f.T2[r + (int64_t)c * J];
   }
-  // T2[0:n] = chol(P) = Q ; D = P^{-1} = Q^{-T} Q^{-1}
-  copy_lower(f.T2, J, f.T1, J, n);
-  __syncthreads();
-  cta_potrf_partial(f.T2, J, n, n, st, CHD_ERR_NOT_COMPLETABLE, k, f.col0);
-  double* Dk = Dd + S.d_off[k];
-  set_identity(Dk, n, n);
-  __syncthreads();
-  cta_trsm_rLT(n, n, DnTW{Dk, n}, f.T2, J);  // Dk = Q^{-1}
-  cta_gemm(n, n, n, 1.0, TriLT{Dk, n}, TriL{Dk, n}, 0.0, Dn{f.T1, J}, true);  // T1 = D (lower)
-  copy_lower(Dk, n, f.T1, J, n);
-  __syncthreads();
-  // C = chol(D) in T1[0:n]; B = L_AN C
-  cta_potrf_partial(f.T1, J, n, n, st, CHD_ERR_NOT_COMPLETABLE, k, f.col0);
-  for (int e = threadIdx.x; e < n * n; e += NT) {
-    int r = e % n, c = e / n;
-    if (r >= c) Lc[f.base + csc_off(J, r, c)] = f.T1[r + (int64_t)c * J];
-  }
-  cta_gemm(a, n, n, 1.0, Dn{f.T2 + n, J}, TriL{f.T1, J}, 0.0, Csc{Lc + f.base, J, n}, false);
-  if (threadIdx.x < 32) {
-    double s = 0.0;
-    for (int i = threadIdx.x; i < n; i += 32) s += 2.0 * log(f.T1[i + (int64_t)i * J]);
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-    if (threadIdx.x == 0) ldet[k] = s;
-  }
-  __syncthreads();
+  complete_nn(S, f, Lc, Dd, ldet, st);
 }
 
 // ---------------------------------------------------------------------------
 // kernels: blockIdx.x = task within the launch, blockIdx.y = right-hand side
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(NT) k_product(SymDev S, int task0, const double* Lc, double* X, double* ws) {
-  const int t = task0 + blockIdx.x;
-  for (int q = S.task_ptr[t]; q < S.task_ptr[t + 1]; ++q) product_front(S, S.task_fronts[q], Lc, X, ws);
-}
-// The factor, the gradient and the Hessian-type passes of the CTA-tier fronts
+// The factor, the product, the gradient and the Hessian-type passes of the CTA-tier fronts
 // that the grouped tier leaves out (wider than kGroupCols columns):
 // blockIdx.x = front of a sub-level's list
 __global__ void __launch_bounds__(NT) k_factor(SymDev S, const int32_t* list, const double* X, double* Lc,
                                                double* Wc, double* Dd, double* ws, double* ldet,
                                                int64_t* st) {
   factor_front(S, list[blockIdx.x], X, Lc, Wc, Dd, ws, ldet, st);
+}
+__global__ void __launch_bounds__(NT) k_product(SymDev S, const int32_t* list, const double* Lc, double* X,
+                                                double* ws) {
+  product_front(S, list[blockIdx.x], Lc, X, ws);
 }
 __global__ void __launch_bounds__(NT) k_gradient(SymDev S, const int32_t* list, const double* Wc, double* Sc,
                                                  double* g, double* Vd, double* ws) {
@@ -855,13 +862,31 @@ __global__ void __launch_bounds__(kScanT) k_active(SymDev S, int32_t* cnt, uint8
     act[y * S.nsn + k] = (c[hi] - (lo > 0 ? c[lo - 1] : 0)) > 0 ? 1 : 0;
   }
 }
-// all CTA-tier fronts at once, one CTA each
-__global__ void __launch_bounds__(NT) k_complete(SymDev S, const double* Sin, double* Lc, double* Wc, double* Dd,
-                                                 double* Vd, double* Rd, const double* Gq, double* ws, double* ldet,
-                                                 int64_t* st) {
-  const int k = S.cta_fronts[blockIdx.x];
+// fronts of `list` at once, one CTA each
+__global__ void __launch_bounds__(NT) k_complete(SymDev S, const int32_t* list, const double* Sin, double* Lc,
+                                                 double* Wc, double* Dd, double* Vd, double* Rd, const double* Gq,
+                                                 double* ws, double* ldet, int64_t* st) {
+  const int k = list[blockIdx.x];
   complete_load_front(S, k, Sin, ws);
   complete_front(S, k, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, st);
+}
+// the end of the grouped completion (group_tier.cu) for fronts wider than one
+// block: P is the N block of the S-front in the order (A, N), L_AN in Wc
+__global__ void __launch_bounds__(NT) k_complete_wide(SymDev S, const int32_t* list, double* Lc, double* Wc,
+                                                      double* Dd, double* ws, double* ldet, int64_t* st) {
+  const FrontInfo f = front_info(S, list[blockIdx.x], ws);
+  const int J = f.J, n = f.n, a = f.a;
+  copy_lower(f.T1, J, f.F + a + (int64_t)a * J, J, n);
+  for (int e = threadIdx.x; e < a * n; e += NT) {
+    const int r = e % a, c = e / a;
+    f.T2[n + r + (int64_t)c * J] = Wc[f.base + csc_off(J, n + r, c)];
+  }
+  __syncthreads();
+  for (int e = threadIdx.x; e < n * n; e += NT) {
+    const int r = e % n, c = e / n;
+    if (r >= c) Wc[f.base + csc_off(J, r, c)] = f.T1[r + (int64_t)c * J];
+  }
+  complete_nn(S, f, Lc, Dd, ldet, st);
 }
 // Completion with factored update matrices, one level of the clique tree
 // (parents done): G_k = P R_k P of every front of fc_fronts[first ..], one
@@ -1099,6 +1124,9 @@ void group_ihess_k(const chd_symbolic* s, cudaStream_t st, int m, const double* 
                    double* Y, int64_t ldy, double* ws);
 void group_ihess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const double* Wc, double* Y, int64_t ldy,
                     double* ws);
+void group_product(const chd_symbolic* s, cudaStream_t st, int q, const double* Lc, double* X, double* ws);
+void group_complete(const chd_symbolic* s, cudaStream_t st, const double* Sin, double* Lc, double* Wc, double* Dd,
+                    double* Vd, double* ws, double* ldet, int64_t* status);
 void group_inv_v(const chd_symbolic* s, cudaStream_t st, const double* Vd, double* Rd, double* ws, int64_t* status);
 
 // warp-tier launches (warp_tier.cu): w32 for |J| <= 32, w64 for |J| <= 64
@@ -1259,15 +1287,21 @@ void product(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doubl
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
-    bf.run(v.nbig, [&](int i, const Slot& sl) {
-      big_product(s, sl, big_front(s, v, i), Lc, X, ws);
+    const std::vector<int> dense = dense_fronts(s, v);
+    bf.run((int)dense.size(), [&](int i, const Slot& sl) {
+      big_product(s, sl, dense[i], Lc, X, ws);
     });
     if (v.nr32 + v.nr64) chain_product(s, st, v.tr, v.nr32 + v.nr64, Lc, X, ws);
     if (v.nwarp) w32::warp_product(s, st, v.t0, v.nwarp, Lc, X, ws);
     if (v.nw64) w64::warp_product(s, st, v.tw, v.nw64, Lc, X, ws);
-    if (v.ncta) {
-      k_product<<<v.ncta, NT, 0, st>>>(s->dev, v.tc, Lc, X, ws);
-      count();
+    for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
+      group_product(s, st, q, Lc, X, ws);
+      int nleft;
+      const int32_t* left = left_out(s, q, nleft);
+      if (nleft) {
+        k_product<<<nleft, NT, 0, st>>>(s->dev, left, Lc, X, ws);
+        count();
+      }
     }
     bf.join_now();
   }
@@ -1461,15 +1495,31 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
       bf.join_now();
     }
   }
-  std::vector<int32_t> bigs = s->big_fronts;  // dense fronts and leaf groups
+  // the grouped form (group_tier.cu) factors V_k itself; with Gq every front
+  // takes the per-front kernels
+  const bool grouped = !Gq;
+  std::vector<int32_t> bigs;  // dense fronts and leaf groups
+  for (int32_t k : s->big_fronts)
+    if (!(grouped && s->in_gc[k])) bigs.push_back(k);
   for (int64_t g0 : s->grp_first) bigs.push_back((int32_t)g0);
+  // the largest V_k first: its blocked Cholesky is the longest chain
+  std::stable_sort(bigs.begin(), bigs.end(), [&](int32_t x, int32_t y) {
+    return front_J(s, x) - front_n(s, x) > front_J(s, y) - front_n(s, y);
+  });
   BigFork bf{ex, st};
   bf.run((int)bigs.size(), [&](int i, const Slot& sl) {
     big_complete_load(s, sl.st, bigs[i], Sin, ws);
     big_complete(s, sl, bigs[i], Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, status);
   });
-  if (s->dev.cta_count > 0) {
-    k_complete<<<(int)s->dev.cta_count, NT, 0, st>>>(s->dev, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, status);
+  if (grouped) group_complete(s, st, Sin, Lc, Wc, Dd, Vd, ws, ldet, status);
+  if (grouped && !s->gc_wide.empty()) {
+    k_complete_wide<<<(int)s->gc_wide.size(), NT, 0, st>>>(s->dev, s->dev.gc_wide, Lc, Wc, Dd, ws, ldet, status);
+    count();
+  }
+  const int nrest = grouped ? (int)s->gc_rest.size() : (int)s->dev.cta_count;
+  if (nrest > 0) {
+    k_complete<<<nrest, NT, 0, st>>>(s->dev, grouped ? s->dev.gc_rest : s->dev.cta_fronts, Sin, Lc, Wc, Dd, Vd, Rd, Gq,
+                                     ws, ldet, status);
     count();
   }
   if (s->dev.warp_count > 0) w32::warp_complete_all(s, st, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ldet, status);

@@ -573,6 +573,76 @@ static void group_inverse_plan(chd_symbolic* s) {
   }
 }
 
+// Work lists of the grouped completion (kp_* in group_tier.cu): the CTA and
+// wide warp tiers, and dense fronts whose V_k is too small for its products
+// to gain from the tensor cores.
+static void group_completion_plan(chd_symbolic* s) {
+  s->gc.clear();
+  s->in_gc.assign(s->nsn, 0);
+  for (auto* v : {&s->gc_all, &s->gc_sol, &s->gc_upd, &s->gc_back, &s->gc_b, &s->gc_thin, &s->gc_wide, &s->gc_rest})
+    v->clear();
+  s->gc_sol_ptr.assign(1, 0);
+  s->gc_upd_ptr.assign(1, 0);
+  s->gc_amax = 0;
+  auto blocks = [](int64_t v) { return (int32_t)((v + kGroupBlock - 1) / kGroupBlock); };
+  for (int64_t k = 0; k < s->nsn; ++k) {
+    const int t = s->tier[k];
+    const int64_t n = front_n(s, k), J = front_J(s, k), a = J - n;
+    if (t != 1 && t != 3 && !(t == 2 && s->tc_mode != 1)) continue;
+    if (n > kGroupCols || a > kInvVGroup) {
+      if (t != 2) s->gc_rest.push_back((int32_t)k);
+      continue;
+    }
+    s->in_gc[k] = 1;
+    GComp c{};
+    c.base = s->colptr[s->sn_ptr[k]];
+    c.f_off = s->f_off[k];
+    c.v_off = s->v_off[k];
+    c.d_off = s->d_off[k];
+    c.rows_off = s->rows_ptr[k];
+    c.k = (int32_t)k;
+    c.n = (int32_t)n;
+    c.a = (int32_t)a;
+    c.J = (int32_t)J;
+    c.nA = blocks(a);
+    s->gc.push_back(c);
+  }
+  if (s->gc.empty()) return;
+  std::stable_sort(s->gc.begin(), s->gc.end(), [](const GComp& x, const GComp& y) { return x.a > y.a; });
+  const int32_t nf = (int32_t)s->gc.size();
+  s->gc_amax = s->gc[0].a;
+  auto push = [](std::vector<int32_t>& v, int32_t f, int32_t i, int32_t j) {
+    v.push_back(f);
+    v.push_back(i | (j << 10));
+  };
+  auto nblk = [&](const GComp& c) { return c.nA + blocks(c.n); };
+  for (int32_t f = 0; f < nf; ++f) {
+    const GComp& c = s->gc[f];
+    for (int32_t j = 0; j < nblk(c); ++j)
+      for (int32_t i = j; i < nblk(c); ++i) push(s->gc_all, f, i, j);
+    if (c.a > 0)
+      for (int32_t b = 0; b < (c.n + 7) / 8; ++b) push(s->gc_back, f, b, 0);
+    if (c.n <= kGroupBlock) {
+      s->gc_thin.push_back(f);
+      for (int32_t b = 0; b < c.nA; ++b) push(s->gc_b, f, b, 0);
+    } else {
+      s->gc_wide.push_back(c.k);
+    }
+  }
+  for (int32_t p = 0; p < s->gc[0].nA; ++p) {
+    for (int32_t f = 0; f < nf && s->gc[f].nA > p; ++f)
+      for (int32_t i = p + 1; i < nblk(s->gc[f]); ++i) push(s->gc_sol, f, i, 0);
+    s->gc_sol_ptr.push_back((int32_t)(s->gc_sol.size() / 2));
+    // the diagonal blocks first: their CTAs go on to factor them
+    for (int32_t f = 0; f < nf && s->gc[f].nA > p + 1; ++f) push(s->gc_upd, f, p + 1, p + 1);
+    for (int32_t f = 0; f < nf && s->gc[f].nA > p; ++f)
+      for (int32_t j = p + 1; j < nblk(s->gc[f]); ++j)
+        for (int32_t i = j; i < nblk(s->gc[f]); ++i)
+          if (i > p + 1 || s->gc[f].nA <= p + 1) push(s->gc_upd, f, i, j);
+    s->gc_upd_ptr.push_back((int32_t)(s->gc_upd.size() / 2));
+  }
+}
+
 chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* rowind,
                               const chd_opts& opts, chd_symbolic* s) {
   if (n < 1 || !colptr || !rowind) return CHD_ERR_INVALID;
@@ -1121,5 +1191,6 @@ chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* r
   factored_completion_plan(s);
   group_plan(s);
   group_inverse_plan(s);
+  group_completion_plan(s);
   return CHD_OK;
 }

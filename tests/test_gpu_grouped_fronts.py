@@ -89,6 +89,18 @@ def _check(pattern, seed, **opts):
         assert err(ws[i], w[i]) < 1e-12
         assert err(ta[i], want[i]) < TOL  # R^adj(R(Y)) = H(Y)
     assert f.status() == 0
+    # completion: P(X-hat^{-1}) = S, f* and the factor's other blocks
+    s = W.projected_gram(N, cp, ri, rng.standard_normal((N, 12)), 0.7)
+    fx, fstar = sym.complete(_dev(s))
+    xh = _host(fx.product())
+    assert err(-OD.gradient(N, cp, ri, xh), s) < 1e-9 and err(-_host(fx.gradient()), s) < 1e-9
+    assert abs(fstar - (OD.logdet(N, cp, ri, xh) - N)) <= 1e-9 * max(1.0, abs(fstar))
+    back = _host(fx.inv_hessian(fx.hessian(_dev(ys[:1]))))[0]
+    assert err(back, ys[0]) < 1e-7
+    bad = s.copy()
+    bad[cp[-2]] = -1.0  # the last pivot of the root: in every V_k, or in the root's P
+    fx.recomplete(_dev(bad), want_fstar=False)
+    assert fx.status() == 3
     # a failing pivot in the last column of the first supernode
     bad = x.copy()
     col = int(sym.supernodes()[0][1]) - 1
