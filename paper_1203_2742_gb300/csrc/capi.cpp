@@ -160,6 +160,15 @@ chd_status alloc_factor(chd_symbolic* s, cudaStream_t stream, chd_factor** out) 
       f->ex.nside = 0;  // run every big front on the caller's stream
     }
   }
+  for (int j = 0; j < kAuxStreams; ++j) {
+    if (cudaStreamCreateWithFlags(&f->ex.aux[j], cudaStreamNonBlocking) != cudaSuccess ||
+        cudaEventCreateWithFlags(&f->ex.aux_fork[j], cudaEventDisableTiming) != cudaSuccess ||
+        cudaEventCreateWithFlags(&f->ex.aux_join[j], cudaEventDisableTiming) != cudaSuccess) {
+      cudaGetLastError();  // run every launch of a level on the caller's stream
+      break;
+    }
+    f->ex.naux = j + 1;
+  }
   if (cudaStreamCreateWithFlags(&f->gs, cudaStreamNonBlocking) != cudaSuccess ||
       cudaEventCreateWithFlags(&f->g_in, cudaEventDisableTiming) != cudaSuccess ||
       cudaEventCreateWithFlags(&f->g_out, cudaEventDisableTiming) != cudaSuccess) {
@@ -937,6 +946,14 @@ void chd_factor_free(chd_factor* f) {
     if (f->ex.join[j]) cudaEventDestroy(f->ex.join[j]);
   }
   if (f->ex.fork) cudaEventDestroy(f->ex.fork);
+  for (int j = 0; j < kAuxStreams; ++j) {
+    if (f->ex.aux[j]) {
+      cudaStreamSynchronize(f->ex.aux[j]);
+      cudaStreamDestroy(f->ex.aux[j]);
+    }
+    if (f->ex.aux_fork[j]) cudaEventDestroy(f->ex.aux_fork[j]);
+    if (f->ex.aux_join[j]) cudaEventDestroy(f->ex.aux_join[j]);
+  }
   for (auto& g : f->graphs) drop_graph(g);
   if (f->gs) {
     cudaStreamSynchronize(f->gs);
@@ -1011,6 +1028,7 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   size_t iGj = add(s->gj.data(), s->gj.size() * sizeof(GJob));
   size_t iGva = add(s->gv_all.data(), s->gv_all.size() * 4);
   size_t iGvs = add(s->gv_sol.data(), s->gv_sol.size() * 4);
+  size_t iGvm = add(s->gv_small.data(), s->gv_small.size() * 4);
   size_t iGvu = add(s->gv_upd.data(), s->gv_upd.size() * 4);
   std::vector<char> host(off, 0);
   for (auto& p : pcs)
@@ -1090,6 +1108,7 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   d.gj = reinterpret_cast<const GJob*>(b + pcs[iGj].off);
   d.gv_all = reinterpret_cast<const int2*>(b + pcs[iGva].off);
   d.gv_sol = reinterpret_cast<const int2*>(b + pcs[iGvs].off);
+  d.gv_small = reinterpret_cast<const int32_t*>(b + pcs[iGvm].off);
   d.gv_upd = reinterpret_cast<const int2*>(b + pcs[iGvu].off);
   d.ninst = (int64_t)s->inst_sn.size() - 1;
   d.f_total = s->f_off[s->nsn];

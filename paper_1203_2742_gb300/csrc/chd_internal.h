@@ -110,6 +110,7 @@ struct SymDev {
   const int32_t* gleg = nullptr;
   const GJob* gj = nullptr;
   const int2 *gv_all = nullptr, *gv_sol = nullptr, *gv_upd = nullptr;
+  const int32_t* gv_small = nullptr;
   const GComp* gc = nullptr;
   const int2 *gc_all = nullptr, *gc_sol = nullptr, *gc_upd = nullptr, *gc_back = nullptr, *gc_b = nullptr;
   const int32_t *gc_thin = nullptr, *gc_wide = nullptr, *gc_rest = nullptr;
@@ -150,6 +151,8 @@ struct chd_symbolic {
   // per level: the first lvl_r32[l] + lvl_r64[l] tasks are chain-tier runs
   // (|J| <= 32, then |J| <= 64; all zero unless chain_runs)
   std::vector<int32_t> lvl_r32, lvl_r64;
+  // lowest level that waits for a chain run, and whether other tasks lie below it
+  int32_t run_join = 0, run_overlap = 0;
   // per level l, five counts at 5*l: chain runs (|J| <= 32), chain runs
   // (|J| <= 64), warp, wide warp and dense-tier tasks (chd_symbolic_schedule)
   std::vector<int32_t> lvl_counts;
@@ -200,6 +203,7 @@ struct chd_symbolic {
   std::vector<GJob> gj;
   std::vector<char> in_gj;  // per supernode
   std::vector<int32_t> gv_all, gv_sol, gv_upd, gv_sol_ptr, gv_upd_ptr;
+  std::vector<int32_t> gv_small;  // supernodes of at most 32 ancestors
   // grouped completion: fronts by decreasing a and the lists of its steps;
   // gc_thin: indices of fronts of at most 32 columns, gc_wide: supernodes of
   // the others, gc_rest: CTA-tier supernodes outside the grouped form
@@ -220,6 +224,7 @@ struct chd_symbolic {
 // the Cholesky panel kernel.  The first kWideSlices slices are large; the
 // rest hold the counter and small partial products only.
 constexpr int kSideStreams = 32;
+constexpr int kAuxStreams = 3;  // chain runs, warp tier, wide warp tier beside the caller's stream
 constexpr int kWideSlices = 9;
 struct Exec {
   int nside = 0;
@@ -233,17 +238,19 @@ struct Exec {
   size_t tc_cap[kSideStreams + 1] = {};
   int64_t* status = nullptr;  // the factor's status (tensor-core timeouts)
   int tc_mode = 0;
+  // streams for the other launches of a level, with their fork and join events
+  int naux = 0;
+  cudaStream_t aux[kAuxStreams] = {};
+  cudaEvent_t aux_fork[kAuxStreams] = {}, aux_join[kAuxStreams] = {};
 };
 
-// Formation of V_k^{-1} by the size a of V_k: up to kInvVGroupMin - 1 rows one
-// CTA per front (k_inv_v; on one SM the a^3 FP64 operations of a larger V_k
-// take milliseconds), up to kInvVGroup rows the grouped kernels over all
-// fronts at once (kv_* in group_tier.cu), beyond that a launch sequence per
-// front whose trailing products run on the tensor cores.  The upper factor
-// of V_k alone (Hessian factor) has no grouped form: one CTA below
+// Formation of V_k^{-1} by the size a of V_k: up to kInvVGroup rows the
+// grouped kernels over all fronts at once (kv_* in group_tier.cu; 12000 fronts
+// of 61 rows: 9.4 ms with one CTA per front before), beyond that a launch
+// sequence per front whose trailing products run on the tensor cores.  The upper
+// factor of V_k (Hessian factor) has no grouped form: one CTA (k_inv_v) below
 // kInvVMulti rows, else a sequence per front.
 constexpr int kInvVMulti = 96;
-constexpr int kInvVGroupMin = 65;
 constexpr int kInvVGroup = 512;
 
 // What one dense-tier front sequence runs with: its stream, the split-K

@@ -750,6 +750,39 @@ __device__ __forceinline__ void factor_diag(double (*T)[GB + 1], double* rinv, d
   for (int c = tid >> 5; c < pb; c += 8)
     if (r < pb && r >= c) D[r + (int64_t)c * J.a] = T[r][c];
 }
+// fronts of one block (a <= 32): everything in one CTA, V^{-1} to R
+__global__ void __launch_bounds__(128) kv_small(SymDev S, const int32_t* list, const double* Vd, double* Rd,
+                                               int64_t* st) {
+  __shared__ double T[GB][GB + 1], X[GB][GB + 1], rinv[GB], col[3][GB];
+  const int k = list[blockIdx.x], tid = threadIdx.x;
+  const int n = (int)(S.sn_ptr[k + 1] - S.sn_ptr[k]), a = (int)(S.rows_ptr[k + 1] - S.rows_ptr[k]) - n;
+  const double* V = Vd + S.v_off[k];
+  double* R = Rd + S.v_off[k];
+  for (int e = tid; e < GB * GB; e += 128) {
+    const int i = e & 31, j = e >> 5;
+    T[i][j] = i < a && j <= i ? V[i + (int64_t)j * a] : (i == j ? 1.0 : 0.0);
+  }
+  __syncthreads();
+  panel::chol32(T, rinv, col, a, tid, 1, st, CHD_ERR_NOT_PD, k, -1);
+  __syncthreads();
+  const int row = tid >> 2, q = tid & 3;
+  if ((tid & ~31) / 4 < a) {  // X = L^{-T}, rows of the identity
+    double b[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) b[u] = row == q + 4 * u ? 1.0 : 0.0;
+    panel::solve_row(b, T, rinv, a, tid & 31);
+#pragma unroll
+    for (int u = 0; u < 8; ++u) X[row][q + 4 * u] = b[u];
+  }
+  __syncthreads();
+  for (int e = tid; e < a * GB; e += 128) {
+    const int i = e & 31, j = e >> 5;
+    if (i >= a || j > i) continue;
+    double v = 0.0;
+    for (int c = i; c < a; ++c) v = fma(X[i][c], X[j][c], v);
+    R[i + (int64_t)j * a] = v;
+  }
+}
 // V into R, I into X (upper block triangle), and the first diagonal block's factor
 __global__ void __launch_bounds__(256) kv_init(SymDev S, const int2* tiles, const double* Vd, double* Rd, double* ws,
                                               int64_t* st) {
@@ -1576,6 +1609,10 @@ void group_ihess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const 
 }
 // V_k^{-1} of the fronts of the grouped inverse (gj), into Rd
 void group_inv_v(const chd_symbolic* s, cudaStream_t st, const double* Vd, double* Rd, double* ws, int64_t* status) {
+  if (!s->gv_small.empty()) {
+    kv_small<<<(unsigned)s->gv_small.size(), 128, 0, st>>>(s->dev, s->dev.gv_small, Vd, Rd, status);
+    count_launch();
+  }
   if (s->gj.empty()) return;
   const int nt = (int)s->gv_all.size() / 2;
   kv_init<<<nt, 256, 0, st>>>(s->dev, s->dev.gv_all, Vd, Rd, ws, status);

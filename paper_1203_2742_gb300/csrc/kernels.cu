@@ -917,39 +917,23 @@ __global__ void __launch_bounds__(NT) k_fc(SymDev S, int first, const double* Si
     cta_potrf_partial(At, f.a, pp, pp, st, CHD_ERR_NOT_COMPLETABLE, k, -1);
   }
 }
-// Inverses of the cached V_k (inverse Hessian step 2), one CTA per front of
-// `front_list` (no dependencies between fronts; big fronts use the dense
-// tier): R = chol(V), R^{-1} in the front's workspace, V^{-1} = R^{-T} R^{-1}.
-// what & 1: V_k^{-1} into Rd (inverse Hessian); what & 2: chol(P V_k P) into
-// Qd (Hessian factor)
-__global__ void __launch_bounds__(NT) k_inv_v(SymDev S, const double* Vd, double* Rd, double* Qd, double* ws,
-                                              int64_t* st, const int32_t* front_list, int what) {
+// Upper factors of the cached V_k (Hessian factor, §5.4), one CTA per front of
+// `front_list` (no dependencies between fronts): V = Q Q^T with Q upper
+// triangular, kept as Q' = chol(P V P) = P Q P, P the order reversal
+__global__ void __launch_bounds__(NT) k_inv_v(SymDev S, const double* Vd, double* Qd, int64_t* st,
+                                              const int32_t* front_list) {
   const int k = front_list[blockIdx.x];
   const int n = (int)(S.sn_ptr[k + 1] - S.sn_ptr[k]);
   const int a = (int)(S.rows_ptr[k + 1] - S.rows_ptr[k]) - n;
-  if (a == 0 || a >= (what == 1 ? kInvVGroupMin : kInvVMulti)) return;  // large V_k: multi-CTA kernels
-  double* R = Rd + S.v_off[k];
-  double* Ri = ws + S.f_off[k];  // a x a scratch inside the front's J x J region
+  if (a == 0 || a >= kInvVMulti) return;  // large V_k: multi-CTA kernels (big_inv_v)
   const double* V = Vd + S.v_off[k];
-  // Hessian factor (§5.4): V = Q Q^T with Q upper triangular, kept as
-  // Q' = chol(P V P) = P Q P, P the order reversal
-  if (what & 2) {
-    double* Qk = Qd + S.v_off[k];
-    for (int e = threadIdx.x; e < a * a; e += NT) {
-      const int r = e % a, c = e / a;
-      if (r >= c) Qk[r + (int64_t)c * a] = V[(a - 1 - c) + (int64_t)(a - 1 - r) * a];
-    }
-    __syncthreads();
-    cta_potrf_partial(Qk, a, a, a, st, CHD_ERR_NOT_PD, k, -1);
+  double* Qk = Qd + S.v_off[k];
+  for (int e = threadIdx.x; e < a * a; e += NT) {
+    const int r = e % a, c = e / a;
+    if (r >= c) Qk[r + (int64_t)c * a] = V[(a - 1 - c) + (int64_t)(a - 1 - r) * a];
   }
-  if (what & 1) {
-    copy_lower(R, a, V, a, a);
-    set_identity(Ri, a, a);
-    __syncthreads();
-    cta_potrf_partial(R, a, a, a, st, CHD_ERR_NOT_PD, k, -1);
-    cta_trsm_rLT(a, a, DnTW{Ri, a}, R, a);  // Ri = R^{-1}
-    cta_gemm(a, a, a, 1.0, TriLT{Ri, a}, TriL{Ri, a}, 0.0, Dn{R, a}, true);
-  }
+  __syncthreads();
+  cta_potrf_partial(Qk, a, a, a, st, CHD_ERR_NOT_PD, k, -1);
 }
 // Deterministic sum of the per-front log det contributions.
 __global__ void k_sum(const double* v, int64_t m, double* out) {
@@ -1129,7 +1113,8 @@ void group_complete(const chd_symbolic* s, cudaStream_t st, const double* Sin, d
                     double* Vd, double* ws, double* ldet, int64_t* status);
 void group_inv_v(const chd_symbolic* s, cudaStream_t st, const double* Vd, double* Rd, double* ws, int64_t* status);
 
-// warp-tier launches (warp_tier.cu): w32 for |J| <= 32, w64 for |J| <= 64
+// warp-tier launches (warp_tier.cu): w32 (one warp per front) and w32x (four)
+// for |J| <= 32, w64 for |J| <= 64
 namespace w32 {
 void warp_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws);
 void warp_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* X, double* Lc, double* Wc,
@@ -1166,6 +1151,23 @@ void warp_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int
 void warp_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,
                    int64_t ldy, double* ws);
 }  // namespace w64
+namespace w32x {
+void warp_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws);
+void warp_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* X, double* Lc, double* Wc,
+                 double* Dd, double* ws, double* ldet, int64_t* status);
+void warp_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Wc, double* Sc,
+                   double* g, double* Vd, double* ws);
+void warp_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
+                  const double* Vd, const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws,
+                  const uint8_t* act);
+void warp_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
+                    int64_t ldt, double* ws);
+void warp_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
+                     const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy,
+                     double* ws);
+void warp_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,
+                   int64_t ldy, double* ws);
+}  // namespace w32x
 
 
 // Runs body(i, stream, scratch, cap) for the `count` independent big fronts
@@ -1222,6 +1224,10 @@ struct Level {
   int tr, nr32, nr64;  // chain runs: [tr, tr + nr32) |J| <= 32, then nr64 with |J| <= 64
   int t0, nwarp, tw, nw64, tc, ncta, nbig;
 };
+// Four warps per front while they all run at once with the single warps of
+// the other layout (twelve per SM): up to 152 x 6 fronts; beyond that one warp
+// per front keeps the FP64 pipes as busy with fewer barriers.
+static inline bool w32_few(int tasks, int m) { return (int64_t)tasks * m <= 152 * 6; }
 static inline Level level(const chd_symbolic* s, int l) {
   Level v;
   v.tr = s->lvl_ptr[l];
@@ -1255,19 +1261,60 @@ static inline const int32_t* left_out(const chd_symbolic* s, int q, int& count) 
   return s->dev.gleg + s->gs_leg[q];
 }
 
+// The launches of a level do not depend on each other: with more than one
+// kind of them, the warp tiers run on streams of their own beside the caller's.
+struct Beside {
+  const Exec* ex;
+  cudaStream_t st;
+  bool used[kAuxStreams] = {};
+  Beside(const Exec* e, cudaStream_t s) : ex(e), st(s) {}
+  // stream of kind j, forked here; the caller's stream if `alone`
+  cudaStream_t fork(int j, bool alone) {
+    if (alone || !ex || j >= ex->naux) return st;
+    if (!used[j]) {
+      cudaEventRecord(ex->aux_fork[j], st);
+      cudaStreamWaitEvent(ex->aux[j], ex->aux_fork[j], 0);
+      used[j] = true;
+    }
+    return ex->aux[j];
+  }
+  void join(int j) {
+    if (!used[j]) return;
+    cudaEventRecord(ex->aux_join[j], ex->aux[j]);
+    cudaStreamWaitEvent(st, ex->aux_join[j], 0);
+    used[j] = false;
+  }
+  void join_level() {
+    join(1);
+    join(2);
+  }
+};
+enum { AUX_RUN = 0, AUX_WARP = 1, AUX_WIDE = 2 };
+// whether level l (v) has launches besides its warp-tier ones (wide: besides
+// its wide ones, the plain ones being on a stream of their own)
+static bool alone(const chd_symbolic* s, int l, const Level& v, bool wide) {
+  const bool rest = s->glvl[l + 1] > s->glvl[l] || v.nbig > 0;
+  return wide ? !rest : !rest && v.nw64 == 0;
+}
+
 void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* X, double* Lc, double* Wc,
             double* Dd, double* ws, double* ldet, int64_t* status) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  Beside bs(ex, st);
   for (int l = 0; l < nl; ++l) {
+    if (l == s->run_join) bs.join(AUX_RUN);  // chain runs, forked at level 0
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_factor(s, sl, dense[i], X, Lc, Wc, Dd, ws, ldet, status);
     });
-    if (v.nr32 + v.nr64) chain_factor(s, st, v.tr, v.nr32 + v.nr64, X, Lc, Wc, Dd, ws, ldet, status);
-    if (v.nwarp) w32::warp_factor(s, st, v.t0, v.nwarp, X, Lc, Wc, Dd, ws, ldet, status);
-    if (v.nw64) w64::warp_factor(s, st, v.tw, v.nw64, X, Lc, Wc, Dd, ws, ldet, status);
+    if (v.nr32 + v.nr64) chain_factor(s, bs.fork(AUX_RUN, !s->run_overlap), v.tr, v.nr32 + v.nr64, X, Lc, Wc, Dd, ws, ldet, status);
+    if (v.nwarp)
+      (w32_few(v.nwarp, 1) ? w32x::warp_factor : w32::warp_factor)(s, sw, v.t0, v.nwarp, X, Lc, Wc, Dd, ws, ldet, status);
+    if (v.nw64) w64::warp_factor(s, sv, v.tw, v.nw64, X, Lc, Wc, Dd, ws, ldet, status);
     for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
       group_factor(s, st, q, X, Lc, Dd, ws, status);
       int nleft;
@@ -1278,22 +1325,28 @@ void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double
       }
     }
     bf.join_now();
+    bs.join_level();
   }
+  bs.join(AUX_RUN);
   group_factor_post(s, st, Lc, Wc, ws, ldet);
 }
 // Cholesky product X = L D L^T on V (Algorithm 3.2), bottom-up like the factor.
 void product(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Lc, double* X, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  Beside bs(ex, st);
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_product(s, sl, dense[i], Lc, X, ws);
     });
     if (v.nr32 + v.nr64) chain_product(s, st, v.tr, v.nr32 + v.nr64, Lc, X, ws);
-    if (v.nwarp) w32::warp_product(s, st, v.t0, v.nwarp, Lc, X, ws);
-    if (v.nw64) w64::warp_product(s, st, v.tw, v.nw64, Lc, X, ws);
+    if (v.nwarp)
+      (w32_few(v.nwarp, 1) ? w32x::warp_product : w32::warp_product)(s, sw, v.t0, v.nwarp, Lc, X, ws);
+    if (v.nw64) w64::warp_product(s, sv, v.tw, v.nw64, Lc, X, ws);
     for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
       group_product(s, st, q, Lc, X, ws);
       int nleft;
@@ -1304,15 +1357,26 @@ void product(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doubl
       }
     }
     bf.join_now();
+    bs.join_level();
   }
 }
 void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Wc, double* Sc, double* g,
               double* Vd, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  Beside bs(ex, st);
   group_zero(s, st, 1, ws);
+  // chain runs (level 0) start as soon as their parents are done
+  const Level r = level(s, 0);
+  const int run_at = s->run_overlap ? s->run_join : 1;
+  auto runs = [&](cudaStream_t sr) {
+    if (r.nr32 + r.nr64) chain_gradient(s, sr, r.tr, r.nr32 + r.nr64, Wc, Sc, g, Vd, ws);
+  };
+  if (run_at >= nl) runs(st);
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_gradient(s, sl, dense[i], Wc, Sc, g, Vd, ws);
@@ -1326,27 +1390,35 @@ void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
         count();
       }
     }
-    if (v.nr32 + v.nr64) chain_gradient(s, st, v.tr, v.nr32 + v.nr64, Wc, Sc, g, Vd, ws);
-    if (v.nwarp) w32::warp_gradient(s, st, v.t0, v.nwarp, Wc, Sc, g, Vd, ws);
-    if (v.nw64) w64::warp_gradient(s, st, v.tw, v.nw64, Wc, Sc, g, Vd, ws);
+    if (v.nwarp)
+      (w32_few(v.nwarp, 1) ? w32x::warp_gradient : w32::warp_gradient)(s, sw, v.t0, v.nwarp, Wc, Sc, g, Vd, ws);
+    if (v.nw64) w64::warp_gradient(s, sv, v.tw, v.nw64, Wc, Sc, g, Vd, ws);
     bf.join_now();
+    bs.join_level();
+    if (l == run_at) runs(bs.fork(AUX_RUN, !s->run_overlap));
   }
+  bs.join(AUX_RUN);
 }
 void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, const double* Vd,
                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  Beside bs(ex, st);
   SymDev D = s->dev;
   D.act = act;
   for (int l = 0; l < nl; ++l) {
+    if (l == s->run_join) bs.join(AUX_RUN);  // chain runs, forked at level 0
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_hess_up(s, sl, m, dense[i], Wc, Vd, Y, ldy, T, ldt, ws, act);
     });
-    if (v.nr32 + v.nr64) chain_hess_up(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
-    if (v.nwarp) w32::warp_hess_up(s, st, v.t0, v.nwarp, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
-    if (v.nw64) w64::warp_hess_up(s, st, v.tw, v.nw64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
+    if (v.nr32 + v.nr64) chain_hess_up(s, bs.fork(AUX_RUN, !s->run_overlap), v.tr, v.nr32 + v.nr64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
+    if (v.nwarp)
+      (w32_few(v.nwarp, m) ? w32x::warp_hess_up : w32::warp_hess_up)(s, sw, v.t0, v.nwarp, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
+    if (v.nw64) w64::warp_hess_up(s, sv, v.tw, v.nw64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
     for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
       group_hess_up(s, st, q, m, Wc, Y, ldy, ws, act);
       int nleft;
@@ -1357,16 +1429,28 @@ void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m,
       }
     }
     bf.join_now();
+    bs.join_level();
   }
+  bs.join(AUX_RUN);
   group_hess_m(s, st, m, Wc, Vd, T, ldt, ws, act);
 }
 void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, double* T,
                     int64_t ldt, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  Beside bs(ex, st);
   group_zero(s, st, m, ws);
+  // chain runs (level 0) start as soon as their parents are done
+  const Level r = level(s, 0);
+  const int run_at = s->run_overlap ? s->run_join : 1;
+  auto runs = [&](cudaStream_t sr) {
+    if (r.nr32 + r.nr64) chain_hess_down(s, sr, r.tr, r.nr32 + r.nr64, m, Wc, T, ldt, ws);
+  };
+  if (run_at >= nl) runs(st);
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_hess_down(s, sl, m, dense[i], Wc, T, ldt, ws);
@@ -1380,11 +1464,14 @@ void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int 
         count();
       }
     }
-    if (v.nr32 + v.nr64) chain_hess_down(s, st, v.tr, v.nr32 + v.nr64, m, Wc, T, ldt, ws);
-    if (v.nwarp) w32::warp_hess_down(s, st, v.t0, v.nwarp, m, Wc, T, ldt, ws);
-    if (v.nw64) w64::warp_hess_down(s, st, v.tw, v.nw64, m, Wc, T, ldt, ws);
+    if (v.nwarp)
+      (w32_few(v.nwarp, m) ? w32x::warp_hess_down : w32::warp_hess_down)(s, sw, v.t0, v.nwarp, m, Wc, T, ldt, ws);
+    if (v.nw64) w64::warp_hess_down(s, sv, v.tw, v.nw64, m, Wc, T, ldt, ws);
     bf.join_now();
+    bs.join_level();
+    if (l == run_at) runs(bs.fork(AUX_RUN, !s->run_overlap));
   }
+  bs.join(AUX_RUN);
 }
 void hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, const double* Vd,
              const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws) {
@@ -1423,9 +1510,12 @@ void rtrans(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, int d
 void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, const double* Dd,
                  const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
+  Beside bs(ex, st);
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_ihess_down(s, sl, m, dense[i], Wc, Dd, Rd, T, ldt, Y, ldy, ws);
@@ -1440,21 +1530,26 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
       }
     }
     if (v.nr32 + v.nr64) chain_ihess_down(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
-    if (v.nwarp) w32::warp_ihess_down(s, st, v.t0, v.nwarp, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
-    if (v.nw64) w64::warp_ihess_down(s, st, v.tw, v.nw64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+    if (v.nwarp)
+      (w32_few(v.nwarp, m) ? w32x::warp_ihess_down : w32::warp_ihess_down)(s, sw, v.t0, v.nwarp, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+    if (v.nw64) w64::warp_ihess_down(s, sv, v.tw, v.nw64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
     bf.join_now();
+    bs.join_level();
   }
   group_ihess_k(s, st, m, Wc, Dd, Rd, Y, ldy, ws);
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
+    const cudaStream_t sw = v.nwarp ? bs.fork(AUX_WARP, alone(s, l, v, false)) : st;
+    const cudaStream_t sv = v.nw64 ? bs.fork(AUX_WIDE, alone(s, l, v, true)) : st;
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_ihess_up(s, sl, m, dense[i], Wc, Y, ldy, ws);
     });
     if (v.nr32 + v.nr64) chain_ihess_up(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Y, ldy, ws);
-    if (v.nwarp) w32::warp_ihess_up(s, st, v.t0, v.nwarp, m, Wc, Y, ldy, ws);
-    if (v.nw64) w64::warp_ihess_up(s, st, v.tw, v.nw64, m, Wc, Y, ldy, ws);
+    if (v.nwarp)
+      (w32_few(v.nwarp, m) ? w32x::warp_ihess_up : w32::warp_ihess_up)(s, sw, v.t0, v.nwarp, m, Wc, Y, ldy, ws);
+    if (v.nw64) w64::warp_ihess_up(s, sv, v.tw, v.nw64, m, Wc, Y, ldy, ws);
     for (int q = s->glvl[l]; q < s->glvl[l + 1]; ++q) {
       group_ihess_up(s, st, q, m, Wc, Y, ldy, ws);
       int nleft;
@@ -1465,6 +1560,7 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
       }
     }
     bf.join_now();
+    bs.join_level();
   }
 }
 // Completion: the arithmetic of Algorithm 7.3 for one front needs only the
@@ -1495,6 +1591,8 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
       bf.join_now();
     }
   }
+  Beside bs(ex, st);
+  const cudaStream_t sw = s->dev.warp_count > 0 ? bs.fork(AUX_WARP, s->gc.empty()) : st;
   // the grouped form (group_tier.cu) factors V_k itself; with Gq every front
   // takes the per-front kernels
   const bool grouped = !Gq;
@@ -1522,8 +1620,9 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
                                      ws, ldet, status);
     count();
   }
-  if (s->dev.warp_count > 0) w32::warp_complete_all(s, st, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ldet, status);
+  if (s->dev.warp_count > 0) w32::warp_complete_all(s, sw, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ldet, status);
   bf.join_now();
+  bs.join_level();
 }
 void big_inv_v(const chd_symbolic* s, const Slot& sl, int k, const double* Vd,
                double* Rd, double* Qd, double* ws, int64_t* status, int what);
@@ -1543,8 +1642,8 @@ void inv_v(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double*
     big_inv_v(s, sl, bigs[i], Vd, Rd, Qd, ws, status, what);
   });
   if (grouped) group_inv_v(s, st, Vd, Rd, ws, status);
-  if (s->dev.small_count > 0) {
-    k_inv_v<<<(int)s->dev.small_count, NT, 0, st>>>(s->dev, Vd, Rd, Qd, ws, status, s->dev.small_fronts, what);
+  if (!grouped && s->dev.small_count > 0) {
+    k_inv_v<<<(int)s->dev.small_count, NT, 0, st>>>(s->dev, Vd, Qd, status, s->dev.small_fronts);
     count();
   }
   bf.join_now();

@@ -528,14 +528,18 @@ static void group_plan(chd_symbolic* s) {
 static void group_inverse_plan(chd_symbolic* s) {
   s->gj.clear();
   s->in_gj.assign(s->nsn, 0);
-  for (auto* v : {&s->gv_all, &s->gv_sol, &s->gv_upd}) v->clear();
+  for (auto* v : {&s->gv_all, &s->gv_sol, &s->gv_upd, &s->gv_small}) v->clear();
   s->gv_sol_ptr.assign(1, 0);
   s->gv_upd_ptr.assign(1, 0);
   for (int64_t k = 0; k < s->nsn; ++k) {
     const int64_t a = front_J(s, k) - front_n(s, k);
-    if (a < kInvVGroupMin || a > kInvVGroup || (s->is_big[k] && s->tc_mode == 1)) continue;
+    if (a < 1 || a > kInvVGroup || (s->is_big[k] && s->tc_mode == 1)) continue;
     if (s->grp_of[k] >= 0 && s->grp_first[s->grp_of[k]] != k) continue;  // a leaf group shares one V
     s->in_gj[k] = 1;
+    if (a <= kGroupBlock) {
+      s->gv_small.push_back((int32_t)k);
+      continue;
+    }
     GJob j{};
     j.v_off = s->v_off[k];
     j.w_off = s->f_off[k];
@@ -1131,6 +1135,27 @@ chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* r
     }
     int64_t nlev = 0;
     for (int64_t l : tlevel) nlev = std::max(nlev, l + 1);
+    // A chain run is a long serial kernel, and only its parent waits for it:
+    // a task that holds such a parent goes to the latest level its own parent
+    // allows, so that the runs overlap with all levels before run_join.
+    s->run_join = (int32_t)nlev;
+    s->run_overlap = 0;
+    {
+      vector<char> over_run(tasks.size(), 0);
+      bool any = false;
+      for (int64_t t = 0; t < nsn; ++t)
+        if (run_of[t] >= 0 && s->sn_par[t] >= 0 && task_of[s->sn_par[t]] != task_of[t])
+          over_run[task_of[s->sn_par[t]]] = 1, any = true;
+      for (int64_t t = nsn - 1; any && t >= 0; --t) {
+        const int64_t tk = task_of[t];
+        if (!over_run[tk] || tasks[tk].back() != t) continue;
+        const int64_t p = s->sn_par[t];
+        tlevel[tk] = std::max(tlevel[tk], (p < 0 ? nlev : tlevel[task_of[p]]) - 1);
+        s->run_join = std::min(s->run_join, (int32_t)tlevel[tk]);
+      }
+      for (size_t q = 0; any && q < tasks.size(); ++q)
+        if (ttier[q] != 5 && ttier[q] != 6 && tlevel[q] < s->run_join) s->run_overlap = 1;
+    }
     vector<vector<int64_t>> bylev(nlev);
     for (size_t q = 0; q < tasks.size(); ++q) bylev[tlevel[q]].push_back((int64_t)q);
     s->task_ptr.assign(1, 0);

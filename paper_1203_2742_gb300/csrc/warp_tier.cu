@@ -36,6 +36,20 @@ void count_launch();
 #undef WT_WPB
 #undef WT_TPF
 
+// the same fronts, four warps (one CTA) each: one warp issues an FP64
+// instruction every 64 clocks at best, so a front of 24 ancestors and 8
+// columns is a chain of 20 to 35 us for it.  Taken where the launch has too few
+// fronts to fill the SMs' FP64 pipes with single warps (w32_few).
+#define WT_NS w32x
+#define WT_J 32
+#define WT_WPB 1
+#define WT_TPF 128
+#include "warp_tier_body.cuh"
+#undef WT_NS
+#undef WT_J
+#undef WT_WPB
+#undef WT_TPF
+
 // chains of fronts with 32 < |J| <= 64 (bands of half-bandwidth up to 63):
 // eight warps (one CTA) per front, which shortens the serial chain
 #define WT_NS w64
