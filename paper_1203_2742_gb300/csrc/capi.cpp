@@ -29,6 +29,7 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
 void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Sin, double* Lc,
               double* Wc, double* Dd, double* Vd, double* Rd, double* Gq, double* fcs, double* ws, double* ldet,
               int64_t* status);
+void chain_psi(const chd_symbolic* s, cudaStream_t st, const double* Wc, double* psi);
 void inv_v(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Vd, double* Rd, double* Qd,
            double* ws, int64_t* status, int what);
 void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, const double* Vd,
@@ -83,6 +84,7 @@ chd_status alloc_factor(chd_symbolic* s, cudaStream_t stream, chd_factor** out) 
   const size_t oVd = off; off = align_up(off + (size_t)s->v_off[s->nsn] * 8);
   const size_t oRd = off; off = align_up(off + (size_t)s->v_off[s->nsn] * 8);
   const size_t oQd = off; off = align_up(off + (size_t)s->v_off[s->nsn] * 8);
+  const size_t ops = off; off = align_up(off + (size_t)s->cseg_psi * 8);
   const size_t old = off; off = align_up(off + (size_t)s->nsn * 8);
   const size_t osc = off; off = align_up(off + 4 * 8);
   const size_t ost = off; off = align_up(off + 4 * 8);
@@ -129,6 +131,7 @@ chd_status alloc_factor(chd_symbolic* s, cudaStream_t stream, chd_factor** out) 
   f->Vd = reinterpret_cast<double*>(b + oVd);
   f->Rd = reinterpret_cast<double*>(b + oRd);
   f->Qd = reinterpret_cast<double*>(b + oQd);
+  if (!s->cseg.empty()) f->ex.psi = reinterpret_cast<double*>(b + ops);
   f->ldet = reinterpret_cast<double*>(b + old);
   f->scalar = reinterpret_cast<double*>(b + osc);
   f->status = reinterpret_cast<int64_t*>(b + ost);
@@ -323,7 +326,16 @@ chd_status ensure_projected_inverse(chd_factor* f) {
   rc = run_sequence(f, G_GRADIENT, key, [&](cudaStream_t st) {
     chd_launch::gradient(f->sym, st, &f->ex, f->Wc, f->Sc, nullptr, f->Vd, f->ws);
   });
-  if (rc == CHD_OK) f->have_S = true;
+  if (rc == CHD_OK) f->have_S = f->have_psi = true;
+  return rc;
+}
+// the chain segments' matrices of an object whose projected inverse did not
+// come from the gradient (a completion)
+chd_status ensure_psi(chd_factor* f) {
+  if (f->have_psi || !f->ex.psi) return CHD_OK;
+  chd_launch::chain_psi(f->sym, f->stream, f->Wc, f->ex.psi);
+  chd_status rc = launch_status();
+  if (rc == CHD_OK) f->have_psi = true;
   return rc;
 }
 
@@ -566,7 +578,7 @@ chd_status chd_refactor(chd_factor* f, const double* x, void* stream) {
   f->stream = static_cast<cudaStream_t>(stream);
   chd_status rc = ensure_ws(f, 1);
   if (rc != CHD_OK) return rc;
-  f->have_S = f->have_R = f->have_Q = false;
+  f->have_S = f->have_psi = f->have_R = f->have_Q = false;
   rc = cuda_ok(cudaMemsetAsync(f->status, 0, 4 * 8, f->stream));
   if (rc != CHD_OK) return rc;
   GraphKey key;
@@ -618,7 +630,7 @@ chd_status chd_gradient(chd_factor* f, double* g, void* stream) {
   rc = run_sequence(f, G_GRADIENT, key, [&](cudaStream_t st) {
     chd_launch::gradient(f->sym, st, &f->ex, f->Wc, f->Sc, g, f->Vd, f->ws);
   });
-  if (rc == CHD_OK) f->have_S = true;
+  if (rc == CHD_OK) f->have_S = f->have_psi = true;
   return rc;
 }
 
@@ -633,6 +645,7 @@ chd_status chd_hessian(chd_factor* f, int m, const double* y, int64_t ldy, doubl
   if (rc != CHD_OK) return rc;
   const int64_t chunk = rhs_chunk(f, m);
   rc = ensure_ws(f, chunk);
+  if (rc == CHD_OK) rc = ensure_psi(f);
   if (rc != CHD_OK) return rc;
   for (int64_t i = 0; i < m; i += chunk) {
     const int mc = (int)std::min<int64_t>(chunk, m - i);
@@ -664,6 +677,7 @@ static chd_status hessian_factor(chd_factor* f, int m, const double* y, int64_t 
   const int64_t chunk = rhs_chunk(f, m);
   rc = ensure_ws(f, chunk);
   if (rc == CHD_OK) rc = ensure_q(f);
+  if (rc == CHD_OK) rc = ensure_psi(f);
   if (rc == CHD_OK && prune) rc = ensure_act(f, chunk);
   if (rc != CHD_OK) return rc;
   const int64_t nsn = f->sym->nsn;
@@ -716,6 +730,7 @@ chd_status chd_hessian_factor_adj(chd_factor* f, int m, const double* w, int64_t
   const int64_t chunk = rhs_chunk(f, m);
   rc = ensure_ws(f, chunk);
   if (rc == CHD_OK) rc = ensure_q(f);
+  if (rc == CHD_OK) rc = ensure_psi(f);
   if (rc != CHD_OK) return rc;
   for (int64_t i = 0; i < m; i += chunk) {
     const int mc = (int)std::min<int64_t>(chunk, m - i);
@@ -800,6 +815,7 @@ chd_status chd_recomplete(chd_factor* f, const double* sv, void* stream, double*
   }
   if (rc != CHD_OK) return rc;
   f->have_S = true;
+  f->have_psi = false;
   f->have_R = false;  // Rd holds chol(V_k) or nothing here; V_k^{-1} is formed on first use
   // the factored form leaves G_k = P R_k P = chol(P V_k P) in Qd: the Hessian
   // factor's upper factors of V_k
@@ -1025,6 +1041,8 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   const std::vector<int32_t>* gq[8] = {&s->gc_all, &s->gc_sol,  &s->gc_upd,  &s->gc_back,
                                        &s->gc_b,   &s->gc_thin, &s->gc_wide, &s->gc_rest};
   for (int i = 0; i < 8; ++i) iGq[i] = add(gq[i]->data(), gq[i]->size() * 4);
+  size_t iCs = add(s->cseg.data(), s->cseg.size() * sizeof(ChainSeg));
+  size_t iCr = add(s->crun.data(), s->crun.size() * 4);
   size_t iGj = add(s->gj.data(), s->gj.size() * sizeof(GJob));
   size_t iGva = add(s->gv_all.data(), s->gv_all.size() * 4);
   size_t iGvs = add(s->gv_sol.data(), s->gv_sol.size() * 4);
@@ -1105,6 +1123,8 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   for (int i = 0; i < 5; ++i) *dq[i] = reinterpret_cast<const int2*>(b + pcs[iGq[i]].off);
   const int32_t** dl[3] = {&d.gc_thin, &d.gc_wide, &d.gc_rest};
   for (int i = 0; i < 3; ++i) *dl[i] = reinterpret_cast<const int32_t*>(b + pcs[iGq[5 + i]].off);
+  d.cseg = reinterpret_cast<const ChainSeg*>(b + pcs[iCs].off);
+  d.crun = reinterpret_cast<const int2*>(b + pcs[iCr].off);
   d.gj = reinterpret_cast<const GJob*>(b + pcs[iGj].off);
   d.gv_all = reinterpret_cast<const int2*>(b + pcs[iGva].off);
   d.gv_sol = reinterpret_cast<const int2*>(b + pcs[iGvs].off);

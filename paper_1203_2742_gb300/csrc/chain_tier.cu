@@ -120,10 +120,22 @@ struct UpArgs {
   double* dd;         // UP_FACTOR: Dd of the first column
   int64_t* st;
 };
+// Columns i0 .. L - 1 of the run.  in: the window before column i0 (a x a,
+// lower, ld a) or null for zeros; outs: whether the columns' outputs are
+// stored; the window after column L - 1 goes to G[p + q ldg], p >= q (or
+// nowhere, G null).
+struct Span {
+  int i0, L;
+  const double* in;
+  bool outs;
+  double* G;
+  int64_t ldg;
+};
 template <int NT, int PP, int MODE>
-__device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double* G) {
+__device__ void up_run(const Run& R, const Span& sp_, const UpArgs& A, UpSmem& sm) {
   constexpr int EL = NT <= 32 ? 1 : NT <= 96 ? 1 : 3;  // slots per lane of warp 0
-  const int a = R.a, W = a + 1, tid = threadIdx.x, L = R.L;
+  const int a = R.a, W = a + 1, tid = threadIdx.x, L = sp_.L, i0 = sp_.i0;
+  const bool outs = sp_.outs;
   if (tid >= NT + 32) return;
   for (int e = tid; e < 2 * WP; e += NT + 32) (&sm.uc[0][0])[e] = 0.0;
   bar(NT + 32);
@@ -158,10 +170,12 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
         if (o < W) {
           val[e] = sm.ring[0][c % RING][o];
           if (MODE == UP_HESS) l[e] = sm.ring[1][c % RING][o];
-          if (c > i0 && o != sp) {  // slot sp: the row that enters, untouched so far
+          if (o != sp) {  // slot sp: the row that enters, untouched so far
             val[e] += sm.uc[cur][o];
-            val[e] = fma(-sm.f[prv][o], gs, val[e]);
-            if (MODE == UP_HESS) val[e] = fma(-sm.g[prv][o], fs, val[e]);
+            if (c > i0) {
+              val[e] = fma(-sm.f[prv][o], gs, val[e]);
+              if (MODE == UP_HESS) val[e] = fma(-sm.g[prv][o], fs, val[e]);
+            }
           }
         }
       }
@@ -185,11 +199,13 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
             sm.g[cur][o] = gv;
             int p = o - s0;
             if (p < 0) p += W;
-            A.o0[(int64_t)c * W + p] = p == 0 ? d : val[e];
-            A.o1[(int64_t)c * W + p] = p == 0 ? r2 : gv;
+            if (outs) {
+              A.o0[(int64_t)c * W + p] = p == 0 ? d : val[e];
+              A.o1[(int64_t)c * W + p] = p == 0 ? r2 : gv;
+            }
           }
         }
-        if (lane == 0) A.dd[4 * (int64_t)c] = d;
+        if (outs && lane == 0) A.dd[4 * (int64_t)c] = d;
       } else {
         // P = h_A - L h_0 / 2: U' = Yh_AA - (P L^T + L P^T); K_A = P - L h_0 / 2
         const double hh = 0.5 * d;
@@ -202,14 +218,14 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
             sm.g[cur][o] = l[e];
             int p = o - s0;
             if (p < 0) p += W;
-            A.o0[(int64_t)c * W + p] = p == 0 ? d : fma(-l[e], hh, pv);
+            if (outs) A.o0[(int64_t)c * W + p] = p == 0 ? d : fma(-l[e], hh, pv);
           }
         }
       }
     };
     for (int c = i0; c < i0 + AHEAD; ++c) prefetch(c);
     cp_async_wait<AHEAD - 1>();
-    __syncwarp();
+    bar(NT + 32);  // the window's columns i0 and i0 + 1 are in uc
     column(i0);
     bar(NT + 32);
     for (int i = i0; i < L; ++i) {
@@ -240,8 +256,22 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
       pv[t] = v;
       U[t] = 0.0;
     }
-    bar(NT + 32);
     int s0 = i0 % W;
+    if (sp_.in) {
+      const int t1 = s0 + 1 == W ? 0 : s0 + 1;
+#pragma unroll
+      for (int t = 0; t < PP; ++t) {
+        if (ut + NT * t >= np) break;
+        const int u = pu[t], v = pv[t];
+        const int p = u >= s0 ? u - s0 : u - s0 + W, q = v >= s0 ? v - s0 : v - s0 + W;
+        const double x = p < a && q < a ? sp_.in[max(p, q) + (int64_t)min(p, q) * a] : 0.0;
+        if (u == s0 || v == s0) sm.uc[i0 & 1][u == s0 ? v : u] = x;
+        else if (i0 + 1 < L && (u == t1 || v == t1)) sm.uc[(i0 + 1) & 1][u == t1 ? v : u] = x;
+        else U[t] = x;
+      }
+    }
+    bar(NT + 32);
+    bar(NT + 32);
     for (int i = i0; i < L; ++i) {
       const int s1 = i + 1 < L ? (s0 + 1 == W ? 0 : s0 + 1) : s0;
       int s2 = s0 + 2;
@@ -266,9 +296,9 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
       bar(NT + 32);
       s0 = s0 + 1 == W ? 0 : s0 + 1;
     }
-    // update block of the top front for the parent (lower, ld J = a + 1):
+    if (!sp_.G) return;
     // rows L .. L + a - 1, i.e. every slot but that of row L - 1
-    const int sL = L % W, out = sL == 0 ? W - 1 : sL - 1, J = W;
+    const int sL = L % W, out = sL == 0 ? W - 1 : sL - 1;
 #pragma unroll
     for (int t = 0; t < PP; ++t) {
       if (ut + NT * t >= np) break;
@@ -277,7 +307,7 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
       int p = u - sL, q = v - sL;
       if (p < 0) p += W;
       if (q < 0) q += W;
-      G[(1 + max(p, q)) + (int64_t)(1 + min(p, q)) * J] = U[t];
+      sp_.G[max(p, q) + (int64_t)min(p, q) * sp_.ldg] = U[t];
     }
   }
 }
@@ -286,10 +316,19 @@ __device__ void up_run(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double
 // instructions (one warp up to a = 9, three up to a = 31, seven up to 64).
 constexpr int UPT = 256;
 template <int MODE>
-__device__ __forceinline__ void up_dispatch(const Run& R, int i0, const UpArgs& A, UpSmem& sm, double* G) {
-  if (R.a <= 9) up_run<32, 2, MODE>(R, i0, A, sm, G);
-  else if (R.a <= 31) up_run<96, 6, MODE>(R, i0, A, sm, G);
-  else up_run<224, 10, MODE>(R, i0, A, sm, G);
+__device__ __forceinline__ void up_dispatch(const Run& R, const Span& sp, const UpArgs& A, UpSmem& sm) {
+  if (R.a <= 9) up_run<32, 2, MODE>(R, sp, A, sm);
+  else if (R.a <= 31) up_run<96, 6, MODE>(R, sp, A, sm);
+  else up_run<224, 10, MODE>(R, sp, A, sm);
+}
+// the top front's update block for the parent (its A x A part, ld J = a + 1)
+__device__ __forceinline__ double* update_block(const Run& R, double* ws) {
+  return ws + R.f0 + (int64_t)(R.L - 1) * R.fstride + R.a + 2;
+}
+// window handed over at the lower end of segment [s, ..): a x a, ld a, in the
+// workspace front of its first column; the second column's holds a temporary
+__device__ __forceinline__ double* seg_window(const Run& R, int s, double* ws) {
+  return ws + R.f0 + (int64_t)s * R.fstride;
 }
 
 // Algorithm 7.1 for one-column fronts (Algorithm 3.1): D = F_11, L_AN =
@@ -300,7 +339,7 @@ __global__ void __launch_bounds__(UPT) kc_factor(SymDev S, int task0, const doub
   __shared__ UpSmem sm;
   const Run R = run_of(S, task0 + blockIdx.x);
   UpArgs A{X + R.base0, nullptr, Lc + R.base0, Wc + R.base0, Dd + R.d0, st};
-  up_dispatch<UP_FACTOR>(R, 0, A, sm, ws + R.f0 + (int64_t)(R.L - 1) * R.fstride);
+  up_dispatch<UP_FACTOR>(R, Span{0, R.L, nullptr, true, update_block(R, ws), R.a + 1}, A, sm);
 }
 // C, B and log D of every column of every run, one warp per column
 __global__ void __launch_bounds__(128) kc_factor_post(SymDev S, int task0, double* Lc, const double* Dd,
@@ -338,7 +377,25 @@ __global__ void __launch_bounds__(UPT) kc_hess_up(SymDev S, int task0, const dou
     i0 = lo;
   }
   UpArgs A{Y + y * ldy + R.base0, Wc + R.base0, T + y * ldt + R.base0, nullptr, nullptr, nullptr};
-  up_dispatch<UP_HESS>(R, i0, A, sm, ws + y * S.f_total + R.f0 + (int64_t)(R.L - 1) * R.fstride);
+  up_dispatch<UP_HESS>(R, Span{i0, R.L, nullptr, true, update_block(R, ws + y * S.f_total), R.a + 1}, A, sm);
+}
+// the same by segments (phase 1: every segment but the last from a zero
+// window, the first one for good; phase 2: the others from their windows)
+__global__ void __launch_bounds__(UPT) kc_hess_up_seg(SymDev S, int task0, int phase, const double* Wc,
+                                                     const double* Y, int64_t ldy, double* T, int64_t ldt,
+                                                     double* ws) {
+  __shared__ UpSmem sm;
+  const ChainSeg g = S.cseg[blockIdx.x];
+  if (phase == 1 ? g.p == g.P - 1 && g.P > 1 : g.p == 0) return;
+  const Run R = run_of(S, task0 + g.run);
+  const int64_t y = blockIdx.y;
+  ws += y * S.f_total;
+  UpArgs A{Y + y * ldy + R.base0, Wc + R.base0, T + y * ldt + R.base0, nullptr, nullptr, nullptr};
+  const bool last = g.p == g.P - 1;
+  const double* in = phase == 2 ? seg_window(R, S.cseg[blockIdx.x - 1].s, ws) : nullptr;
+  double* win = last ? update_block(R, ws) : phase == 1 ? seg_window(R, g.s, ws) : nullptr;
+  const Span sp{g.s, g.e, in, phase == 2 || g.p == 0, win, last ? R.a + 1 : R.a};
+  up_dispatch<UP_HESS>(R, sp, A, sm);
 }
 
 // ---------------------------------------------------------------------------
@@ -458,10 +515,21 @@ enum { DOWN_GRAD = 0, DOWN_HESS = 1 };
 // second barrier of a column: the window threads wait, warp 0 only arrives
 __device__ __forceinline__ void bar2_sync(int n) { asm volatile("bar.sync 2, %0;\n" ::"r"(n) : "memory"); }
 __device__ __forceinline__ void bar2_arrive(int n) { asm volatile("bar.arrive 2, %0;\n" ::"r"(n) : "memory"); }
+// Columns hi .. lo (downwards).  in: the window above column hi (rows hi + 1
+// .. hi + a; a x a, lower, ld a), or the parent's front where it is null and
+// `top`, or zeros; outs: whether outputs are stored; win: receives the window
+// after column lo (rows lo .. lo + a - 1), or null.
+struct DownSpan {
+  int hi, lo;
+  const double* in;
+  bool top, outs;
+  double* win;
+};
 template <int NT, int CP, int TP, int MODE>
-__device__ void down_run(const SymDev& S, const Run& R, const double* wc, const double* src, double* out,
-                         const double* ws, DownSmem& sm) {
-  const int a = R.a, W = a + 1, tid = threadIdx.x, L = R.L;
+__device__ void down_run(const SymDev& S, const Run& R, const DownSpan& sp, const double* wc, const double* src,
+                         double* out, const double* ws, DownSmem& sm) {
+  const int a = R.a, W = a + 1, tid = threadIdx.x, L = sp.hi + 1, lo = sp.lo;
+  const bool outs = sp.outs;
   if (tid >= NT + 32) return;
   // slots past the window are multiplied by zeros: they must hold numbers
   for (int e = tid; e < 2 * RING * WP; e += NT + 32) (&sm.ring[0][0][0])[e] = 0.0;
@@ -470,7 +538,7 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
     const int lane = tid;
     int sload = (L - 1) % a;
     auto prefetch = [&](int c) {
-      if (c >= 0) {
+      if (c >= lo) {
         const int sc = sload;
         sload = sload == 0 ? a - 1 : sload - 1;
         for (int p = lane; p <= a; p += 32) {
@@ -490,7 +558,7 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
     bar(NT + 32);
     int s1 = -1;  // slot of row c + 1, whose diagonal entry d the window lacks
     double d = 0.0;
-    for (int c = L - 1; c >= 0; --c) {
+    for (int c = L - 1; c >= lo; --c) {
       cp_async_wait<AHEAD - 2>();  // column c - 1 has arrived
       bar(NT + 32);
       const double* l = sm.ring[0][c % RING];
@@ -509,36 +577,37 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
       d = __shfl_sync(0xffffffffu, acc, 0);
       if (lane == 0) {
         sm.dg[c & 1] = d;
-        out[(int64_t)c * W] = d;
+        if (outs) out[(int64_t)c * W] = d;
       }
       s1 = s1 < 0 ? (L - 1) % a : (s1 == 0 ? a - 1 : s1 - 1);
       prefetch(c - AHEAD);
     }
+    bar(NT + 32);  // the last diagonal entry
   } else {
     const int rt = tid - 32, u = rt / TP, part = rt % TP;
     double V[CP];
     {
-      // rows L .. L + a - 1 from the parent's front
-      const int k1 = R.k0 + L - 1;
+      const int sL = L % a;
+      auto off = [&](int v) { return v >= sL ? v - sL : v - sL + a; };
+      const int k1 = R.k0 + R.L - 1;
       const int64_t p = S.sn_par[k1];
       const int Jp = (int)(S.rows_ptr[p + 1] - S.rows_ptr[p]);
       const double* Fp = ws + S.f_off[p];
       const int32_t* rel = S.rel + S.rows_ptr[k1] + 1;
-      const int sL = L % a;
-      auto pos = [&](int s) { return __ldg(rel + (s >= sL ? s - sL : s - sL + a)); };
 #pragma unroll
       for (int j = 0; j < CP; ++j) {
         const int v = part + TP * j;
         V[j] = 0.0;
         if (u < a && v < a) {
-          const int pr = pos(u), pc = pos(v);
-          V[j] = __ldcg(Fp + (pr >= pc ? pr + (int64_t)pc * Jp : pc + (int64_t)pr * Jp));
+          const int x = max(off(u), off(v)), y = min(off(u), off(v));
+          if (sp.in) V[j] = sp.in[x + (int64_t)y * a];
+          else if (sp.top) V[j] = __ldcg(Fp + __ldg(rel + x) + (int64_t)__ldg(rel + y) * Jp);
         }
       }
     }
     bar(NT + 32);
     int s = (L - 1) % a;
-    for (int c = L - 1; c >= 0; --c) {
+    for (int c = L - 1; c >= lo; --c) {
       const double* l = sm.ring[0][c % RING];
       const double* mm = sm.ring[1][c % RING];
       // one accumulator: a warp issues an FP64 instruction every 64 clocks at
@@ -561,7 +630,7 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
         tv[rt] = t;
         int p = rt - s;
         if (p <= 0) p += a;
-        out[(int64_t)c * W + p] = t;
+        if (outs) out[(int64_t)c * W + p] = t;
       }
       bar2_sync(NT + 32);
       // the new row into the registers: column slot s of every row, the
@@ -586,16 +655,36 @@ __device__ void down_run(const SymDev& S, const Run& R, const double* wc, const 
       }
       s = s == 0 ? a - 1 : s - 1;
     }
+    bar(NT + 32);
+    if (sp.win && u < a) {
+      const int sw = lo % a;
+      const int p = u >= sw ? u - sw : u - sw + a;
+#pragma unroll
+      for (int j = 0; j < CP; ++j) {
+        const int v = part + TP * j, q = v >= sw ? v - sw : v - sw + a;
+        if (v < a && p >= q) sp.win[p + (int64_t)q * a] = p == 0 ? sm.dg[lo & 1] : V[j];
+      }
+    }
   }
 }
 constexpr int DNT = 288;
 template <int MODE>
-__device__ __forceinline__ void down_dispatch(const SymDev& S, const Run& R, const double* wc, const double* src,
-                                             double* out, const double* ws, DownSmem& sm) {
-  if (R.a <= 8) down_run<32, 2, 4, MODE>(S, R, wc, src, out, ws, sm);
-  else if (R.a <= 16) down_run<64, 4, 4, MODE>(S, R, wc, src, out, ws, sm);
-  else if (R.a <= 32) down_run<128, 8, 4, MODE>(S, R, wc, src, out, ws, sm);
-  else down_run<256, 16, 4, MODE>(S, R, wc, src, out, ws, sm);
+__device__ __forceinline__ void down_dispatch(const SymDev& S, const Run& R, const DownSpan& sp, const double* wc,
+                                             const double* src, double* out, const double* ws, DownSmem& sm) {
+  if (R.a <= 8) down_run<32, 2, 4, MODE>(S, R, sp, wc, src, out, ws, sm);
+  else if (R.a <= 16) down_run<64, 4, 4, MODE>(S, R, sp, wc, src, out, ws, sm);
+  else if (R.a <= 32) down_run<128, 8, 4, MODE>(S, R, sp, wc, src, out, ws, sm);
+  else down_run<256, 16, 4, MODE>(S, R, sp, wc, src, out, ws, sm);
+}
+// by segments: phase 1: every segment but the first from a zero window, the
+// last one from the parent and for good; phase 2: the others from their windows
+__device__ __forceinline__ bool down_seg(const SymDev& S, const ChainSeg& g, const Run& R, int phase, double* ws,
+                                         DownSpan& sp) {
+  const bool last = g.p == g.P - 1;
+  if (phase == 1 ? g.p == 0 && g.P > 1 : last) return false;
+  sp = DownSpan{g.e - 1, g.s, phase == 2 ? seg_window(R, g.e, ws) : nullptr, last, phase == 2 || last,
+                phase == 1 && g.p > 0 ? seg_window(R, g.s, ws) : nullptr};
+  return true;
 }
 
 // Algorithm 7.2 for one-column fronts (Algorithm 4.1): S_AN = -V L_AN,
@@ -605,7 +694,17 @@ __global__ void __launch_bounds__(DNT) kc_gradient(SymDev S, int task0, const do
                                                   const double* ws) {
   __shared__ DownSmem sm;
   const Run R = run_of(S, task0 + blockIdx.x);
-  down_dispatch<DOWN_GRAD>(S, R, Wc + R.base0, nullptr, Sc + R.base0, ws, sm);
+  down_dispatch<DOWN_GRAD>(S, R, DownSpan{R.L - 1, 0, nullptr, true, true, nullptr}, Wc + R.base0, nullptr,
+                           Sc + R.base0, ws, sm);
+}
+__global__ void __launch_bounds__(DNT) kc_gradient_seg(SymDev S, int task0, int phase, const double* Wc, double* Sc,
+                                                      double* ws) {
+  __shared__ DownSmem sm;
+  const ChainSeg g = S.cseg[blockIdx.x];
+  const Run R = run_of(S, task0 + g.run);
+  DownSpan sp;
+  if (!down_seg(S, g, R, phase, ws, sp)) return;
+  down_dispatch<DOWN_GRAD>(S, R, sp, Wc + R.base0, nullptr, Sc + R.base0, ws, sm);
 }
 __global__ void __launch_bounds__(MT) kc_grad_post(SymDev S, int task0, const double* Sc, double* g, double* Vd,
                                                   const double* ws) {
@@ -657,7 +756,135 @@ __global__ void __launch_bounds__(DNT) kc_hess_down(SymDev S, int task0, const d
   const Run R = run_of(S, task0 + blockIdx.x);
   const int64_t y = blockIdx.y;
   double* t = T + y * ldt + R.base0;
-  down_dispatch<DOWN_HESS>(S, R, Wc + R.base0, t, t, ws + y * S.f_total, sm);
+  down_dispatch<DOWN_HESS>(S, R, DownSpan{R.L - 1, 0, nullptr, true, true, nullptr}, Wc + R.base0, t, t,
+                           ws + y * S.f_total, sm);
+}
+__global__ void __launch_bounds__(DNT) kc_hess_down_seg(SymDev S, int task0, int phase, const double* Wc, double* T,
+                                                       int64_t ldt, double* ws) {
+  __shared__ DownSmem sm;
+  const ChainSeg g = S.cseg[blockIdx.x];
+  const Run R = run_of(S, task0 + g.run);
+  const int64_t y = blockIdx.y;
+  ws += y * S.f_total;
+  DownSpan sp;
+  if (!down_seg(S, g, R, phase, ws, sp)) return;
+  double* t = T + y * ldt + R.base0;
+  down_dispatch<DOWN_HESS>(S, R, sp, Wc + R.base0, t, t, ws, sm);
+}
+
+// ---------------------------------------------------------------------------
+// Segments.  Along a run the gradient and both Hessian passes are affine in
+// the window that passes from front to front: over a segment of columns
+//   top-down   V_low  = Psi V_high Psi^T + C,
+//   bottom-up  U_high = Psi^T U_low Psi + B,
+// with the same a x a matrix Psi (rows: the window at the segment's lower end,
+// in terms of the one at its upper end), which depends on L only.  So all
+// segments run at once from a zero window (phase 1), the windows at their
+// ends follow from one small congruence per segment, and all run again from
+// their true windows (phase 2).  Twice the work, but on as many SMs as there
+// are segments instead of one: every value is computed by the same recursion
+// as in the serial kernels, from windows whose error is that of one more
+// congruence.  kc_psi propagates the rows of Psi; its columns are independent
+// of each other, so it needs no exchange between threads.
+// ---------------------------------------------------------------------------
+constexpr int PSX = 16;  // columns of Psi per CTA, four threads each
+__global__ void __launch_bounds__(4 * PSX) kc_psi(SymDev S, int task0, const double* Wc, double* Psi) {
+  __shared__ double Lb[2][RING][WP];
+  const ChainSeg g = S.cseg[blockIdx.x];
+  const int tid = threadIdx.x, part = tid & 3, x = blockIdx.y * PSX + (tid >> 2);
+  const Run R = run_of(S, task0 + g.run);
+  const int a = R.a, W = a + 1;
+  if (g.p == 0 || g.p == g.P - 1 || (int)(blockIdx.y * PSX) >= a) return;
+  const double* wc = Wc + R.base0;
+  double X[AMAX / 4];
+  const int se = g.e % a;
+#pragma unroll
+  for (int j = 0; j < AMAX / 4; ++j) {
+    const int v = part + 4 * j, q = v >= se ? v - se : v - se + a;
+    X[j] = v < a && q == x ? 1.0 : 0.0;
+  }
+  auto load = [&](int c0, int b) {  // columns c0, c0 - 1, .. c0 - RING + 1
+    for (int k = 0; k < RING; ++k)
+      if (c0 - k >= g.s)
+        for (int p = tid; p < W; p += 4 * PSX) cp_async8(&Lb[b][k][p], wc + (int64_t)(c0 - k) * W + p);
+    cp_async_commit();
+  };
+  int b = 0, sc = (g.e - 1) % a;
+  load(g.e - 1, 0);
+  for (int c0 = g.e - 1; c0 >= g.s; c0 -= RING, b ^= 1) {
+    __syncthreads();
+    load(c0 - RING, b ^ 1);
+    cp_async_wait<1>();
+    __syncthreads();
+    for (int k = 0; k < RING && c0 - k >= g.s; ++k) {
+      const double* l = Lb[b][k];
+      double y = 0.0;
+#pragma unroll
+      for (int j = 0; j < AMAX / 4; ++j) {
+        const int v = part + 4 * j;
+        int p = v - sc;
+        if (p <= 0) p += a;
+        if (4 * j < a) y = fma(X[j], v < a ? l[p] : 0.0, y);
+      }
+      y += __shfl_xor_sync(0xffffffffu, y, 1);
+      y += __shfl_xor_sync(0xffffffffu, y, 2);
+      if (part == (sc & 3)) {
+#pragma unroll
+        for (int j = 0; j < AMAX / 4; ++j)
+          if (j == sc >> 2) X[j] = -y;
+      }
+      sc = sc == 0 ? a - 1 : sc - 1;
+    }
+  }
+  if (x >= a) return;
+  const int ss = g.s % a;
+#pragma unroll
+  for (int j = 0; j < AMAX / 4; ++j) {
+    const int v = part + 4 * j, p = v >= ss ? v - ss : v - ss + a;
+    if (v < a) Psi[g.psi + p + (int64_t)x * a] = X[j];
+  }
+}
+// One step of the windows' recursion on every run: Z = M V (half 0), then
+// win += Z M^T (half 1, lower), M = Psi (top-down) or Psi^T (bottom-up);
+// 16 x 16 outputs per CTA
+template <bool UP>
+__global__ void __launch_bounds__(256) kc_scan(SymDev S, int task0, int step, int half, const double* Psi,
+                                              double* ws) {
+  __shared__ double A[16][AMAX + 1], B[AMAX][17];
+  const int r = blockIdx.y;
+  const int2 rs = S.crun[r];
+  const int p = UP ? 1 + step : rs.y - 2 - step;
+  if (p < 1 || p > rs.y - 2) return;
+  const Run R = run_of(S, task0 + r);
+  const int a = R.a, i0 = (blockIdx.x & 3) * 16, j0 = (blockIdx.x >> 2) * 16, tid = threadIdx.x;
+  if (i0 >= a || j0 >= a || (half && i0 < j0)) return;
+  ws += (int64_t)blockIdx.z * S.f_total;
+  const ChainSeg g = S.cseg[rs.x + p], src = S.cseg[UP ? rs.x + p - 1 : rs.x + p + 1];
+  const double* M = Psi + g.psi;
+  double* win = seg_window(R, g.s, ws);
+  double* Z = win + R.fstride;
+  const double* V = seg_window(R, src.s, ws);
+  auto m = [&](int i, int k) { return UP ? M[k + (int64_t)i * a] : M[i + (int64_t)k * a]; };
+  for (int e = tid; e < 16 * AMAX; e += 256) {
+    const int i = e & 15, k = e >> 4;
+    double x = 0.0, y = 0.0;
+    if (k < a) {
+      if (i0 + i < a) x = half ? Z[i0 + i + (int64_t)k * a] : m(i0 + i, k);
+      if (j0 + i < a) {
+        const int j = j0 + i;
+        y = half ? m(j, k) : V[max(k, j) + (int64_t)min(k, j) * a];
+      }
+    }
+    A[i][k] = x;
+    B[k][i] = y;
+  }
+  __syncthreads();
+  const int i = tid & 15, j = tid >> 4;
+  double acc = 0.0;
+  for (int k = 0; k < a; ++k) acc = fma(A[i][k], B[k][j], acc);
+  if (i0 + i >= a || j0 + j >= a) return;
+  if (half == 0) Z[i0 + i + (int64_t)(j0 + j) * a] = acc;
+  else if (i0 + i >= j0 + j) win[i0 + i + (int64_t)(j0 + j) * a] += acc;
 }
 
 // Algorithm 5.2 steps 1-2 for one-column fronts: V' is the input T on
@@ -776,6 +1003,33 @@ static unsigned columns(const chd_symbolic* s, int t0, int nt, int per, int extr
   for (int t = t0; t < t0 + nt; ++t) L = std::max<int64_t>(L, s->task_ptr[t + 1] - s->task_ptr[t] + extra);
   return (unsigned)std::min<int64_t>((L + per - 1) / per, 32768);
 }
+// Whether m right-hand sides run by segments (the times of the analysis, in
+// us): the serial kernels take one SM per run and right-hand side for
+// cseg_serial; by segments every column is done twice, all segments sharing
+// the SMs, and every segment adds two launches of small products.
+static bool by_segments(const chd_symbolic* s, int m, const double* psi) {
+  if (!psi || s->cseg.empty()) return false;
+  const double runs = (double)s->crun.size() / 2, segs = (double)s->cseg.size();
+  const double serial = std::max(1.0, m * runs / 152.0) * s->cseg_serial;
+  const double seg = 2.0 * std::max(1.0, m * segs / 152.0) * s->cseg_column +
+                     s->cseg_steps * s->cseg_step * std::max(1.0, m * runs / 40.0);
+  return seg < 0.8 * serial;
+}
+template <bool UP>
+static void scan(const chd_symbolic* s, cudaStream_t st, int t0, int m, const double* psi, double* ws) {
+  const int nr = (int)s->crun.size() / 2;
+  for (int step = 0; step < s->cseg_steps; ++step)
+    for (int half = 0; half < 2; ++half) {
+      kc_scan<UP><<<dim3(16, nr, m), 256, 0, st>>>(s->dev, t0, step, half, psi, ws);
+      count_launch();
+    }
+}
+// Psi of every inner segment (once per factor)
+void chain_psi(const chd_symbolic* s, cudaStream_t st, const double* Wc, double* psi) {
+  if (s->cseg.empty() || !psi) return;
+  kc_psi<<<dim3((unsigned)s->cseg.size(), AMAX / PSX), 4 * PSX, 0, st>>>(s->dev, s->lvl_ptr[0], Wc, psi);
+  count_launch();
+}
 void chain_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* X, double* Lc, double* Wc,
                   double* Dd, double* ws, double* ldet, int64_t* status) {
   kc_factor<<<nt, UPT, 0, st>>>(s->dev, t0, X, Lc, Wc, Dd, ws, status);
@@ -788,25 +1042,53 @@ void chain_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const
   count_launch();
 }
 void chain_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Wc, double* Sc, double* g,
-                    double* Vd, double* ws) {
-  kc_gradient<<<nt, DNT, 0, st>>>(s->dev, t0, Wc, Sc, ws);
-  count_launch();
+                    double* Vd, double* ws, double* psi) {
+  if (by_segments(s, 1, psi)) {
+    const unsigned ns = (unsigned)s->cseg.size();
+    kc_gradient_seg<<<ns, DNT, 0, st>>>(s->dev, t0, 1, Wc, Sc, ws);
+    count_launch();
+    scan<false>(s, st, t0, 1, psi, ws);
+    kc_gradient_seg<<<ns, DNT, 0, st>>>(s->dev, t0, 2, Wc, Sc, ws);
+    count_launch();
+  } else {
+    kc_gradient<<<nt, DNT, 0, st>>>(s->dev, t0, Wc, Sc, ws);
+    count_launch();
+  }
   kc_grad_post<<<dim3(nt, columns(s, t0, nt, 1, 0)), MT, 0, st>>>(s->dev, t0, Sc, g, Vd, ws);
   count_launch();
 }
 void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, const double* Vd,
-                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act) {
-  kc_hess_up<<<dim3(nt, m), UPT, 0, st>>>(s->dev, t0, Wc, Y, ldy, T, ldt, ws, act);
-  count_launch();
+                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act,
+                   const double* psi) {
+  if (!act && by_segments(s, m, psi)) {
+    const unsigned ns = (unsigned)s->cseg.size();
+    kc_hess_up_seg<<<dim3(ns, m), UPT, 0, st>>>(s->dev, t0, 1, Wc, Y, ldy, T, ldt, ws);
+    count_launch();
+    scan<true>(s, st, t0, m, psi, ws);
+    kc_hess_up_seg<<<dim3(ns, m), UPT, 0, st>>>(s->dev, t0, 2, Wc, Y, ldy, T, ldt, ws);
+    count_launch();
+  } else {
+    kc_hess_up<<<dim3(nt, m), UPT, 0, st>>>(s->dev, t0, Wc, Y, ldy, T, ldt, ws, act);
+    count_launch();
+  }
   kc_hess_m<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Vd, T, ldt, act);
   count_launch();
 }
 void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
-                     int64_t ldt, double* ws) {
+                     int64_t ldt, double* ws, const double* psi) {
   kc_down_pre<<<dim3(nt, columns(s, t0, nt, 4, 0), m), 128, 0, st>>>(s->dev, t0, Wc, T, ldt);
   count_launch();
-  kc_hess_down<<<dim3(nt, m), DNT, 0, st>>>(s->dev, t0, Wc, T, ldt, ws);
-  count_launch();
+  if (by_segments(s, m, psi)) {
+    const unsigned ns = (unsigned)s->cseg.size();
+    kc_hess_down_seg<<<dim3(ns, m), DNT, 0, st>>>(s->dev, t0, 1, Wc, T, ldt, ws);
+    count_launch();
+    scan<false>(s, st, t0, m, psi, ws);
+    kc_hess_down_seg<<<dim3(ns, m), DNT, 0, st>>>(s->dev, t0, 2, Wc, T, ldt, ws);
+    count_launch();
+  } else {
+    kc_hess_down<<<dim3(nt, m), DNT, 0, st>>>(s->dev, t0, Wc, T, ldt, ws);
+    count_launch();
+  }
 }
 void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
                       const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy,

@@ -50,6 +50,12 @@ struct alignas(16) GChild {
   int32_t pad;
 };
 
+// one segment of a chain run (chain_tier.cu): columns s .. e - 1 of run
+// `run` (index among level 0's runs), p-th of P from the bottom
+struct alignas(16) ChainSeg {
+  int32_t run, p, P, s, e, pad;
+  int64_t psi;  // offset of its a x a matrix Psi
+};
 // grouped inverse of V_k: one front
 struct alignas(16) GJob {
   int64_t v_off, w_off;  // V_k slot, workspace (a x a)
@@ -108,6 +114,8 @@ struct SymDev {
   const int2 *gt_up = nullptr, *gt_row = nullptr, *gt_asm = nullptr, *gt_p = nullptr, *gt_gat = nullptr,
              *gt_nn = nullptr, *gt_asmf = nullptr, *gt_wb = nullptr, *gt_fr = nullptr;
   const int32_t* gleg = nullptr;
+  const ChainSeg* cseg = nullptr;
+  const int2* crun = nullptr;  // per run: first segment, number of segments
   const GJob* gj = nullptr;
   const int2 *gv_all = nullptr, *gv_sol = nullptr, *gv_upd = nullptr;
   const int32_t* gv_small = nullptr;
@@ -153,6 +161,14 @@ struct chd_symbolic {
   std::vector<int32_t> lvl_r32, lvl_r64;
   // lowest level that waits for a chain run, and whether other tasks lie below it
   int32_t run_join = 0, run_overlap = 0;
+  // segments of the runs (none when the serial kernels are faster), (first,
+  // count) per run, doubles of all Psi, most inner segments of a run; modelled
+  // times in us: longest run, longest segment, one step of the windows
+  std::vector<ChainSeg> cseg;
+  std::vector<int32_t> crun;
+  int64_t cseg_psi = 0;
+  int cseg_steps = 0;
+  double cseg_serial = 0, cseg_column = 0, cseg_step = 0;
   // per level l, five counts at 5*l: chain runs (|J| <= 32), chain runs
   // (|J| <= 64), warp, wide warp and dense-tier tasks (chd_symbolic_schedule)
   std::vector<int32_t> lvl_counts;
@@ -238,6 +254,7 @@ struct Exec {
   size_t tc_cap[kSideStreams + 1] = {};
   int64_t* status = nullptr;  // the factor's status (tensor-core timeouts)
   int tc_mode = 0;
+  double* psi = nullptr;      // chain segments' matrices, when the pattern has segments
   // streams for the other launches of a level, with their fork and join events
   int naux = 0;
   cudaStream_t aux[kAuxStreams] = {};
@@ -325,6 +342,7 @@ struct chd_factor {
   int64_t act_rhs = 0;       // capacity of act_buf in right-hand sides
   size_t ws_limit = 0;       // caller's cap on the workspace (0: library default)
   bool have_S = false;
+  bool have_psi = false;     // ex.psi belongs to the current factor
   bool have_R = false;
   bool have_Q = false;
   // CUDA graphs of the launch sequences, replayed on the private stream gs

@@ -1077,11 +1077,13 @@ void chain_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const 
                   double* Dd, double* ws, double* ldet, int64_t* status);
 void chain_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws);
 void chain_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Wc, double* Sc, double* g,
-                    double* Vd, double* ws);
+                    double* Vd, double* ws, double* psi);
+void chain_psi(const chd_symbolic* s, cudaStream_t st, const double* Wc, double* psi);
 void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, const double* Vd,
-                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act);
+                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act,
+                   const double* psi);
 void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
-                     int64_t ldt, double* ws);
+                     int64_t ldt, double* ws, const double* psi);
 void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
                       const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy,
                       double* ws);
@@ -1364,12 +1366,13 @@ void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
               double* Vd, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
   Beside bs(ex, st);
+  if (ex) chain_psi(s, st, Wc, ex->psi);
   group_zero(s, st, 1, ws);
   // chain runs (level 0) start as soon as their parents are done
   const Level r = level(s, 0);
   const int run_at = s->run_overlap ? s->run_join : 1;
   auto runs = [&](cudaStream_t sr) {
-    if (r.nr32 + r.nr64) chain_gradient(s, sr, r.tr, r.nr32 + r.nr64, Wc, Sc, g, Vd, ws);
+    if (r.nr32 + r.nr64) chain_gradient(s, sr, r.tr, r.nr32 + r.nr64, Wc, Sc, g, Vd, ws, ex ? ex->psi : nullptr);
   };
   if (run_at >= nl) runs(st);
   for (int l = nl - 1; l >= 0; --l) {
@@ -1415,7 +1418,7 @@ void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m,
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_hess_up(s, sl, m, dense[i], Wc, Vd, Y, ldy, T, ldt, ws, act);
     });
-    if (v.nr32 + v.nr64) chain_hess_up(s, bs.fork(AUX_RUN, !s->run_overlap), v.tr, v.nr32 + v.nr64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
+    if (v.nr32 + v.nr64) chain_hess_up(s, bs.fork(AUX_RUN, !s->run_overlap), v.tr, v.nr32 + v.nr64, m, Wc, Vd, Y, ldy, T, ldt, ws, act, ex ? ex->psi : nullptr);
     if (v.nwarp)
       (w32_few(v.nwarp, m) ? w32x::warp_hess_up : w32::warp_hess_up)(s, sw, v.t0, v.nwarp, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
     if (v.nw64) w64::warp_hess_up(s, sv, v.tw, v.nw64, m, Wc, Vd, Y, ldy, T, ldt, ws, act);
@@ -1443,7 +1446,7 @@ void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int 
   const Level r = level(s, 0);
   const int run_at = s->run_overlap ? s->run_join : 1;
   auto runs = [&](cudaStream_t sr) {
-    if (r.nr32 + r.nr64) chain_hess_down(s, sr, r.tr, r.nr32 + r.nr64, m, Wc, T, ldt, ws);
+    if (r.nr32 + r.nr64) chain_hess_down(s, sr, r.tr, r.nr32 + r.nr64, m, Wc, T, ldt, ws, ex ? ex->psi : nullptr);
   };
   if (run_at >= nl) runs(st);
   for (int l = nl - 1; l >= 0; --l) {

@@ -647,6 +647,65 @@ static void group_completion_plan(chd_symbolic* s) {
   }
 }
 
+// Segments of the chain runs (chain_tier.cu).  A column costs about 0.3 + 0.02 a
+// us in the serial kernels (0.4 at a = 8, 1.6 at a = 61), one step of the
+// windows' recursion 12 us (two launches of a x a products).  With P segments of
+// the longest run the two phases take 2 T / P and the windows 12 P: P =
+// sqrt(T / 6).  Runs too short to gain 30 % keep the serial kernels.
+static void chain_segments_plan(chd_symbolic* s) {
+  s->cseg.clear();
+  s->crun.clear();
+  s->cseg_psi = 0;
+  s->cseg_steps = 0;
+  if (s->lvl_r32.empty()) return;
+  const int nr = s->lvl_r32[0] + s->lvl_r64[0];
+  if (nr == 0) return;
+  const int t0 = s->lvl_ptr[0];
+  auto len = [&](int r) { return s->task_ptr[t0 + r + 1] - s->task_ptr[t0 + r]; };
+  auto anc = [&](int r) { return front_J(s, s->task_fronts[s->task_ptr[t0 + r]]) - 1; };
+  auto time = [&](int r) { return len(r) * (0.3 + 0.02 * anc(r)); };
+  double tmax = 0;
+  for (int r = 0; r < nr; ++r) tmax = std::max(tmax, time(r));
+  constexpr double kStep = 12.0;
+  const double pbest = std::min(64.0, std::max(1.0, std::floor(std::sqrt(tmax / (0.5 * kStep)))));
+  double tau = tmax / pbest;
+  auto count = [&](int r, double t) {
+    const int P = (int)std::floor(time(r) / t + 0.5);
+    return std::max(1, std::min(P, len(r) / 16));
+  };
+  int64_t total = 0;
+  for (;; tau *= 1.25) {
+    total = 0;
+    for (int r = 0; r < nr; ++r) total += count(r, tau);
+    if (total <= std::max(152, 2 * nr) || tau >= tmax) break;
+  }
+  int pmax = 1;
+  for (int r = 0; r < nr; ++r) pmax = std::max(pmax, count(r, tau));
+  const double waves = std::max(1.0, total / 152.0);
+  s->cseg_serial = tmax;
+  s->cseg_column = tau;
+  s->cseg_step = kStep;
+  if (pmax < 2 || 2.0 * tau * waves + kStep * (pmax - 2) > 0.7 * tmax * std::max(1.0, nr / 152.0)) return;
+  for (int r = 0; r < nr; ++r) {
+    const int P = count(r, tau), L = len(r);
+    const int64_t a = anc(r);
+    s->crun.push_back((int32_t)s->cseg.size());
+    s->crun.push_back(P);
+    for (int p = 0; p < P; ++p) {
+      ChainSeg g{};
+      g.run = r;
+      g.p = p;
+      g.P = P;
+      g.s = (int32_t)((int64_t)L * p / P);
+      g.e = (int32_t)((int64_t)L * (p + 1) / P);
+      g.psi = s->cseg_psi;
+      s->cseg_psi += (a * a + 3) & ~int64_t(3);
+      s->cseg.push_back(g);
+    }
+  }
+  s->cseg_steps = std::max(0, pmax - 2);
+}
+
 chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* rowind,
                               const chd_opts& opts, chd_symbolic* s) {
   if (n < 1 || !colptr || !rowind) return CHD_ERR_INVALID;
@@ -1217,5 +1276,6 @@ chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* r
   group_plan(s);
   group_inverse_plan(s);
   group_completion_plan(s);
+  chain_segments_plan(s);
   return CHD_OK;
 }

@@ -55,6 +55,38 @@ def test_chain_window_sizes(a, extra):
             assert err(r_on[k][i], r_off[k][i]) < 1e-11, k
 
 
+@pytest.mark.parametrize("bands", [[(5000, 1)], [(2500, 8)], [(1300, 24)], [(701, 61)], [(900, 64)],
+                                   [(1500, 30), (200, 5), (620, 47), (1400, 12)]])
+def test_chain_segments(bands):
+    """Runs long enough to be cut into segments (alone, and of several lengths
+    in one object): the gradient and both Hessian passes against the same
+    patterns without chain runs, on a factor and on a completion (whose
+    segments' matrices do not come from a gradient)."""
+    from paper_1203_2742_gb300 import binding as B
+    pats = [W.band(n, w) for n, w in bands]
+    make = (lambda **o: B.Symbolic(*pats[0], **o)) if len(pats) == 1 else (lambda **o: B.SymbolicBatch(pats, **o))
+    rng = np.random.default_rng(len(pats) + bands[0][0])
+    on, off = make(chain_runs=True), make(chain_runs=False)
+    n, cp, ri = on.n, on.colptr, on.rowind
+    x = W.diag_dominant(n, cp, ri, rng)
+    ys = W.uniform_sym(n, cp, ri, rng, count=2)
+    s = W.projected_gram(n, cp, ri, rng.standard_normal((n, 6)), 1.0)
+    err = lambda p, q: OD.rel_err(n, cp, ri, p, q)
+    res = []
+    for sym in (on, off):
+        f = sym.factor(_dev(x))
+        fx, _ = sym.complete(_dev(s))
+        res.append((_host(f.gradient()), _host(f.hessian(_dev(ys))), _host(f.inv_hessian(f.hessian(_dev(ys)))),
+                    _host(fx.hessian(_dev(ys))), _host(fx.gradient())))
+        assert f.status() == 0 and fx.status() == 0
+    assert err(res[0][0], res[1][0]) < 1e-12
+    assert err(-res[0][4], s) < 1e-10
+    for i in range(2):
+        assert err(res[0][1][i], res[1][1][i]) < 1e-12
+        assert err(res[0][2][i], ys[i]) < 1e-9
+        assert err(res[0][3][i], res[1][3][i]) < 1e-9
+
+
 @pytest.mark.parametrize("col", [0, 1, 2, 17])
 def test_chain_not_pd(col):
     """A non-positive pivot inside a run is reported with its column."""
