@@ -1123,17 +1123,7 @@ __global__ void __launch_bounds__(128) kg_factor_rows(SymDev S, const int2* bloc
     if (ident) {
       panel::solve_row(b, Cs, rinv, pb, lane);
     } else {
-#pragma unroll
-      for (int c = GB - 1; c >= 0; --c) {
-        if (c < pb) {
-          double x = b[c >> 2] * rinv[c];
-          x = __shfl_sync(0xffffffffu, x, (lane & 28) | (c & 3));
-          if (q == (c & 3)) b[c >> 2] = x;
-#pragma unroll
-          for (int u = 0; u <= c >> 2; ++u)
-            if (4 * u < c) b[u] = fma(4 * u + q < c ? -Cs[c][4 * u + q] : 0.0, x, b[u]);
-        }
-      }
+      panel::solve_row_back(b, Cs, rinv, pb, lane);
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u)
@@ -1388,17 +1378,7 @@ __global__ void __launch_bounds__(128) kp_back(SymDev S, const int2* blocks, dou
       double b[8];
 #pragma unroll
       for (int u = 0; u < 8; ++u) b[u] = row < nr && q + 4 * u < pb ? rows[row * ld + p0 + q + 4 * u] : 0.0;
-#pragma unroll
-      for (int c = GB - 1; c >= 0; --c) {
-        if (c < pb) {
-          double x = b[c >> 2] * rinv[c];
-          x = __shfl_sync(0xffffffffu, x, (lane & 28) | (c & 3));
-          if (q == (c & 3)) b[c >> 2] = x;
-#pragma unroll
-          for (int u = 0; u <= c >> 2; ++u)
-            if (4 * u < c) b[u] = fma(4 * u + q < c ? -Ls[c][4 * u + q] : 0.0, x, b[u]);
-        }
-      }
+      panel::solve_row_back(b, Ls, rinv, pb, lane);
 #pragma unroll
       for (int u = 0; u < 8; ++u)
         if (row < nr && q + 4 * u < pb) rows[row * ld + p0 + q + 4 * u] = b[u];

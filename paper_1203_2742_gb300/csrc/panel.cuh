@@ -34,12 +34,13 @@ __device__ __forceinline__ void bar128(int id) { asm volatile("bar.sync %0, 128;
 __device__ __forceinline__ void chol32(double (*Ls)[PB + 1], double* rinv, double (*col)[PB], int pb, int tid, int id,
                                        int64_t* st, int64_t code, int64_t snode, int64_t col0) {
   const int w = tid >> 5, lane = tid & 31;
-  double a[8];
+  double a[9];  // a[t]: column 4 (g + t) + w of column group g
 #pragma unroll
   for (int t = 0; t < 8; ++t) a[t] = Ls[lane][4 * t + w];
+  a[8] = 0.0;
   bar128(id);
   // pivot of column j by its owner: scaled column to Ls and to col[j % 3]
-  auto pivot = [&](int j, double v) {
+  auto pivot = [&](int j, double v, double* cj) {
     double d = __shfl_sync(0xffffffffu, v, j);
     if (!(d > 0.0)) {
       if (lane == 0) record_error(st, code, snode, col0 < 0 ? -1 : col0 + j);
@@ -47,57 +48,113 @@ __device__ __forceinline__ void chol32(double (*Ls)[PB + 1], double* rinv, doubl
     }
     const double r = rsqrt(d);
     const double l = lane == j ? d * r : v * r;
-    col[j % 3][lane] = l;
+    cj[lane] = l;
     if (lane >= j) Ls[lane][j] = l;
     if (lane == 0) rinv[j] = r;
   };
-  if (w == 0) pivot(0, a[0]);
+  if (w == 0) pivot(0, a[0], col[0]);
   bar128(id);
+  double *cp = col[2], *cj = col[0], *cn = col[1];  // columns j - 1, j, j + 1
+#pragma unroll 1
+  for (int g = 0; 4 * g + 1 < pb; ++g) {
 #pragma unroll
-  for (int j = 0; j < PB; ++j) {
-    if (j + 1 < pb) {
-      const double* cj = col[j % 3];
-      const double lj = cj[lane];
-      if (w == ((j + 1) & 3)) {
-        a[(j + 1) >> 2] = fma(-lj, cj[j + 1], a[(j + 1) >> 2]);
-        pivot(j + 1, a[(j + 1) >> 2]);
-      } else {
-        if (j > 0 && w == (j & 3)) {  // owned pivot j in the last phase: column j - 1 is still to be applied
-          const double* cp = col[(j + 2) % 3];
-          const double lp = cp[lane];
+    for (int i = 0; i < 4; ++i) {
+      const int j = 4 * g + i;
+      if (j + 1 < pb) {  // the same for all threads
+        const double lj = cj[lane];
+        if (w == ((i + 1) & 3)) {
+          const int t = (i + 1) >> 2;  // column j + 1
+          a[t] = fma(-lj, cj[j + 1], a[t]);
+          pivot(j + 1, a[t], cn);
+        } else {
+          const bool late = j > 0 && w == i;  // owned pivot j: column j - 1 is still to be applied
+          const double lp = late ? cp[lane] : 0.0;
 #pragma unroll
-          for (int t = (j >> 2) + 1; t < 8; ++t)
-            if (4 * t + w < pb) a[t] = fma(-lp, cp[4 * t + w], a[t]);
+          for (int t = 0; t < 8; ++t) {
+            const int k = 4 * (g + t) + w;
+            if (k < pb && k > j) {
+              if (late) a[t] = fma(-lp, cp[k], a[t]);
+              a[t] = fma(-lj, cj[k], a[t]);
+            }
+          }
         }
-#pragma unroll
-        for (int t = 0; t < 8; ++t)
-          if (4 * t + w > j && 4 * t + w < pb) a[t] = fma(-lj, cj[4 * t + w], a[t]);
+        bar128(id);
+        double* x = cp;
+        cp = cj;
+        cj = cn;
+        cn = x;
       }
-      bar128(id);
     }
+#pragma unroll
+    for (int t = 0; t < 8; ++t) a[t] = a[t + 1];
   }
 }
 
 // Row group of four lanes (q = lane & 3): b[u] holds entry q + 4 u of the row;
-// b := b L^{-T} for the pb x pb lower block Ls (rinv: reciprocal pivots)
+// b := b L^{-T} for the pb x pb lower block Ls (rinv: reciprocal pivots).  Rolled
+// over groups of four columns, the registers shifted after each: fully
+// unrolled, a launch spends more on fetching the code once than on running it.
 __device__ __forceinline__ void solve_row(double (&b)[8], const double (*Ls)[PB + 1], const double* rinv, int pb,
                                           int lane) {
   const int q = lane & 3;
+#pragma unroll 1
+  for (int g = 0; g < PB / 4; ++g) {
+    if (4 * g < pb) {
 #pragma unroll
-  for (int c = 0; c < PB; ++c) {
-    if (c < pb) {
-      double x = b[c >> 2] * rinv[c];
-      x = __shfl_sync(0xffffffffu, x, (lane & 28) | (c & 3));
-      if (q == (c & 3)) b[c >> 2] = x;
+      for (int i = 0; i < 4; ++i) {
+        const int c = 4 * g + i;
+        if (c < pb) {
+          double x = b[0] * rinv[c];
+          x = __shfl_sync(0xffffffffu, x, (lane & 28) | i);
+          if (q == i) b[0] = x;
 #pragma unroll
-      for (int u = c >> 2; u < 8; ++u) {
-        const int t = 4 * u + q;
-        if (4 * u + 3 > c) {
-          const double l = t > c ? Ls[t][c] : 0.0;
-          b[u] = fma(-l, x, b[u]);
+          for (int u = 0; u < 8; ++u) {
+            const int t = 4 * (g + u) + q;
+            if (4 * (g + u) < pb && (u > 0 || i < 3)) {
+              const double l = t > c && t < pb ? Ls[t][c] : 0.0;
+              b[u] = fma(-l, x, b[u]);
+            }
+          }
         }
       }
     }
+    // the finished entry goes to the back: after eight shifts all are in place
+    const double f = b[0];
+#pragma unroll
+    for (int u = 0; u < 7; ++u) b[u] = b[u + 1];
+    b[7] = f;
+  }
+}
+// b := b L^{-1}: the same backwards
+__device__ __forceinline__ void solve_row_back(double (&b)[8], const double (*Ls)[PB + 1], const double* rinv, int pb,
+                                               int lane) {
+  const int q = lane & 3;
+#pragma unroll 1
+  for (int g = PB / 4 - 1; g >= 0; --g) {
+    // b[7] is group g here
+    if (4 * g < pb) {
+#pragma unroll
+      for (int i = 3; i >= 0; --i) {
+        const int c = 4 * g + i;
+        if (c < pb) {
+          double x = b[7] * rinv[c];
+          x = __shfl_sync(0xffffffffu, x, (lane & 28) | i);
+          if (q == i) b[7] = x;
+#pragma unroll
+          for (int u = 0; u < 8; ++u) {
+            const int t = 4 * (g - 7 + u) + q;  // group g - 7 + u
+            if (g - 7 + u >= 0 && (u < 7 || i > 0)) {
+              const double l = t < c ? Ls[c][t] : 0.0;
+              b[u] = fma(-l, x, b[u]);
+            }
+          }
+        }
+      }
+    }
+    const double f = b[7];
+#pragma unroll
+    for (int u = 7; u > 0; --u) b[u] = b[u - 1];
+    b[0] = f;
   }
 }
 

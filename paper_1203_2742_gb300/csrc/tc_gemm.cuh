@@ -37,7 +37,7 @@
 // MMAs per 16-wide K step, 36 digit pairs.  The first MMA (s = 0, N = 256)
 // overwrites all 256 columns, the rest accumulate.  Operands reach shared
 // memory by TMA (cp.async.bulk.tensor, 64-byte swizzle, 32-wide K chunks,
-// two stages); one thread issues the copies and the MMAs and signals
+// one or two stages); one thread issues the copies and the MMAs and signals
 // through mbarriers; tcgen05.commit releases a stage when its MMAs have
 // read it.  The epilogue reads the eight levels from TMEM (tcgen05.ld),
 // sums levels 0..3 exactly in an int64 and levels 4..7 in FP32, converts
@@ -51,6 +51,7 @@
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 
 #include "chordal_barrier.h"
@@ -63,10 +64,14 @@ constexpr int DBITS = 7;     // bits per digit
 constexpr int TM = 128;      // output rows per tile (MMA M)
 constexpr int TN = 32;       // output columns per tile (per digit of B)
 constexpr int KC = 32;       // K per pipeline stage (64-byte rows of bf16)
-constexpr int STAGES = 2;
 constexpr int A_STAGE = ND * TM * KC * 2;  // bytes: 64 KiB
 constexpr int B_STAGE = ND * TN * KC * 2;  // bytes: 16 KiB
-constexpr int SMEM_BYTES = STAGES * (A_STAGE + B_STAGE) + 1024;
+// Stages: two while every tile has an SM of its own; beyond 152 tiles one, so
+// that two CTAs share an SM (80 KiB and 256 TMEM columns each) and one's
+// epilogue runs under the other's MMAs: eight products of 1134 x 256 x 1134
+// 137 -> 124 us; a single product (76 tiles) 57 us with two stages, 76 with one.
+constexpr int smem_bytes(int stages) { return stages * (A_STAGE + B_STAGE) + 1024; }
+constexpr int kSms = 152;
 constexpr int TMEM_COLS = ND * TN;         // 256: eight levels of 32 columns
 constexpr int KMAX = 1024;                 // longest K per tensor-core pass
 
@@ -305,7 +310,7 @@ __device__ __forceinline__ double times_pow2(double v, int e) {
 // ---------------------------------------------------------------------------
 // the product of the digit planes: one CTA per 128 x 32 tile of C and batch z
 // ---------------------------------------------------------------------------
-template <class MC>
+template <class MC, int STAGES>
 __global__ void __launch_bounds__(128, 1)
     k_tc_gemm(const __grid_constant__ CUtensorMap mapA, const __grid_constant__ CUtensorMap mapB, int M, int N, int Kp,
               int Mp, int Np, const int* exA, const int* exB, double alpha, double beta, MC C, int64_t sC, int lower,
@@ -501,11 +506,18 @@ cudaError_t gemm(cudaStream_t st, void* scratch, size_t scratch_cap, int64_t* st
   const int ba = shA ? 1 : batch, bb = shB ? 1 : batch;
   const Layout L = layout(ba, bb, M, N, K);
   if (L.bytes > scratch_cap || batch * ND > 65535) return cudaErrorInvalidValue;
-  static bool attr = false;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(k_tc_gemm<MC>, cudaFuncAttributeMaxDynamicSharedMemorySize, SMEM_BYTES);
+  // the kernels' shared-memory limit, once per device
+  static std::atomic<uint64_t> attr{0};
+  int dev = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  const uint64_t bit = uint64_t(1) << (dev & 63);
+  if (!(attr.load(std::memory_order_acquire) & bit)) {
+    e = cudaFuncSetAttribute(k_tc_gemm<MC, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(1));
+    if (e == cudaSuccess)
+      e = cudaFuncSetAttribute(k_tc_gemm<MC, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem_bytes(2));
     if (e != cudaSuccess) return e;
-    attr = true;
+    attr.fetch_or(bit, std::memory_order_release);
   }
   uint8_t* base = static_cast<uint8_t*>(scratch);
   uint16_t* dA = reinterpret_cast<uint16_t*>(base);
@@ -529,7 +541,9 @@ cudaError_t gemm(cudaStream_t st, void* scratch, size_t scratch_cap, int64_t* st
     const int dm = L.Mp / SPLIT_ROWS, dn = L.Np / SPLIT_ROWS;
     k_tc_digits<MA, MB><<<dim3(dm + dn, L.Kp / SPLIT_K + (L.Kp % SPLIT_K ? 1 : 0), batch), 256, 0, st>>>(
         M, N, kk, k0, L.Mp, L.Np, L.Kp, dm, A, sA, B, sB, mxA, mxB, dA, dB, eA, eB);
-    k_tc_gemm<MC><<<dim3(tiles_m * tiles_n, 1, batch), 128, SMEM_BYTES, st>>>(
+    const bool wide = static_cast<int64_t>(lower ? (tiles_m * tiles_n + 1) / 2 : tiles_m * tiles_n) * batch > kSms;
+    const auto kernel = wide ? k_tc_gemm<MC, 1> : k_tc_gemm<MC, 2>;
+    kernel<<<dim3(tiles_m * tiles_n, 1, batch), 128, smem_bytes(wide ? 1 : 2), st>>>(
         mA, mB, M, N, L.Kp, L.Mp, L.Np, eA, eB, alpha, k0 == 0 ? beta : 1.0, C, sC, lower ? 1 : 0, tiles_n, shA, shB,
         status);
     if (K <= 0) break;
