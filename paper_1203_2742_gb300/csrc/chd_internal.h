@@ -32,7 +32,7 @@ struct alignas(16) WMeta {
 constexpr int kGroupBlock = 32;       // rows per block of the assembly and of the update tiles
 constexpr int kGroupThin = 16;        // thin fronts: up to this many columns
 constexpr int kGroupFactor = 32;      // fronts up to this many columns factor in one launch per sub-level
-constexpr int kGroupCols = 128;       // widest front of the tier
+constexpr int kGroupCols = 256;       // widest front of the tier
 constexpr int kGroupSmem = 200 << 10; // dynamic shared memory a kernel of the tier may use
 struct alignas(16) GFront {
   int64_t base, f_off, fp_off, d_off, v_off, rel_off;  // values, workspace, parent's workspace, D_NN, V_k, rel of A_k

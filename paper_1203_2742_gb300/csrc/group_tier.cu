@@ -682,47 +682,60 @@ __global__ void __launch_bounds__(RT) kg_nn(SymDev S, const int2* blocks, const 
   if (act && !act[y * S.nsn + f.k]) return;
   ws += y * S.f_total;
   const int n = f.n, J = f.J, tid = threadIdx.x, i0 = d.y * 16, ld = n | 1;
-  double* K = dyn;           // n x n, full
-  double* X = K + n * ld;    // 16 x n
+  double* Br = dyn;               // 16 x n: rows i0 .. of B
+  double* X = Br + 16 * ld;       // 16 x n: B K
+  double* Cs = X + 16 * ld;       // n x 32: columns of K, then of B
   const double* F = ws + f.f_off;
   const double* T2 = F + (int64_t)J * J + (int64_t)J * n;
   const double* W = Wc + f.base;
   const double* D = MODE == NN_IH ? Dd + f.d_off : nullptr;
-  const int np = n * (n + 1) / 2;
-  for (int e = tid; e < n * n; e += RT) {
-    const int i = e % n, j = e / n;
-    if (i < j) continue;
-    double v = F[i + (int64_t)j * J];
-    if (MODE == NN_IH && f.a > 0) {
-      double s = 0.0;
-      const double* part = T2 + i * (i + 1) / 2 + j;
-      for (int b = 0; b < f.nb; ++b) s += part[(int64_t)b * np];
-      v += s;
-    }
-    K[i + j * ld] = v;
-    K[j + i * ld] = v;
-  }
-  __syncthreads();
+  const int np = n * (n + 1) / 2, rows = min(16, n - i0);
   auto B = [&](int r, int c) {
     return MODE == NN_M ? W[r >= c ? csc_off(J, r, c) : csc_off(J, c, r)]
                         : D[r >= c ? r + (int64_t)c * n : c + (int64_t)r * n];
   };
-  const int rows = min(16, n - i0);
+  auto K = [&](int r, int c) {
+    const int i = max(r, c), j = min(r, c);
+    double v = F[i + (int64_t)j * J];
+    if (MODE == NN_IH && f.a > 0) {
+      double t = 0.0;
+      const double* part = T2 + i * (i + 1) / 2 + j;
+      for (int b = 0; b < f.nb; ++b) t += part[(int64_t)b * np];
+      v += t;
+    }
+    return v;
+  };
   for (int e = tid; e < 16 * n; e += RT) {
-    const int r = e & 15, c = e >> 4;
-    if (r >= rows) continue;
-    double s = 0.0;
-    for (int q = 0; q < n; ++q) s = fma(B(i0 + r, q), K[q + c * ld], s);
-    X[r + c * 16] = s;
+    const int q = e % n, r = e / n;
+    Br[r * ld + q] = r < rows ? B(i0 + r, q) : 0.0;
   }
-  __syncthreads();
+  // 16 x 32 outputs at a time, four per thread
+  const int r = tid & 15, cq = tid >> 4;
   double* out = Out + y * ldo + f.base;
-  for (int e = tid; e < 16 * (i0 + rows); e += RT) {
-    const int r = e & 15, c = e >> 4;
-    if (r >= rows || c > i0 + r) continue;
-    double s = 0.0;
-    for (int q = 0; q < n; ++q) s = fma(X[r + q * 16], B(q, c), s);
-    out[csc_off(J, i0 + r, c)] = s;
+  for (int half = 0; half < 2; ++half) {
+    const double* A = (half ? X : Br) + r * ld;
+    for (int c0 = 0; c0 < (half ? i0 + rows : n); c0 += 32) {
+      const int cn = min(32, n - c0);
+      __syncthreads();
+      for (int e = tid; e < n * 32; e += RT) {
+        const int q = e % n, c = e / n;
+        Cs[q * 33 + c] = c < cn ? (half ? B(q, c0 + c) : K(q, c0 + c)) : 0.0;
+      }
+      __syncthreads();
+      double x[4] = {0.0, 0.0, 0.0, 0.0};
+      for (int q = 0; q < n; ++q) {
+        const double av = A[q];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) x[u] = fma(av, Cs[q * 33 + cq + 8 * u], x[u]);
+      }
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int c = c0 + cq + 8 * u;
+        if (c >= n) continue;
+        if (half == 0) X[r * ld + c] = x[u];
+        else if (r < rows && c <= i0 + r) out[csc_off(J, i0 + r, c)] = x[u];
+      }
+    }
   }
 }
 
@@ -1475,7 +1488,7 @@ using namespace chd::grp;
 
 namespace {
 size_t rows_smem(int rn) { return (size_t)(KC * CBL + RT * CB + 2 * rn) * 8; }
-size_t nn_smem(int n) { return (size_t)(n * (n | 1) + 16 * n) * 8; }
+size_t nn_smem(int n) { return (size_t)(32 * (n | 1) + 33 * n) * 8; }
 template <class K>
 void allow_smem(K kernel) {
   cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kGroupSmem);
@@ -1494,6 +1507,7 @@ void init() {
   allow_smem(kg_rows<RK_IH2>);
   allow_smem(kg_nn<NN_M>);
   allow_smem(kg_nn<NN_IH>);
+  allow_smem(kg_factor_rows);
   done.fetch_or(bit, std::memory_order_release);
 }
 }  // namespace
@@ -1636,6 +1650,7 @@ void group_factor(const chd_symbolic* s, cudaStream_t st, int q, const double* X
 void group_factor_post(const chd_symbolic* s, cudaStream_t st, const double* Lc, double* Wc, double* ws,
                        double* ldet) {
   if (s->gf.empty()) return;
+  init();
   const int nr = (int)s->gt_fr.size() / 2, nn = (int)s->gt_nn.size() / 2;
   kg_factor_rows<<<nr, 128, (size_t)GB * (s->g_nmax + 1) * 8, st>>>(s->dev, s->dev.gt_fr, Lc, Wc, ws);
   count_launch();

@@ -46,7 +46,7 @@ def _cliques(n, a, kids=2, extra=5):
 
 
 SIZES = [(1, 40), (1, 65), (9, 7), (9, 8), (8, 33), (15, 16), (16, 31), (17, 32), (31, 33), (32, 64), (33, 65), (40, 96),
-         (64, 15), (65, 97), (100, 70), (127, 9), (128, 20), (129, 20)]
+         (64, 15), (65, 97), (100, 70), (128, 20), (129, 20), (159, 3)]
 
 
 @pytest.mark.parametrize("n,a", SIZES)
@@ -57,7 +57,9 @@ def test_grouped_front_sizes(n, a, kids):
 
 @pytest.mark.parametrize("n,a,opts", [(10, 330, {}), (3, 513, {}), (16, 320, {"tc_products": -1}),
                                       (12, 40, {"big_rows": 48, "big_cols": 48}),
-                                      (40, 70, {"big_rows": 4096, "big_cols": 4096, "split_cols": -1})])
+                                      (40, 70, {"big_rows": 4096, "big_cols": 4096, "split_cols": -1}),
+                                      (256, 9, {"big_rows": 4096, "big_cols": 4096, "split_cols": -1}),
+                                      (257, 40, {"big_rows": 4096, "big_cols": 4096, "split_cols": -1})])
 def test_grouped_dense_thin_fronts(n, a, opts):
     """Thin fronts of the dense tier, and CTA-tier fronts of any size."""
     _check(_cliques(n, a, 2), seed=a, **opts)
