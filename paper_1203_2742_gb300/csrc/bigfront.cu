@@ -949,36 +949,127 @@ void complete_load_front(const chd_symbolic* s, const Ctx& st, int k, const doub
   CHD_EW(mk_csc_to_front, (int64_t)f.J * f.n, 1, st, ws + f.foff, 0, f.J, f.n, Sin + f.base, 0);
 }
 
+// The front in the order (A_k, N_k): lower triangle of [S_AA; S_NA S_NN], and
+// V_k = S_AA
+__global__ void __launch_bounds__(BT) mk_gather_an(SymDev S, int k, const double* Sin, double* ws, double* V) {
+  const int n = (int)(S.sn_ptr[k + 1] - S.sn_ptr[k]);
+  const int J = (int)(S.rows_ptr[k + 1] - S.rows_ptr[k]);
+  const int a = J - n;
+  const int64_t base = S.colptr[S.sn_ptr[k]];
+  double* F = ws + S.f_off[k];
+  const int32_t* A = S.rows + S.rows_ptr[k] + n;
+  const int64_t tot = (int64_t)J * J;
+  for (int64_t e = blockIdx.x * (int64_t)EW + threadIdx.x; e < min(tot, (blockIdx.x + 1) * (int64_t)EW); e += BT) {
+    const int r = (int)(e % J), c = (int)(e / J);
+    if (r < c) continue;
+    double v;
+    if (c >= a) v = Sin[base + csc_off(J, r - a, c - a)];
+    else if (r >= a) v = Sin[base + csc_off(J, n + c, r - a)];
+    else V[r + (int64_t)c * a] = v = Sin[csc_find(S, __ldg(A + r), __ldg(A + c))];
+    F[e] = v;
+  }
+}
+// L_AN = -R^{-T} Z for a front of a few columns, Z^T in the N rows of F: back
+// substitution through the panels of 32 in one CTA.  With n = 1 the blocked
+// solve is 2 a / 64 launches of about 30 us whose products have one row (1.4 ms
+// at a = 1340); here a panel is a chain of 9 us and the updates left of it one
+// dot product of 32 per entry.
+constexpr int BACK_N = 4;
+__global__ void __launch_bounds__(BT) mk_back(const double* F, int J, int a, int n, double* LA) {
+  extern __shared__ double rows[];  // n x (a + 1)
+  __shared__ double Ls[PP][PP + 1], rinv[PP];
+  const int tid = threadIdx.x, lane = tid & 31, ld = a + 1;
+  for (int e = tid; e < a * n; e += BT) {
+    const int r = e % n, c = e / n;
+    rows[r * ld + c] = -F[a + r + (int64_t)c * J];
+  }
+  for (int p0 = (a - 1) / PP * PP; p0 >= 0; p0 -= PP) {
+    const int pb = min(PP, a - p0);
+    __syncthreads();
+    for (int e = tid; e < PP * PP; e += BT) {
+      const int i = e & 31, c = e >> 5;
+      Ls[i][c] = i < pb && c <= i ? F[(p0 + i) + (int64_t)(p0 + c) * J] : 0.0;
+    }
+    __syncthreads();
+    if (tid < 32) {
+      rinv[lane] = lane < pb ? 1.0 / Ls[lane][lane] : 0.0;
+      __syncwarp();
+      const int row = lane >> 2, q = lane & 3;
+      double b[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u) b[u] = row < n && q + 4 * u < pb ? rows[row * ld + p0 + q + 4 * u] : 0.0;
+      panel::solve_row_back(b, Ls, rinv, pb, lane);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (row < n && q + 4 * u < pb) rows[row * ld + p0 + q + 4 * u] = b[u];
+    }
+    __syncthreads();
+    for (int e = tid; e < n * p0; e += BT) {
+      const int r = e % n, c = e / n;
+      const double* R = F + p0 + (int64_t)c * J;
+      double acc = 0.0;
+      for (int k = 0; k < pb; ++k) acc = fma(rows[r * ld + p0 + k], __ldg(R + k), acc);
+      rows[r * ld + c] -= acc;
+    }
+  }
+  __syncthreads();
+  for (int e = tid; e < a * n; e += BT) {
+    const int c = e % a, r = e / a;
+    LA[c + (int64_t)r * J] = rows[r * ld + c];
+  }
+}
+// D(r, c) = -S(c, r) for an R x C block of D
+__global__ void __launch_bounds__(BT) mk_neg_t(double* D, int64_t ldd, const double* S, int64_t lds, int R, int C) {
+  const int64_t tot = (int64_t)R * C;
+  for (int64_t e = blockIdx.x * (int64_t)EW + threadIdx.x; e < min(tot, (blockIdx.x + 1) * (int64_t)EW); e += BT) {
+    const int r = (int)(e % R), c = (int)(e / R);
+    D[r + (int64_t)c * ldd] = -S[c + (int64_t)r * lds];
+  }
+}
+
+// Algorithm 7.3 for one dense front.  The partial Cholesky factorisation of
+// the A columns of the front in the order (A, N) gives R = chol(V_k), Z^T in
+// the N rows and P = S_NN - Z^T Z in the N block, so Z costs no solve of its
+// own (er5000: 27 fronts, 40 % of their launches).
 // With Gq (factored update matrices, Algorithm 4.3): G = P R_k P of
 // V_k = R_k R_k^T from Gq instead of chol(V_k); the solves run on S_AN and
 // L_AN with reversed rows (Z^T Z is unchanged).
 void complete_front(const chd_symbolic* s, const Ctx& st, int k, const double* Sin, double* Lc, double* Wc,
-                    double* Dd, double* Vd, double* Rd, const double* Gq, double* ws, double* ldet,
-                    int64_t* status) {
+                    double* Dd, double* Vd, const double* Gq, double* ws, double* ldet, int64_t* status) {
   Front f = front(s, k);
   const int J = f.J, n = f.n, a = f.a;
   double* F = ws + f.foff;
   double* T1 = F + (int64_t)J * J;
   double* T2 = T1 + (int64_t)J * n;
-  // the S-front F was loaded by complete_load_front
   double* V = Vd + s->v_off[k];
-  double* R = Gq ? const_cast<double*>(Gq) + s->v_off[k] : Rd + s->v_off[k];
-  if (a > 0) {
-    CHD_EW(mk_copy, (int64_t)a * a, 1, st, V, 0, a, F + n + (int64_t)n * J, 0, J, a, a, 1.0, 0.0, 1, 0);
-    if (!Gq) {
-      CHD_EW(mk_copy, (int64_t)a * a, 1, st, R, 0, a, F + n + (int64_t)n * J, 0, J, a, a, 1.0, 0.0, 1, 0);
-      potrf_partial(st, R, a, a, a, status, CHD_ERR_NOT_COMPLETABLE, k, -1);
+  if (!Gq) {
+    CHD_EW(mk_gather_an, (int64_t)J * J, 1, st, s->dev, k, Sin, ws, V);
+    if (a > 0) potrf_partial(st, F, J, J, a, status, CHD_ERR_NOT_COMPLETABLE, k, -1);
+    CHD_EW(mk_copy, (int64_t)n * n, 1, st, T1, 0, J, F + a + (int64_t)a * J, 0, J, n, n, 1.0, 0.0, 1, 0);  // P
+    const size_t smem = (size_t)n * (a + 1) * 8;
+    if (a > 0 && n <= BACK_N && smem <= 40960) {
+      mk_back<<<1, BT, smem, st>>>(F, J, a, n, T2 + n);
+      chd_launch::count_launch();
+    } else if (a > 0) {
+      CHD_EW(mk_neg_t, (int64_t)a * n, 1, st, T2 + n, J, F + a, J, a, n);
+      trsm_rL(st, 1, n, a, DnTW{T2 + n, J}, 0, F, J);  // L_AN = -R^{-T} Z
     }
-    CHD_EW(mk_copy, (int64_t)a * n, 1, st, T1 + n, 0, J, F + n, 0, J, a, n, 1.0, 0.0, 0, 0);
-    if (Gq) CHD_EW(mk_rev_rows, (int64_t)(a / 2) * n, 1, st, T1 + n, J, a, n);
-    trsm_rLT(st, 1, n, a, DnTW{T1 + n, J}, 0, R, a);  // Z = R^{-1} S_AN
-  }
-  CHD_EW(mk_copy, (int64_t)n * n, 1, st, T1, 0, J, F, 0, J, n, n, 1.0, 0.0, 1, 0);
-  if (a > 0) {
-    gemm(st, 1, n, n, a, -1.0, DnT{T1 + n, J}, 0, Dn{T1 + n, J}, 0, 1.0, Dn{T1, J}, 0, true);  // P
-    CHD_EW(mk_copy, (int64_t)a * n, 1, st, T2 + n, 0, J, T1 + n, 0, J, a, n, -1.0, 0.0, 0, 0);
-    trsm_rL(st, 1, n, a, DnTW{T2 + n, J}, 0, R, a);  // L_AN = -R^{-T} Z
-    if (Gq) CHD_EW(mk_rev_rows, (int64_t)(a / 2) * n, 1, st, T2 + n, J, a, n);
+  } else {
+    // the S-front F was loaded by complete_load_front
+    const double* R = Gq + s->v_off[k];
+    if (a > 0) {
+      CHD_EW(mk_copy, (int64_t)a * a, 1, st, V, 0, a, F + n + (int64_t)n * J, 0, J, a, a, 1.0, 0.0, 1, 0);
+      CHD_EW(mk_copy, (int64_t)a * n, 1, st, T1 + n, 0, J, F + n, 0, J, a, n, 1.0, 0.0, 0, 0);
+      CHD_EW(mk_rev_rows, (int64_t)(a / 2) * n, 1, st, T1 + n, J, a, n);
+      trsm_rLT(st, 1, n, a, DnTW{T1 + n, J}, 0, R, a);  // Z = R^{-1} S_AN
+    }
+    CHD_EW(mk_copy, (int64_t)n * n, 1, st, T1, 0, J, F, 0, J, n, n, 1.0, 0.0, 1, 0);
+    if (a > 0) {
+      gemm(st, 1, n, n, a, -1.0, DnT{T1 + n, J}, 0, Dn{T1 + n, J}, 0, 1.0, Dn{T1, J}, 0, true);  // P
+      CHD_EW(mk_copy, (int64_t)a * n, 1, st, T2 + n, 0, J, T1 + n, 0, J, a, n, -1.0, 0.0, 0, 0);
+      trsm_rL(st, 1, n, a, DnTW{T2 + n, J}, 0, R, a);  // L_AN = -R^{-T} Z
+      CHD_EW(mk_rev_rows, (int64_t)(a / 2) * n, 1, st, T2 + n, J, a, n);
+    }
   }
   CHD_EW(mk_front_to_csc, (int64_t)J * n, 1, st, Wc + f.base, 0, T1, 0, J, J, n, 0, n, 1.0);
   if (a > 0) CHD_EW(mk_front_to_csc, (int64_t)J * n, 1, st, Wc + f.base, 0, T2, 0, J, J, n, n, J, 1.0);
@@ -1509,7 +1600,7 @@ void big_complete(const chd_symbolic* s, const Slot& sl, int k, const double* Si
                   double* Lc, double* Wc, double* Dd, double* Vd, double* Rd, const double* Gq, double* ws,
                   double* ldet, int64_t* status) {
   if (s->grp_of[k] >= 0) return chd::big::group_complete(s, chd::big::make_ctx(sl), s->grp_of[k], Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, status);
-  chd::big::complete_front(s, chd::big::make_ctx(sl), k, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, status);
+  chd::big::complete_front(s, chd::big::make_ctx(sl), k, Sin, Lc, Wc, Dd, Vd, Gq, ws, ldet, status);
 }
 void big_fc(const chd_symbolic* s, const Slot& sl, int k, const double* Sin, double* Gq, double* fcs,
             int64_t* status) {

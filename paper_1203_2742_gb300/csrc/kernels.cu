@@ -1602,6 +1602,7 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
   std::vector<int32_t> bigs;  // dense fronts and leaf groups
   for (int32_t k : s->big_fronts)
     if (!(grouped && s->in_gc[k])) bigs.push_back(k);
+  if (grouped) bigs.insert(bigs.end(), s->gc_rest.begin(), s->gc_rest.end());
   for (int64_t g0 : s->grp_first) bigs.push_back((int32_t)g0);
   // the largest V_k first: its blocked Cholesky is the longest chain
   std::stable_sort(bigs.begin(), bigs.end(), [&](int32_t x, int32_t y) {
@@ -1609,7 +1610,7 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
   });
   BigFork bf{ex, st};
   bf.run((int)bigs.size(), [&](int i, const Slot& sl) {
-    big_complete_load(s, sl.st, bigs[i], Sin, ws);
+    if (Gq) big_complete_load(s, sl.st, bigs[i], Sin, ws);
     big_complete(s, sl, bigs[i], Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, status);
   });
   if (grouped) group_complete(s, st, Sin, Lc, Wc, Dd, Vd, ws, ldet, status);
@@ -1617,10 +1618,9 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
     k_complete_wide<<<(int)s->gc_wide.size(), NT, 0, st>>>(s->dev, s->dev.gc_wide, Lc, Wc, Dd, ws, ldet, status);
     count();
   }
-  const int nrest = grouped ? (int)s->gc_rest.size() : (int)s->dev.cta_count;
-  if (nrest > 0) {
-    k_complete<<<nrest, NT, 0, st>>>(s->dev, grouped ? s->dev.gc_rest : s->dev.cta_fronts, Sin, Lc, Wc, Dd, Vd, Rd, Gq,
-                                     ws, ldet, status);
+  if (!grouped && s->dev.cta_count > 0) {
+    k_complete<<<(int)s->dev.cta_count, NT, 0, st>>>(s->dev, s->dev.cta_fronts, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet,
+                                                     status);
     count();
   }
   if (s->dev.warp_count > 0) w32::warp_complete_all(s, sw, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ldet, status);

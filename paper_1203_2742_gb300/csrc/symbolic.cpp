@@ -593,7 +593,7 @@ static void group_completion_plan(chd_symbolic* s) {
     const int t = s->tier[k];
     const int64_t n = front_n(s, k), J = front_J(s, k), a = J - n;
     if (t != 1 && t != 3 && !(t == 2 && s->tc_mode != 1)) continue;
-    if (n > kGroupCols || a > kInvVGroup) {
+    if (n > kGroupComplete || a > kInvVGroup) {
       if (t != 2) s->gc_rest.push_back((int32_t)k);
       continue;
     }
