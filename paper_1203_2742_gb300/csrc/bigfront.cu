@@ -734,13 +734,11 @@ void gather_parent(const chd_symbolic* s, const Ctx& st, int batch, const Front&
   CHD_EW(mk_gather_parent, (int64_t)f.a * f.a, batch, st, s->dev, f.k, ws, sws);
 }
 
-void factor_front(const chd_symbolic* s, const Ctx& st, int k, const double* X, double* Lc, double* Wc,
-                  double* Dd, double* ws, double* ldet, int64_t* status) {
+void factor_front(const chd_symbolic* s, const Ctx& st, int k, const double* X, double* Lc, double* Dd,
+                  double* ws, double* ldet, int64_t* status) {
   Front f = front(s, k);
   const int J = f.J, n = f.n, a = f.a;
   double* F = ws + f.foff;
-  double* T1 = F + (int64_t)J * J;
-  double* T2 = T1 + (int64_t)J * n;
   CHD_EW(mk_csc_to_front, (int64_t)J * n, 1, st, F, 0, J, n, X + f.base, 0);
   if (a > 0) CHD_EW(mk_copy, (int64_t)a * a, 1, st, F + n + (int64_t)n * J, 0, J, nullptr, 0, 0, a, a, 0.0, 0.0, 1, 0);
   assemble_children(s, st, 1, k, ws, 0);
@@ -749,6 +747,14 @@ void factor_front(const chd_symbolic* s, const Ctx& st, int k, const double* X, 
   CHD_EW(mk_front_to_csc, (int64_t)J * n, 1, st, Lc + f.base, 0, F, 0, J, J, n, 0, J, 1.0);
   k_logdet_diag<<<1, BT, 0, st>>>(F, J, n, ldet + k);
   chd_launch::count_launch();
+}
+// D_NN^{-1} and L_AN of a factored front: no other front waits for them
+void factor_post(const chd_symbolic* s, const Ctx& st, int k, double* Wc, double* ws) {
+  Front f = front(s, k);
+  const int J = f.J, n = f.n, a = f.a;
+  double* F = ws + f.foff;
+  double* T1 = F + (int64_t)J * J;
+  double* T2 = T1 + (int64_t)J * n;
   // Cinv = C^{-1} (T1), D^{-1} = Cinv^T Cinv (T2 top), L_AN = B C^{-1} (T2 bottom)
   CHD_EW(mk_identity, (int64_t)n * n, 1, st, T1, J, n);
   trsm_rLT(st, 1, n, n, DnTW{T1, J}, 0, F, J);
@@ -760,8 +766,7 @@ void factor_front(const chd_symbolic* s, const Ctx& st, int k, const double* X, 
   CHD_EW(mk_front_to_csc, (int64_t)J * n, 1, st, Wc + f.base, 0, T2, 0, J, J, n, 0, J, 1.0);
 }
 
-void gradient_front(const chd_symbolic* s, const Ctx& st, int k, const double* Wc, double* Sc, double* g,
-                    double* Vd, double* ws) {
+void gradient_front(const chd_symbolic* s, const Ctx& st, int k, const double* Wc, double* ws) {
   Front f = front(s, k);
   const int J = f.J, n = f.n, a = f.a;
   double* F = ws + f.foff;
@@ -770,19 +775,23 @@ void gradient_front(const chd_symbolic* s, const Ctx& st, int k, const double* W
   CHD_EW(mk_csc_to_front, (int64_t)J * n, 1, st, F, 0, J, n, W, 0);  // D^{-1}; rows >= n overwritten next
   gemm(st, 1, a, n, a, -1.0, SymL{F + n + (int64_t)n * J, J}, 0, CscRO{W, J, n}, 0, 0.0, Dn{F + n, J}, 0, false);
   gemm(st, 1, n, n, a, -1.0, DnT{F + n, J}, 0, CscRO{W, J, n}, 0, 1.0, Dn{F, J}, 0, true);
+}
+void gradient_post(const chd_symbolic* s, const Ctx& st, int k, double* Sc, double* g, double* Vd, double* ws) {
+  Front f = front(s, k);
+  const int J = f.J, n = f.n, a = f.a;
+  double* F = ws + f.foff;
   CHD_EW(mk_front_to_csc, (int64_t)J * n, 1, st, Sc + f.base, 0, F, 0, J, J, n, 0, J, 1.0);
   if (g) CHD_EW(mk_front_to_csc, (int64_t)J * n, 1, st, g + f.base, 0, F, 0, J, J, n, 0, J, -1.0);
   if (a > 0) CHD_EW(mk_copy, (int64_t)a * a, 1, st, Vd + s->v_off[k], 0, a, F + n + (int64_t)n * J, 0, J, a, a, 1.0, 0.0, 1, 0);
 }
 
-void hess_up_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc, const double* Vd,
-                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act) {
+void hess_up_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc,
+                   const double* Y, int64_t ldy, double* ws, const uint8_t* act) {
   Front f = front(s, k);
   const int J = f.J, n = f.n, a = f.a;
   const int64_t sw = s->dev.f_total;
   double* F = ws + f.foff;
   double* T1 = F + (int64_t)J * J;
-  double* T2 = T1 + (int64_t)J * n;
   const double* W = Wc + f.base;
   CscRO L{W, J, n};
   CHD_EW(mk_csc_to_front, (int64_t)J * n, m, st, F, sw, J, n, Y + f.base, ldy);
@@ -794,6 +803,18 @@ void hess_up_front(const chd_symbolic* s, const Ctx& st, int m, int k, const dou
     gemm(st, m, a, a, n, -1.0, Dn{T1 + n, J}, sw, CscT{W, J, n}, 0, 1.0, Dn{F + n + (int64_t)n * J, J}, sw, true);
     gemm(st, m, a, a, n, -1.0, L, 0, DnT{F + n, J}, sw, 1.0, Dn{F + n + (int64_t)n * J, J}, sw, true);
   }
+}
+// Step 2 of Algorithm 5.1 for a front whose step 1 is done (no other front
+// waits for it): M_NN = D^{-1} K_NN D^{-1}, M_AN = V K_AN D^{-1}
+void hess_m_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc, const double* Vd, double* T,
+                  int64_t ldt, double* ws) {
+  Front f = front(s, k);
+  const int J = f.J, n = f.n, a = f.a;
+  const int64_t sw = s->dev.f_total;
+  double* F = ws + f.foff;
+  double* T1 = F + (int64_t)J * J;
+  double* T2 = T1 + (int64_t)J * n;
+  const double* W = Wc + f.base;
   CscSym Dinv{W, J};
   gemm(st, m, n, n, n, 1.0, SymL{F, J}, sw, Dinv, 0, 0.0, Dn{T2, J}, sw, false);
   gemm(st, m, n, n, n, 1.0, Dinv, 0, Dn{T2, J}, sw, 0.0, Csc{T + f.base, J, 0}, ldt, true);
@@ -803,7 +824,7 @@ void hess_up_front(const chd_symbolic* s, const Ctx& st, int m, int k, const dou
   }
 }
 
-void hess_down_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc, double* T,
+void hess_down_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc, const double* T,
                      int64_t ldt, double* ws) {
   Front f = front(s, k);
   const int J = f.J, n = f.n, a = f.a;
@@ -821,11 +842,24 @@ void hess_down_front(const chd_symbolic* s, const Ctx& st, int m, int k, const d
     gemm(st, m, n, n, a, -1.0, CscT{W, J, n}, 0, Dn{F + n, J}, sw, 1.0, Dn{F, J}, sw, true);
     CHD_EW(mk_copy, (int64_t)a * n, m, st, F + n, sw, J, T1 + n, sw, J, a, n, -0.5, 1.0, 0, 0);
   }
-  CHD_EW(mk_front_to_csc, (int64_t)J * n, m, st, T + f.base, ldt, F, sw, J, J, n, 0, J, 1.0);
+}
+void hess_down_post(const chd_symbolic* s, const Ctx& st, int m, int k, double* T, int64_t ldt, double* ws) {
+  Front f = front(s, k);
+  const int J = f.J, n = f.n;
+  CHD_EW(mk_front_to_csc, (int64_t)J * n, m, st, T + f.base, ldt, ws + f.foff, s->dev.f_total, J, J, n, 0, J, 1.0);
 }
 
-void ihess_down_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc, const double* Dd,
-                      const double* Rd, const double* Tin, int64_t ldt, double* Yout, int64_t ldy, double* ws) {
+// Inverse Hessian, top-down: the children read the front's input and its
+// parent's rows only, so the products all belong to the second half.
+void ihess_down_front(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Tin, int64_t ldt,
+                      double* ws) {
+  Front f = front(s, k);
+  const int64_t sw = s->dev.f_total;
+  gather_parent(s, st, m, f, ws, sw);
+  CHD_EW(mk_csc_to_front, (int64_t)f.J * f.n, m, st, ws + f.foff, sw, f.J, f.n, Tin + f.base, ldt);
+}
+void ihess_down_post(const chd_symbolic* s, const Ctx& st, int m, int k, const double* Wc, const double* Dd,
+                     const double* Rd, double* Yout, int64_t ldy, double* ws) {
   Front f = front(s, k);
   const int J = f.J, n = f.n, a = f.a;
   const int64_t sw = s->dev.f_total;
@@ -834,8 +868,6 @@ void ihess_down_front(const chd_symbolic* s, const Ctx& st, int m, int k, const 
   double* T2 = T1 + (int64_t)J * n;
   const double* W = Wc + f.base;
   CscRO L{W, J, n};
-  gather_parent(s, st, m, f, ws, sw);
-  CHD_EW(mk_csc_to_front, (int64_t)J * n, m, st, F, sw, J, n, Tin + f.base, ldt);
   // T1 = [M_NN (full); M_AN]
   CHD_EW(mk_copy, (int64_t)n * n, m, st, T1, sw, J, F, sw, J, n, n, 1.0, 0.0, 0, 1);
   if (a > 0) {
@@ -1559,7 +1591,10 @@ using chd::big::Ctx;
 void big_factor(const chd_symbolic* s, const Slot& sl, int k, const double* X,
                 double* Lc, double* Wc, double* Dd, double* ws, double* ldet, int64_t* status) {
   if (s->grp_of[k] >= 0) return chd::big::group_factor(s, chd::big::make_ctx(sl), s->grp_of[k], X, Lc, Wc, Dd, ws, ldet, status);
-  chd::big::factor_front(s, chd::big::make_ctx(sl), k, X, Lc, Wc, Dd, ws, ldet, status);
+  chd::big::factor_front(s, chd::big::make_ctx(sl), k, X, Lc, Dd, ws, ldet, status);
+}
+void big_factor_post(const chd_symbolic* s, const Slot& sl, int k, double* Wc, double* ws) {
+  chd::big::factor_post(s, chd::big::make_ctx(sl), k, Wc, ws);
 }
 void big_product(const chd_symbolic* s, const Slot& sl, int k, const double* Lc,
                  double* X, double* ws) {
@@ -1569,7 +1604,10 @@ void big_product(const chd_symbolic* s, const Slot& sl, int k, const double* Lc,
 void big_gradient(const chd_symbolic* s, const Slot& sl, int k, const double* Wc,
                   double* Sc, double* g, double* Vd, double* ws) {
   if (s->grp_of[k] >= 0) return chd::big::group_gradient(s, chd::big::make_ctx(sl), s->grp_of[k], Wc, Sc, g, Vd, ws);
-  chd::big::gradient_front(s, chd::big::make_ctx(sl), k, Wc, Sc, g, Vd, ws);
+  chd::big::gradient_front(s, chd::big::make_ctx(sl), k, Wc, ws);
+}
+void big_gradient_post(const chd_symbolic* s, const Slot& sl, int k, double* Sc, double* g, double* Vd, double* ws) {
+  chd::big::gradient_post(s, chd::big::make_ctx(sl), k, Sc, g, Vd, ws);
 }
 void big_hess_up(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc,
                  const double* Vd, const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws,
@@ -1578,18 +1616,29 @@ void big_hess_up(const chd_symbolic* s, const Slot& sl, int m, int k, const doub
   // front still runs, skipping pruned children, and gives exact zeros where
   // its own subtree is pruned
   if (s->grp_of[k] >= 0) return chd::big::group_hess_up(s, chd::big::make_ctx(sl), m, s->grp_of[k], Wc, Vd, Y, ldy, T, ldt, ws);
-  chd::big::hess_up_front(s, chd::big::make_ctx(sl), m, k, Wc, Vd, Y, ldy, T, ldt, ws, act);
+  chd::big::hess_up_front(s, chd::big::make_ctx(sl), m, k, Wc, Y, ldy, ws, act);
+}
+void big_hess_m(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc, const double* Vd, double* T,
+                int64_t ldt, double* ws) {
+  chd::big::hess_m_front(s, chd::big::make_ctx(sl), m, k, Wc, Vd, T, ldt, ws);
 }
 void big_hess_down(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc,
                    double* T, int64_t ldt, double* ws) {
   if (s->grp_of[k] >= 0) return chd::big::group_hess_down(s, chd::big::make_ctx(sl), m, s->grp_of[k], Wc, T, ldt, ws);
   chd::big::hess_down_front(s, chd::big::make_ctx(sl), m, k, Wc, T, ldt, ws);
 }
+void big_hess_down_post(const chd_symbolic* s, const Slot& sl, int m, int k, double* T, int64_t ldt, double* ws) {
+  chd::big::hess_down_post(s, chd::big::make_ctx(sl), m, k, T, ldt, ws);
+}
 void big_ihess_down(const chd_symbolic* s, const Slot& sl, int m, int k,
                     const double* Wc, const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y,
                     int64_t ldy, double* ws) {
   if (s->grp_of[k] >= 0) return chd::big::group_ihess_down(s, chd::big::make_ctx(sl), m, s->grp_of[k], Wc, Dd, Rd, T, ldt, Y, ldy, ws);
-  chd::big::ihess_down_front(s, chd::big::make_ctx(sl), m, k, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+  chd::big::ihess_down_front(s, chd::big::make_ctx(sl), m, k, T, ldt, ws);
+}
+void big_ihess_down_post(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc, const double* Dd,
+                         const double* Rd, double* Y, int64_t ldy, double* ws) {
+  chd::big::ihess_down_post(s, chd::big::make_ctx(sl), m, k, Wc, Dd, Rd, Y, ldy, ws);
 }
 void big_ihess_up(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc,
                   double* Y, int64_t ldy, double* ws) {

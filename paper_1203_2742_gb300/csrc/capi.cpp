@@ -60,10 +60,13 @@ constexpr size_t kWorkspaceCap = size_t(48) << 30;
 inline size_t align_up(size_t x) { return (x + 255) & ~size_t(255); }
 
 // Scratch of the dense tier per stream: 2 Mi doubles (16 MiB) for the first
-// kWideSlices streams, 64 Ki doubles for the others.
+// kWideSlices streams and for those of the second halves, 64 Ki doubles for
+// the others.
 constexpr int64_t kSplitScratch = int64_t(2) << 20;
 constexpr int64_t kSmallScratch = int64_t(64) << 10;
-inline int64_t slice_doubles(int j) { return j < kWideSlices ? kSplitScratch : kSmallScratch; }
+inline int64_t slice_doubles(int j) {
+  return j < kWideSlices || j > kSideStreams - kPostStreams ? kSplitScratch : kSmallScratch;
+}
 
 chd_status cuda_ok(cudaError_t e) {
   if (e == cudaSuccess) return CHD_OK;
@@ -101,8 +104,9 @@ chd_status alloc_factor(chd_symbolic* s, cudaStream_t stream, chd_factor** out) 
   }
   // tensor-core product scratch (digit planes): one slice for the caller's
   // stream and for each side stream, sized for the largest dense front's
-  // products (up to eight right-hand sides at once on the caller's stream,
-  // two on a side stream; a call with more right-hand sides runs them in
+  // products (up to eight right-hand sides at once on the caller's stream
+  // and on those of the second halves, two on the other side streams; a call
+  // with more right-hand sides runs them in
   // turn, and a product that does not fit runs on the FP64 units)
   size_t tc_slice[kSideStreams + 1] = {};
   const size_t otc = off;
@@ -113,8 +117,9 @@ chd_status alloc_factor(chd_symbolic* s, cudaStream_t stream, chd_factor** out) 
     if (jmax >= 64) {
       const size_t need = chd_launch::tc_scratch_bytes(1, (int)jmax, (int)jmax, (int)jmax);
       for (int j = 0; j <= nside; ++j) {
-        tc_slice[j] = align_up(std::min<size_t>(j == 0 ? (size_t(256) << 20) : (size_t(48) << 20),
-                                                (j == 0 ? 8 : 2) * need));
+        const bool wide = j == 0 || j > kSideStreams - kPostStreams;
+        tc_slice[j] = align_up(std::min<size_t>(wide ? (size_t(256) << 20) : (size_t(48) << 20),
+                                                (wide ? 8 : 2) * need));
         off += tc_slice[j];
       }
     }

@@ -244,6 +244,7 @@ struct chd_symbolic {
 // the Cholesky panel kernel.  The first kWideSlices slices are large; the
 // rest hold the counter and small partial products only.
 constexpr int kSideStreams = 32;
+constexpr int kPostStreams = 2;   // the last of the side streams
 constexpr int kAuxStreams = 3;  // chain runs, warp tier, wide warp tier beside the caller's stream
 constexpr int kWideSlices = 9;
 struct Exec {

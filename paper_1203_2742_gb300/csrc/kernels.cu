@@ -1054,6 +1054,13 @@ static inline void count() { ++g_launches; }
 // dense-tier sequences (bigfront.cu); xs/xcap: split-K scratch (may be null)
 void big_factor(const chd_symbolic* s, const Slot& sl, int k, const double* X,
                 double* Lc, double* Wc, double* Dd, double* ws, double* ldet, int64_t* status);
+void big_factor_post(const chd_symbolic* s, const Slot& sl, int k, double* Wc, double* ws);
+void big_hess_m(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc, const double* Vd, double* T,
+                int64_t ldt, double* ws);
+void big_gradient_post(const chd_symbolic* s, const Slot& sl, int k, double* Sc, double* g, double* Vd, double* ws);
+void big_hess_down_post(const chd_symbolic* s, const Slot& sl, int m, int k, double* T, int64_t ldt, double* ws);
+void big_ihess_down_post(const chd_symbolic* s, const Slot& sl, int m, int k, const double* Wc, const double* Dd,
+                         const double* Rd, double* Y, int64_t ldy, double* ws);
 void big_product(const chd_symbolic* s, const Slot& sl, int k, const double* Lc,
                  double* X, double* ws);
 void big_gradient(const chd_symbolic* s, const Slot& sl, int k, const double* Wc,
@@ -1177,6 +1184,20 @@ void warp_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m
 // streams, else round-robin over the side streams, forked after the work
 // already queued on `st` and joined back into `st` at `join_now` (the caller
 // may queue independent work on `st` in between).
+// the last kPostStreams side streams take what no other front waits for (Posts)
+static inline Slot exec_slot(const Exec* ex, int j, cudaStream_t bs) {
+  Slot sl;
+  sl.st = bs;
+  if (ex) {
+    sl.xs = ex->slice[j];
+    sl.xcap = ex->slice_cap[j];
+    sl.tc = ex->tc[j];
+    sl.tc_cap = ex->tc_cap[j];
+    sl.status = ex->status;
+    sl.tc_mode = ex->tc_mode;
+  }
+  return sl;
+}
 struct BigFork {
   const Exec* ex;
   cudaStream_t st;
@@ -1184,30 +1205,17 @@ struct BigFork {
   template <class Body>
   void run(int count, Body&& body) {
     if (count <= 0) return;
-    auto slot = [&](int j, cudaStream_t bs) {
-      Slot sl;
-      sl.st = bs;
-      if (ex) {
-        sl.xs = ex->slice[j];
-        sl.xcap = ex->slice_cap[j];
-        sl.tc = ex->tc[j];
-        sl.tc_cap = ex->tc_cap[j];
-        sl.status = ex->status;
-        sl.tc_mode = ex->tc_mode;
-      }
-      return sl;
-    };
     if (!ex || ex->nside == 0 || count == 1) {
-      const Slot sl = slot(0, st);
+      const Slot sl = exec_slot(ex, 0, st);
       for (int i = 0; i < count; ++i) body(i, sl);
       return;
     }
-    used = std::min(count, ex->nside);
+    used = std::min(count, ex->nside > kPostStreams ? ex->nside - kPostStreams : ex->nside);
     cudaEventRecord(ex->fork, st);
     for (int j = 0; j < used; ++j) cudaStreamWaitEvent(ex->side[j], ex->fork, 0);
     for (int i = 0; i < count; ++i) {
       const int j = i % used;
-      body(i, slot(1 + j, ex->side[j]));
+      body(i, exec_slot(ex, 1 + j, ex->side[j]));
     }
   }
   void join_now() {
@@ -1216,6 +1224,40 @@ struct BigFork {
       cudaStreamWaitEvent(st, ex->join[j], 0);
     }
     used = 0;
+  }
+};
+
+// The second halves of dense fronts that no other front waits for (D^{-1} and
+// L_AN of the factor, M of the Hessian, the products of the inverse Hessian's
+// top-down pass, the outputs of the others): on the levels of the root chain
+// they are queued on side streams of their own behind the front's first half,
+// beside the next fronts of the chain, and joined at the end of the pass.  A
+// level of more dense fronts than those streams keeps each second half behind
+// its first one, on as many streams as fronts.
+struct Posts {
+  const chd_symbolic* s;
+  const Exec* ex;
+  cudaStream_t st;
+  int next = 0;
+  bool used[kPostStreams] = {};
+  template <class Body>
+  void add(const Slot& first, const std::vector<int>& dense, int i, Body&& body) {
+    if (s->grp_of[dense[i]] >= 0) return;  // leaf groups: in one piece
+    if (!ex || ex->nside <= kPostStreams || (int)dense.size() > kPostStreams) return body(first);
+    const int p = next++ % kPostStreams, j = ex->nside - kPostStreams + p;
+    cudaEventRecord(ex->join[j], first.st);
+    cudaStreamWaitEvent(ex->side[j], ex->join[j], 0);
+    used[p] = true;
+    body(exec_slot(ex, 1 + j, ex->side[j]));
+  }
+  void join() {
+    for (int p = 0; p < kPostStreams; ++p)
+      if (used[p]) {
+        const int j = ex->nside - kPostStreams + p;
+        cudaEventRecord(ex->join[j], ex->side[j]);
+        cudaStreamWaitEvent(st, ex->join[j], 0);
+        used[p] = false;
+      }
   }
 };
 
@@ -1303,6 +1345,7 @@ void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double
             double* Dd, double* ws, double* ldet, int64_t* status) {
   const int nl = (int)s->lvl_ptr.size() - 1;
   Beside bs(ex, st);
+  Posts posts{s, ex, st};
   for (int l = 0; l < nl; ++l) {
     if (l == s->run_join) bs.join(AUX_RUN);  // chain runs, forked at level 0
     Level v = level(s, l);
@@ -1312,6 +1355,7 @@ void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_factor(s, sl, dense[i], X, Lc, Wc, Dd, ws, ldet, status);
+      posts.add(sl, dense, i, [&](const Slot& ps) { big_factor_post(s, ps, dense[i], Wc, ws); });
     });
     if (v.nr32 + v.nr64) chain_factor(s, bs.fork(AUX_RUN, !s->run_overlap), v.tr, v.nr32 + v.nr64, X, Lc, Wc, Dd, ws, ldet, status);
     if (v.nwarp)
@@ -1329,6 +1373,7 @@ void factor(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double
     bf.join_now();
     bs.join_level();
   }
+  posts.join();
   bs.join(AUX_RUN);
   group_factor_post(s, st, Lc, Wc, ws, ldet);
 }
@@ -1366,6 +1411,7 @@ void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
               double* Vd, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
   Beside bs(ex, st);
+  Posts posts{s, ex, st};
   if (ex) chain_psi(s, st, Wc, ex->psi);
   group_zero(s, st, 1, ws);
   // chain runs (level 0) start as soon as their parents are done
@@ -1383,6 +1429,7 @@ void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_gradient(s, sl, dense[i], Wc, Sc, g, Vd, ws);
+      posts.add(sl, dense, i, [&](const Slot& ps) { big_gradient_post(s, ps, dense[i], Sc, g, Vd, ws); });
     });
     for (int q = s->glvl[l + 1] - 1; q >= s->glvl[l]; --q) {
       group_gradient(s, st, q, Wc, Sc, g, Vd, ws);
@@ -1400,12 +1447,14 @@ void gradient(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
     bs.join_level();
     if (l == run_at) runs(bs.fork(AUX_RUN, !s->run_overlap));
   }
+  posts.join();
   bs.join(AUX_RUN);
 }
 void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, const double* Vd,
                   const double* Y, int64_t ldy, double* T, int64_t ldt, double* ws, const uint8_t* act) {
   const int nl = (int)s->lvl_ptr.size() - 1;
   Beside bs(ex, st);
+  Posts posts{s, ex, st};
   SymDev D = s->dev;
   D.act = act;
   for (int l = 0; l < nl; ++l) {
@@ -1417,6 +1466,7 @@ void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m,
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_hess_up(s, sl, m, dense[i], Wc, Vd, Y, ldy, T, ldt, ws, act);
+      posts.add(sl, dense, i, [&](const Slot& ps) { big_hess_m(s, ps, m, dense[i], Wc, Vd, T, ldt, ws); });
     });
     if (v.nr32 + v.nr64) chain_hess_up(s, bs.fork(AUX_RUN, !s->run_overlap), v.tr, v.nr32 + v.nr64, m, Wc, Vd, Y, ldy, T, ldt, ws, act, ex ? ex->psi : nullptr);
     if (v.nwarp)
@@ -1434,6 +1484,7 @@ void hess_up_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m,
     bf.join_now();
     bs.join_level();
   }
+  posts.join();
   bs.join(AUX_RUN);
   group_hess_m(s, st, m, Wc, Vd, T, ldt, ws, act);
 }
@@ -1441,6 +1492,7 @@ void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int 
                     int64_t ldt, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
   Beside bs(ex, st);
+  Posts posts{s, ex, st};
   group_zero(s, st, m, ws);
   // chain runs (level 0) start as soon as their parents are done
   const Level r = level(s, 0);
@@ -1457,6 +1509,7 @@ void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int 
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_hess_down(s, sl, m, dense[i], Wc, T, ldt, ws);
+      posts.add(sl, dense, i, [&](const Slot& ps) { big_hess_down_post(s, ps, m, dense[i], T, ldt, ws); });
     });
     for (int q = s->glvl[l + 1] - 1; q >= s->glvl[l]; --q) {
       group_hess_down(s, st, q, m, Wc, T, ldt, ws);
@@ -1474,6 +1527,7 @@ void hess_down_pass(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int 
     bs.join_level();
     if (l == run_at) runs(bs.fork(AUX_RUN, !s->run_overlap));
   }
+  posts.join();
   bs.join(AUX_RUN);
 }
 void hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, const double* Wc, const double* Vd,
@@ -1514,6 +1568,7 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
                  const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy, double* ws) {
   const int nl = (int)s->lvl_ptr.size() - 1;
   Beside bs(ex, st);
+  Posts posts{s, ex, st};
   for (int l = nl - 1; l >= 0; --l) {
     Level v = level(s, l);
     BigFork bf{ex, st};
@@ -1522,6 +1577,7 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
     const std::vector<int> dense = dense_fronts(s, v);
     bf.run((int)dense.size(), [&](int i, const Slot& sl) {
       big_ihess_down(s, sl, m, dense[i], Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+      posts.add(sl, dense, i, [&](const Slot& ps) { big_ihess_down_post(s, ps, m, dense[i], Wc, Dd, Rd, Y, ldy, ws); });
     });
     for (int q = s->glvl[l + 1] - 1; q >= s->glvl[l]; --q) {
       group_ihess_gather(s, st, q, m, T, ldt, ws);
@@ -1539,6 +1595,7 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
     bf.join_now();
     bs.join_level();
   }
+  posts.join();
   group_ihess_k(s, st, m, Wc, Dd, Rd, Y, ldy, ws);
   for (int l = 0; l < nl; ++l) {
     Level v = level(s, l);
