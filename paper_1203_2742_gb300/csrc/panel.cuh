@@ -94,12 +94,13 @@ __device__ __forceinline__ void chol32(double (*Ls)[PB + 1], double* rinv, doubl
 // b := b L^{-T} for the pb x pb lower block Ls (rinv: reciprocal pivots).  Rolled
 // over groups of four columns, the registers shifted after each: fully
 // unrolled, a launch spends more on fetching the code once than on running it.
+// g0: the entries before column 4 g0 are zero in all rows of the warp.
 __device__ __forceinline__ void solve_row(double (&b)[8], const double (*Ls)[PB + 1], const double* rinv, int pb,
-                                          int lane) {
+                                          int lane, int g0 = 0) {
   const int q = lane & 3;
 #pragma unroll 1
   for (int g = 0; g < PB / 4; ++g) {
-    if (4 * g < pb) {
+    if (g >= g0 && 4 * g < pb) {
 #pragma unroll
       for (int i = 0; i < 4; ++i) {
         const int c = 4 * g + i;
