@@ -106,8 +106,8 @@ chd_status alloc_factor(chd_symbolic* s, cudaStream_t stream, chd_factor** out) 
   // stream and for each side stream, sized for the largest dense front's
   // products (up to eight right-hand sides at once on the caller's stream
   // and on those of the second halves, two on the other side streams; a call
-  // with more right-hand sides runs them in
-  // turn, and a product that does not fit runs on the FP64 units)
+  // with more right-hand sides runs them in turn, and a product that does not
+  // fit runs on the FP64 units)
   size_t tc_slice[kSideStreams + 1] = {};
   const size_t otc = off;
   if (any_big && s->tc_mode >= 0) {

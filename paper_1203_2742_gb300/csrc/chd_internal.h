@@ -244,7 +244,12 @@ struct chd_symbolic {
 // the Cholesky panel kernel.  The first kWideSlices slices are large; the
 // rest hold the counter and small partial products only.
 constexpr int kSideStreams = 32;
-constexpr int kPostStreams = 2;   // the last of the side streams
+// The last of the side streams take second halves of dense fronts (Posts in
+// kernels.cu), with the scratch sizes of the caller's stream.  Two: four gave
+// the same times (er5000 factor 5.95 against 5.98 ms), and four with the other
+// side streams' scratch lost 2 of 41 ms on the Hessian of 64 right-hand sides
+// of a 150 x 150 grid, whose products then ran two right-hand sides at a time.
+constexpr int kPostStreams = 2;
 constexpr int kAuxStreams = 3;  // chain runs, warp tier, wide warp tier beside the caller's stream
 constexpr int kWideSlices = 9;
 struct Exec {
@@ -268,7 +273,7 @@ struct Exec {
 
 // Formation of V_k^{-1} by the size a of V_k: up to kInvVGroup rows the
 // grouped kernels over all fronts at once (kv_* in group_tier.cu; 12000 fronts
-// of 61 rows: 9.4 ms with one CTA per front before), beyond that a launch
+// of 61 rows: 9.4 ms with one CTA per front, 5.0 ms grouped), beyond that a launch
 // sequence per front whose trailing products run on the tensor cores.  The upper
 // factor of V_k (Hessian factor) has no grouped form: one CTA (k_inv_v) below
 // kInvVMulti rows, else a sequence per front.

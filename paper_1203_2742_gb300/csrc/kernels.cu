@@ -17,8 +17,7 @@
 //   Wc  (CSC)  : [D_NN^{-1}; L_AN]
 //   Dd  (n x n): D_NN
 //   Vd  (a x a): V_k = S_{A_k A_k}  (Algorithm 7.2)
-//   Rd  (a x a): V_k^{-1} (lower triangle; inverse Hessian, §5.3) for the
-//                warp and CTA tiers, R = chol(V_k) for dense-tier fronts
+//   Rd  (a x a): V_k^{-1} (lower triangle; inverse Hessian, §5.3)
 //   Qd  (a x a): chol(P V_k P), P the order reversal (Hessian factor, §5.4)
 //   Sc  (CSC)  : S = P(X^{-1})
 #include <cuda_runtime.h>
@@ -722,20 +721,17 @@ __device__ void complete_nn(const SymDev& S, const FrontInfo& f, double* Lc, dou
 // is read from Gq instead of factoring V_k: the solves then run on S_AN and
 // L_AN with their rows in reversed order (Z^T Z is unchanged).
 __device__ void complete_front(const SymDev& S, int k, const double* Sin, double* Lc, double* Wc,
-                               double* Dd, double* Vd, double* Rd, const double* Gq, double* ws, double* ldet,
+                               double* Dd, double* Vd, const double* Gq, double* ws, double* ldet,
                                int64_t* st) {
   FrontInfo f = front_info(S, k, ws);
   const int J = f.J, n = f.n, a = f.a;
   double* V = Vd + S.v_off[k];
-  double* R = Gq ? const_cast<double*>(Gq) + S.v_off[k] : Rd + S.v_off[k];
+  const double* R = Gq + S.v_off[k];
   copy_lower(V, a, f.F + n + (int64_t)n * J, J, a);
-  if (!Gq) copy_lower(R, a, f.F + n + (int64_t)n * J, J, a);
-  __syncthreads();
-  if (a > 0 && !Gq) cta_potrf_partial(R, a, a, a, st, CHD_ERR_NOT_COMPLETABLE, k, -1);
   // T1[n:J] = Z = R^{-1} S_AN
   copy_rect(f.T1 + n, J, f.F + n, J, a, n);
   __syncthreads();
-  if (Gq) reverse_rows(f.T1 + n, J, a, n);
+  reverse_rows(f.T1 + n, J, a, n);
   if (a > 0) cta_trsm_rLT(n, a, DnTW{f.T1 + n, J}, R, a);
   // T1[0:n] (lower) = P = S_NN - Z^T Z
   copy_lower(f.T1, J, f.F, J, n);
@@ -748,7 +744,7 @@ __device__ void complete_front(const SymDev& S, int k, const double* Sin, double
   }
   __syncthreads();
   if (a > 0) cta_trsm_rL(n, a, DnTW{f.T2 + n, J}, R, a);
-  if (Gq) reverse_rows(f.T2 + n, J, a, n);
+  reverse_rows(f.T2 + n, J, a, n);
   // Wc = [P; L_AN]
   for (int e = threadIdx.x; e < J * n; e += NT) {
     int r = e % J, c = e / J;
@@ -864,11 +860,11 @@ __global__ void __launch_bounds__(kScanT) k_active(SymDev S, int32_t* cnt, uint8
 }
 // fronts of `list` at once, one CTA each
 __global__ void __launch_bounds__(NT) k_complete(SymDev S, const int32_t* list, const double* Sin, double* Lc,
-                                                 double* Wc, double* Dd, double* Vd, double* Rd, const double* Gq,
+                                                 double* Wc, double* Dd, double* Vd, const double* Gq,
                                                  double* ws, double* ldet, int64_t* st) {
   const int k = list[blockIdx.x];
   complete_load_front(S, k, Sin, ws);
-  complete_front(S, k, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet, st);
+  complete_front(S, k, Sin, Lc, Wc, Dd, Vd, Gq, ws, ldet, st);
 }
 // the end of the grouped completion (group_tier.cu) for fronts wider than one
 // block: P is the N block of the S-front in the order (A, N), L_AN in Wc
@@ -1263,7 +1259,8 @@ struct Posts {
 
 // Level l holds tasks [t0, t0 + nwarp) of the warp tier (|J| <= 32), then
 // [tw, tw + nw64) of the wide warp tier (|J| <= 64), then [tc, tc + ncta) of
-// the CTA tier, then nbig single big fronts of the dense tier.
+// the grouped tier and the fronts too wide for it, then nbig single fronts of
+// the dense tier.
 struct Level {
   int tr, nr32, nr64;  // chain runs: [tr, tr + nr32) |J| <= 32, then nr64 with |J| <= 64
   int t0, nwarp, tw, nw64, tc, ncta, nbig;
@@ -1625,15 +1622,17 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
 }
 // Completion: the arithmetic of Algorithm 7.3 for one front needs only the
 // input S (its columns N_k and the submatrix V_k = S_{A_k A_k}), so every
-// front is independent: the big fronts run on the side streams, all CTA-tier
-// fronts in one launch and all warp-tier fronts in one launch, concurrently.
+// front is independent: the dense fronts run on the side streams, the fronts
+// of the grouped tier in launches over all of them, all warp-tier fronts in one
+// launch, concurrently.
 void big_complete_load(const chd_symbolic* s, cudaStream_t st, int k, const double* Sin, double* ws);
 void big_fc(const chd_symbolic* s, const Slot& sl, int k, const double* Sin, double* Gq, double* fcs,
             int64_t* status);
 // Algorithm 7.3 over all fronts (independent).  With Gq (chd_opts.completion
 // = 1), first the factored update matrices of Algorithm 4.3: G_k = P R_k P
 // for every front, level by level from the roots (one launch of k_fc per
-// level, dense-tier sequences on the side streams), then the fronts use G_k.
+// level, dense-tier sequences on the side streams), then the fronts use G_k
+// (k_complete, one CTA per front, in place of the grouped form).
 void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const double* Sin, double* Lc, double* Wc,
               double* Dd, double* Vd, double* Rd, double* Gq, double* fcs, double* ws, double* ldet,
               int64_t* status) {
@@ -1676,7 +1675,7 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
     count();
   }
   if (!grouped && s->dev.cta_count > 0) {
-    k_complete<<<(int)s->dev.cta_count, NT, 0, st>>>(s->dev, s->dev.cta_fronts, Sin, Lc, Wc, Dd, Vd, Rd, Gq, ws, ldet,
+    k_complete<<<(int)s->dev.cta_count, NT, 0, st>>>(s->dev, s->dev.cta_fronts, Sin, Lc, Wc, Dd, Vd, Gq, ws, ldet,
                                                      status);
     count();
   }

@@ -991,15 +991,16 @@ chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* r
 
   // ---- schedule -------------------------------------------------------------
   // Each front gets a tier: warp (|N| <= 8 and |J| <= 32, one warp per front),
-  // wide warp (|N| <= 8 and |J| <= 64, one warp per front), CTA (one
-  // 256-thread CTA per front) or dense (|J| >= big_rows or |N| >= big_cols,
-  // multi-CTA sequence).  Maximal subtrees of warp-tier
+  // wide warp (|N| <= 8 and |J| <= 64, one warp per front), grouped (launches
+  // over all fronts of a sub-level; one CTA per front for those too wide for it)
+  // or dense (|J| >= big_rows or |N| >= big_cols, multi-CTA sequence).  Maximal subtrees of warp-tier
   // fronts whose total work is at most total/(8*152) become single-warp
   // tasks processed in postorder (tree parallelism, §8); the fronts above
   // form chains (a front joins its only such child when both have the same
   // tier, dense fronts never chain), one task each.  A task's level exceeds
   // the levels of the tasks it depends on; every level is launched as one
-  // warp-tier kernel, one CTA-tier kernel and one dense sequence per front.
+  // warp-tier kernel, the grouped tier's kernels per sub-level and one dense
+  // sequence per front.
   {
     const int64_t big_rows = opts.big_rows > 0 ? opts.big_rows : 320;
     const int64_t big_cols = opts.big_cols > 0 ? opts.big_cols : 160;
