@@ -73,7 +73,7 @@ def hbm_peak_gbs():
 # DRAM bytes (read + write) of one Hessian call, summed over the call's
 # launches in one ncu capture of the current kernels (dram__bytes_read.sum +
 # dram__bytes_write.sum); absent where there is none.
-TRAFFIC_PER_HESSIAN_CALL = {"er5000": 9.716e9}
+TRAFFIC_PER_HESSIAN_CALL = {}
 
 
 def make_workload(name):
