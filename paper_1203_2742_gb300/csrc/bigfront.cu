@@ -1003,8 +1003,8 @@ __global__ void __launch_bounds__(BT) mk_gather_an(SymDev S, int k, const double
 }
 // L_AN = -R^{-T} Z for a front of a few columns, Z^T in the N rows of F: back
 // substitution through the panels of 32 in one CTA.  With n = 1 the blocked
-// solve is 2 a / 64 launches of about 30 us whose products have one row (1.4 ms
-// at a = 1340); here a panel is a chain of 9 us and the updates left of it one
+// solve is 2 a / 64 launches of about 30 us whose products have one row (1.4 ms,
+// now 0.5, at a = 1340); here a panel is a chain of 9 us and the updates left of it one
 // dot product of 32 per entry.
 constexpr int BACK_N = 4;
 __global__ void __launch_bounds__(BT) mk_back(const double* F, int J, int a, int n, double* LA) {
