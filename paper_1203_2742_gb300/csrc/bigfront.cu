@@ -1007,6 +1007,10 @@ __global__ void __launch_bounds__(BT) mk_gather_an(SymDev S, int k, const double
 // now 0.5, at a = 1340); here a panel is a chain of 9 us and the updates left of it one
 // dot product of 32 per entry.
 constexpr int BACK_N = 4;
+// Dynamic shared memory that leaves room for Ls and rinv below within the 48 KiB
+// a launch gets without raising its limit: n (a + 1) <= 5056.  Longer rows take
+// the blocked solve.
+constexpr size_t BACK_SMEM = (size_t(48) << 10) - (PP * (PP + 1) + PP) * sizeof(double);
 __global__ void __launch_bounds__(BT) mk_back(const double* F, int J, int a, int n, double* LA) {
   extern __shared__ double rows[];  // n x (a + 1)
   __shared__ double Ls[PP][PP + 1], rinv[PP];
@@ -1079,7 +1083,7 @@ void complete_front(const chd_symbolic* s, const Ctx& st, int k, const double* S
     if (a > 0) potrf_partial(st, F, J, J, a, status, CHD_ERR_NOT_COMPLETABLE, k, -1);
     CHD_EW(mk_copy, (int64_t)n * n, 1, st, T1, 0, J, F + a + (int64_t)a * J, 0, J, n, n, 1.0, 0.0, 1, 0);  // P
     const size_t smem = (size_t)n * (a + 1) * 8;
-    if (a > 0 && n <= BACK_N && smem <= 40960) {
+    if (a > 0 && n <= BACK_N && smem <= BACK_SMEM) {
       mk_back<<<1, BT, smem, st>>>(F, J, a, n, T2 + n);
       chd_launch::count_launch();
     } else if (a > 0) {
