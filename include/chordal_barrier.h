@@ -340,7 +340,9 @@ chd_status chd_hessian_factor_sparse(chd_factor* fac, int m, const double* y_dev
 /*
  * Inverse-Hessian products Y_i = H^{-1}(T_i) (§5.3, Algorithm 5.2 in
  * supernodal block form): the solution in S^n_V of P(X^{-1} Y X^{-1}) = T.
- * Uses cached Cholesky factors of V_k = S_{A_k A_k}.
+ * Uses cached inverses of V_k = S_{A_k A_k}, formed by the first call on a
+ * factor.  y_dev may equal t_dev with ldy == ldt (in place); other overlaps
+ * are not allowed.
  */
 chd_status chd_inv_hessian(chd_factor* fac, int m, const double* t_dev, int64_t ldt,
                            double* y_dev, int64_t ldy, void* stream);

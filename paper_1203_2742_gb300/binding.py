@@ -651,6 +651,7 @@ class Factor:
         return out
 
     def inv_hessian(self, t, out=None, stream=None):
+        """Y = H^{-1}(T); `out` may be `t` itself."""
         import torch
         if out is None:
             out = torch.empty_like(t)

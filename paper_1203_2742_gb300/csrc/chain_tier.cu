@@ -891,11 +891,13 @@ __global__ void __launch_bounds__(256) kc_scan(SymDev S, int task0, int step, in
 // Algorithm 5.2 steps 1-2 for one-column fronts: V' is the input T on
 // A_j x A_j, M_A = T_A + V' L_A, M_jj = T_jj + L_A^T (T_A + M_A),
 // K_jj = D M_jj D, K_A = V^{-1} (M_A D).  No column waits for another.
-// Writes what step 3 starts from: Y_jj = K_jj, Y_A = K_A + L_A K_jj, and
-// P = K_A + L_A K_jj / 2 into the first temporary of the front.
+// Writes what step 3 starts from into the front's temporaries: P = K_A + L_A
+// K_jj / 2 into the first, Y_jj = K_jj and Y_A = K_A + L_A K_jj into the second.
+// Not into the output, which may be the input: other CTAs still read the
+// input's columns j+1 .. j+a.
 __global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const double* Wc, const double* Dd,
-                                                   const double* Rd, const double* Tin, int64_t ldt, double* Y,
-                                                   int64_t ldy, double* ws) {
+                                                   const double* Rd, const double* Tin, int64_t ldt,
+                                                   double* ws) {
   __shared__ double B[AMAX][BLD];
   __shared__ double lw[AMAX], tt[AMAX], x[AMAX], yv[AMAX];
   __shared__ double kjj;
@@ -903,7 +905,6 @@ __global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const d
   const int a = R.a, tid = threadIdx.x, lane = tid & 31;
   const int64_t y = blockIdx.z;
   Tin += y * ldt + R.base0;
-  Y += y * ldy + R.base0;
   ws += y * S.f_total;
   const Parent P = parent_of(S, R, ws);
   for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
@@ -932,12 +933,13 @@ __global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const d
     sym_dot(B, x, a, yv);
     __syncthreads();
     double* Pv = ws + R.f0 + (int64_t)i * R.fstride + (int64_t)(a + 1) * (a + 1);
+    double* Yv = Pv + a + 1;
     if (tid < a) {
       const double k = kjj, p = fma(0.5 * lw[tid], k, yv[tid]);
       Pv[1 + tid] = p;
-      Y[b + 1 + tid] = 2.0 * p - yv[tid];
+      Yv[1 + tid] = 2.0 * p - yv[tid];
     }
-    if (tid == MT - 1) Y[b] = kjj;
+    if (tid == MT - 1) Yv[0] = kjj;
     __syncthreads();
   }
 }
@@ -945,11 +947,12 @@ __global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const d
 // Sums of the columns' rank-one (rank-two) blocks over a run: entry
 // (j + r, j) of Z = sum_k x_k y_k^T, the k-th column's vectors covering rows
 // k .. k+a.  Nothing depends on the order of the columns, so a warp takes one
-// column j of Z, its lanes the rows r, for the columns of the run (subtracted
-// from or stored to the output) and for the a columns beyond it (the update
-// block the parent adds).
+// column j of Z, its lanes the rows r, for the columns of the run (stored to
+// the output) and for the a columns beyond it (the update block the parent
+// adds).
 //   product (Algorithm 3.2): x = y = [C; B];
-//   inverse Hessian step 3:  -(P L^T + L P^T), rows k+1 .. k+a.
+//   inverse Hessian step 3:  -(P L^T + L P^T), rows k+1 .. k+a, added to what
+//   kc_ihess_down left in the second temporaries.
 template <bool PROD>
 __global__ void __launch_bounds__(128) kc_band_sum(SymDev S, int task0, const double* Gc, double* Out, int64_t ldo,
                                                   double* ws) {
@@ -982,8 +985,7 @@ __global__ void __launch_bounds__(128) kc_band_sum(SymDev S, int task0, const do
       }
       if (r <= rmax) {
         if (j < R.L) {
-          double* o = Out + (int64_t)j * W + r;
-          *o = PROD ? acc : *o + acc;
+          Out[(int64_t)j * W + r] = PROD ? acc : Pw[(int64_t)j * R.fstride + W + r] + acc;
         } else {
           const int q = j - R.L;
           G[(1 + q + r) + (int64_t)(1 + q) * W] = PROD ? acc : -acc;
@@ -1092,9 +1094,8 @@ void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int
   }
 }
 void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
-                      const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy,
-                      double* ws) {
-  kc_ihess_down<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+                      const double* Dd, const double* Rd, const double* T, int64_t ldt, double* ws) {
+  kc_ihess_down<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Dd, Rd, T, ldt, ws);
   count_launch();
 }
 void chain_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,

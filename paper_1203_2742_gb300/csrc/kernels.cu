@@ -1088,8 +1088,7 @@ void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m
 void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
                      int64_t ldt, double* ws, const double* psi);
 void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
-                      const double* Dd, const double* Rd, const double* T, int64_t ldt, double* Y, int64_t ldy,
-                      double* ws);
+                      const double* Dd, const double* Rd, const double* T, int64_t ldt, double* ws);
 void chain_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,
                     int64_t ldy, double* ws);
 
@@ -1588,7 +1587,7 @@ void inv_hessian(const chd_symbolic* s, cudaStream_t st, const Exec* ex, int m, 
         count();
       }
     }
-    if (v.nr32 + v.nr64) chain_ihess_down(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
+    if (v.nr32 + v.nr64) chain_ihess_down(s, st, v.tr, v.nr32 + v.nr64, m, Wc, Dd, Rd, T, ldt, ws);
     if (v.nwarp)
       (w32_few(v.nwarp, m) ? w32x::warp_ihess_down : w32::warp_ihess_down)(s, sw, v.t0, v.nwarp, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
     if (v.nw64) w64::warp_ihess_down(s, sv, v.tw, v.nw64, m, Wc, Dd, Rd, T, ldt, Y, ldy, ws);
