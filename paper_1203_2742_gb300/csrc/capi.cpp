@@ -1042,9 +1042,10 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   for (int i = 0; i < 9; ++i) iGt[i] = add(gt[i]->data(), gt[i]->size() * 4);
   size_t iGl = add(s->gleg.data(), s->gleg.size() * 4);
   size_t iGc2 = add(s->gc.data(), s->gc.size() * sizeof(GComp));
-  size_t iGq[7];
-  const std::vector<int32_t>* gq[7] = {&s->gc_all, &s->gc_sol, &s->gc_upd, &s->gc_back, &s->gc_b, &s->gc_thin, &s->gc_wide};
-  for (int i = 0; i < 7; ++i) iGq[i] = add(gq[i]->data(), gq[i]->size() * 4);
+  size_t iGq[8];
+  const std::vector<int32_t>* gq[8] = {&s->gc_all, &s->gc_sol,  &s->gc_upd,  &s->gc_back,
+                                       &s->gc_b,   &s->gc_thin, &s->gc_wide, &s->gc_root};
+  for (int i = 0; i < 8; ++i) iGq[i] = add(gq[i]->data(), gq[i]->size() * 4);
   size_t iCs = add(s->cseg.data(), s->cseg.size() * sizeof(ChainSeg));
   size_t iCr = add(s->crun.data(), s->crun.size() * 4);
   size_t iGj = add(s->gj.data(), s->gj.size() * sizeof(GJob));
@@ -1125,8 +1126,8 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   d.gc = reinterpret_cast<const GComp*>(b + pcs[iGc2].off);
   const int2** dq[5] = {&d.gc_all, &d.gc_sol, &d.gc_upd, &d.gc_back, &d.gc_b};
   for (int i = 0; i < 5; ++i) *dq[i] = reinterpret_cast<const int2*>(b + pcs[iGq[i]].off);
-  const int32_t** dl[2] = {&d.gc_thin, &d.gc_wide};
-  for (int i = 0; i < 2; ++i) *dl[i] = reinterpret_cast<const int32_t*>(b + pcs[iGq[5 + i]].off);
+  const int32_t** dl[3] = {&d.gc_thin, &d.gc_wide, &d.gc_root};
+  for (int i = 0; i < 3; ++i) *dl[i] = reinterpret_cast<const int32_t*>(b + pcs[iGq[5 + i]].off);
   d.cseg = reinterpret_cast<const ChainSeg*>(b + pcs[iCs].off);
   d.crun = reinterpret_cast<const int2*>(b + pcs[iCr].off);
   d.gj = reinterpret_cast<const GJob*>(b + pcs[iGj].off);

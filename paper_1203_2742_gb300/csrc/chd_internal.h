@@ -33,8 +33,8 @@ constexpr int kGroupBlock = 32;       // rows per block of the assembly and of t
 constexpr int kGroupThin = 16;        // thin fronts: up to this many columns
 constexpr int kGroupFactor = 32;      // fronts up to this many columns factor in one launch per sub-level
 constexpr int kGroupCols = 256;       // widest front of the tier
-// widest front of the grouped completion: its N x N part ends in one CTA from 33
-// columns on, 0.2 to 0.4 ms up to here, 17 ms at 256 columns
+// the grouped completion ends the N x N part of a front in one CTA from 33 columns
+// on, 0.2 to 0.4 ms up to here; wider ones by the rule at wide_by_sequence
 constexpr int kGroupComplete = 64;
 constexpr int kGroupSmem = 200 << 10; // dynamic shared memory a kernel of the tier may use
 struct alignas(16) GFront {
@@ -124,7 +124,7 @@ struct SymDev {
   const int32_t* gv_small = nullptr;
   const GComp* gc = nullptr;
   const int2 *gc_all = nullptr, *gc_sol = nullptr, *gc_upd = nullptr, *gc_back = nullptr, *gc_b = nullptr;
-  const int32_t *gc_thin = nullptr, *gc_wide = nullptr;
+  const int32_t *gc_thin = nullptr, *gc_wide = nullptr, *gc_root = nullptr;
   const int64_t* inst_sn = nullptr;       // instances x supernode ranges
   int64_t ninst = 1;
   int64_t f_total = 0;               // workspace doubles per right-hand side
@@ -225,11 +225,12 @@ struct chd_symbolic {
   std::vector<int32_t> gv_small;  // supernodes of at most 32 ancestors
   // grouped completion: fronts by decreasing a and the lists of its steps;
   // gc_thin: indices of fronts of at most 32 columns, gc_wide: supernodes of
-  // the others, gc_rest: CTA-tier supernodes outside the grouped form, which take the
+  // the others, gc_root: supernodes of more than 32 columns and no ancestors, one
+  // CTA each, gc_rest: CTA-tier supernodes outside the grouped form, which take the
   // dense tier's sequences
   std::vector<GComp> gc;
   std::vector<char> in_gc;
-  std::vector<int32_t> gc_all, gc_sol, gc_upd, gc_sol_ptr, gc_upd_ptr, gc_back, gc_b, gc_thin, gc_wide, gc_rest;
+  std::vector<int32_t> gc_all, gc_sol, gc_upd, gc_sol_ptr, gc_upd_ptr, gc_back, gc_b, gc_thin, gc_wide, gc_root, gc_rest;
   int gc_amax = 0;
   // device mirror
   SymDev dev;

@@ -858,7 +858,8 @@ __global__ void __launch_bounds__(kScanT) k_active(SymDev S, int32_t* cnt, uint8
     act[y * S.nsn + k] = (c[hi] - (lo > 0 ? c[lo - 1] : 0)) > 0 ? 1 : 0;
   }
 }
-// fronts of `list` at once, one CTA each
+// fronts of `list` at once, one CTA each; without Gq only fronts that have no
+// ancestors
 __global__ void __launch_bounds__(NT) k_complete(SymDev S, const int32_t* list, const double* Sin, double* Lc,
                                                  double* Wc, double* Dd, double* Vd, const double* Gq,
                                                  double* ws, double* ldet, int64_t* st) {
@@ -1657,6 +1658,13 @@ void complete(const chd_symbolic* s, cudaStream_t st, const Exec* ex, const doub
   // the grouped form (group_tier.cu) factors V_k itself; with Gq every front
   // takes the per-front kernels
   const bool grouped = !Gq;
+  if (grouped && !s->gc_root.empty()) {
+    const bool only = s->gc.empty() && s->gc_rest.empty() && s->big_fronts.empty() && s->grp_first.empty();
+    const cudaStream_t sr = bs.fork(AUX_WIDE, only);
+    k_complete<<<(int)s->gc_root.size(), NT, 0, sr>>>(s->dev, s->dev.gc_root, Sin, Lc, Wc, Dd, Vd, nullptr, ws, ldet,
+                                                      status);
+    count();
+  }
   std::vector<int32_t> bigs;  // dense fronts and leaf groups
   for (int32_t k : s->big_fronts)
     if (!(grouped && s->in_gc[k])) bigs.push_back(k);

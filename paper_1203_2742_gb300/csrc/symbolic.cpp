@@ -577,27 +577,77 @@ static void group_inverse_plan(chd_symbolic* s) {
   }
 }
 
+// Which CTA-tier fronts wider than kGroupComplete columns the completion ends by
+// the dense tier's launch sequences (1) instead of in one CTA each (0).
+// Measured, in us (n columns, p panels of 32 of them, q panels of the ancestors):
+//   CTA       1.63 n p^1.5, up to one per SM at once (590 at n = 66, 1280 at 100,
+//             2670 at 150, 9520 at 256), after a (3 + 0.05 n) for its a ancestors
+//   sequence  40 p + 1.9 n + 65 q (250, 315, 520, 750), one after another on the
+//             caller's stream; with dense fronts, whose objects have side streams,
+//             twenty and more at once when the call is replayed, three when the
+//             host issues its launches: sixteen
+// Sequences for the widest m, with the m that gives the smallest sum: one block of
+// 150 columns 2670 -> 540, but 12 of 100 1285 instead of 3780, 300 of 66 0.8
+// instead of 77 ms, 100 grids of 70 x 70 12.7 instead of 46 ms.
+std::vector<char> wide_by_sequence(const chd_symbolic* s) {
+  struct Wide {
+    int64_t k;
+    double seq, cta;
+  };
+  std::vector<Wide> w;
+  bool dense = false;
+  for (int64_t k = 0; k < s->nsn; ++k) {
+    dense = dense || s->is_big[k];
+    const int64_t n = front_n(s, k), a = front_J(s, k) - n;
+    if (s->tier[k] != 1 || n <= kGroupComplete || a > kInvVGroup) continue;
+    const double dn = (double)n, p = (double)((n + 31) / 32), q = (double)((a + 31) / 32);
+    w.push_back({k, 40.0 * p + 1.9 * dn + 65.0 * q, 1.63 * dn * p * std::sqrt(p) + (double)a * (3.0 + 0.05 * dn)});
+  }
+  std::stable_sort(w.begin(), w.end(), [](const Wide& x, const Wide& y) { return x.cta > y.cta; });
+  const double streams = dense ? 16.0 : 1.0;
+  const size_t nw = w.size();
+  size_t best = 0;
+  double cost = 1e300, seq = 0.0;
+  for (size_t m = 0; m <= nw; ++m) {
+    const double waves = std::ceil((double)(nw - m) / 152.0);
+    const double c = seq / streams + (m < nw ? waves * w[m].cta : 0.0);
+    if (c < cost) cost = c, best = m;
+    if (m < nw) seq += w[m].seq;
+  }
+  std::vector<char> by(s->nsn, 0);
+  for (size_t m = 0; m < best; ++m) by[w[m].k] = 1;
+  return by;
+}
+
 // Work lists of the grouped completion (kp_* in group_tier.cu): the CTA and
 // wide warp tiers, and dense fronts whose V_k is too small for its products
-// to gain from the tensor cores.
+// to gain from the tensor cores.  Fronts of more than one block of columns and no
+// ancestors have no part in its panels and run beside them, one CTA each (the
+// root of a 40 x 40 grid: 480 -> 360 us for the call).
 static void group_completion_plan(chd_symbolic* s) {
   s->gc.clear();
   s->in_gc.assign(s->nsn, 0);
-  for (auto* v : {&s->gc_all, &s->gc_sol, &s->gc_upd, &s->gc_back, &s->gc_b, &s->gc_thin, &s->gc_wide, &s->gc_rest})
+  for (auto* v : {&s->gc_all, &s->gc_sol, &s->gc_upd, &s->gc_back, &s->gc_b, &s->gc_thin, &s->gc_wide, &s->gc_root,
+                  &s->gc_rest})
     v->clear();
   s->gc_sol_ptr.assign(1, 0);
   s->gc_upd_ptr.assign(1, 0);
   s->gc_amax = 0;
   auto blocks = [](int64_t v) { return (int32_t)((v + kGroupBlock - 1) / kGroupBlock); };
+  const std::vector<char> by_sequence = wide_by_sequence(s);
   for (int64_t k = 0; k < s->nsn; ++k) {
     const int t = s->tier[k];
     const int64_t n = front_n(s, k), J = front_J(s, k), a = J - n;
     if (t != 1 && t != 3 && !(t == 2 && s->tc_mode != 1)) continue;
-    if (n > kGroupComplete || a > kInvVGroup) {
+    if ((t == 2 && n > kGroupComplete) || by_sequence[k] || a > kInvVGroup) {
       if (t != 2) s->gc_rest.push_back((int32_t)k);
       continue;
     }
     s->in_gc[k] = 1;
+    if (a == 0 && n > kGroupBlock && t != 2) {
+      s->gc_root.push_back((int32_t)k);
+      continue;
+    }
     GComp c{};
     c.base = s->colptr[s->sn_ptr[k]];
     c.f_off = s->f_off[k];
