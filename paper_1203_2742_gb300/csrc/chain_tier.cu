@@ -845,22 +845,21 @@ __global__ void __launch_bounds__(4 * PSX) kc_psi(SymDev S, int task0, const dou
     if (v < a) Psi[g.psi + p + (int64_t)x * a] = X[j];
   }
 }
-// One step of the windows' recursion on every run: Z = M V (half 0), then
-// win += Z M^T (half 1, lower), M = Psi (top-down) or Psi^T (bottom-up);
-// 16 x 16 outputs per CTA
+// One step of the windows' recursion on every run of three segments or more:
+// Z = M V (half 0), then win += Z M^T (half 1, lower), M = Psi (top-down) or
+// Psi^T (bottom-up); 16 x 16 outputs per CTA
 template <bool UP>
 __global__ void __launch_bounds__(256) kc_scan(SymDev S, int task0, int step, int half, const double* Psi,
                                               double* ws) {
   __shared__ double A[16][AMAX + 1], B[AMAX][17];
-  const int r = blockIdx.y;
-  const int2 rs = S.crun[r];
+  const int2 rs = S.crun[blockIdx.y];
   const int p = UP ? 1 + step : rs.y - 2 - step;
   if (p < 1 || p > rs.y - 2) return;
-  const Run R = run_of(S, task0 + r);
+  const ChainSeg g = S.cseg[rs.x + p], src = S.cseg[UP ? rs.x + p - 1 : rs.x + p + 1];
+  const Run R = run_of(S, task0 + g.run);
   const int a = R.a, i0 = (blockIdx.x & 3) * 16, j0 = (blockIdx.x >> 2) * 16, tid = threadIdx.x;
   if (i0 >= a || j0 >= a || (half && i0 < j0)) return;
   ws += (int64_t)blockIdx.z * S.f_total;
-  const ChainSeg g = S.cseg[rs.x + p], src = S.cseg[UP ? rs.x + p - 1 : rs.x + p + 1];
   const double* M = Psi + g.psi;
   double* win = seg_window(R, g.s, ws);
   double* Z = win + R.fstride;
@@ -1006,17 +1005,10 @@ static unsigned columns(const chd_symbolic* s, int t0, int nt, int per, int extr
   for (int t = t0; t < t0 + nt; ++t) L = std::max<int64_t>(L, s->task_ptr[t + 1] - s->task_ptr[t] + extra);
   return (unsigned)std::min<int64_t>((L + per - 1) / per, 32768);
 }
-// Whether m right-hand sides run by segments (the times of the analysis, in
-// us): the serial kernels take one SM per run and right-hand side for
-// cseg_serial; by segments every column is done twice, all segments sharing
-// the SMs, and every segment adds two launches of small products.
+// Whether m right-hand sides run by segments (chain_by_segments: the rule and
+// its evidence)
 static bool by_segments(const chd_symbolic* s, int m, const double* psi) {
-  if (!psi || s->cseg.empty()) return false;
-  const double runs = (double)s->crun.size() / 2, segs = (double)s->cseg.size();
-  const double serial = std::max(1.0, m * runs / 152.0) * s->cseg_serial;
-  const double seg = 2.0 * std::max(1.0, m * segs / 152.0) * s->cseg_column +
-                     s->cseg_steps * s->cseg_step * std::max(1.0, m * runs / 40.0);
-  return seg < 0.8 * serial;
+  return psi && !s->cseg.empty() && chain_by_segments(s, m, 0.8);
 }
 template <bool UP>
 static void scan(const chd_symbolic* s, cudaStream_t st, int t0, int m, const double* psi, double* ws) {

@@ -118,7 +118,7 @@ struct SymDev {
              *gt_nn = nullptr, *gt_asmf = nullptr, *gt_wb = nullptr, *gt_fr = nullptr;
   const int32_t* gleg = nullptr;
   const ChainSeg* cseg = nullptr;
-  const int2* crun = nullptr;  // per run: first segment, number of segments
+  const int2* crun = nullptr;  // runs of at least three segments: first segment, number of segments
   const GJob* gj = nullptr;
   const int2 *gv_all = nullptr, *gv_sol = nullptr, *gv_upd = nullptr;
   const int32_t* gv_small = nullptr;
@@ -165,13 +165,14 @@ struct chd_symbolic {
   // lowest level that waits for a chain run, and whether other tasks lie below it
   int32_t run_join = 0, run_overlap = 0;
   // segments of the runs (none when the serial kernels are faster), (first,
-  // count) per run, doubles of all Psi, most inner segments of a run; modelled
-  // times in us: longest run, longest segment, one step of the windows
+  // count) of the runs of at least three, doubles of all Psi, most inner segments
+  // of a run; modelled times in us: longest run, longest segment, all runs, one
+  // step of the windows
   std::vector<ChainSeg> cseg;
   std::vector<int32_t> crun;
   int64_t cseg_psi = 0;
   int cseg_steps = 0;
-  double cseg_serial = 0, cseg_column = 0, cseg_step = 0;
+  double cseg_serial = 0, cseg_column = 0, cseg_total = 0, cseg_step = 0;
   // per level l, five counts at 5*l: chain runs (|J| <= 32), chain runs
   // (|J| <= 64), warp, wide warp and dense-tier tasks (chd_symbolic_schedule)
   std::vector<int32_t> lvl_counts;
@@ -271,6 +272,21 @@ struct Exec {
   cudaStream_t aux[kAuxStreams] = {};
   cudaEvent_t aux_fork[kAuxStreams] = {}, aux_join[kAuxStreams] = {};
 };
+
+// Whether m right-hand sides of the chain runs are faster by segments than `gain`
+// times the serial kernels, with the times of the analysis (us): the serial
+// kernels take an SM per run and right-hand side, at least as long as the longest
+// run; by segments every column is done twice, all segments sharing the SMs, and
+// every inner segment adds two launches of small products over the runs that have
+// one (kMaxScanRuns of them at most: a grid dimension indexes them).
+constexpr size_t kMaxScanRuns = 65535;
+inline bool chain_by_segments(const chd_symbolic* s, int m, double gain) {
+  const double share = m * s->cseg_total / 152.0, runs = (double)s->crun.size() / 2;
+  const double serial = share > s->cseg_serial ? share : s->cseg_serial;
+  const double seg = 2.0 * (share > s->cseg_column ? share : s->cseg_column) +
+                     s->cseg_steps * s->cseg_step * (m * runs > 40.0 ? m * runs / 40.0 : 1.0);
+  return seg < gain * serial;
+}
 
 // Formation of V_k^{-1} by the size a of V_k: up to kInvVGroup rows the
 // grouped kernels over all fronts at once (kv_* in group_tier.cu; 12000 fronts

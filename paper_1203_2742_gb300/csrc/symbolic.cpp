@@ -729,18 +729,20 @@ static void chain_segments_plan(chd_symbolic* s) {
     for (int r = 0; r < nr; ++r) total += count(r, tau);
     if (total <= std::max(152, 2 * nr) || tau >= tmax) break;
   }
-  int pmax = 1;
-  for (int r = 0; r < nr; ++r) pmax = std::max(pmax, count(r, tau));
-  const double waves = std::max(1.0, total / 152.0);
   s->cseg_serial = tmax;
   s->cseg_column = tau;
   s->cseg_step = kStep;
-  if (pmax < 2 || 2.0 * tau * waves + kStep * (pmax - 2) > 0.7 * tmax * std::max(1.0, nr / 152.0)) return;
+  s->cseg_total = 0;
+  int pmax = 1;
   for (int r = 0; r < nr; ++r) {
     const int P = count(r, tau), L = len(r);
     const int64_t a = anc(r);
-    s->crun.push_back((int32_t)s->cseg.size());
-    s->crun.push_back(P);
+    pmax = std::max(pmax, P);
+    s->cseg_total += time(r);
+    if (P > 2) {
+      s->crun.push_back((int32_t)s->cseg.size());
+      s->crun.push_back(P);
+    }
     for (int p = 0; p < P; ++p) {
       ChainSeg g{};
       g.run = r;
@@ -754,6 +756,12 @@ static void chain_segments_plan(chd_symbolic* s) {
     }
   }
   s->cseg_steps = std::max(0, pmax - 2);
+  if (pmax < 2 || s->crun.size() / 2 > kMaxScanRuns || !chain_by_segments(s, 1, 0.7)) {
+    s->cseg.clear();
+    s->crun.clear();
+    s->cseg_psi = 0;
+    s->cseg_steps = 0;
+  }
 }
 
 chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* rowind,
