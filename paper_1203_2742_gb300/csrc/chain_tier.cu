@@ -59,24 +59,58 @@ struct Run {
   int k0;                         // first supernode (the others follow)
   int64_t base0, col0, d0, v0, vstride, f0, fstride;
 };
-__device__ __forceinline__ Run run_of(const SymDev& S, int t) {
+// ... from the record of its i-th front
+__device__ __forceinline__ Run run_with(const WMeta& w, int i, int L) {
   Run r;
-  const int q0 = S.task_ptr[t], q1 = S.task_ptr[t + 1];
-  const WMeta w = S.tmeta[q0];
-  r.L = q1 - q0;
+  r.L = L;
   r.a = w.J - 1;
-  r.k0 = w.k;
-  r.base0 = w.base;
-  r.col0 = w.col0;
-  r.d0 = w.d_off;
-  r.v0 = w.v_off;
   // per-front offsets of one-column fronts (the symbolic phase rounds each
   // block up to a multiple of four doubles)
   r.vstride = ((int64_t)r.a * r.a + 3) & ~int64_t(3);
   const int64_t J = r.a + 1;
-  r.f0 = w.f_off;
   r.fstride = (J * J + 2 * J + 3) & ~int64_t(3);
+  r.k0 = w.k - i;
+  r.base0 = w.base - i * J;
+  r.col0 = w.col0 - i;
+  r.d0 = w.d_off - 4 * (int64_t)i;
+  r.v0 = w.v_off - i * r.vstride;
+  r.f0 = w.f_off - i * r.fstride;
   return r;
+}
+__device__ __forceinline__ Run run_of(const SymDev& S, int t) {
+  const int q0 = S.task_ptr[t], q1 = S.task_ptr[t + 1];
+  return run_with(S.tmeta[q0], 0, q1 - q0);
+}
+// Kernels over all columns of the launch's runs.  A grid of runs x longest run is
+// empty nearly everywhere when one run is long and many are short (30000 runs of ten
+// columns beside one of 1275: 24.6 ms for a gradient, 1.2 without the empty
+// CTAs), so such runs' columns are taken one after another over all runs (LIST),
+// each through its own record.  An empty CTA costs about 0.55 ns, the record,
+// which neighbours in a run do not share, 0.4: the grid while it adds less than three
+// quarters of the columns.
+struct Columns {
+  int task0;
+  int q0, n;  // LIST: task positions q0 .. q0 + n - 1
+};
+// The run of the CTA's columns (its sub-th, `per` of them a CTA); they are i, i + step,
+// .. while below R.L
+template <bool LIST>
+__device__ __forceinline__ Run run_of_columns(const SymDev& S, const Columns& c, int per, int sub, int& i, int& step) {
+  if (!LIST) {
+    i = blockIdx.y * per + sub;
+    step = gridDim.y * per;
+    return run_of(S, c.task0 + blockIdx.x);
+  }
+  const int q = blockIdx.x * per + sub;
+  step = 1 << 30;
+  if (q >= c.n) {
+    Run none{};
+    i = 0;
+    return none;
+  }
+  const WMeta w = S.tmeta[c.q0 + q];
+  i = w.place;
+  return run_with(w, i, S.task_ptr[w.task + 1] - (c.q0 + q - i));
 }
 
 __device__ __forceinline__ void cp_async8(double* dst, const double* src) {
@@ -343,11 +377,13 @@ __global__ void __launch_bounds__(UPT) kc_factor(SymDev S, int task0, const doub
   up_dispatch<UP_FACTOR>(R, Span{0, R.L, nullptr, true, update_block(R, ws), R.a + 1}, A, sm);
 }
 // C, B and log D of every column of every run, one warp per column
-__global__ void __launch_bounds__(128) kc_factor_post(SymDev S, int task0, double* Lc, const double* Dd,
+template <bool LIST>
+__global__ void __launch_bounds__(128) kc_factor_post(SymDev S, Columns cols, double* Lc, const double* Dd,
                                                      double* ldet) {
-  const Run R = run_of(S, task0 + blockIdx.x);
+  int i, step;
+  const Run R = run_of_columns<LIST>(S, cols, 4, threadIdx.x >> 5, i, step);
   const int lane = threadIdx.x & 31;
-  for (int i = blockIdx.y * 4 + (threadIdx.x >> 5); i < R.L; i += gridDim.y * 4) {
+  for (; i < R.L; i += step) {
     const double d = Dd[R.d0 + 4 * (int64_t)i], r = rsqrt(d);
     double* c = Lc + R.base0 + (int64_t)i * (R.a + 1);
     for (int p = lane; p <= R.a; p += 32) c[p] *= r;
@@ -469,14 +505,16 @@ __device__ __forceinline__ Parent parent_of(const SymDev& S, const Run& R, const
 }
 
 // Algorithm 5.1 step 2: M_jj = K_jj / D^2, M_A = V K_A / D (K in T, in place)
-__global__ void __launch_bounds__(MT) kc_hess_m(SymDev S, int task0, const double* Wc, const double* Vd, double* T,
+template <bool LIST>
+__global__ void __launch_bounds__(MT) kc_hess_m(SymDev S, Columns cols, const double* Wc, const double* Vd, double* T,
                                                int64_t ldt, const uint8_t* act) {
   __shared__ double B[AMAX][BLD];
   __shared__ double x[AMAX], yv[AMAX];
-  const Run R = run_of(S, task0 + blockIdx.x);
+  int i, step;
+  const Run R = run_of_columns<LIST>(S, cols, 1, 0, i, step);
   const int a = R.a, tid = threadIdx.x;
   const int64_t y = blockIdx.z;
-  for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
+  for (; i < R.L; i += step) {
     if (act && !act[y * S.nsn + R.k0 + i]) continue;
     double* t = T + y * ldt + R.base0 + (int64_t)i * (a + 1);
     const double dinv = Wc[R.base0 + (int64_t)i * (a + 1)];
@@ -707,13 +745,15 @@ __global__ void __launch_bounds__(DNT) kc_gradient_seg(SymDev S, int task0, int 
   if (!down_seg(S, g, R, phase, ws, sp)) return;
   down_dispatch<DOWN_GRAD>(S, R, sp, Wc + R.base0, nullptr, Sc + R.base0, ws, sm);
 }
-__global__ void __launch_bounds__(MT) kc_grad_post(SymDev S, int task0, const double* Sc, double* g, double* Vd,
+template <bool LIST>
+__global__ void __launch_bounds__(MT) kc_grad_post(SymDev S, Columns cols, const double* Sc, double* g, double* Vd,
                                                   const double* ws) {
-  const Run R = run_of(S, task0 + blockIdx.x);
+  int i, step;
+  const Run R = run_of_columns<LIST>(S, cols, 1, 0, i, step);
   const Parent P = parent_of(S, R, ws);
   const int a = R.a, lane = threadIdx.x & 31;
   const double* v = Sc + R.base0;
-  for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
+  for (; i < R.L; i += step) {
     double* Vb = Vd + R.v0 + (int64_t)i * R.vstride;
     for (int c = threadIdx.x >> 5; c < a; c += MT / 32) {
       const int col = i + 1 + c;
@@ -738,11 +778,13 @@ __global__ void __launch_bounds__(MT) kc_grad_post(SymDev S, int task0, const do
 // T_jj = M_jj - 2 L_A^T M_A + L_A^T w; V' of the child = [T_jj T_A^T; T_A V']
 // on its rows.  T in place; first
 // what of T_jj does not depend on the recursion, in place: M_jj - 2 L_A^T M_A
-__global__ void __launch_bounds__(128) kc_down_pre(SymDev S, int task0, const double* Wc, double* T, int64_t ldt) {
-  const Run R = run_of(S, task0 + blockIdx.x);
+template <bool LIST>
+__global__ void __launch_bounds__(128) kc_down_pre(SymDev S, Columns cols, const double* Wc, double* T, int64_t ldt) {
+  int i, step;
+  const Run R = run_of_columns<LIST>(S, cols, 4, threadIdx.x >> 5, i, step);
   const int lane = threadIdx.x & 31, W = R.a + 1;
   T += (int64_t)blockIdx.z * ldt + R.base0;
-  for (int i = blockIdx.y * 4 + (threadIdx.x >> 5); i < R.L; i += gridDim.y * 4) {
+  for (; i < R.L; i += step) {
     double* t = T + (int64_t)i * W;
     const double* l = Wc + R.base0 + (int64_t)i * W;
     double acc = 0.0;
@@ -894,19 +936,21 @@ __global__ void __launch_bounds__(256) kc_scan(SymDev S, int task0, int step, in
 // K_jj / 2 into the first, Y_jj = K_jj and Y_A = K_A + L_A K_jj into the second.
 // Not into the output, which may be the input: other CTAs still read the
 // input's columns j+1 .. j+a.
-__global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const double* Wc, const double* Dd,
+template <bool LIST>
+__global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, Columns cols, const double* Wc, const double* Dd,
                                                    const double* Rd, const double* Tin, int64_t ldt,
                                                    double* ws) {
   __shared__ double B[AMAX][BLD];
   __shared__ double lw[AMAX], tt[AMAX], x[AMAX], yv[AMAX];
   __shared__ double kjj;
-  const Run R = run_of(S, task0 + blockIdx.x);
+  int i, step;
+  const Run R = run_of_columns<LIST>(S, cols, 1, 0, i, step);
   const int a = R.a, tid = threadIdx.x, lane = tid & 31;
   const int64_t y = blockIdx.z;
   Tin += y * ldt + R.base0;
   ws += y * S.f_total;
   const Parent P = parent_of(S, R, ws);
-  for (int i = blockIdx.y; i < R.L; i += gridDim.y) {
+  for (; i < R.L; i += step) {
     const int64_t b = (int64_t)i * (a + 1);
     const double dd = Dd[R.d0 + 4 * (int64_t)i];
     stage_window(S, R, i, Tin, P.F, P.J, P.rel, B);
@@ -952,10 +996,20 @@ __global__ void __launch_bounds__(MT) kc_ihess_down(SymDev S, int task0, const d
 //   product (Algorithm 3.2): x = y = [C; B];
 //   inverse Hessian step 3:  -(P L^T + L P^T), rows k+1 .. k+a, added to what
 //   kc_ihess_down left in the second temporaries.
-template <bool PROD>
-__global__ void __launch_bounds__(128) kc_band_sum(SymDev S, int task0, const double* Gc, double* Out, int64_t ldo,
-                                                  double* ws) {
-  const Run R = run_of(S, task0 + blockIdx.x);
+// LIST: the grid ends with `beyond` CTAs for the columns beyond each run
+template <bool PROD, bool LIST>
+__global__ void __launch_bounds__(128) kc_band_sum(SymDev S, Columns cols, int beyond, const double* Gc, double* Out,
+                                                  int64_t ldo, double* ws) {
+  int j, step;
+  Run R;
+  const int e = (int)blockIdx.x - (cols.n + 3) / 4;
+  if (!LIST || e < 0) {
+    R = run_of_columns<LIST>(S, cols, 4, threadIdx.x >> 5, j, step);
+  } else {
+    R = run_of(S, cols.task0 + e / beyond);
+    j = R.L + e % beyond * 4 + (threadIdx.x >> 5);
+    step = 1 << 30;
+  }
   const int a = R.a, lane = threadIdx.x & 31, W = a + 1;
   const int64_t y = blockIdx.z;
   Out += y * ldo + R.base0;
@@ -963,7 +1017,7 @@ __global__ void __launch_bounds__(128) kc_band_sum(SymDev S, int task0, const do
   const double* Lw = Gc + R.base0;
   const double* Pw = ws + R.f0 + (int64_t)W * W;
   double* G = ws + R.f0 + (int64_t)(R.L - 1) * R.fstride;
-  for (int j = blockIdx.y * 4 + (threadIdx.x >> 5); j < R.L + a; j += gridDim.y * 4) {
+  for (; j < R.L + a; j += step) {
     const int rmax = j < R.L ? a : R.L + a - 1 - j;
     const int kend = PROD ? min(j, R.L - 1) : min(j, R.L) - 1;
     for (int r0 = 0; r0 <= rmax; r0 += 32) {
@@ -999,11 +1053,16 @@ __global__ void __launch_bounds__(128) kc_band_sum(SymDev S, int task0, const do
 
 namespace chd_launch {
 using namespace chd::chain;
-// columns of the longest run of the launch, as a grid dimension
-static unsigned columns(const chd_symbolic* s, int t0, int nt, int per, int extra) {
-  int64_t L = 1;
-  for (int t = t0; t < t0 + nt; ++t) L = std::max<int64_t>(L, s->task_ptr[t + 1] - s->task_ptr[t] + extra);
-  return (unsigned)std::min<int64_t>((L + per - 1) / per, 32768);
+// the columns of the launch's runs, and a grid of m x `per` of them per CTA
+// (extra: as many more beyond each run)
+static Columns columns(const chd_symbolic* s, int t0, int nt) {
+  if (s->run_lmax > 0) return Columns{t0, 0, 0};
+  return Columns{t0, s->task_ptr[t0], s->task_ptr[t0 + nt] - s->task_ptr[t0]};
+}
+static dim3 column_grid(const chd_symbolic* s, const Columns& c, int nt, int per, int m, int extra = 0) {
+  auto ctas = [&](int v) { return (v + per - 1) / per; };
+  if (c.n > 0) return dim3(ctas(c.n) + nt * ctas(extra), 1, m);
+  return dim3(nt, std::min(ctas(s->run_lmax + extra), 32768), m);
 }
 // Whether m right-hand sides run by segments (chain_by_segments: the rule and
 // its evidence)
@@ -1029,11 +1088,15 @@ void chain_factor(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const 
                   double* Dd, double* ws, double* ldet, int64_t* status) {
   kc_factor<<<nt, UPT, 0, st>>>(s->dev, t0, X, Lc, Wc, Dd, ws, status);
   count_launch();
-  kc_factor_post<<<dim3(nt, columns(s, t0, nt, 4, 0)), 128, 0, st>>>(s->dev, t0, Lc, Dd, ldet);
+  const Columns c = columns(s, t0, nt);
+  const auto post = c.n > 0 ? kc_factor_post<true> : kc_factor_post<false>;
+  post<<<column_grid(s, c, nt, 4, 1), 128, 0, st>>>(s->dev, c, Lc, Dd, ldet);
   count_launch();
 }
 void chain_product(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Lc, double* X, double* ws) {
-  kc_band_sum<true><<<dim3(nt, columns(s, t0, nt, 4, AMAX)), 128, 0, st>>>(s->dev, t0, Lc, X, 0, ws);
+  const Columns c = columns(s, t0, nt);
+  const auto sum = c.n > 0 ? kc_band_sum<true, true> : kc_band_sum<true, false>;
+  sum<<<column_grid(s, c, nt, 4, 1, s->run_amax), 128, 0, st>>>(s->dev, c, (s->run_amax + 3) / 4, Lc, X, 0, ws);
   count_launch();
 }
 void chain_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, const double* Wc, double* Sc, double* g,
@@ -1049,7 +1112,9 @@ void chain_gradient(const chd_symbolic* s, cudaStream_t st, int t0, int nt, cons
     kc_gradient<<<nt, DNT, 0, st>>>(s->dev, t0, Wc, Sc, ws);
     count_launch();
   }
-  kc_grad_post<<<dim3(nt, columns(s, t0, nt, 1, 0)), MT, 0, st>>>(s->dev, t0, Sc, g, Vd, ws);
+  const Columns c = columns(s, t0, nt);
+  const auto post = c.n > 0 ? kc_grad_post<true> : kc_grad_post<false>;
+  post<<<column_grid(s, c, nt, 1, 1), MT, 0, st>>>(s->dev, c, Sc, g, Vd, ws);
   count_launch();
 }
 void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, const double* Vd,
@@ -1066,12 +1131,16 @@ void chain_hess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m
     kc_hess_up<<<dim3(nt, m), UPT, 0, st>>>(s->dev, t0, Wc, Y, ldy, T, ldt, ws, act);
     count_launch();
   }
-  kc_hess_m<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Vd, T, ldt, act);
+  const Columns c = columns(s, t0, nt);
+  const auto step2 = c.n > 0 ? kc_hess_m<true> : kc_hess_m<false>;
+  step2<<<column_grid(s, c, nt, 1, m), MT, 0, st>>>(s->dev, c, Wc, Vd, T, ldt, act);
   count_launch();
 }
 void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* T,
                      int64_t ldt, double* ws, const double* psi) {
-  kc_down_pre<<<dim3(nt, columns(s, t0, nt, 4, 0), m), 128, 0, st>>>(s->dev, t0, Wc, T, ldt);
+  const Columns c = columns(s, t0, nt);
+  const auto pre = c.n > 0 ? kc_down_pre<true> : kc_down_pre<false>;
+  pre<<<column_grid(s, c, nt, 4, m), 128, 0, st>>>(s->dev, c, Wc, T, ldt);
   count_launch();
   if (by_segments(s, m, psi)) {
     const unsigned ns = (unsigned)s->cseg.size();
@@ -1087,12 +1156,16 @@ void chain_hess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int
 }
 void chain_ihess_down(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc,
                       const double* Dd, const double* Rd, const double* T, int64_t ldt, double* ws) {
-  kc_ihess_down<<<dim3(nt, columns(s, t0, nt, 1, 0), m), MT, 0, st>>>(s->dev, t0, Wc, Dd, Rd, T, ldt, ws);
+  const Columns c = columns(s, t0, nt);
+  const auto down = c.n > 0 ? kc_ihess_down<true> : kc_ihess_down<false>;
+  down<<<column_grid(s, c, nt, 1, m), MT, 0, st>>>(s->dev, c, Wc, Dd, Rd, T, ldt, ws);
   count_launch();
 }
 void chain_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m, const double* Wc, double* Y,
                     int64_t ldy, double* ws) {
-  kc_band_sum<false><<<dim3(nt, columns(s, t0, nt, 4, AMAX), m), 128, 0, st>>>(s->dev, t0, Wc, Y, ldy, ws);
+  const Columns c = columns(s, t0, nt);
+  const auto sum = c.n > 0 ? kc_band_sum<false, true> : kc_band_sum<false, false>;
+  sum<<<column_grid(s, c, nt, 4, m, s->run_amax), 128, 0, st>>>(s->dev, c, (s->run_amax + 3) / 4, Wc, Y, ldy, ws);
   count_launch();
 }
 }  // namespace chd_launch

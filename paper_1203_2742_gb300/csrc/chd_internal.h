@@ -24,7 +24,7 @@ struct alignas(16) WMeta {
   int64_t v_off;     // offset of the a x a block
   int32_t k, n, J, flags;
   int32_t ch_beg, ch_end;  // children of k in ch[ch_beg..ch_end)
-  int32_t pad[2];
+  int32_t task, place;     // the task that holds the front, and where in it
 };
 
 // Grouped tier (group_tier.cu): the fronts whose gradient, Hessian and
@@ -164,6 +164,9 @@ struct chd_symbolic {
   std::vector<int32_t> lvl_r32, lvl_r64;
   // lowest level that waits for a chain run, and whether other tasks lie below it
   int32_t run_join = 0, run_overlap = 0;
+  // largest a of the runs, and the longest run if a grid of runs x columns of it
+  // is full enough (Columns in chain_tier.cu), else 0
+  int run_amax = 0, run_lmax = 0;
   // segments of the runs (none when the serial kernels are faster), (first,
   // count) of the runs of at least three, doubles of all Psi, most inner segments
   // of a run; modelled times in us: longest run, longest segment, all runs, one

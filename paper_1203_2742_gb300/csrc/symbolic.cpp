@@ -707,6 +707,7 @@ static void chain_segments_plan(chd_symbolic* s) {
   s->crun.clear();
   s->cseg_psi = 0;
   s->cseg_steps = 0;
+  s->run_amax = s->run_lmax = 0;
   if (s->lvl_r32.empty()) return;
   const int nr = s->lvl_r32[0] + s->lvl_r64[0];
   if (nr == 0) return;
@@ -715,7 +716,13 @@ static void chain_segments_plan(chd_symbolic* s) {
   auto anc = [&](int r) { return front_J(s, s->task_fronts[s->task_ptr[t0 + r]]) - 1; };
   auto time = [&](int r) { return len(r) * (0.3 + 0.02 * anc(r)); };
   double tmax = 0;
-  for (int r = 0; r < nr; ++r) tmax = std::max(tmax, time(r));
+  for (int r = 0; r < nr; ++r) {
+    tmax = std::max(tmax, time(r));
+    s->run_amax = std::max(s->run_amax, (int)anc(r));
+    s->run_lmax = std::max(s->run_lmax, len(r));
+  }
+  const double cols = s->task_ptr[t0 + nr] - s->task_ptr[t0];
+  if ((double)nr * s->run_lmax > 1.75 * cols) s->run_lmax = 0;
   constexpr double kStep = 12.0;
   const double pbest = std::min(64.0, std::max(1.0, std::floor(std::sqrt(tmax / (0.5 * kStep)))));
   double tau = tmax / pbest;
@@ -1318,6 +1325,8 @@ chd_status chd_symbolic_build(int64_t n, const int64_t* colptr, const int32_t* r
         w.d_off = s->d_off[k];
         w.v_off = s->v_off[k];
         w.k = (int32_t)k;
+        w.task = (int32_t)t;
+        w.place = q - q0;
         w.n = (int32_t)(s->sn_ptr[k + 1] - s->sn_ptr[k]);
         w.J = (int32_t)(s->rows_ptr[k + 1] - s->rows_ptr[k]);
         w.ch_beg = (int32_t)s->ea_ptr[k];

@@ -1,6 +1,7 @@
 """Many short chain runs in one object beside one long enough to be cut into
 segments: more of them than a grid dimension of a launch holds, every value
-against dense references (the long band alone on the CPU oracle)."""
+against dense references (the long band alone on the CPU oracle); and the time
+of a call stays near that of the two kinds on their own."""
 import numpy as np
 import pytest
 
@@ -55,3 +56,39 @@ def test_more_runs_than_a_grid_dimension():
     h = z @ full(y) @ z
     assert np.abs(g[nz1:].reshape(COUNT, nz) + z[:, rs, cols]).max() < 1e-12 * np.abs(z).max()
     assert np.abs(t[nz1:].reshape(COUNT, nz) - h[:, rs, cols]).max() < 1e-12 * np.abs(h).max()
+
+
+def test_short_runs_beside_a_long_one_cost_no_more():
+    """Kernels over all columns of all runs: time by columns, not by runs times the
+    longest run (a factor of ten and more here)."""
+    import torch
+    from paper_1203_2742_gb300 import binding as B
+
+    def times(pattern):
+        sym = B.Symbolic(*pattern)
+        rng = np.random.default_rng(4)
+        x = _dev(W.diag_dominant(sym.n, sym.colptr, sym.rowind, rng))
+        y = _dev(W.uniform_sym(sym.n, sym.colptr, sym.rowind, rng, count=2))
+        f = sym.factor(x)
+        g, t, u = f.gradient(), f.hessian(y), None
+        u = f.inv_hessian(t)
+        p = f.product()
+        out = []
+        for call in (lambda: f.refactor(x), lambda: f.gradient(out=g), lambda: f.hessian(y, out=t),
+                     lambda: f.inv_hessian(t, out=u), lambda: f.product(out=p)):
+            best = 1e30
+            for _ in range(8):
+                a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                a.record()
+                call()
+                b.record()
+                torch.cuda.synchronize()
+                best = min(best, a.elapsed_time(b))
+            out.append(best)
+        return out
+
+    long = W.band(1300, 24)
+    short = _pattern((0, np.zeros(1, np.int64), np.zeros(0, np.int32)), 30000)[0]
+    both = times(_pattern(long, 30000)[0])
+    for t, a, b in zip(both, times(long), times(short)):
+        assert t < 3.0 * (a + b), (both, a, b)
