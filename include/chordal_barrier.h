@@ -476,6 +476,7 @@ chd_status chd_probe_tc_bf16_peak(void* stream, double* tflops);
  */
 chd_status chd_probe_units(void* stream, double out[4]);
 
+/* Waits for the object's work on the stream of its last call, then frees it. */
 void chd_factor_free(chd_factor* fac);
 
 /*

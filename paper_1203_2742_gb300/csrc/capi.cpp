@@ -960,7 +960,9 @@ chd_status chd_probe_fp64_peak(void* stream, double* gflops) {
 
 void chd_factor_free(chd_factor* f) {
   if (!f) return;
-  if (f->stream) cudaStreamSynchronize(f->stream);
+  // The default stream (null) too: cudaFree of a stream-ordered allocation assumes
+  // that nothing uses it any more and waits for nothing.
+  cudaStreamSynchronize(f->stream);
   for (int j = 0; j < f->ex.nside; ++j) {
     cudaStreamSynchronize(f->ex.side[j]);
     cudaStreamDestroy(f->ex.side[j]);
