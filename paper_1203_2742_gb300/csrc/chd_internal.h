@@ -220,7 +220,7 @@ struct chd_symbolic {
   std::vector<int32_t> gptr, gidx, glvl;
   std::vector<int32_t> gt_up, gt_row, gt_asm, gt_p, gt_gat, gt_nn, gt_asmf, gt_wb, gt_fr, gleg;
   std::vector<int32_t> gs_up, gs_row, gs_asm, gs_p, gs_gat, gs_asmf, gs_wb, gs_rn, gs_np, gs_thin, gs_leg;
-  int g_rnmax = 0, g_nmax = 0;
+  int g_rnmax = 0, g_nmax = 0, g_amax = 0;
   // grouped inverse: fronts by decreasing a, their lower tiles, and per panel
   // of 32 columns the row blocks to solve and the tiles to update
   std::vector<GJob> gj;

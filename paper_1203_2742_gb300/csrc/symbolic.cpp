@@ -400,7 +400,7 @@ static void group_plan(chd_symbolic* s) {
     v->assign(1, 0);
   s->gf.clear();
   s->gch.clear();
-  s->g_rnmax = s->g_nmax = 0;
+  s->g_rnmax = s->g_nmax = s->g_amax = 0;
   auto blocks = [](int64_t v) { return (v + kGroupBlock - 1) / kGroupBlock; };
   // rows per block of the row-block kernels: as few as the front's second
   // temporary holds partial n x n sums for (and a counter); 16 or more for
@@ -482,6 +482,7 @@ static void group_plan(chd_symbolic* s) {
     s->gs_rn.back() = std::max(s->gs_rn.back(), (int32_t)(R * n));
     s->g_rnmax = std::max(s->g_rnmax, (int)(R * n));
     s->g_nmax = std::max(s->g_nmax, (int)n);
+    s->g_amax = std::max(s->g_amax, (int)a);
   };
   auto eligible = [&](int64_t k) {
     const int64_t n = front_n(s, k), a = front_J(s, k) - n;
