@@ -1038,10 +1038,10 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   size_t iGf = add(s->gf.data(), s->gf.size() * sizeof(GFront));
   size_t iGc = add(s->gch.data(), s->gch.size() * sizeof(GChild));
   size_t iGp = add(s->gptr.data(), s->gptr.size() * 4);
-  size_t iGt[9];
-  const std::vector<int32_t>* gt[9] = {&s->gt_up,  &s->gt_row,  &s->gt_asm, &s->gt_p, &s->gt_gat,
-                                       &s->gt_nn, &s->gt_asmf, &s->gt_wb,  &s->gt_fr};
-  for (int i = 0; i < 9; ++i) iGt[i] = add(gt[i]->data(), gt[i]->size() * 4);
+  size_t iGt[10];
+  const std::vector<int32_t>* gt[10] = {&s->gt_up,  &s->gt_row,  &s->gt_asm, &s->gt_p, &s->gt_gat,
+                                       &s->gt_nn, &s->gt_asmf, &s->gt_wb,  &s->gt_fr, &s->gt_out};
+  for (int i = 0; i < 10; ++i) iGt[i] = add(gt[i]->data(), gt[i]->size() * 4);
   size_t iGl = add(s->gleg.data(), s->gleg.size() * 4);
   size_t iGc2 = add(s->gc.data(), s->gc.size() * sizeof(GComp));
   size_t iGq[8];
@@ -1122,8 +1122,9 @@ chd_status chd_symbolic_upload(chd_symbolic* s) {
   d.gf = reinterpret_cast<const GFront*>(b + pcs[iGf].off);
   d.gch = reinterpret_cast<const GChild*>(b + pcs[iGc].off);
   d.gptr = reinterpret_cast<const int32_t*>(b + pcs[iGp].off);
-  const int2** dgt[9] = {&d.gt_up, &d.gt_row, &d.gt_asm, &d.gt_p, &d.gt_gat, &d.gt_nn, &d.gt_asmf, &d.gt_wb, &d.gt_fr};
-  for (int i = 0; i < 9; ++i) *dgt[i] = reinterpret_cast<const int2*>(b + pcs[iGt[i]].off);
+  const int2** dgt[10] = {&d.gt_up, &d.gt_row,  &d.gt_asm, &d.gt_p,  &d.gt_gat,
+                          &d.gt_nn, &d.gt_asmf, &d.gt_wb,  &d.gt_fr, &d.gt_out};
+  for (int i = 0; i < 10; ++i) *dgt[i] = reinterpret_cast<const int2*>(b + pcs[iGt[i]].off);
   d.gleg = reinterpret_cast<const int32_t*>(b + pcs[iGl].off);
   d.gc = reinterpret_cast<const GComp*>(b + pcs[iGc2].off);
   const int2** dq[5] = {&d.gc_all, &d.gc_sol, &d.gc_upd, &d.gc_back, &d.gc_b};

@@ -115,7 +115,7 @@ struct SymDev {
   const GChild* gch = nullptr;
   const int32_t* gptr = nullptr;
   const int2 *gt_up = nullptr, *gt_row = nullptr, *gt_asm = nullptr, *gt_p = nullptr, *gt_gat = nullptr,
-             *gt_nn = nullptr, *gt_asmf = nullptr, *gt_wb = nullptr, *gt_fr = nullptr;
+             *gt_nn = nullptr, *gt_asmf = nullptr, *gt_wb = nullptr, *gt_fr = nullptr, *gt_out = nullptr;
   const int32_t* gleg = nullptr;
   const ChainSeg* cseg = nullptr;
   const int2* crun = nullptr;  // runs of at least three segments: first segment, number of segments
@@ -218,8 +218,8 @@ struct chd_symbolic {
   std::vector<GFront> gf;
   std::vector<GChild> gch;
   std::vector<int32_t> gptr, gidx, glvl;
-  std::vector<int32_t> gt_up, gt_row, gt_asm, gt_p, gt_gat, gt_nn, gt_asmf, gt_wb, gt_fr, gleg;
-  std::vector<int32_t> gs_up, gs_row, gs_asm, gs_p, gs_gat, gs_asmf, gs_wb, gs_rn, gs_np, gs_thin, gs_leg;
+  std::vector<int32_t> gt_up, gt_row, gt_asm, gt_p, gt_gat, gt_nn, gt_asmf, gt_wb, gt_fr, gt_out, gleg;
+  std::vector<int32_t> gs_up, gs_row, gs_asm, gs_p, gs_gat, gs_asmf, gs_wb, gs_out, gs_rn, gs_np, gs_thin, gs_leg;
   int g_rnmax = 0, g_nmax = 0, g_amax = 0;
   // grouped inverse: fronts by decreasing a, their lower tiles, and per panel
   // of 32 columns the row blocks to solve and the tiles to update

@@ -205,17 +205,23 @@ __global__ void __launch_bounds__(256) kg_p(SymDev S, const int2* tiles, const d
 //           launch per sub-level instead of three); wide ones find the front
 //           assembled and P in T1.  The first tile column stores F_AN, P and
 //           F_NN for step 2.
-// UP_IHESS: P is in the N-part of F (left by step 2); the first tile column
-//           subtracts the children's part from the output's columns N_k.
+// UP_IHESS: P is in the N-part of F (left by step 2).  The CTAs beyond the tiles
+//           subtract the children's part from the output's columns N_k, a 32 x 32
+//           block each (fronts with children only).  A CTA walks the children
+//           one by one, so a block per CTA: 400 children of five columns
+//           under one front of 40, one right-hand side: 2020 us with all blocks of the
+//           front's rows in the CTAs of the first tile column, 907 so.
 // ---------------------------------------------------------------------------
 enum { UP_HESS = 0, UP_IHESS = 1 };
 template <int MODE>
 __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const double* Wc, const double* Y,
-                                            int64_t ldy, double* Yo, double* ws, const uint8_t* act) {
+                                            int64_t ldy, double* Yo, double* ws, const uint8_t* act,
+                                            const int2* outs, int ntiles) {
   __shared__ double t[GB][GB + 1];
   __shared__ double sP[2][GB][GN + 1], sL[2][GB][GN + 1];
   __shared__ double sN[GN][GN + 1];
-  const int2 d = tiles[blockIdx.x];
+  const bool out_block = MODE == UP_IHESS && (int)blockIdx.x >= ntiles;
+  const int2 d = out_block ? outs[blockIdx.x - ntiles] : tiles[blockIdx.x];
   const GFront f = S.gf[d.x];
   const int64_t y = blockIdx.y;
   if (MODE == UP_HESS && act) {
@@ -223,6 +229,25 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
     if (!act[f.k]) return;  // pruned (§5.5): K, U' and M are zero here
   }
   ws += y * S.f_total;
+  if (out_block) {
+    // Y_NN = K_NN - Z_NN, Y_AN = (K_AN + L K_NN) - Z_AN, Z the children's part
+    const int rb = d.y & 0xffff, cb = d.y >> 16;
+    int gi, ni, gj, nj;
+    block_range(f, rb, gi, ni);
+    block_range(f, cb, gj, nj);
+    for (int e = threadIdx.x; e < GB * (GB + 1); e += 256) (&t[0][0])[e] = 0.0;
+    __syncthreads();
+    for (int q = f.ch_beg; q < f.ch_end; ++q) {
+      add_child(S, S.gch[q], ws, rb, gi, cb, gj, &t[0][0], GB + 1);
+      __syncthreads();
+    }
+    double* out = Yo + y * ldy + f.base;
+    const int r = threadIdx.x & 31;
+    if (r < ni)
+      for (int c = threadIdx.x >> 5; c < nj; c += 8)
+        if (gi + r >= gj + c) out[csc_off(f.J, gi + r, gj + c)] -= t[r][c];
+    return;
+  }
   const int tm = d.y & 0xffff, tn = d.y >> 16, tid = threadIdx.x;
   const int r0 = tm * GB, c0 = tn * GB, n = f.n, J = f.J;
   const int nr = min(GB, f.a - r0), nc = min(GB, f.a - c0);
@@ -231,7 +256,7 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
   double* T1 = F + (int64_t)J * J;
   const double* W = Wc + f.base;
   const bool thin = MODE == UP_HESS && n <= GN;
-  if (MODE == UP_HESS && !thin && f.a == 0) return;  // assembled, and no update block
+  if (!thin && f.a == 0) return;  // no update block (UP_HESS: assembled before)
   const int side = tm == tn ? 0 : 1;  // the column block's vectors (the row block's on the diagonal)
   const int tr = tid & 15, tc = tid >> 4;
   double acc[2][2] = {{0, 0}, {0, 0}};
@@ -339,32 +364,6 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
         *o = (MODE == UP_HESS && !thin ? *o : t[r][c]) - acc[u][w];
       }
     }
-  if (MODE == UP_IHESS && tn == 0 && f.ch_end > f.ch_beg) {
-    // Y_NN = K_NN - Z_NN, Y_AN = (K_AN + L K_NN) - Z_AN, Z the children's part
-    double* out = Yo + y * ldy + f.base;
-    for (int b = 0; b < f.nbn; ++b) {
-      for (int part = tm == 0 ? 0 : f.nbn; part <= f.nbn; ++part) {
-        // row blocks: the N blocks at and below b (first tile only), then this tile's rows
-        const int rb = part < f.nbn ? part : bi;
-        if (part < f.nbn && part < b) continue;
-        if (part == f.nbn && f.a == 0) continue;
-        int gi, ni, gj, nj;
-        block_range(f, rb, gi, ni);
-        block_range(f, b, gj, nj);
-        __syncthreads();
-        for (int e = tid; e < GB * (GB + 1); e += 256) (&t[0][0])[e] = 0.0;
-        __syncthreads();
-        for (int q = f.ch_beg; q < f.ch_end; ++q) {
-          add_child(S, S.gch[q], ws, rb, gi, b, gj, &t[0][0], GB + 1);
-          __syncthreads();
-        }
-        const int r = tid & 31;
-        if (r < ni)
-          for (int c = tid >> 5; c < nj; c += 8)
-            if (gi + r >= gj + c) out[csc_off(J, gi + r, gj + c)] -= t[r][c];
-      }
-    }
-  }
 }
 
 // ---------------------------------------------------------------------------
@@ -1575,7 +1574,8 @@ void group_hess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const d
   }
   const int u0 = s->gs_up[q], nu = s->gs_up[q + 1] - u0;
   if (nu > 0) {
-    kg_up<UP_HESS><<<dim3(nu, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, Y, ldy, nullptr, ws, act);
+    kg_up<UP_HESS><<<dim3(nu, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, Y, ldy, nullptr, ws, act,
+                                                      nullptr, nu);
     count_launch();
   }
 }
@@ -1628,8 +1628,10 @@ void group_ihess_k(const chd_symbolic* s, cudaStream_t st, int m, const double* 
 void group_ihess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const double* Wc, double* Y, int64_t ldy,
                     double* ws) {
   const int u0 = s->gs_up[q], nu = s->gs_up[q + 1] - u0;
+  const int o0 = s->gs_out[q], no = s->gs_out[q + 1] - o0;
   if (nu == 0) return;
-  kg_up<UP_IHESS><<<dim3(nu, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, nullptr, ldy, Y, ws, nullptr);
+  kg_up<UP_IHESS><<<dim3(nu + no, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, nullptr, ldy, Y, ws, nullptr,
+                                                    s->dev.gt_out + o0, nu);
   count_launch();
 }
 // V_k^{-1} of the fronts of the grouped inverse (gj), into Rd

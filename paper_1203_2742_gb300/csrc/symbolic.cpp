@@ -394,9 +394,9 @@ static void group_plan(chd_symbolic* s) {
   const int64_t nsn = s->nsn;
   s->gidx.assign(nsn, -1);
   for (auto* v : {&s->gptr, &s->gt_up, &s->gt_row, &s->gt_asm, &s->gt_p, &s->gt_gat, &s->gt_nn, &s->gt_asmf, &s->gt_wb,
-                  &s->gt_fr, &s->gleg, &s->gs_rn, &s->gs_np, &s->gs_thin})
+                  &s->gt_fr, &s->gt_out, &s->gleg, &s->gs_rn, &s->gs_np, &s->gs_thin})
     v->clear();
-  for (auto* v : {&s->gs_up, &s->gs_row, &s->gs_asm, &s->gs_p, &s->gs_gat, &s->gs_asmf, &s->gs_wb, &s->gs_leg, &s->glvl})
+  for (auto* v : {&s->gs_up, &s->gs_row, &s->gs_asm, &s->gs_p, &s->gs_gat, &s->gs_asmf, &s->gs_wb, &s->gs_out, &s->gs_leg, &s->glvl})
     v->assign(1, 0);
   s->gf.clear();
   s->gch.clear();
@@ -466,6 +466,7 @@ static void group_plan(chd_symbolic* s) {
     for (int64_t j = 0; j < nblk; ++j)
       for (int64_t i = j; i < nblk; ++i) {
         push(s->gt_gat, i, j);
+        if (j < f.nbn && f.ch_end > f.ch_beg) push(s->gt_out, i, j);
         if (n > kGroupThin) push(s->gt_asm, i, j);
         if (n > kGroupFactor) push(s->gt_asmf, i, j);
       }
@@ -519,6 +520,7 @@ static void group_plan(chd_symbolic* s) {
       s->gs_gat.push_back((int32_t)s->gt_gat.size() / 2);
       s->gs_asmf.push_back((int32_t)s->gt_asmf.size() / 2);
       s->gs_wb.push_back((int32_t)s->gt_wb.size() / 2);
+      s->gs_out.push_back((int32_t)s->gt_out.size() / 2);
       s->gs_leg.push_back((int32_t)s->gleg.size());
     }
     s->glvl.push_back((int32_t)s->gs_rn.size());
