@@ -260,6 +260,41 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
   const int side = tm == tn ? 0 : 1;  // the column block's vectors (the row block's on the diagonal)
   const int tr = tid & 15, tc = tid >> 4;
   double acc[2][2] = {{0, 0}, {0, 0}};
+  // acc += P L^T + L P^T over jn columns; FP64-bound, so 16 x 16 quarters beyond
+  // the block's rows or above the diagonal are left out (600 fronts of 20 columns and
+  // 40 ancestors, Hessian of eight: 3950 -> 3720 us)
+  auto products = [&](int jn) {
+    auto run = [&](auto row1, auto col1) {  // whether (1, .) and (0, 1) are wanted
+      for (int j = 0; j < jn; ++j) {
+        const double p0 = sP[0][tr][j], l0 = sL[0][tr][j], lc = sL[side][tc][j], pc = sP[side][tc][j];
+        acc[0][0] = fma(p0, lc, acc[0][0]);
+        acc[0][0] = fma(l0, pc, acc[0][0]);
+        if constexpr (row1.value || col1.value) {
+          const double ld = sL[side][tc + 16][j], pd = sP[side][tc + 16][j];
+          if constexpr (col1.value) {
+            acc[0][1] = fma(p0, ld, acc[0][1]);
+            acc[0][1] = fma(l0, pd, acc[0][1]);
+          }
+          if constexpr (row1.value) {
+            const double p1 = sP[0][tr + 16][j], l1 = sL[0][tr + 16][j];
+            acc[1][0] = fma(p1, lc, acc[1][0]);
+            acc[1][0] = fma(l1, pc, acc[1][0]);
+            acc[1][1] = fma(p1, ld, acc[1][1]);
+            acc[1][1] = fma(l1, pd, acc[1][1]);
+          }
+        }
+      }
+    };
+    using yes = std::true_type;
+    using no = std::false_type;
+    if (nr > 16) {
+      if (side) run(yes{}, yes{});
+      else run(yes{}, no{});
+    } else {
+      if (side) run(no{}, yes{});
+      else run(no{}, no{});
+    }
+  };
   for (int e = tid; e < GB * (GB + 1); e += 256) (&t[0][0])[e] = 0.0;
   if (thin) {
     const double* v = Y + y * ldy + f.base;
@@ -319,15 +354,7 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
         if (s == 0 && tn == 0 && r < nr) T1[fi + r + (int64_t)j * J] = x;
       }
     __syncthreads();
-    for (int j = 0; j < n; ++j) {
-#pragma unroll
-      for (int u = 0; u < 2; ++u)
-#pragma unroll
-        for (int w = 0; w < 2; ++w) {
-          acc[u][w] = fma(sP[0][tr + 16 * u][j], sL[side][tc + 16 * w][j], acc[u][w]);
-          acc[u][w] = fma(sL[0][tr + 16 * u][j], sP[side][tc + 16 * w][j], acc[u][w]);
-        }
-    }
+    products(n);
   } else if (f.a > 0) {
     const double* P = MODE == UP_HESS ? T1 : F;
     for (int j0 = 0; j0 < n; j0 += GN) {
@@ -341,16 +368,7 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
         }
       }
       __syncthreads();
-      const int jn = min(GN, n - j0);
-      for (int j = 0; j < jn; ++j) {
-#pragma unroll
-        for (int u = 0; u < 2; ++u)
-#pragma unroll
-          for (int w = 0; w < 2; ++w) {
-            acc[u][w] = fma(sP[0][tr + 16 * u][j], sL[side][tc + 16 * w][j], acc[u][w]);
-            acc[u][w] = fma(sL[0][tr + 16 * u][j], sP[side][tc + 16 * w][j], acc[u][w]);
-          }
-      }
+      products(min(GN, n - j0));
       __syncthreads();
     }
   }
