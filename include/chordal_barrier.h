@@ -250,8 +250,9 @@ chd_status chd_completion_plan(const chd_symbolic* sym, int64_t* nlevels, int64_
  * only on tasks of lower levels.  Level l holds tasks lvl_ptr[l] ..
  * lvl_ptr[l+1]-1 of task_ptr (nlevels+1 entries), in this order: chain runs
  * with |J| <= 32, chain runs with |J| <= 64, warp-tier, wide warp-tier,
- * CTA-tier tasks and dense-tier fronts; lvl_counts[5*l .. 5*l+4] are the
- * counts of those kinds except the CTA tier.  Task q holds the fronts
+ * CTA-tier tasks (chains whose i-th fronts the grouped kernels take together) and
+ * dense-tier fronts; lvl_counts[5*l .. 5*l+4] are the counts of those kinds
+ * except the CTA tier.  Task q holds the fronts
  * task_fronts[task_ptr[q] .. task_ptr[q+1]-1].  For tests and tools.
  * Errors: CHD_ERR_INVALID for NULL arguments.
  */

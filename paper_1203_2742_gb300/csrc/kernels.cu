@@ -1175,12 +1175,7 @@ void warp_ihess_up(const chd_symbolic* s, cudaStream_t st, int t0, int nt, int m
 }  // namespace w32x
 
 
-// Runs body(i, stream, scratch, cap) for the `count` independent big fronts
-// of one level: on the caller's stream if there is one front or no side
-// streams, else round-robin over the side streams, forked after the work
-// already queued on `st` and joined back into `st` at `join_now` (the caller
-// may queue independent work on `st` in between).
-// the last kPostStreams side streams take what no other front waits for (Posts)
+// what a front sequence on stream bs runs with: the caller's stream (j = 0) or side stream j - 1
 static inline Slot exec_slot(const Exec* ex, int j, cudaStream_t bs) {
   Slot sl;
   sl.st = bs;
@@ -1194,6 +1189,12 @@ static inline Slot exec_slot(const Exec* ex, int j, cudaStream_t bs) {
   }
   return sl;
 }
+// Runs body(i, slot) for the `count` independent dense fronts of one level: on
+// the caller's stream if there is one front or no side streams, else round-robin
+// over the side streams (but the last kPostStreams, which take what no other
+// front waits for: Posts), forked after the work already queued on `st` and
+// joined back into `st` at `join_now` (the caller may queue independent work on
+// `st` in between).
 struct BigFork {
   const Exec* ex;
   cudaStream_t st;

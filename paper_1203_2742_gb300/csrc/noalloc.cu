@@ -79,8 +79,9 @@ extern "C" chd_status chd_hessian_noalloc(chd_factor* f, int m, const double* y,
   if (rc != CHD_OK) return rc;
   // Every workspace entry the Hessian passes read is written earlier in the
   // same call, so no clearing is needed between calls.
-  // The dense tier runs on the caller's stream without split-K here (no
-  // scratch beyond the array).
+  // The dense tier runs on the caller's stream without scratch beyond the array:
+  // its products are not split, but those of leaf groups, whose partial sums lie in
+  // the members' own workspace.
   chd_launch::hessian(f->sym, static_cast<cudaStream_t>(stream), nullptr, m, f->Wc, f->Vd, y, ldy, t, ldt, ws);
   const cudaError_t e = cudaGetLastError();
   return e == cudaSuccess ? CHD_OK : CHD_ERR_CUDA;
