@@ -33,6 +33,9 @@ constexpr int kGroupBlock = 32;       // rows per block of the assembly and of t
 constexpr int kGroupThin = 16;        // thin fronts: up to this many columns
 constexpr int kGroupFactor = 32;      // fronts up to this many columns factor in one launch per sub-level
 constexpr int kGroupCols = 256;       // widest front of the tier
+// sub-levels with a front of more children than this use add_children: 40 children gain
+// 7 %, 400 a third, and fronts of few children lose up to 10 % (group_tier.cu)
+constexpr int kManyChildren = 64;
 // the grouped completion ends the N x N part of a front in one CTA from 33 columns
 // on, 0.2 to 0.4 ms up to here; wider ones by the rule at wide_by_sequence
 constexpr int kGroupComplete = 64;
@@ -219,7 +222,7 @@ struct chd_symbolic {
   std::vector<GChild> gch;
   std::vector<int32_t> gptr, gidx, glvl;
   std::vector<int32_t> gt_up, gt_row, gt_asm, gt_p, gt_gat, gt_nn, gt_asmf, gt_wb, gt_fr, gt_out, gleg;
-  std::vector<int32_t> gs_up, gs_row, gs_asm, gs_p, gs_gat, gs_asmf, gs_wb, gs_out, gs_rn, gs_np, gs_thin, gs_leg;
+  std::vector<int32_t> gs_up, gs_row, gs_asm, gs_p, gs_gat, gs_asmf, gs_wb, gs_out, gs_rn, gs_np, gs_thin, gs_many, gs_leg;
   int g_rnmax = 0, g_nmax = 0, g_amax = 0;
   // grouped inverse: fronts by decreasing a, their lower tiles, and per panel
   // of 32 columns the row blocks to solve and the tiles to update

@@ -84,6 +84,79 @@ __device__ __forceinline__ void add_child(const SymDev& S, const GChild& c, cons
     if (i >= j) t[r * ld + (__ldg(rel + j) - fj)] += __ldcg(U + i + (int64_t)j * c.Jc);
 }
 
+// The same for all children of a front that has many.  One child after another behind
+// a barrier each is a chain of dependent loads (record, range, rows, entries), 1.5 us a
+// child.  Here lane r of warp w owns the entries (r, w), (r, w + 8), .. (c < nc) and
+// adds every child to them in order, so no barrier is needed and two children are in
+// flight: the lane of a row finds its place in a child's range by counting the rows
+// before it.  Pruned children (act[k] == 0) are left out 32 at a time.  The caller writes
+// and reads other threads' entries behind barriers of its own.  A root of 20 columns
+// under 2000 children: factor 3210 -> 2010 us, Hessian of eight 3670 -> 2510.  It takes 64
+// registers instead of 40 and costs fronts of few children that much occupancy (20 x 20 x
+// 20 grid, Hessian of eight 37.5 -> 39.6 ms), hence the rule at kManyChildren.
+__device__ __forceinline__ void add_children(const SymDev& S, const GFront& f, const double* ws, const uint8_t* act,
+                                             int bi, int fi, int bj, int fj, double* t, int ld, int nc) {
+  constexpr int CHB = 2;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const unsigned below = (1u << lane) - 1;
+  double x[4];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) x[k] = w + 8 * k < nc ? t[lane * ld + w + 8 * k] : 0.0;
+  for (int q0 = f.ch_beg; q0 < f.ch_end; q0 += 32) {
+    const bool mine = q0 + lane < f.ch_end && (!act || act[S.gch[q0 + lane].k]);
+    unsigned todo = __ballot_sync(0xffffffffu, mine);  // the same in all warps
+    while (todo) {
+      const double* U[CHB];
+      int Jc[CHB], i0[CHB], ni[CHB], j0[CHB], nj[CHB], ri[CHB], rj[CHB];
+#pragma unroll
+      for (int u = 0; u < CHB; ++u) {
+        ni[u] = nj[u] = 0;
+        ri[u] = rj[u] = -1;
+        if (todo) {
+          const GChild c = S.gch[q0 + __ffs(todo) - 1];
+          todo &= todo - 1;
+          const int32_t* ptr = S.gptr + c.ptr_off;
+          i0[u] = __ldg(ptr + bi);
+          ni[u] = __ldg(ptr + bi + 1) - i0[u];
+          j0[u] = __ldg(ptr + bj);
+          nj[u] = __ldg(ptr + bj + 1) - j0[u];
+          const int32_t* rel = S.rel + c.rel_off;
+          if (lane < ni[u]) ri[u] = __ldg(rel + i0[u] + lane) - fi;
+          if (lane < nj[u]) rj[u] = __ldg(rel + j0[u] + lane) - fj;
+          U[u] = ws + c.u_off;
+          Jc[u] = c.Jc;
+        }
+      }
+      double v[CHB][4];
+      bool in[CHB][4];
+#pragma unroll
+      for (int u = 0; u < CHB; ++u) {
+#pragma unroll
+        for (int k = 0; k < 4; ++k) in[u][k] = false;
+        if (ni[u] > 0 && nj[u] > 0) {  // the same for all threads
+          const unsigned mi = __reduce_or_sync(0xffffffffu, ri[u] >= 0 ? 1u << ri[u] : 0u);
+          const unsigned mj = __reduce_or_sync(0xffffffffu, rj[u] >= 0 ? 1u << rj[u] : 0u);
+          const int i = i0[u] + __popc(mi & below);
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int c = w + 8 * k, j = j0[u] + __popc(mj & ((1u << c) - 1));
+            in[u][k] = (mi >> lane & 1) && (mj >> c & 1) && i >= j && c < nc;
+            if (in[u][k]) v[u][k] = __ldcg(U[u] + i + (int64_t)j * Jc[u]);
+          }
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < CHB; ++u)
+#pragma unroll
+        for (int k = 0; k < 4; ++k)
+          if (in[u][k]) x[k] += v[u][k];
+    }
+  }
+#pragma unroll
+  for (int k = 0; k < 4; ++k)
+    if (w + 8 * k < nc) t[lane * ld + w + 8 * k] = x[k];
+}
+
 // the counters of the row-block kernels (last double of T2), before a pass
 __global__ void __launch_bounds__(256) kg_zero(SymDev S, int first, int count, double* ws) {
   const int g = blockIdx.x * 256 + threadIdx.x;
@@ -101,7 +174,8 @@ __global__ void __launch_bounds__(256) kg_zero(SymDev S, int first, int count, d
 //   ASM_FACTOR: as ASM_UP, and D_NN = F_NN
 // ---------------------------------------------------------------------------
 enum { ASM_UP = 0, ASM_GATHER, ASM_FACTOR };
-template <int MODE>
+// MANY: some front of the launch has many children (add_children)
+template <int MODE, bool MANY>
 __global__ void __launch_bounds__(256) kg_assemble(SymDev S, const int2* tiles, const double* Y, int64_t ldy,
                                                   double* ws, const uint8_t* act, double* Dd) {
   __shared__ double t[GB][GB + 1];
@@ -138,11 +212,15 @@ __global__ void __launch_bounds__(256) kg_assemble(SymDev S, const int2* tiles, 
     t[r][c] = r < ni && c < nj && row >= col && col < f.n ? v[csc_off(f.J, row, col)] : 0.0;
   }
   __syncthreads();
-  for (int q = f.ch_beg; q < f.ch_end; ++q) {
-    const GChild c = S.gch[q];
-    if (act && !act[c.k]) continue;  // pruned child (§5.5): its update block is zero
-    add_child(S, c, ws, bi, fi, bj, fj, &t[0][0], GB + 1);
-    __syncthreads();
+  if constexpr (MANY) {
+    add_children(S, f, ws, MODE == ASM_UP ? act : nullptr, bi, fi, bj, fj, &t[0][0], GB + 1, GB);
+  } else {
+    for (int q = f.ch_beg; q < f.ch_end; ++q) {
+      const GChild c = S.gch[q];
+      if (act && !act[c.k]) continue;  // pruned child (§5.5): its update block is zero
+      add_child(S, c, ws, bi, fi, bj, fj, &t[0][0], GB + 1);
+      __syncthreads();
+    }
   }
   if (r < ni)
     for (int c = tid >> 5; c < nj; c += 8) {
@@ -210,16 +288,16 @@ __global__ void __launch_bounds__(256) kg_p(SymDev S, const int2* tiles, const d
 //           block each (fronts with children only).  A CTA walks the children
 //           one by one, so a block per CTA: 400 children of five columns
 //           under one front of 40, one right-hand side: 2020 us with all blocks of the
-//           front's rows in the CTAs of the first tile column, 907 so.
+//           front's rows in the CTAs of the first tile column, 907 so (620 with add_children).
 // ---------------------------------------------------------------------------
 enum { UP_HESS = 0, UP_IHESS = 1 };
-template <int MODE>
+template <int MODE, bool MANY>
 __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const double* Wc, const double* Y,
                                             int64_t ldy, double* Yo, double* ws, const uint8_t* act,
                                             const int2* outs, int ntiles) {
   __shared__ double t[GB][GB + 1];
   __shared__ double sP[2][GB][GN + 1], sL[2][GB][GN + 1];
-  __shared__ double sN[GN][GN + 1];
+  __shared__ double sN[MANY ? GB : GN][GN + 1];  // add_children passes over GB rows
   const bool out_block = MODE == UP_IHESS && (int)blockIdx.x >= ntiles;
   const int2 d = out_block ? outs[blockIdx.x - ntiles] : tiles[blockIdx.x];
   const GFront f = S.gf[d.x];
@@ -237,9 +315,13 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
     block_range(f, cb, gj, nj);
     for (int e = threadIdx.x; e < GB * (GB + 1); e += 256) (&t[0][0])[e] = 0.0;
     __syncthreads();
-    for (int q = f.ch_beg; q < f.ch_end; ++q) {
-      add_child(S, S.gch[q], ws, rb, gi, cb, gj, &t[0][0], GB + 1);
-      __syncthreads();
+    if constexpr (MANY) {
+      add_children(S, f, ws, nullptr, rb, gi, cb, gj, &t[0][0], GB + 1, GB);
+    } else {
+      for (int q = f.ch_beg; q < f.ch_end; ++q) {
+        add_child(S, S.gch[q], ws, rb, gi, cb, gj, &t[0][0], GB + 1);
+        __syncthreads();
+      }
     }
     double* out = Yo + y * ldy + f.base;
     const int r = threadIdx.x & 31;
@@ -314,7 +396,20 @@ __global__ void __launch_bounds__(256) kg_up(SymDev S, const int2* tiles, const 
     }
   }
   __syncthreads();
-  if (thin || MODE == UP_IHESS) {
+  if (MANY && (thin || MODE == UP_IHESS)) {
+    if constexpr (MANY) {
+      const uint8_t* ac = MODE == UP_HESS ? act : nullptr;
+      if (f.a > 0) add_children(S, f, ws, ac, bi, fi, bj, fj, &t[0][0], GB + 1, GB);
+      if (thin) {
+        add_children(S, f, ws, ac, 0, 0, 0, 0, &sN[0][0], GN + 1, GN);
+        if (f.a > 0) {
+          add_children(S, f, ws, ac, bi, fi, 0, 0, &sP[0][0][0], GN + 1, GN);
+          if (side) add_children(S, f, ws, ac, bj, fj, 0, 0, &sP[1][0][0], GN + 1, GN);
+        }
+      }
+      __syncthreads();
+    }
+  } else if (thin || MODE == UP_IHESS) {
     for (int q = f.ch_beg; q < f.ch_end; ++q) {
       const GChild c = S.gch[q];
       if (MODE == UP_HESS && act && !act[c.k]) continue;
@@ -987,6 +1082,7 @@ __global__ void __launch_bounds__(256) kv_product(SymDev S, const int2* tiles, d
 //     rows; then the trailing tiles.
 // ---------------------------------------------------------------------------
 constexpr int GF = kGroupFactor;
+template <bool MANY>
 __global__ void __launch_bounds__(256) kg_factor(SymDev S, const int2* tiles, const double* X, double* Lc, double* Dd,
                                                 double* ws, int64_t* st) {
   __shared__ double t[GB][GB + 1], Ns[GB][GB + 1], Bs[2][GB][GB + 1], rinv[GB], col[3][GB];
@@ -1011,15 +1107,25 @@ __global__ void __launch_bounds__(256) kg_factor(SymDev S, const int2* tiles, co
     }
   }
   __syncthreads();
-  for (int q = f.ch_beg; q < f.ch_end; ++q) {
-    const GChild c = S.gch[q];
-    add_child(S, c, ws, 0, 0, 0, 0, &Ns[0][0], GB + 1);
+  if constexpr (MANY) {
+    add_children(S, f, ws, nullptr, 0, 0, 0, 0, &Ns[0][0], GB + 1, GB);
     if (f.a > 0) {
-      add_child(S, c, ws, bi, fi, bj, fj, &t[0][0], GB + 1);
-      add_child(S, c, ws, bi, fi, 0, 0, &Bs[0][0][0], GB + 1);
-      if (side) add_child(S, c, ws, bj, fj, 0, 0, &Bs[1][0][0], GB + 1);
+      add_children(S, f, ws, nullptr, bi, fi, bj, fj, &t[0][0], GB + 1, GB);
+      add_children(S, f, ws, nullptr, bi, fi, 0, 0, &Bs[0][0][0], GB + 1, GB);
+      if (side) add_children(S, f, ws, nullptr, bj, fj, 0, 0, &Bs[1][0][0], GB + 1, GB);
     }
     __syncthreads();
+  } else {
+    for (int q = f.ch_beg; q < f.ch_end; ++q) {
+      const GChild c = S.gch[q];
+      add_child(S, c, ws, 0, 0, 0, 0, &Ns[0][0], GB + 1);
+      if (f.a > 0) {
+        add_child(S, c, ws, bi, fi, bj, fj, &t[0][0], GB + 1);
+        add_child(S, c, ws, bi, fi, 0, 0, &Bs[0][0][0], GB + 1);
+        if (side) add_child(S, c, ws, bj, fj, 0, 0, &Bs[1][0][0], GB + 1);
+      }
+      __syncthreads();
+    }
   }
   const bool first = tm == 0 && tn == 0;
   if (first)
@@ -1236,6 +1342,7 @@ __global__ void __launch_bounds__(RT) kg_factor_nn(SymDev S, const int2* blocks,
 // so the product G G^T comes first in each CTA.  17 x 20 x 13 grid: 23.1 ms
 // (one CTA per front) before.
 // ---------------------------------------------------------------------------
+template <bool MANY>
 __global__ void __launch_bounds__(256) kg_product(SymDev S, const int2* tiles, const double* Lc, double* Xo,
                                                  double* ws) {
   __shared__ double t[GB][GB + 1], A[GB][GB + 1], B[GB][GB + 1];
@@ -1266,9 +1373,13 @@ __global__ void __launch_bounds__(256) kg_product(SymDev S, const int2* tiles, c
 #pragma unroll
     for (int w = 0; w < 2; ++w) t[tr + 16 * u][tc + 16 * w] = s.v[u][w];
   __syncthreads();
-  for (int q = f.ch_beg; q < f.ch_end; ++q) {
-    add_child(S, S.gch[q], ws, bi, fi, bj, fj, &t[0][0], GB + 1);
-    __syncthreads();
+  if constexpr (MANY) {
+    add_children(S, f, ws, nullptr, bi, fi, bj, fj, &t[0][0], GB + 1, GB);
+  } else {
+    for (int q = f.ch_beg; q < f.ch_end; ++q) {
+      add_child(S, S.gch[q], ws, bi, fi, bj, fj, &t[0][0], GB + 1);
+      __syncthreads();
+    }
   }
   double* F = ws + f.f_off;
   if (r < ni)
@@ -1582,7 +1693,8 @@ void group_hess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const d
                    int64_t ldy, double* ws, const uint8_t* act) {
   const int a0 = s->gs_asm[q], na = s->gs_asm[q + 1] - a0;
   if (na > 0) {
-    kg_assemble<ASM_UP><<<dim3(na, m), 256, 0, st>>>(s->dev, s->dev.gt_asm + a0, Y, ldy, ws, act, nullptr);
+    const auto assemble = s->gs_many[q] ? kg_assemble<ASM_UP, true> : kg_assemble<ASM_UP, false>;
+    assemble<<<dim3(na, m), 256, 0, st>>>(s->dev, s->dev.gt_asm + a0, Y, ldy, ws, act, nullptr);
     count_launch();
   }
   const int p0 = s->gs_p[q], np = s->gs_p[q + 1] - p0;
@@ -1592,8 +1704,8 @@ void group_hess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const d
   }
   const int u0 = s->gs_up[q], nu = s->gs_up[q + 1] - u0;
   if (nu > 0) {
-    kg_up<UP_HESS><<<dim3(nu, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, Y, ldy, nullptr, ws, act,
-                                                      nullptr, nu);
+    const auto up = s->gs_many[q] ? kg_up<UP_HESS, true> : kg_up<UP_HESS, false>;
+    up<<<dim3(nu, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, Y, ldy, nullptr, ws, act, nullptr, nu);
     count_launch();
   }
 }
@@ -1618,7 +1730,7 @@ void group_ihess_gather(const chd_symbolic* s, cudaStream_t st, int q, int m, co
                         double* ws) {
   const int t0 = s->gs_gat[q], nt = s->gs_gat[q + 1] - t0;
   if (nt == 0) return;
-  kg_assemble<ASM_GATHER><<<dim3(nt, m), 256, 0, st>>>(s->dev, s->dev.gt_gat + t0, T, ldt, ws, nullptr, nullptr);
+  kg_assemble<ASM_GATHER, false><<<dim3(nt, m), 256, 0, st>>>(s->dev, s->dev.gt_gat + t0, T, ldt, ws, nullptr, nullptr);
   count_launch();
 }
 // steps 1 and 2 of Algorithm 5.2 over all fronts (K_NN only where none has
@@ -1648,8 +1760,9 @@ void group_ihess_up(const chd_symbolic* s, cudaStream_t st, int q, int m, const 
   const int u0 = s->gs_up[q], nu = s->gs_up[q + 1] - u0;
   const int o0 = s->gs_out[q], no = s->gs_out[q + 1] - o0;
   if (nu == 0) return;
-  kg_up<UP_IHESS><<<dim3(nu + no, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, nullptr, ldy, Y, ws, nullptr,
-                                                    s->dev.gt_out + o0, nu);
+  const auto up = s->gs_many[q] ? kg_up<UP_IHESS, true> : kg_up<UP_IHESS, false>;
+  up<<<dim3(nu + no, m), 256, 0, st>>>(s->dev, s->dev.gt_up + u0, Wc, nullptr, ldy, Y, ws, nullptr, s->dev.gt_out + o0,
+                                       nu);
   count_launch();
 }
 // V_k^{-1} of the fronts of the grouped inverse (gj), into Rd
@@ -1681,7 +1794,8 @@ void group_factor(const chd_symbolic* s, cudaStream_t st, int q, const double* X
                   int64_t* status) {
   const int a0 = s->gs_asmf[q], na = s->gs_asmf[q + 1] - a0;
   if (na > 0) {
-    kg_assemble<ASM_FACTOR><<<na, 256, 0, st>>>(s->dev, s->dev.gt_asmf + a0, X, 0, ws, nullptr, Dd);
+    const auto assemble = s->gs_many[q] ? kg_assemble<ASM_FACTOR, true> : kg_assemble<ASM_FACTOR, false>;
+    assemble<<<na, 256, 0, st>>>(s->dev, s->dev.gt_asmf + a0, X, 0, ws, nullptr, Dd);
     count_launch();
     const int b0 = s->gs_wb[q], nb = s->gs_wb[q + 1] - b0;
     for (int p = 0; p < s->gs_np[q]; ++p) {
@@ -1693,7 +1807,8 @@ void group_factor(const chd_symbolic* s, cudaStream_t st, int q, const double* X
   }
   const int u0 = s->gs_up[q], nu = s->gs_up[q + 1] - u0;
   if (nu > 0 && s->gs_thin[q]) {
-    kg_factor<<<nu, 256, 0, st>>>(s->dev, s->dev.gt_up + u0, X, Lc, Dd, ws, status);
+    const auto factor = s->gs_many[q] ? kg_factor<true> : kg_factor<false>;
+    factor<<<nu, 256, 0, st>>>(s->dev, s->dev.gt_up + u0, X, Lc, Dd, ws, status);
     count_launch();
   }
 }
@@ -1712,7 +1827,8 @@ void group_factor_post(const chd_symbolic* s, cudaStream_t st, const double* Lc,
 void group_product(const chd_symbolic* s, cudaStream_t st, int q, const double* Lc, double* X, double* ws) {
   const int t0 = s->gs_gat[q], nt = s->gs_gat[q + 1] - t0;
   if (nt == 0) return;
-  kg_product<<<nt, 256, 0, st>>>(s->dev, s->dev.gt_gat + t0, Lc, X, ws);
+  const auto product = s->gs_many[q] ? kg_product<true> : kg_product<false>;
+  product<<<nt, 256, 0, st>>>(s->dev, s->dev.gt_gat + t0, Lc, X, ws);
   count_launch();
 }
 // completion of the tier's fronts up to L_AN, and of those of at most 32

@@ -394,7 +394,7 @@ static void group_plan(chd_symbolic* s) {
   const int64_t nsn = s->nsn;
   s->gidx.assign(nsn, -1);
   for (auto* v : {&s->gptr, &s->gt_up, &s->gt_row, &s->gt_asm, &s->gt_p, &s->gt_gat, &s->gt_nn, &s->gt_asmf, &s->gt_wb,
-                  &s->gt_fr, &s->gt_out, &s->gleg, &s->gs_rn, &s->gs_np, &s->gs_thin})
+                  &s->gt_fr, &s->gt_out, &s->gleg, &s->gs_rn, &s->gs_np, &s->gs_thin, &s->gs_many})
     v->clear();
   for (auto* v : {&s->gs_up, &s->gs_row, &s->gs_asm, &s->gs_p, &s->gs_gat, &s->gs_asmf, &s->gs_wb, &s->gs_out, &s->gs_leg, &s->glvl})
     v->assign(1, 0);
@@ -480,6 +480,7 @@ static void group_plan(chd_symbolic* s) {
     }
     if (n > kGroupFactor) s->gs_np.back() = std::max(s->gs_np.back(), f.nbn);
     else s->gs_thin.back() = 1;
+    if (f.ch_end - f.ch_beg > kManyChildren) s->gs_many.back() = 1;
     s->gs_rn.back() = std::max(s->gs_rn.back(), (int32_t)(R * n));
     s->g_rnmax = std::max(s->g_rnmax, (int)(R * n));
     s->g_nmax = std::max(s->g_nmax, (int)n);
@@ -511,6 +512,7 @@ static void group_plan(chd_symbolic* s) {
       s->gs_rn.push_back(0);
       s->gs_np.push_back(0);
       s->gs_thin.push_back(0);
+      s->gs_many.push_back(0);
       for (int64_t k : in) add(k);
       for (int64_t k : out) s->gleg.push_back((int32_t)k);
       s->gs_up.push_back((int32_t)s->gt_up.size() / 2);
